@@ -339,7 +339,7 @@ extern "C" int wsbm_lu_dense(void* A, int64_t lda, int32_t n, int32_t* piv, void
   rc = wsbm_lu_big((double2*)A, lda, n, piv, nullptr, ws, st);
   if (rc == -1) return WSBM_ERR_INVALID_ARG;
   if (rc) return WSBM_ERR_CUDA;
-  rc = wsbm_zgemm_tc_status(st);
+  rc = wsbm_lu_big_status(st);
   return rc == 0 ? WSBM_OK : (rc == -5 ? WSBM_ERR_TIMEOUT : WSBM_ERR_CUDA);
 }
 

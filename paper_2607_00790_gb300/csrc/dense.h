@@ -189,6 +189,8 @@ int wsbm_lu_big(double2* A, int64_t lda, int n, int* piv, int* d_info, void* ws,
 int wsbm_lu_big_nb(double2* A, int64_t lda, int n, int* piv, int* d_info, void* ws, cudaStream_t st, int nb);
 int wsbm_lu_big_large_n();  // n from which the root LU takes the large-class panel width
 size_t wsbm_lu_big_ws_bytes(int n);
+// wsbm_zgemm_tc_status for a large LU: the waits of its panels and of its products.
+int wsbm_lu_big_status(cudaStream_t st);
 int wsbm_trsm_batched(const TrsmDesc* d_desc, int nbatch, int max_n, int max_nrhs, int lower,
                       cudaStream_t st);
 int wsbm_lu_solve_batched(const TrsmDesc* d_desc_lower, const TrsmDesc* d_desc_upper, int nbatch,

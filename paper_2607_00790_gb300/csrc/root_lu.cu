@@ -1,0 +1,449 @@
+// LU with partial pivoting of one large complex matrix (the dense root of a build).
+//
+// Right-looking, outer panels of LUB_NB columns (LUB_NB_BIG for large n, where the deeper
+// tensor-core products pay for the longer panels).  An outer panel is factored recursively by
+// halves down to base panels of at most 32 columns; a base panel is one cooperative launch over
+// the whole GPU (k_lub_panel).  The updates between the halves, U12 = L11^-1 A12 and the
+// trailing update A22 -= L21 U12 run on the tensor cores (wsbm_zgemm_tc).  Factors and piv as
+// for wsbm_lu_batched.  Pivot: the row of largest max(|re|, |im|) compared on the upper 32 bits
+// of its bit pattern (within 2^-20 of the largest), first row on ties.
+#include <algorithm>
+
+#include "cplx.cuh"
+#include "dense.h"
+
+#ifndef LUB_NB
+#define LUB_NB 128      // outer panel width
+#endif
+#ifndef LUB_NB_BIG
+#define LUB_NB_BIG 256  // outer panel width from LUB_BIG_N on: deeper tensor-core products
+#endif
+#ifndef LUB_BIG_N
+#define LUB_BIG_N 12288
+#endif
+#define LUB_W 32            // widest base panel: one lane per column
+#define LUB_T 256           // threads of a base-panel CTA
+#define LUB_MINROWS 32      // fewest rows per CTA (the base panel's pivot rows all start in CTA 0)
+#define LUB_MAXCTA 256      // CTAs a base panel can use (key slots per column)
+#define LUB_SMEM (200 * 1024)
+#define LUB_WAIT_NS 2000000000ull  // bound of every wait (2 s)
+
+static __device__ int g_lub_error;  // set when a bounded wait ran out
+
+__device__ __forceinline__ unsigned long long lub_key(double2 v, int row) {
+  const unsigned long long m = 0x7fffffffffffffffull;
+  const unsigned long long a = (unsigned long long)__double_as_longlong(v.x) & m;
+  const unsigned long long b = (unsigned long long)__double_as_longlong(v.y) & m;
+  const unsigned long long hi = (a > b ? a : b) >> 32;
+  return (hi << 32) | (unsigned long long)(0xFFFFFFFFu - (unsigned)row);
+}
+
+__device__ __forceinline__ unsigned long long lub_warp_max(unsigned long long best) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const unsigned long long x = __shfl_xor_sync(0xFFFFFFFFu, best, o);
+    best = x > best ? x : best;
+  }
+  return best;
+}
+
+__device__ __forceinline__ unsigned long long ld_acquire(const unsigned long long* p) {
+  unsigned long long v;
+  asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
+  return v;
+}
+__device__ __forceinline__ void st_release(unsigned long long* p, unsigned long long v) {
+  asm volatile("st.release.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
+}
+__device__ __forceinline__ unsigned long long lub_time() {
+  unsigned long long t;
+  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
+  return t;
+}
+
+// Base panel: columns [c0, c0 + w) (w <= 32) of rows [c0, n), rows spread over the CTAs of one
+// cooperative launch, R consecutive rows each (R >= w), held in shared memory from the first to
+// the last column.  Per column every CTA publishes its best candidate (key) and that candidate's
+// panel row; every CTA then reads all the keys, takes the winner's row as the pivot row and
+// updates its own rows, so a column costs one exchange through L2 instead of two launches: about
+// 6 us a column at n = 8200 (49 ms in all; the launches per column and their gaps took 100 ms).
+// Bound by that exchange (release, 152 polled keys, one row read); the FP64 work is 1 us of it.
+//   slots  key slots [w][LUB_MAXCTA], zero on entry (a key is never zero)
+//   cand   published rows [2][LUB_MAXCTA][32]; a slot of one parity is rewritten two columns
+//          later, after every CTA has published the column between (and so has read it)
+//   diag   row c as its owner holds it before the swap, [2][32]
+__global__ void __launch_bounds__(LUB_T, 1)
+    k_lub_panel(double2* __restrict__ A, int64_t lda, int n, int c0, int w, int R, unsigned long long* slots,
+                double2* cand, double2* diag, int* __restrict__ piv, int* __restrict__ info) {
+  extern __shared__ double2 sm[];
+  const int RS = R | 1;  // odd stride: a row read across the columns meets no bank twice
+  double2* lcol = sm + (size_t)w * RS;
+  __shared__ double2 prow[LUB_W];
+  __shared__ double2 s_inv;
+  __shared__ unsigned long long red[LUB_T / 32];
+  __shared__ int s_err;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int b = blockIdx.x, G = gridDim.x;
+  const int r0 = c0 + b * R, cnt = min(R, n - r0);
+  for (int e = tid; e < R * w; e += LUB_T) {
+    const int t = e / R, i = e - t * R;
+    if (i < cnt) sm[t * RS + i] = A[(int64_t)(r0 + i) + (int64_t)(c0 + t) * lda];
+  }
+  if (tid == 0) s_err = 0;
+  __syncthreads();
+  unsigned long long best = 0;
+  for (int i = tid; i < cnt; i += LUB_T) {
+    const unsigned long long k = lub_key(sm[i], r0 + i);
+    best = k > best ? k : best;
+  }
+  // rows per pass of the update: threads in groups of `span` rows, the groups over the columns
+  int span = 32;
+  while (span < cnt && span < LUB_T) span *= 2;
+  const int ng = LUB_T / span, g = tid / span, ri = tid - g * span;
+
+  for (int j = 0; j < w; ++j) {
+    const int c = c0 + j, par = j & 1;
+    best = lub_warp_max(best);
+    if (lane == 0) red[warp] = best;
+    __syncthreads();
+    if (warp == 0) {
+      unsigned long long k = lub_warp_max(lane < LUB_T / 32 ? red[lane] : 0ull);
+      const int loc = (int)(0xFFFFFFFFu - (unsigned)k) - r0;
+      double2* mine = cand + ((size_t)par * LUB_MAXCTA + b) * LUB_W;
+      if (lane < w) __stcg(mine + lane, sm[lane * RS + loc]);
+      if (b == 0 && lane < w) __stcg(diag + par * LUB_W + lane, sm[lane * RS + j]);
+      __syncwarp();
+      unsigned long long* row = slots + (size_t)j * LUB_MAXCTA;
+      if (lane == 0) st_release(row + b, k);
+      // all keys of this column (bounded)
+      unsigned long long top = 0;
+      bool ok = true;
+      for (int x = lane; x < G; x += 32) {
+        unsigned long long v = ld_acquire(row + x);
+        if (v == 0) {
+          const unsigned long long t0 = lub_time();
+          for (unsigned it = 1; (v = ld_acquire(row + x)) == 0; ++it) {
+            if ((it & 63) == 0 && (*(volatile int*)&g_lub_error || lub_time() - t0 > LUB_WAIT_NS)) {
+              atomicExch(&g_lub_error, 1);
+              ok = false;
+              break;
+            }
+          }
+        }
+        top = v > top ? v : top;
+      }
+      ok = __all_sync(0xFFFFFFFFu, ok);
+      top = lub_warp_max(top);
+      if (!ok) {
+        if (lane == 0) s_err = 1;
+      } else {
+        const int p = (int)(0xFFFFFFFFu - (unsigned)top), bp = (p - c0) / R;
+        if (lane < w) {
+          const double2 v = __ldcg(cand + ((size_t)par * LUB_MAXCTA + bp) * LUB_W + lane);
+          prow[lane] = v;
+          if (p != c) {
+            if (b == bp) sm[lane * RS + (p - r0)] = __ldcg(diag + par * LUB_W + lane);
+            if (b == 0) sm[lane * RS + j] = v;
+          }
+          if (lane == j) {
+            const bool zero = v.x == 0.0 && v.y == 0.0;
+            s_inv = zero ? make_double2(0.0, 0.0) : cdiv(make_double2(1.0, 0.0), v);
+            if (b == 0) {
+              piv[c] = p;
+              if (zero && info) info[0] = c + 1;
+            }
+          }
+        }
+      }
+    }
+    __syncthreads();
+    if (s_err) return;
+    // rows below c: multipliers, then the rank-1 update of the columns to the right
+    const int first = b == 0 ? j + 1 : 0;
+    const double2 iv = s_inv;
+    for (int i = tid; i < cnt; i += LUB_T)
+      if (i >= first) {
+        const double2 l = cmul(sm[j * RS + i], iv);
+        sm[j * RS + i] = l;
+        lcol[i] = l;
+      }
+    __syncthreads();
+    best = 0;
+    for (int i = ri; i < cnt; i += span) {
+      if (i < first) continue;
+      const double2 l = lcol[i];
+      for (int t = j + 1 + g; t < w; t += ng) {
+        const double2 v = cfms(l, prow[t], sm[t * RS + i]);
+        sm[t * RS + i] = v;
+        if (t == j + 1) {
+          const unsigned long long k = lub_key(v, r0 + i);
+          best = k > best ? k : best;
+        }
+      }
+    }
+  }
+  __syncthreads();
+  for (int e = tid; e < R * w; e += LUB_T) {
+    const int t = e / R, i = e - t * R;
+    if (i < cnt) A[(int64_t)(r0 + i) + (int64_t)(c0 + t) * lda] = sm[t * RS + i];
+  }
+}
+
+// Row interchanges piv[j0 .. j0 + nb) (nb <= 256) on the columns [a0, a1) and [b0, b1).  The nb
+// swaps are turned into one gather per column (at most 2 nb rows move): with a[j] the row whose
+// content sits in row j0 + j just before swap j, row j0 + j receives the content of row piv[j]
+// and a row below the panel the content a[j] of the last swap that names it.  One warp per
+// column, so the top nb rows are read and written contiguously (5 us a call at n = 8200).
+__global__ void __launch_bounds__(256) k_lub_rowswap(double2* __restrict__ A, int64_t lda, int n, int j0, int nb,
+                                                     const int* __restrict__ piv, int a0, int a1, int b0, int b1) {
+  __shared__ int sp[256], ptr[256], src[512], dst[512];
+  const int t = threadIdx.x, lane = t & 31;
+  if (t < nb) {
+    const int p = piv[j0 + t];  // out of range only after a panel that gave up waiting
+    sp[t] = p >= j0 + t && p < n ? p : j0 + t;
+  }
+  __syncthreads();
+  int par = -1, prev = -1;
+  bool last = true;
+  if (t < nb) {
+    for (int i = 0; i < nb; ++i) {
+      const int q = sp[i];
+      if (i < t && q == j0 + t) par = i;
+      if (i < t && q == sp[t]) prev = i;
+      if (i > t && q == sp[t]) last = false;
+    }
+    ptr[t] = par >= 0 ? par : t;
+  }
+  __syncthreads();
+  for (int s = 1; s < nb; s <<= 1) {  // root of each chain by pointer jumping
+    const int v = t < nb ? ptr[ptr[t]] : 0;
+    __syncthreads();
+    if (t < nb) ptr[t] = v;
+    __syncthreads();
+  }
+  if (t < nb) {
+    const int at = j0 + ptr[t];
+    dst[t] = j0 + t;
+    src[t] = sp[t] == j0 + t ? at : (prev >= 0 ? j0 + ptr[prev] : sp[t]);
+    dst[nb + t] = sp[t] >= j0 + nb && last ? sp[t] : -1;
+    src[nb + t] = at;
+  }
+  __syncthreads();
+  const int na = a1 - a0, tot = na + (b1 - b0);
+  for (int q = blockIdx.x * 8 + (t >> 5); q < tot; q += gridDim.x * 8) {
+    double2* col = A + (int64_t)(q < na ? a0 + q : b0 + (q - na)) * lda;
+    double2 v[16];
+#pragma unroll
+    for (int s = 0; s < 16; ++s) {
+      const int e = s * 32 + lane;
+      if (e < 2 * nb && dst[e] >= 0) v[s] = col[src[e]];
+    }
+    __syncwarp();
+#pragma unroll
+    for (int s = 0; s < 16; ++s) {
+      const int e = s * 32 + lane;
+      if (e < 2 * nb && dst[e] >= 0) col[dst[e]] = v[s];
+    }
+  }
+}
+
+// X = L^-1 B for the unit lower triangle L of A[r0 : r0 + nb, r0 : r0 + nb] (nb <= 256), one warp
+// per column, the column spread over the lanes' registers: step t broadcasts x_t and takes
+// column t of L (contiguous) off the rows below (80 us for a 128 x 128 inverse; one thread per
+// column, whose chain of dependent loads bound it, took 1.7 ms).  B: the ncols columns at B (leading dimension
+// ldb), in place; B = NULL: the identity, X into `out` (leading dimension nb).
+__global__ void k_lub_trsm(const double2* __restrict__ A, int64_t lda, int r0, int nb, double2* B, int64_t ldb,
+                           int ncols, double2* __restrict__ out) {
+  const int lane = threadIdx.x & 31, q = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+  if (q >= ncols) return;
+  double2 x[8];
+  double2* col = B ? B + (int64_t)q * ldb : nullptr;
+#pragma unroll
+  for (int s = 0; s < 8; ++s) {
+    const int i = s * 32 + lane;
+    x[s] = i < nb ? (B ? col[i] : make_double2(i == q ? 1.0 : 0.0, 0.0)) : make_double2(0.0, 0.0);
+  }
+  const double2* L = A + r0 + (int64_t)r0 * lda;
+#pragma unroll
+  for (int s = 0; s < 8; ++s) {
+    if (s * 32 >= nb) break;
+    if (!B && s * 32 + 31 < q) continue;  // leading zeros of a column of the inverse
+    const int te = min(32, nb - s * 32);
+#pragma unroll 4
+    for (int tt = 0; tt < te; ++tt) {
+      const double2* lc = L + (int64_t)(s * 32 + tt) * lda;
+      double2 xt;
+      xt.x = __shfl_sync(0xFFFFFFFFu, x[s].x, tt);
+      xt.y = __shfl_sync(0xFFFFFFFFu, x[s].y, tt);
+#pragma unroll
+      for (int s2 = s; s2 < 8; ++s2) {
+        const int i = s2 * 32 + lane;
+        if (s2 * 32 < nb && i < nb && (s2 > s || lane > tt)) x[s2] = cfms(lc[i], xt, x[s2]);
+      }
+    }
+  }
+  double2* o = B ? col : out + (int64_t)q * nb;
+#pragma unroll
+  for (int s = 0; s < 8; ++s) {
+    const int i = s * 32 + lane;
+    if (i < nb) o[i] = x[s];
+  }
+}
+
+namespace {
+struct LubCtx {
+  double2* A;
+  int64_t lda;
+  int n;
+  int* piv;
+  int* info;
+  unsigned long long* slots;  // [LUB_NB_BIG][LUB_MAXCTA], by column of the outer panel
+  double2 *cand, *diag;
+  cudaStream_t st;
+  int cs, ce;  // current outer panel
+  void* tcws;  // work space of the tensor-core products
+};
+
+// columns a base panel can take: every CTA holds its rows of them in shared memory
+int lub_base_width(int n) {
+  const int64_t per = std::max<int64_t>(LUB_MINROWS, (n + wsbm_sm_count() - 1) / wsbm_sm_count()) + 1;
+  for (int w = LUB_W; w > 1; w /= 2)
+    if (per * (w + 1) * (int64_t)sizeof(double2) <= LUB_SMEM) return w;
+  return 1;
+}
+
+int lub_swap(const LubCtx& x, int j0, int nb, int a0, int a1, int b0, int b1) {
+  const int tot = (a1 - a0) + (b1 - b0);
+  if (tot <= 0) return 0;
+  k_lub_rowswap<<<std::min((tot + 7) / 8, wsbm_sm_count() * 4), 256, 0, x.st>>>(x.A, x.lda, x.n, j0, nb, x.piv, a0,
+                                                                               a1, b0, b1);
+  wsbm_count_launch();
+  return 0;
+}
+
+void lub_trsm(const LubCtx& x, int r0, int nb, double2* B, int ncols, double2* out) {
+  const int wpb = ncols > wsbm_sm_count() * 4 ? 4 : 1;
+  k_lub_trsm<<<(ncols + wpb - 1) / wpb, 32 * wpb, 0, x.st>>>(x.A, x.lda, r0, nb, B, x.lda, ncols, out);
+  wsbm_count_launch();
+}
+
+// factor columns [c0, c1) of rows [c0, n); row swaps across the whole outer panel
+int lub_rec(const LubCtx& x, int c0, int c1, int base) {
+  const int w = c1 - c0;
+  if (w <= base) {
+    int rows = x.n - c0, nsm = std::min(wsbm_sm_count(), LUB_MAXCTA);
+    int R = std::max(LUB_MINROWS, (rows + nsm - 1) / nsm);
+    int G = (rows + R - 1) / R, width = w, c = c0;
+    size_t smem = ((size_t)w * (R | 1) + R) * sizeof(double2);
+    if (wsbm_smem_optin((const void*)k_lub_panel, LUB_SMEM) != cudaSuccess) return -3;
+    double2* A = x.A;
+    int64_t lda = x.lda;
+    int n = x.n;
+    unsigned long long* slots = x.slots + (size_t)(c0 - x.cs) * LUB_MAXCTA;
+    double2 *cand = x.cand, *diag = x.diag;
+    int *piv = x.piv, *info = x.info;
+    void* args[] = {&A, &lda, &n, &c, &width, &R, &slots, &cand, &diag, &piv, &info};
+    if (cudaLaunchCooperativeKernel((const void*)k_lub_panel, dim3(G), dim3(LUB_T), args, smem, x.st) != cudaSuccess)
+      return -3;
+    wsbm_count_launch();
+    return lub_swap(x, c0, w, x.cs, c0, c1, x.ce);
+  }
+  const int mid = c0 + ((w / 2 + base - 1) / base) * base;
+  if (int rc = lub_rec(x, c0, mid, base)) return rc;
+  // A[c0:mid, mid:c1] = L11^-1 A[c0:mid, mid:c1];  A[mid:n, mid:c1] -= A[mid:n, c0:mid] A[c0:mid, mid:c1]
+  lub_trsm(x, c0, mid - c0, x.A + c0 + (int64_t)mid * x.lda, c1 - mid, nullptr);
+  const double2 mone = make_double2(-1.0, 0.0), one = make_double2(1.0, 0.0);
+  if (int rc = wsbm_zgemm_tc(x.n - mid, c1 - mid, mid - c0, mone, x.A + mid + (int64_t)c0 * x.lda, x.lda,
+                             x.A + c0 + (int64_t)mid * x.lda, x.lda, one, x.A + mid + (int64_t)mid * x.lda, x.lda,
+                             x.tcws, x.st))
+    return rc;
+  return lub_rec(x, mid, c1, base);
+}
+
+// work space behind the products' planes: key slots, published rows, L11^-1
+size_t lub_layout(int n, size_t* o_slots, size_t* o_cand, size_t* o_inv) {
+  size_t b = (wsbm_zgemm_tc_ws_bytes(n, n, LUB_NB_BIG) + 255) & ~(size_t)255;  // either panel width fits
+  *o_slots = b;
+  b += (size_t)LUB_NB_BIG * LUB_MAXCTA * sizeof(unsigned long long);
+  *o_cand = b;
+  b += (size_t)2 * (LUB_MAXCTA + 1) * LUB_W * sizeof(double2);
+  *o_inv = b;
+  return b + (size_t)LUB_NB_BIG * LUB_NB_BIG * sizeof(double2) + 256;
+}
+}  // namespace
+
+int wsbm_lu_big_large_n() { return LUB_BIG_N; }
+
+// outer panel width: the tuned one of n's size class (LUB_NB / LUB_NB_BIG by default)
+static int lub_nb(int n) {
+  const WsbmTune t = wsbm_tune_current();
+  return n >= LUB_BIG_N ? t.root_nb_large : t.root_nb_mid;
+}
+
+size_t wsbm_lu_big_ws_bytes(int n) {
+  size_t a, b, c;
+  return lub_layout(n, &a, &b, &c);
+}
+
+int wsbm_lu_big(double2* A, int64_t lda, int n, int* piv, int* d_info, void* ws, cudaStream_t st) {
+  return wsbm_lu_big_nb(A, lda, n, piv, d_info, ws, st, lub_nb(n));
+}
+
+int wsbm_lu_big_nb(double2* A, int64_t lda, int n, int* piv, int* d_info, void* ws, cudaStream_t st, int nb) {
+  if (n <= 0) return 0;
+  if (!A || !piv || !ws || lda < n || ((uintptr_t)ws & 255)) return -1;
+  if (nb != LUB_NB && nb != LUB_NB_BIG) return -1;
+  size_t o_slots, o_cand, o_inv;
+  lub_layout(n, &o_slots, &o_cand, &o_inv);
+  double2* Linv = (double2*)((char*)ws + o_inv);
+  LubCtx x;
+  x.A = A;
+  x.lda = lda;
+  x.n = n;
+  x.piv = piv;
+  x.info = d_info;
+  x.slots = (unsigned long long*)((char*)ws + o_slots);
+  x.cand = (double2*)((char*)ws + o_cand);
+  x.diag = x.cand + (size_t)2 * LUB_MAXCTA * LUB_W;
+  x.st = st;
+  x.tcws = ws;
+  const int base = lub_base_width(n);
+  const double2 mone = make_double2(-1.0, 0.0), one = make_double2(1.0, 0.0), zero = make_double2(0.0, 0.0);
+  for (int j0 = 0; j0 < n; j0 += nb) {
+    const int jb = std::min(nb, n - j0), je = j0 + jb;
+    x.cs = j0;
+    x.ce = je;
+    if (cudaMemsetAsync(x.slots, 0, (size_t)jb * LUB_MAXCTA * sizeof(unsigned long long), st) != cudaSuccess)
+      return -3;
+    if (int rc = lub_rec(x, j0, je, base)) return rc;
+    lub_swap(x, j0, jb, 0, j0, je, n);
+    if (je < n) {
+      // U12 = L11^-1 A12 as a tensor-core product with the explicit inverse of the unit lower
+      // L11 (the digit planes of A12 are formed before A12 is overwritten)
+      const int m = n - je;
+      lub_trsm(x, j0, jb, nullptr, jb, Linv);
+      if (int rc = wsbm_zgemm_tc(jb, m, jb, one, Linv, jb, A + j0 + (int64_t)je * lda, lda, zero,
+                                 A + j0 + (int64_t)je * lda, lda, ws, st))
+        return rc;
+      if (int rc = wsbm_zgemm_tc(m, m, jb, mone, A + je + (int64_t)j0 * lda, lda, A + j0 + (int64_t)je * lda, lda,
+                                 one, A + je + (int64_t)je * lda, lda, ws, st))
+        return rc;
+    }
+  }
+  return cudaGetLastError() == cudaSuccess ? 0 : -3;
+}
+
+// Error flags of the bounded waits of the panel and of its products: reads and clears both
+// (synchronizes the stream).
+int wsbm_lu_big_status(cudaStream_t st) {
+  const int rc = wsbm_zgemm_tc_status(st);
+  if (rc == -3) return rc;
+  int v = 0;
+  if (cudaMemcpyFromSymbol(&v, g_lub_error, sizeof(int)) != cudaSuccess) return -3;
+  if (v) {
+    const int z = 0;
+    cudaMemcpyToSymbol(g_lub_error, &z, sizeof(int));
+    return -5;
+  }
+  return rc;
+}
