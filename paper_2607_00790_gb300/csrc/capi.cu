@@ -8,6 +8,7 @@
 #include <utility>
 
 #include "wsbm_internal.h"
+#include "hankel.cuh"
 
 static std::atomic<int64_t> g_launches{0};
 void wsbm_count_launch() { g_launches.fetch_add(1, std::memory_order_relaxed); }
@@ -170,7 +171,29 @@ int wsbm_phys_from_params(const wsbm_params* p, Phys* ph) {
   ph->finv_k0 = (float)ph->inv_k0;
   ph->feps0 = (float)ph->eps0;
   ph->feps1 = (float)ph->eps1;
-  ph->fpad = 0.0f;
+  {
+    const double kmin = fmin(ph->k0, ph->k1), kmax = fmax(ph->k0, ph->k1);
+    const double lo = HX_Z_LO / kmin, hi = HX_Z_HI / kmax, fr = HX_Z_FAR / kmin;
+    const double lo2 = lo * lo, hi2 = hi * hi;
+    uint64_t bl, bh;
+    memcpy(&bl, &lo2, 8);
+    memcpy(&bh, &hi2, 8);
+    ph->fix_lo = (int32_t)(bl >> 32);
+    ph->fix_hi = (int32_t)(bh >> 32);
+    // a wavenumber so extreme that r^2 leaves the normal range takes the general path
+    if (!(lo2 > 1e-290) || !(hi2 < 1e290)) ph->fix_lo = INT32_MAX;
+    ph->near_r2 = (float)lo2;
+    ph->far_r2 = (float)(fr * fr);
+    const double a0 = WSBM_SQRT_2_OVER_PI, a1 = a0 * ph->s01, n = ph->k1 / ph->k0;
+    ph->c_v = 0.25 * ph->k0 * a0;
+    ph->c_d0 = 0.25 * a0;
+    ph->c_d1 = 0.25 * n * a1;
+    ph->c_c1 = 0.25 * ph->k1 * n * a1;
+    ph->c_s11 = 0.25 * ph->k1 * a1;
+    ph->c_s12 = -0.25 * eps1 * a1;
+    ph->c_e0 = 0.25 * eps0 * a0;
+    ph->c_u1 = 0.25 * n * eps1 * a1;
+  }
   return WSBM_OK;
 }
 

@@ -14,9 +14,12 @@
 
 #include "entry_blocks.cuh"
 
+#define PAIR_CLASSES 4  // far, middle, near, diagonal (k_pairs)
+
 struct SlotData {
   double x, y, nx, ny, w, kap;
   float fnx, fny, fw;  // FP32 copies for the mixed-precision algebra
+  float fx, fy;        // and for the grouping of the pairs
   int32_t node, p0, p1;
 };
 
@@ -46,6 +49,8 @@ __device__ __forceinline__ void load_slot(const DevGeom& g, const int32_t* nodes
   s.fnx = (float)s.nx;
   s.fny = (float)s.ny;
   s.fw = (float)s.w;
+  s.fx = (float)s.x;
+  s.fy = (float)s.y;
   s.p0 = pos[2 * t];
   s.p1 = pos[2 * t + 1];
 }
@@ -54,13 +59,14 @@ __device__ __forceinline__ void load_slot(const DevGeom& g, const int32_t* nodes
 // other (TF a power of two, 16..64).
 template <int TF>
 __global__ void __launch_bounds__(WSBM_PAIR_THREADS)
-    k_pairs(DevGeom g0, Phys ph0, const PairTask* __restrict__ tasks, int ntasks, int64_t ntiles,
+    k_pairs(DevGeom g0, const __grid_constant__ Phys ph0, const PairTask* __restrict__ tasks, int ntasks, int64_t ntiles,
             const DevGeom* __restrict__ geos, const Phys* __restrict__ phys) {
   constexpr int TS = WSBM_PAIR_THREADS / TF;
   __shared__ HkTables T;
   __shared__ SlotData sf[TF];
   __shared__ SlotData ss[TS];
-  __shared__ int s_cnt[WSBM_PAIR_THREADS / 32][3];
+  __shared__ Phys ph;  // of the tile's curve (shared memory: FP64 operands, not registers)
+  __shared__ int s_cnt[WSBM_PAIR_THREADS / 32][PAIR_CLASSES];
   __shared__ int16_t s_list[WSBM_PAIR_THREADS];
   __shared__ int s_ntot;
   hk_stage_tables(&T);
@@ -71,7 +77,6 @@ __global__ void __launch_bounds__(WSBM_PAIR_THREADS)
     int ti = find_task_by_tile(&tasks[0].tile0, stride, ntasks, tile);
     const PairTask tk = tasks[ti];
     const DevGeom g = geos ? geos[tk.inst] : g0;
-    const Phys ph = phys ? phys[tk.inst] : ph0;
     const bool fc = tk.fastc != 0;
     const int nf = fc ? tk.nc : tk.nr;
     const int ns = fc ? tk.nr : tk.nc;
@@ -80,6 +85,8 @@ __global__ void __launch_bounds__(WSBM_PAIR_THREADS)
     const int f0 = (int)(lt % nft) * TF;
     const int s0 = (int)(lt / nft) * TS;
     __syncthreads();  // previous tile done with the staged slots (and tables staged)
+    if (threadIdx.x < sizeof(Phys) / 4)
+      reinterpret_cast<int32_t*>(&ph)[threadIdx.x] = reinterpret_cast<const int32_t*>(phys ? phys + tk.inst : &ph0)[threadIdx.x];
     if (threadIdx.x < TF) {
       int f = f0 + threadIdx.x;
       if (f < nf) {
@@ -100,40 +107,37 @@ __global__ void __launch_bounds__(WSBM_PAIR_THREADS)
     }
     __syncthreads();
     // Group the tile's pairs by evaluation path before evaluating them: far pairs (both
-    // Hankel arguments on the large-argument branch), near pairs (at least one ascending
-    // series) and diagonal pairs (one-point correction).  Threads then take pairs from the
-    // grouped list, so a warp mixes paths only at a group boundary instead of wherever the
-    // diagonal band crosses the tile.  (The grouping only orders work; any pair may be
-    // evaluated by any thread.)
-    int cls = 3;  // 3: outside the task
+    // arguments beyond 20), middle pairs (both in fixed point), near pairs (at least one ascending series) and
+    // diagonal pairs (one-point correction).  Threads then take pairs from the grouped list, so
+    // a warp mixes paths only at a group boundary.  (The grouping only orders work, so FP32
+    // coordinates are enough for it: any pair may be evaluated by any thread.)
+    int cls = PAIR_CLASSES;  // outside the task
     {
       const int f = f0 + tx, s = s0 + ty;
       if (f < nf && s < ns) {
         const SlotData& R = fc ? ss[ty] : sf[tx];
         const SlotData& C = fc ? sf[tx] : ss[ty];
         if (R.node == C.node) {
-          cls = 2;
+          cls = 3;
         } else {
-          // near: min(k0, k1) r < HK_Z_SERIES, compared on r^2 (no square root)
-          const double dx = R.x - C.x, dy = R.y - C.y;
-          const double rz = HK_Z_SERIES * fmax(ph.inv_k0, ph.inv_k1);
-          cls = fma(dx, dx, dy * dy) < rz * rz ? 1 : 0;
+          const float dx = R.fx - C.fx, dy = R.fy - C.fy, r2 = fmaf(dx, dx, dy * dy);
+          cls = r2 < ph.near_r2 ? 2 : (r2 < ph.far_r2 ? 1 : 0);
         }
       }
     }
     {
       const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
       const unsigned lt = (1u << lane) - 1u;
-      unsigned bal[3];
+      unsigned bal[PAIR_CLASSES];
 #pragma unroll
-      for (int c = 0; c < 3; ++c) {
+      for (int c = 0; c < PAIR_CLASSES; ++c) {
         bal[c] = __ballot_sync(0xffffffffu, cls == c);
         if (lane == 0) s_cnt[warp][c] = __popc(bal[c]);
       }
       __syncthreads();
       int base = 0, pos = -1;
 #pragma unroll
-      for (int c = 0; c < 3; ++c) {
+      for (int c = 0; c < PAIR_CLASSES; ++c) {
         int before = 0, total = 0;
 #pragma unroll
         for (int w = 0; w < WSBM_PAIR_THREADS / 32; ++w) {
@@ -156,9 +160,7 @@ __global__ void __launch_bounds__(WSBM_PAIR_THREADS)
       if (R.node == C.node) {
         block_diag(ph, R.w, R.kap, e);
       } else {
-        PairGeom G;
-        pair_geom(R.x, R.y, R.nx, R.ny, C.x, C.y, C.nx, C.ny, ph, G);
-        block_offdiag(T, ph, G, C.w, e);
+        pair_block(T, ph, R.x, R.y, R.nx, R.ny, C.x, C.y, C.nx, C.ny, C.w, e);
       }
       const int rp[2] = {R.p0, R.p1};
       const int cp[2] = {C.p0, C.p1};

@@ -61,6 +61,83 @@ __device__ __forceinline__ void block_offdiag(const HkTables& T, const Phys& ph,
                          wj * (-0.25 * ph.eps0 * a.h0r - u * vi));
 }
 
+// r^2 of a pair in the fixed operation order (no contraction).
+__device__ __forceinline__ double pair_r2(double dx, double dy) {
+  return __dadd_rn(__dmul_rn(dx, dx), __dmul_rn(dy, dy));
+}
+__device__ __forceinline__ bool pair_is_fixed(const Phys& ph, double r2) {
+  const int h = __double2hiint(r2);
+  return h > ph.fix_lo && h < ph.fix_hi;
+}
+
+// 1/sqrt(x) to about an ulp for normal x: hardware seed (23 bits) and one third-order step.
+__device__ __forceinline__ double rsqrt3(double x) {
+  double y;
+  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+  const double e = fma(-(x * y), y, 1.0);
+  return fma(y * e, fma(e, 0.375, 0.5), y);
+}
+
+// The same for any x > 0 (subnormal and infinite ones through the library function).
+__device__ __forceinline__ double rsqrt3_any(double x) {
+  const int h = __double2hiint(x);
+  return h >= 0x00100000 && h < 0x7FF00000 ? rsqrt3(x) : rsqrt(x);
+}
+
+// sqrt(x), correctly rounded, from y = 1/sqrt(x): x y plus half its residual times y.
+__device__ __forceinline__ double sqrt_from(double x, double y) {
+  const double r = x * y;
+  return fma(fma(-r, r, x), __hiloint2double(__double2hiint(y) - 0x100000, __double2loint(y)), r);
+}
+
+// Off-diagonal block of a pair with both arguments in the range of hankel_fixed.  Same formulas
+// as block_offdiag, with three savings on the FP64 pipe, which bounds every pair kernel (one
+// FP64 instruction costs as much issue time as 64 others): the Hankel values come from the
+// integer pipe; r (correctly rounded) and 1/r share one reciprocal
+// square root; and the amplitudes sqrt(2/(pi k r)) and every constant are folded into eight real
+// factors of the unit-amplitude values, so that an entry is two to five multiply-adds.  The
+// 1/(k r)^2 poles of F1 cancel in N_k0 - N_k1 and are left out (at z >= 1.5 they are no larger than
+// the values they stand beside).
+// 71 FP64 instructions where the general path takes about 185.
+__device__ __forceinline__ void block_fixed(const HkTables& T, const Phys& ph, double dx, double dy, double r2, double nxi, double nyi,
+                                          double nxj, double nyj, double wj, double2 e[2][2]) {
+  const double ir = rsqrt3(r2);
+  const double r = sqrt_from(r2, ir);
+  const double z0 = __dmul_rn(ph.k0, r), z1 = __dmul_rn(ph.k1, r);
+  HxUnit a, b;
+  hankel_fixed(T.near_, z0, ir * ph.inv_k0, a);
+  hankel_fixed(T.near_, z1, ir * ph.inv_k1, b);
+  const double dny = __dadd_rn(__dmul_rn(dx, nxj), __dmul_rn(dy, nyj)) * ir;
+  const double dnx = __dadd_rn(__dmul_rn(dx, nxi), __dmul_rn(dy, nyi)) * ir;
+  const double nn = __dadd_rn(__dmul_rn(nxi, nxj), __dmul_rn(nyi, nyj));
+  const double c = dnx * dny, m2c = fma(-2.0, c, nn);
+  const double w0 = wj * rsqrt3(z0);
+  const double v0 = w0 * ph.c_v, t0 = v0 * dny, c0 = v0 * c;  // t1 H1(z0), k0 H0(z0) c
+  const double mr = w0 * m2c * ir, d0 = mr * ph.c_d0, d1 = mr * ph.c_d1;
+  const double c1 = w0 * c * ph.c_c1;
+  const double s11 = w0 * dny * ph.c_s11, s12 = w0 * ph.c_s12;
+  const double e0 = w0 * ph.c_e0, u0 = e0 * dnx, u1 = w0 * dnx * ph.c_u1;
+  e[0][0] = make_double2(-s11 * b.i1, s11 * b.r1);
+  e[0][1] = make_double2(-s12 * b.i0, s12 * b.r0);
+  e[1][0] = make_double2(fma(-t0, a.i1, fma(-c0, a.r0, fma(-d0, a.r1, fma(c1, b.r0, d1 * b.r1)))),
+                         fma(t0, a.r1, fma(-c0, a.i0, fma(-d0, a.i1, fma(c1, b.i0, d1 * b.i1)))));
+  e[1][1] = make_double2(fma(e0, a.i0, fma(-u0, a.r1, u1 * b.r1)), fma(-e0, a.r0, fma(-u0, a.i1, u1 * b.i1)));
+}
+
+// Off-diagonal block of target (xi, yi, nxi, nyi) and source (xj, yj, nxj, nyj, wj).
+__device__ __forceinline__ void pair_block(const HkTables& T, const Phys& ph, double xi, double yi, double nxi,
+                                           double nyi, double xj, double yj, double nxj, double nyj, double wj,
+                                           double2 e[2][2]) {
+  const double dx = __dsub_rn(xi, xj), dy = __dsub_rn(yi, yj), r2 = pair_r2(dx, dy);
+  if (pair_is_fixed(ph, r2)) {
+    block_fixed(T, ph, dx, dy, r2, nxi, nyi, nxj, nyj, wj, e);
+  } else {
+    PairGeom G;
+    pair_geom(xi, yi, nxi, nyi, xj, yj, nxj, nyj, ph, G);
+    block_offdiag(T, ph, G, wj, e);
+  }
+}
+
 // Diagonal 2x2 block: one-point corrected trapezoidal rule.  A kernel a ln|x-y| + b gets the
 // weight w_i [a ln(w_i/2pi) + b(x_i, x_i)]; D and D* tend to -kappa/(4 pi).
 __device__ __forceinline__ void block_diag(const Phys& ph, double wi, double kap, double2 e[2][2]) {

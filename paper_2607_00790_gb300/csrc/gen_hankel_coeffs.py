@@ -4,10 +4,11 @@ The evaluator writes, for z >= Z_SERIES,
     H_nu(z) = sqrt(2/(pi z)) (P_nu(z) + i Q_nu(z)) exp(i (z - pi/4 - nu pi/2)),   nu = 0, 1,
 which defines the real functions P_nu, Q_nu exactly (P -> 1, Q -> 0 as z -> infinity).
 
-* Z_SERIES <= z < Z_ASYM: P_nu - 1 and Q_nu on the intervals BOUNDS are polynomials of degree
-  DEG in s = (u - c)/h, u = 1/z (c, h: centre and half-width of the interval in u), obtained by
+* Z_SERIES <= z < Z_ASYM: P_nu - 1 and Q_nu on the intervals BOUNDS are polynomials in
+  s = (u - c)/h, u = 1/z (c, h: centre and half-width of the interval in u), obtained by
   interpolation at Chebyshev points in 50-digit arithmetic (mpmath).  In u the functions are far
-  smoother than in z (degree 10 instead of 16 for the same accuracy).
+  smoother than in z (degree 10 instead of 16 for the same accuracy).  The FP64 evaluator takes
+  these arguments in fixed point (gen_hankel_fixed.py); only the FP32 table is written.
 * z >= Z_ASYM: P_nu - 1 and z Q_nu as polynomials of degree DEG_T in s = (t - c)/h, t = 1/z^2 on
   [0, 1/Z_ASYM^2], interpolated the same way (their values at t = 0 follow the Hankel asymptotic
   expansion, A&S 9.2.5-9.2.10: P -> 1, z Q -> (4 nu^2 - 1)/8).
@@ -215,7 +216,7 @@ def main():
     L = ["// Generated by gen_hankel_coeffs.py -- do not edit.",
          f"// max abs error (emulated): P,Q FP64 {errs[0]:.2e}, FP32 {errs[1]:.2e}; sin {errs[2]:.2e}, cos {errs[3]:.2e}",
          f"#define HK_Z_SERIES {Z_SERIES!r}", f"#define HK_Z_ASYM {Z_ASYM!r}", f"#define HK_NIV {nv}",
-         f"#define HK_DEG {DEG}", f"#define HK_DEG_T {DEG_T}", f"#define HK_NSER {N_SERIES}",
+         f"#define HK_DEG_T {DEG_T}", f"#define HK_NSER {N_SERIES}",
          f"#define HK_DEG_SC {DEG_SC}", f"#define HKF_DEG {DEG_F}", f"#define HKF_DEG_T {DEG_TF}", ""]
     # interval i covers [BOUNDS[i], BOUNDS[i+1]); high 32-bit words of the inner bounds
     import struct
@@ -230,14 +231,6 @@ def main():
     L.append("static __device__ const double hk_iv[HK_NIV][2] = {")
     for (a, b, c, ih) in mids:
         L.append(f"  {{{fmt(c)}, {fmt(ih)}}},  // z in [{a}, {b})")
-    L.append("};")
-    L.append("// fits[iv][fn][k], fn = P0-1, Q0, P1-1, Q1")
-    L.append("static __device__ const double hk_fit[HK_NIV][4][HK_DEG + 1] = {")
-    for row in fits:
-        L.append("  {")
-        for cf in row:
-            L.append("    {" + ", ".join(fmt(v) for v in cf) + "},")
-        L.append("  },")
     L.append("};")
     L.append(f"#define HK_T_C {fmt(tc)}")
     L.append(f"#define HK_T_IH {fmt(tih)}")

@@ -5,15 +5,13 @@
 // instructions per argument:
 //   z < 1.5     ascending series in z^2/4 (A&S 9.1.10, 9.1.11, 9.1.13); the 1/z pole of Y1 is kept
 //               apart so F1 = H1/z + 2i/(pi z^2) is formed without cancellation;
-//   z >= 1.5    H_nu = sqrt(2/(pi z)) (P_nu + i Q_nu) e^{i(z - pi/4 - nu pi/2)};
-//               P_nu - 1, Q_nu are degree-10 polynomials in u = 1/z on seven intervals up to
-//               z = 20 (the functions are smooth in 1/z), and degree-6 polynomials in 1/z^2
-//               beyond (P_nu - 1 and z Q_nu), evaluated there in two-float (hi + lo FP32)
-//               arithmetic on the FP32 pipe: they are small corrections, so 48 significant
-//               bits give them an absolute error below 1e-17;
-//   phase       z - pi/4 is reduced by multiples of pi/2 (Cody-Waite with a two-part pi/2 and
-//               fused multiply-adds) and sin/cos of the remainder |w| <= pi/4 come from fitted
-//               polynomials, so no rounding of z - pi/4 enters the phase.
+//   z >= 1.5    H_nu = sqrt(2/(pi z)) (P_nu + i Q_nu) e^{i(z - pi/4 - nu pi/2)}, the phase factor,
+//               P_nu and Q_nu in 64-bit fixed point on the integer pipe (hankel_fixed.cuh): about
+//               9 FP64 operations an argument;
+//   z >= 2^20   the same in FP64: degree-6 polynomials in 1/z^2 in two-float (hi + lo FP32)
+//               arithmetic (absolute error below 1e-17), z - pi/4 reduced by multiples of pi/2
+//               (Cody-Waite with a two-part pi/2 and fused multiply-adds), sin/cos of the
+//               remainder |w| <= pi/4 from fitted polynomials.
 // The interval is chosen by comparing the high 32-bit word of z as an integer (integer pipe).
 // All coefficients are fitted by gen_hankel_coeffs.py (50-digit arithmetic) and checked there.
 //
@@ -27,12 +25,17 @@
 #include <stdint.h>
 
 #include "hankel_coeffs.inc"
+#include "hankel_fixed.cuh"
 
 #define WSBM_PI 3.14159265358979323846
 #define WSBM_2_OVER_PI 0.63661977236758134308
 #define WSBM_SQRT_2_OVER_PI 0.79788456080286535588
 #define WSBM_INV_SQRT2 0.70710678118654752440
 #define WSBM_EULER 0.57721566490153286061
+
+static __device__ const int64_t hx_near_c[HX_NIV][4][HX_DEG_N + 1] = HX_NEAR;
+static __device__ const uint64_t hx_near_lo[HX_NIV] = HX_NEAR_LO;
+static __device__ const int32_t hx_near_sh[HX_NIV] = HX_NEAR_SH;
 
 struct Hk {
   double h0r, h0i, h1r, h1i, f1r, f1i;
@@ -45,8 +48,7 @@ struct HkF {
 // Coefficient tables staged in shared memory by every kernel that evaluates Hankel values
 // (divergent interval indices within a warp would serialise constant-bank reads).
 struct HkTables {
-  double iv[HK_NIV][2];
-  double fit[HK_NIV][4][HK_DEG + 1];
+  HxNear near_;
   double asy[4][HK_DEG_T + 1];
   double ser[4][HK_NSER];
   double sn[HK_DEG_SC + 1];
@@ -63,8 +65,9 @@ __device__ __forceinline__ void hk_copy(T* dst, const T* src, int n) {
 }
 
 __device__ __forceinline__ void hk_stage_tables(HkTables* t) {
-  hk_copy(&t->iv[0][0], &hk_iv[0][0], HK_NIV * 2);
-  hk_copy(&t->fit[0][0][0], &hk_fit[0][0][0], HK_NIV * 4 * (HK_DEG + 1));
+  hk_copy(&t->near_.c[0][0][0], &hx_near_c[0][0][0], HX_NIV * 4 * (HX_DEG_N + 1));
+  hk_copy(t->near_.lo, hx_near_lo, HX_NIV);
+  hk_copy(t->near_.sh, hx_near_sh, HX_NIV);
   hk_copy(&t->asy[0][0], &hk_asy[0][0], 4 * (HK_DEG_T + 1));
   hk_copy(&t->ser[0][0], &hk_ser[0][0], 4 * HK_NSER);
   hk_copy(t->sn, hk_sin, HK_DEG_SC + 1);
@@ -189,31 +192,20 @@ __device__ __forceinline__ void hk_series(const HkTables& T, double z, double iz
   o.f1i = y1h * iz;
 }
 
-// P_nu - 1 (pm0, pm1) and Q_nu for z >= HK_Z_SERIES, u = 1/z.
-__device__ __forceinline__ void hk_pq(const HkTables& T, int zhi, double u, double* pm0,
-                                      double* Q0, double* pm1, double* Q1) {
-  if (zhi < HK_ASYM_HI) {
-    int iv = hk_interval_hi(zhi);
-    double s = (u - T.iv[iv][0]) * T.iv[iv][1];
-    *pm0 = hk_horner<HK_DEG + 1>(T.fit[iv][0], s);
-    *Q0 = hk_horner<HK_DEG + 1>(T.fit[iv][1], s);
-    *pm1 = hk_horner<HK_DEG + 1>(T.fit[iv][2], s);
-    *Q1 = hk_horner<HK_DEG + 1>(T.fit[iv][3], s);
-  } else {
-    // z >= 20: P - 1 (|.| < 4e-4) and z Q in two-float arithmetic on the FP32 pipe; the
-    // absolute error of P and Q stays below 1e-17
-    const double s = (u * u - HK_T_C) * HK_T_IH;
-    const float sh = __double2float_rn(s), sl = __double2float_rn(s - f2d_exact(sh));
-    float h, l;
-    hk_asy_ff(T, 0, sh, sl, &h, &l);
-    *pm0 = f2d_exact(h) + f2d_exact(l);
-    hk_asy_ff(T, 1, sh, sl, &h, &l);
-    *Q0 = u * (f2d_exact(h) + f2d_exact(l));
-    hk_asy_ff(T, 2, sh, sl, &h, &l);
-    *pm1 = f2d_exact(h) + f2d_exact(l);
-    hk_asy_ff(T, 3, sh, sl, &h, &l);
-    *Q1 = u * (f2d_exact(h) + f2d_exact(l));
-  }
+// P_nu - 1 (pm0, pm1) and Q_nu for z >= 20, u = 1/z: P - 1 (|.| < 4e-4) and z Q in two-float
+// arithmetic on the FP32 pipe; the absolute error of P and Q stays below 1e-17.
+__device__ __forceinline__ void hk_pq(const HkTables& T, double u, double* pm0, double* Q0, double* pm1, double* Q1) {
+  const double s = (u * u - HK_T_C) * HK_T_IH;
+  const float sh = __double2float_rn(s), sl = __double2float_rn(s - f2d_exact(sh));
+  float h, l;
+  hk_asy_ff(T, 0, sh, sl, &h, &l);
+  *pm0 = f2d_exact(h) + f2d_exact(l);
+  hk_asy_ff(T, 1, sh, sl, &h, &l);
+  *Q0 = u * (f2d_exact(h) + f2d_exact(l));
+  hk_asy_ff(T, 2, sh, sl, &h, &l);
+  *pm1 = f2d_exact(h) + f2d_exact(l);
+  hk_asy_ff(T, 3, sh, sl, &h, &l);
+  *Q1 = u * (f2d_exact(h) + f2d_exact(l));
 }
 
 // P_nu - 1 and Q_nu from the FP32 tables (amplitude-only mixed precision, WSBM_MIXED_FINE):
@@ -256,13 +248,26 @@ __device__ __forceinline__ void hankel_fp64_rs(const HkTables& T, double z, doub
     return;
   }
   double A = WSBM_SQRT_2_OVER_PI * rs;
+  if (!PQ32 && zhi < HX_Z_HI_WORD) {
+    HxUnit h;
+    hankel_fixed(T.near_, z, u, h);
+    o.h0r = A * h.r0;
+    o.h0i = A * h.i0;
+    o.h1r = A * h.r1;
+    o.h1i = A * h.i1;
+    if (WITH_F1) {
+      o.f1r = o.h1r * u;
+      o.f1i = fma(WSBM_2_OVER_PI * u, u, o.h1i * u);
+    }
+    return;
+  }
   double E, F;
   hk_phase(T, z, &E, &F);
   double pm0, Q0, pm1, Q1;
   if (PQ32)
     hk_pq_f32(T, zhi, u, &pm0, &Q0, &pm1, &Q1);
   else
-    hk_pq(T, zhi, u, &pm0, &Q0, &pm1, &Q1);
+    hk_pq(T, u, &pm0, &Q0, &pm1, &Q1);
   double P0 = fma(A, pm0, A), AQ0 = A * Q0;
   double P1 = fma(A, pm1, A), AQ1 = A * Q1;
   o.h0r = fma(P0, E, -AQ0 * F);

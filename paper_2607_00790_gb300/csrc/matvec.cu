@@ -72,13 +72,9 @@ __global__ void __launch_bounds__(MV_THREADS)
       if (jc + jj == i) {
         block_diag(ph, wi, ki, e);
       } else if (!TRANS) {  // block (i, j): row node i, column node j
-        PairGeom G;
-        pair_geom(xi, yi, nxi, nyi, s.x, s.y, s.nx, s.ny, ph, G);
-        block_offdiag(T, ph, G, s.w, e);
+        pair_block(T, ph, xi, yi, nxi, nyi, s.x, s.y, s.nx, s.ny, s.w, e);
       } else {  // block (j, i), applied transposed
-        PairGeom G;
-        pair_geom(s.x, s.y, s.nx, s.ny, xi, yi, nxi, nyi, ph, G);
-        block_offdiag(T, ph, G, wi, e);
+        pair_block(T, ph, s.x, s.y, s.nx, s.ny, xi, yi, nxi, nyi, wi, e);
       }
       if (TRANS) {
         double2 t = e[0][1];

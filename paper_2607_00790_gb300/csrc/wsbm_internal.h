@@ -18,7 +18,13 @@ struct Phys {
   double inv_k0, inv_k1;  // 1/k0, 1/k1
   double s01, s10;        // sqrt(k0/k1), sqrt(k1/k0): 1/sqrt(k1 r) = s01/sqrt(k0 r)
   // FP32 copies for the mixed-precision kernels
-  float fk0, fk1, frk0, frk1, finv_k0, feps0, feps1, fpad;  // frk = 1/sqrt(k)
+  float fk0, fk1, frk0, frk1, finv_k0, feps0, feps1;  // frk = 1/sqrt(k)
+  // node pairs by r^2: both arguments on the fixed-point evaluator (fix_lo < high word < fix_hi),
+  // and the FP32 bounds by which the entry kernel groups its pairs (any ascending series, far)
+  float near_r2, far_r2;
+  int32_t fix_lo, fix_hi;
+  // scalar factors of the block (entry_blocks.cuh)
+  double c_v, c_d0, c_d1, c_c1, c_s11, c_s12, c_e0, c_u1;
 };
 
 // One output block of node-pair entries of the WSBM matrix.  A row "slot" t names row node
