@@ -11,56 +11,121 @@
 
 #include <algorithm>
 
-#include "hankel.cuh"
+#include "entry_blocks.cuh"
 #include "wsbm_internal.h"
 
 namespace {
 
 #define FLD_THREADS 128
-#define FLD_RHS 4  // right-hand sides per launch (Hankel values shared by all of them)
 
 struct FldSlot {
-  double x, y, nx, ny, w, pad;
+  double x, y, nx, ny, w;
 };
 
-// side[t] = 1 inside, 0 outside (one thread per target, all sources)
-__global__ void k_field_side(DevGeom g, const double* __restrict__ tx, const double* __restrict__ ty,
-                             int64_t nt, int8_t* __restrict__ side) {
-  __shared__ FldSlot sj[FLD_THREADS];
+// ---- side of the targets.  The Gauss sum is 0 or 1 up to the quadrature error, so FP32 decides
+// it nearly everywhere: coordinate differences from (hi, lo) FP32 pairs, sums of 128 terms in FP32,
+// the sums of those in FP64.  A target whose sum lies within FLD_SIDE_EPS sum_j w_j/r_j of the
+// threshold (every rounding error above is below a tenth of that), or that meets a node closer than
+// FP32 resolves, is summed again in FP64.  0.1 ms for 3001 targets and 16384 nodes, where one FP64
+// thread per target took 10.4 ms.
+#define FLD_SIDE_EPS 1e-4f
+struct SideSlot {
+  float xh, xl, yh, yl, nx, ny, w;
+};
+
+__global__ void __launch_bounds__(FLD_THREADS)
+    k_field_side(DevGeom g, const double* __restrict__ tx, const double* __restrict__ ty, int64_t nt, int64_t jspan,
+                 double2* __restrict__ part) {
+  __shared__ SideSlot sj[FLD_THREADS];
   const int64_t t = (int64_t)blockIdx.x * FLD_THREADS + threadIdx.x;
   const double px = t < nt ? tx[t] : 0.0, py = t < nt ? ty[t] : 0.0;
-  double acc = 0.0;
-  for (int64_t jc = 0; jc < g.n; jc += FLD_THREADS) {
+  const float pxh = (float)px, pyh = (float)py, pxl = (float)(px - (double)pxh), pyl = (float)(py - (double)pyh);
+  const int64_t j0 = (int64_t)blockIdx.y * jspan, j1 = min(g.n, j0 + jspan);
+  double acc = 0.0, mag = 0.0;
+  for (int64_t jc = j0; jc < j1; jc += FLD_THREADS) {
     __syncthreads();
-    int64_t j = jc + threadIdx.x;
-    if (j < g.n) {
-      sj[threadIdx.x].x = g.x[j];
-      sj[threadIdx.x].y = g.y[j];
-      sj[threadIdx.x].nx = g.nx[j];
-      sj[threadIdx.x].ny = g.ny[j];
-      sj[threadIdx.x].w = g.w[j];
+    const int64_t j = jc + threadIdx.x;
+    if (j < j1) {
+      SideSlot& s = sj[threadIdx.x];
+      const double x = g.x[j], y = g.y[j];
+      s.xh = (float)x;
+      s.xl = (float)(x - (double)s.xh);
+      s.yh = (float)y;
+      s.yl = (float)(y - (double)s.yh);
+      s.nx = (float)g.nx[j];
+      s.ny = (float)g.ny[j];
+      s.w = (float)g.w[j];
     }
     __syncthreads();
-    const int nj = (int)min((int64_t)FLD_THREADS, g.n - jc);
+    const int nj = (int)min((int64_t)FLD_THREADS, j1 - jc);
+    float a = 0.0f, m = 0.0f;
     for (int jj = 0; jj < nj; ++jj) {
-      const FldSlot& s = sj[jj];
-      const double dx = px - s.x, dy = py - s.y;
-      const double r2 = dx * dx + dy * dy;
-      if (r2 > 0.0) acc += s.w * (dx * s.nx + dy * s.ny) / r2;
+      const SideSlot& s = sj[jj];
+      const float dx = (pxh - s.xh) + (pxl - s.xl), dy = (pyh - s.yh) + (pyl - s.yl);
+      const float r2 = fmaf(dx, dx, dy * dy);
+      const float ir = rsqrtf(r2);  // infinite at r2 = 0: the FP64 sum decides
+      const float wr = s.w * ir;
+      a = fmaf(wr * ir, fmaf(dx, s.nx, dy * s.ny), a);
+      m += fabsf(wr);
     }
+    acc += (double)a;
+    mag += (double)m;
   }
-  if (t < nt) side[t] = (-acc / (2.0 * WSBM_PI)) > 0.5 ? 1 : 0;
+  if (t < nt) part[(int64_t)blockIdx.y * nt + t] = make_double2(acc, mag);
 }
 
-// Partial sums over the sources [j0, j1) of CTA row blockIdx.y, for FLD_RHS right-hand sides
-// starting at column c0.  part: nsplit x nt x FLD_RHS complex128.
+// side[t] = 1 inside, 0 outside
 __global__ void __launch_bounds__(FLD_THREADS)
-    k_field(DevGeom g, Phys ph, const double2* __restrict__ u, const double2* __restrict__ q, int nrhs,
-            int c0, const double* __restrict__ tx, const double* __restrict__ ty, int64_t nt,
+    k_field_side_finish(DevGeom g, const double* __restrict__ tx, const double* __restrict__ ty, int64_t nt,
+                        int nsplit, const double2* __restrict__ part, int8_t* __restrict__ side) {
+  __shared__ double red[FLD_THREADS];
+  __shared__ int unsure[FLD_THREADS];
+  const int64_t t0 = (int64_t)blockIdx.x * FLD_THREADS, t = t0 + threadIdx.x;
+  double acc = 0.0, mag = 0.0;
+  if (t < nt)
+    for (int p = 0; p < nsplit; ++p) {
+      const double2 v = part[(int64_t)p * nt + t];
+      acc += v.x;
+      mag += v.y;
+    }
+  const double off = fabs(acc + WSBM_PI);  // 2 pi |sum - 1/2|
+  const bool sure = off > (double)FLD_SIDE_EPS * mag;  // false for infinities and NaN
+  unsure[threadIdx.x] = t < nt && !sure;
+  if (t < nt && sure) side[t] = (-acc / (2.0 * WSBM_PI)) > 0.5 ? 1 : 0;
+  __syncthreads();
+  for (int q = 0; q < FLD_THREADS; ++q) {
+    if (!unsure[q]) continue;
+    const double px = tx[t0 + q], py = ty[t0 + q];
+    double s = 0.0;
+    for (int64_t j = threadIdx.x; j < g.n; j += FLD_THREADS) {
+      const double dx = px - g.x[j], dy = py - g.y[j];
+      const double r2 = dx * dx + dy * dy;
+      if (r2 > 0.0) s += g.w[j] * (dx * g.nx[j] + dy * g.ny[j]) / r2;
+    }
+    red[threadIdx.x] = s;
+    __syncthreads();
+    for (int h = FLD_THREADS / 2; h > 0; h >>= 1) {
+      if (threadIdx.x < h) red[threadIdx.x] += red[threadIdx.x + h];
+      __syncthreads();
+    }
+    if (threadIdx.x == 0) side[t0 + q] = (-red[0] / (2.0 * WSBM_PI)) > 0.5 ? 1 : 0;
+    __syncthreads();
+  }
+}
+
+// Partial sums over the sources [j0, j1) of CTA row blockIdx.y, for the nc <= NR right-hand sides
+// starting at column c0.  part: nsplit x nt x NR complex128.  Bound by the FP64 pipe: 31 operations
+// a pair (Hankel values in fixed point, one reciprocal square root each for 1/r and the amplitude,
+// the side's signs and constants folded into two factors) and 8 per right-hand side.  16384 nodes, 3001
+// targets, 8 columns: 8.4 ms (25 ms in two launches of 4 columns with FP64 Hankel values).
+template <int NR>
+__global__ void __launch_bounds__(FLD_THREADS)
+    k_field(DevGeom g, Phys ph, const double2* __restrict__ u, const double2* __restrict__ q, int nc, int c0,
+            const double* __restrict__ tx, const double* __restrict__ ty, int64_t nt,
             const int8_t* __restrict__ side, int64_t jspan, double2* __restrict__ part) {
   __shared__ HkTables T;
   __shared__ FldSlot sj[FLD_THREADS];
-  __shared__ double2 su[FLD_RHS][FLD_THREADS], sq[FLD_RHS][FLD_THREADS];
+  __shared__ double2 su[NR][FLD_THREADS], sq[NR][FLD_THREADS];
   hk_stage_tables(&T);
   const int64_t N = g.n;
   const int64_t t = (int64_t)blockIdx.x * FLD_THREADS + threadIdx.x;
@@ -68,11 +133,13 @@ __global__ void __launch_bounds__(FLD_THREADS)
   const bool valid = t < nt;
   const double px = valid ? tx[t] : 0.0, py = valid ? ty[t] : 0.0;
   const bool in = valid && side[t] != 0;
-  const double k = in ? ph.k1 : ph.k0;
-  const int nc = min(FLD_RHS, nrhs - c0);
-  double2 acc[FLD_RHS];
+  const double k = in ? ph.k1 : ph.k0, ik = in ? ph.inv_k1 : ph.inv_k0;
+  // w G = (i w/4) H0, times eps1 inside, -eps0 outside;  w dG/dn_y = (i k w/4) H1 (d.n)/r, times
+  // -1 inside, 1 outside
+  const double ea = 0.25 * (in ? ph.eps1 : -ph.eps0), eb = (in ? -0.25 : 0.25) * k;
+  double2 acc[NR];
 #pragma unroll
-  for (int c = 0; c < FLD_RHS; ++c) acc[c] = make_double2(0.0, 0.0);
+  for (int c = 0; c < NR; ++c) acc[c] = make_double2(0.0, 0.0);
   for (int64_t jc = j0; jc < j1; jc += FLD_THREADS) {
     __syncthreads();
     {
@@ -85,7 +152,7 @@ __global__ void __launch_bounds__(FLD_THREADS)
         s.ny = g.ny[j];
         s.w = g.w[j];
 #pragma unroll
-        for (int c = 0; c < FLD_RHS; ++c) {
+        for (int c = 0; c < NR; ++c) {
           su[c][threadIdx.x] = c < nc ? u[(int64_t)(c0 + c) * N + j] : make_double2(0.0, 0.0);
           sq[c][threadIdx.x] = c < nc ? q[(int64_t)(c0 + c) * N + j] : make_double2(0.0, 0.0);
         }
@@ -100,44 +167,50 @@ __global__ void __launch_bounds__(FLD_THREADS)
       asm volatile("" ::: "memory");
       const FldSlot& s = sj[jj];
       const double dx = px - s.x, dy = py - s.y;
-      const double r2 = fma(dx, dx, dy * dy);
+      const double r2 = pair_r2(dx, dy);
       if (r2 == 0.0) continue;
-      const double rs = rsqrt(r2);  // 1/r
-      const double r = r2 * rs;
-      const double z = k * r;
-      Hk h;
-      hankel_fp64_rs<false>(T, z, rsqrt(z), h);
-      // w G = (i w/4) H0;  w dG/dn_y = (i k w/4) H1 (d.n)/r
-      const double sg = 0.25 * s.w, sd = 0.25 * s.w * k * (dx * s.nx + dy * s.ny) * rs;
-      const double2 G = make_double2(-sg * h.h0i, sg * h.h0r);
-      const double2 D = make_double2(-sd * h.h1i, sd * h.h1r);
-      const double ea = in ? ph.eps1 : -ph.eps0;  // coefficient of S[q]
-      const double eb = in ? -1.0 : 1.0;          // coefficient of D[u]
+      const double rs = rsqrt3_any(r2);  // 1/r
+      const double z = k * sqrt_from(r2, rs);
+      const double dn = fma(dx, s.nx, dy * s.ny) * rs;
+      const int zhi = __double2hiint(z);
+      double2 G, D;
+      if (zhi >= HK_SERIES_HI && zhi < HX_Z_HI_WORD) {
+        HxUnit h;
+        hankel_fixed(T.near_, z, rs * ik, h);
+        const double wa = s.w * (WSBM_SQRT_2_OVER_PI * rsqrt3(z));
+        const double sg = ea * wa, sd = eb * wa * dn;
+        G = make_double2(-sg * h.i0, sg * h.r0);
+        D = make_double2(-sd * h.i1, sd * h.r1);
+      } else {
+        Hk h;
+        hankel_fp64_rs<false>(T, z, rsqrt(z), h);
+        const double sg = ea * s.w, sd = eb * s.w * dn;
+        G = make_double2(-sg * h.h0i, sg * h.h0r);
+        D = make_double2(-sd * h.h1i, sd * h.h1r);
+      }
 #pragma unroll
-      for (int c = 0; c < FLD_RHS; ++c) {
+      for (int c = 0; c < NR; ++c) {
         const double2 uu = su[c][jj], qq = sq[c][jj];
-        acc[c].x += ea * (G.x * qq.x - G.y * qq.y) + eb * (D.x * uu.x - D.y * uu.y);
-        acc[c].y += ea * (G.x * qq.y + G.y * qq.x) + eb * (D.x * uu.y + D.y * uu.x);
+        acc[c].x = fma(G.x, qq.x, fma(-G.y, qq.y, fma(D.x, uu.x, fma(-D.y, uu.y, acc[c].x))));
+        acc[c].y = fma(G.x, qq.y, fma(G.y, qq.x, fma(D.x, uu.y, fma(D.y, uu.x, acc[c].y))));
       }
     }
   }
   if (valid) {
 #pragma unroll
-    for (int c = 0; c < FLD_RHS; ++c)
-      part[((int64_t)blockIdx.y * nt + t) * FLD_RHS + c] = acc[c];
+    for (int c = 0; c < NR; ++c) part[((int64_t)blockIdx.y * nt + t) * NR + c] = acc[c];
   }
 }
 
-__global__ void k_field_reduce(int64_t nt, int nsplit, int nrhs, int c0,
-                               const double2* __restrict__ part, double2* __restrict__ out) {
-  const int nc = min(FLD_RHS, nrhs - c0);
+__global__ void k_field_reduce(int64_t nt, int nsplit, int nc, int nr, int c0, const double2* __restrict__ part,
+                               double2* __restrict__ out) {
   for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < nt * nc;
        e += (int64_t)gridDim.x * blockDim.x) {
     const int64_t t = e / nc;
     const int c = (int)(e % nc);
     double2 s = make_double2(0.0, 0.0);
     for (int p = 0; p < nsplit; ++p) {
-      double2 v = part[((int64_t)p * nt + t) * FLD_RHS + c];
+      double2 v = part[((int64_t)p * nt + t) * nr + c];
       s.x += v.x;
       s.y += v.y;
     }
@@ -169,28 +242,35 @@ extern "C" int wsbm_field(const wsbm_geom* g, const wsbm_params* p, const void* 
   cudaStream_t st = (cudaStream_t)stream;
   const int64_t N = g->n;
   const int64_t nti = (nt + FLD_THREADS - 1) / FLD_THREADS;
-  int nsm = wsbm_sm_count(), per_sm = 1;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_field, FLD_THREADS, 0) != cudaSuccess ||
-      per_sm < 1)
-    per_sm = 1;
-  int64_t want = (int64_t)nsm * per_sm * 8;  // about eight waves, at least 128 sources a CTA
+  const int nr = nrhs > 4 ? 8 : (nrhs > 2 ? 4 : nrhs);  // right-hand sides per launch
+  const int per_sm = nr == 8 ? 2 : 4;                   // resident CTAs per SM
+  // about eight waves (four of the 8-column kernel, whose partial sums are twice as wide), at least
+  // 128 sources a CTA
+  const int64_t want = (int64_t)wsbm_sm_count() * per_sm * (nr == 8 ? 4 : 8);
   int64_t nsplit = std::max<int64_t>(1, std::min<int64_t>((want + nti - 1) / nti, (N + 127) / 128));
-  const int64_t jspan = (N + nsplit - 1) / nsplit;
+  const int64_t jspan = ((N + nsplit - 1) / nsplit + FLD_THREADS - 1) / FLD_THREADS * FLD_THREADS;
   nsplit = (N + jspan - 1) / jspan;
   WsbmScratch scr(st);
   double2* part = nullptr;
-  if ((rc = scr.get((size_t)nsplit * nt * FLD_RHS * sizeof(double2), (void**)&part))) return rc;
+  if ((rc = scr.get((size_t)nsplit * nt * nr * sizeof(double2), (void**)&part))) return rc;
   DevGeom dg = wsbm_devgeom(g);
-  k_field_side<<<(unsigned)nti, FLD_THREADS, 0, st>>>(dg, tx, ty, nt, inside);
-  wsbm_count_launch();
-  for (int c0 = 0; c0 < nrhs; c0 += FLD_RHS) {
-    k_field<<<dim3((unsigned)nti, (unsigned)nsplit), FLD_THREADS, 0, st>>>(
-        dg, ph, (const double2*)u, (const double2*)q, nrhs, c0, tx, ty, nt, inside, jspan, part);
-    wsbm_count_launch();
-    k_field_reduce<<<grid_cap((nt * FLD_RHS + 255) / 256), 256, 0, st>>>(nt, (int)nsplit, nrhs, c0,
-                                                                         part, (double2*)out);
-    wsbm_count_launch();
+  const dim3 grid((unsigned)nti, (unsigned)nsplit);
+  k_field_side<<<grid, FLD_THREADS, 0, st>>>(dg, tx, ty, nt, jspan, part);
+  k_field_side_finish<<<(unsigned)nti, FLD_THREADS, 0, st>>>(dg, tx, ty, nt, (int)nsplit, part, inside);
+  wsbm_count_launches(2);
+  const double2 *cu = (const double2*)u, *cq = (const double2*)q;
+  for (int c0 = 0; c0 < nrhs; c0 += nr) {
+    const int nc = std::min(nr, nrhs - c0);
+    if (nr == 8)
+      k_field<8><<<grid, FLD_THREADS, 0, st>>>(dg, ph, cu, cq, nc, c0, tx, ty, nt, inside, jspan, part);
+    else if (nr == 4)
+      k_field<4><<<grid, FLD_THREADS, 0, st>>>(dg, ph, cu, cq, nc, c0, tx, ty, nt, inside, jspan, part);
+    else if (nr == 2)
+      k_field<2><<<grid, FLD_THREADS, 0, st>>>(dg, ph, cu, cq, nc, c0, tx, ty, nt, inside, jspan, part);
+    else
+      k_field<1><<<grid, FLD_THREADS, 0, st>>>(dg, ph, cu, cq, nc, c0, tx, ty, nt, inside, jspan, part);
+    k_field_reduce<<<grid_cap((nt * nc + 255) / 256), 256, 0, st>>>(nt, (int)nsplit, nc, nr, c0, part, (double2*)out);
+    wsbm_count_launches(2);
   }
-  rc = cudaGetLastError() == cudaSuccess ? WSBM_OK : WSBM_ERR_CUDA;
-  return rc;
+  return cudaGetLastError() == cudaSuccess ? WSBM_OK : WSBM_ERR_CUDA;
 }
