@@ -541,6 +541,7 @@ __global__ void __launch_bounds__(LUS_T) k_lu_solve_fused(const LuSolveDesc* __r
 #ifndef CPQR_TPC_MAXM
 #define CPQR_TPC_MAXM 2048
 #endif
+#define CPQR_CLUSTER_SMEM (192 * 1024)  // longest reflector of the cluster variant (12288 rows)
 // Warp variant: CB trailing columns per warp per pass (2*CB partial sums, a power of two <= 16).
 template <bool TPC, int CB>
 __global__ void __launch_bounds__(256, CPQR_MINB) k_cpqr(const QrDesc* __restrict__ d, int mode) {
@@ -783,6 +784,213 @@ __global__ void __launch_bounds__(256, CPQR_MINB) k_cpqr(const QrDesc* __restric
   }
 }
 
+// One matrix per cluster of CTAs, for batches too small to fill the GPU with one CTA per matrix
+// (the upper tree levels: few boxes, the largest matrices).  The trailing columns are dealt to
+// the warps of the whole cluster, CB at a time.  Every CTA finds the pivot from the norms in
+// global memory by itself and stages the pivot column as the reflector in its own shared memory,
+// so a step costs two cluster barriers: one between that staging and the update (which overwrites
+// the pivot's slot with column j), one after the update (the ID of the 16384-node star, 64 to 256
+// matrices a level: 257 -> 88 ms).  The reflectors are not kept (only R and
+// the trailing matrix are read later): column j's rows below j stay as they are.
+__device__ __forceinline__ void cluster_sync_all() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
+template <int CB>
+__global__ void __launch_bounds__(256, 3) k_cpqr_cluster(const QrDesc* __restrict__ d, int mode) {
+  constexpr int SH = CB == 1 ? 4 : CB == 2 ? 3 : CB == 4 ? 2 : 1;  // 5 - log2(2 * CB)
+  extern __shared__ double2 su[];  // the reflector u = (column p)[j : m]
+  uint32_t rank, csize;
+  asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
+  asm("mov.u32 %0, %%cluster_nctarank;" : "=r"(csize));
+  const QrDesc q = d[blockIdx.x / csize];
+  const int m = q.m, n = q.n;
+  double2* M = q.A;
+  const int64_t ld = q.lda;
+  const int tid = threadIdx.x, lane = tid & 31, nw = blockDim.x >> 5;
+  const int gw = (int)rank * nw + (tid >> 5), gn = (int)csize * nw;  // this warp and all warps of the cluster
+  __shared__ double sval[8], ssum[8];
+  __shared__ int sidx[8];
+  __shared__ double s_tau;
+  __shared__ double2 s_beta;
+  const int kmax = min(m, n);
+  int j = q.state[0];  // resume point
+  if (j == 0) {
+    for (int c = gw; c < n; c += gn) {
+      double s = 0.0;
+      for (int i = lane; i < m; i += 32) s += cabs2(M[i + (int64_t)c * ld]);
+      for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+      if (lane == 0) {
+        q.norm2[c] = s;
+        q.nref[c] = s;
+        q.perm[c] = c;
+      }
+    }
+  }
+  cluster_sync_all();
+  const int kt = mode == 1 ? min(q.kt, kmax) : kmax;
+  for (; j < kt; ++j) {
+    // pivot: largest remaining norm (lowest index on ties)
+    double best = -1.0;
+    int p = j;
+    for (int c = j + tid; c < n; c += blockDim.x) {
+      const double v = __ldcg(q.norm2 + c);
+      if (v > best) {
+        best = v;
+        p = c;
+      }
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      const double ob = __shfl_xor_sync(0xffffffffu, best, o);
+      const int oi = __shfl_xor_sync(0xffffffffu, p, o);
+      if (ob > best || (ob == best && oi < p)) {
+        best = ob;
+        p = oi;
+      }
+    }
+    if (lane == 0) {
+      sval[tid >> 5] = best;
+      sidx[tid >> 5] = p;
+    }
+    __syncthreads();
+    best = sval[0];
+    p = sidx[0];
+    for (int w = 1; w < nw; ++w)
+      if (sval[w] > best || (sval[w] == best && sidx[w] < p)) {
+        best = sval[w];
+        p = sidx[w];
+      }
+    const double nrm = sqrt(fmax(best, 0.0));
+    if (j == 0 && rank == 0 && tid == 0) q.rdiag0[0] = nrm;
+    const double r00 = j == 0 ? nrm : __ldcg(q.rdiag0);
+    if (mode == 0 && (nrm <= q.tol * r00 || nrm == 0.0)) break;  // the same in every CTA
+    // reflector from x = column p; |x| recomputed exactly
+    const int mm = m - j;
+    double s = 0.0;
+    for (int i = tid; i < mm; i += blockDim.x) {
+      const double2 v = __ldcg(M + j + i + (int64_t)p * ld);
+      su[i] = v;
+      s += cabs2(v);
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if (lane == 0) ssum[tid >> 5] = s;
+    __syncthreads();
+    if (tid == 0) {
+      double t = 0.0;
+      for (int w = 0; w < nw; ++w) t += ssum[w];
+      const double xn = sqrt(t);
+      const double2 x0 = su[0];
+      const double a0 = sqrt(cabs2(x0));
+      const double2 beta = a0 > 0.0 ? make_double2(-x0.x / a0 * xn, -x0.y / a0 * xn) : make_double2(-xn, 0.0);
+      su[0] = make_double2(x0.x - beta.x, x0.y - beta.y);
+      const double uu = 2.0 * xn * (xn + a0);  // u^H u = 2 |x| (|x| + |x0|)
+      s_tau = uu > 0.0 ? 2.0 / uu : 0.0;
+      s_beta = beta;
+    }
+    cluster_sync_all();
+    const double tau = s_tau;
+    if (rank == 0 && tid == 0) {
+      q.tauv[j] = tau;
+      q.betav[j] = s_beta;
+      if (p != j) {
+        const int t = q.perm[j];
+        q.perm[j] = q.perm[p];
+        q.perm[p] = t;
+      }
+    }
+    // P applied to the trailing columns; slot p takes column j (the interchange)
+    for (int c0 = j + 1 + gw * CB; c0 < n; c0 += gn * CB) {
+      const int nc = min(CB, n - c0);
+      const double2* src[CB];
+#pragma unroll
+      for (int v = 0; v < CB; ++v) src[v] = M + j + (int64_t)(c0 + v == p ? j : (v < nc ? c0 + v : c0)) * ld;
+      double acc[2 * CB];  // re of the CB columns, then im
+#pragma unroll
+      for (int v = 0; v < 2 * CB; ++v) acc[v] = 0.0;
+      for (int i = lane; i < mm; i += 32) {
+        const double2 ui = su[i];
+#pragma unroll
+        for (int v = 0; v < CB; ++v) {
+          const double2 ci = src[v][i];
+          acc[v] = fma(ui.x, ci.x, fma(ui.y, ci.y, acc[v]));
+          acc[CB + v] = fma(ui.x, ci.y, fma(-ui.y, ci.x, acc[CB + v]));
+        }
+      }
+      int cur = 2 * CB;
+#pragma unroll
+      for (int o = 16; o >= 1; o >>= 1) {
+        if (cur > 1) {
+          const int h = cur >> 1;
+          const bool up = (lane & o) != 0;
+#pragma unroll
+          for (int v = 0; v < CB; ++v) {
+            if (v < h) {
+              const double send = up ? acc[v] : acc[v + h];
+              const double keep = up ? acc[v + h] : acc[v];
+              acc[v] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+            }
+          }
+          cur = h;
+        } else {
+          acc[0] += __shfl_xor_sync(0xffffffffu, acc[0], o);
+        }
+      }
+      double2 w[CB], top[CB];
+#pragma unroll
+      for (int v = 0; v < CB; ++v) {
+        w[v].x = tau * __shfl_sync(0xffffffffu, acc[0], v << SH);
+        w[v].y = tau * __shfl_sync(0xffffffffu, acc[0], (CB + v) << SH);
+        top[v] = make_double2(0.0, 0.0);
+      }
+      for (int i = lane; i < mm; i += 32) {
+        const double2 ui = su[i];
+#pragma unroll
+        for (int v = 0; v < CB; ++v)
+          if (v < nc) {
+            const double2 x = cfms(ui, w[v], src[v][i]);
+            M[j + i + (int64_t)(c0 + v) * ld] = x;
+            if (i == 0) top[v] = x;
+          }
+      }
+      // remaining norms: downdated by the new row-j entry, recomputed exactly once cancellation
+      // has eaten half their digits
+#pragma unroll
+      for (int v = 0; v < CB; ++v) {
+        if (v >= nc) break;
+        const int c = c0 + v, cs = c == p ? j : c;
+        const double rj = __shfl_sync(0xffffffffu, cabs2(top[v]), 0);
+        const double nf = __ldcg(q.nref + cs);
+        double nv = __ldcg(q.norm2 + cs) - rj;
+        __syncwarp();
+        if (nv <= 1e-8 * nf) {
+          double ns = 0.0;
+          const double2* col = M + (int64_t)c * ld;
+          for (int i = j + 1 + lane; i < m; i += 32) ns += cabs2(col[i]);
+          for (int o = 16; o > 0; o >>= 1) ns += __shfl_xor_sync(0xffffffffu, ns, o);
+          nv = ns;
+          if (lane == 0) q.nref[c] = ns;
+        } else if (cs != c && lane == 0) {
+          q.nref[c] = nf;
+        }
+        if (lane == 0) q.norm2[c] = fmax(nv, 0.0);
+        if (cs != c)  // rows above j of R: plain interchange of columns j and p
+          for (int i = lane; i < j; i += 32) {
+            const double2 t = M[i + (int64_t)j * ld];
+            M[i + (int64_t)j * ld] = M[i + (int64_t)p * ld];
+            M[i + (int64_t)p * ld] = t;
+          }
+      }
+    }
+    cluster_sync_all();
+  }
+  if (rank == 0 && tid == 0) {
+    q.state[0] = j;
+    q.state[1] = j;  // rank reached
+  }
+}
+
 // After the QR: put the diagonal of R back (the reflectors are no longer needed) and zero
 // the part of column t below the diagonal within the first k rows (none: R11 is k x k).
 __global__ void k_cpqr_finish(const QrDesc* __restrict__ d) {
@@ -924,7 +1132,25 @@ int wsbm_lu_solve_fused_batched(const LuSolveDesc* d_desc, int nbatch, int max_n
 int wsbm_cpqr_batched(const QrDesc* d_desc, int nbatch, int mode, int max_m, cudaStream_t st) {
   if (nbatch <= 0) return 0;
   const WsbmTune tu = wsbm_tune_current();
-  if (max_m <= CPQR_TPC_MAXM) {
+  // clusters of 2, 4 or 8 CTAs per matrix while the GPU holds them all at once (three per SM)
+  int cl = 1;
+  while (cl < 8 && (int64_t)nbatch * cl * 2 <= (int64_t)wsbm_sm_count() * 3) cl *= 2;
+  if (cl > 1 && (size_t)max_m * sizeof(double2) <= CPQR_CLUSTER_SMEM) {
+    const size_t sm = (size_t)max_m * sizeof(double2);
+    if (wsbm_smem_optin((const void*)k_cpqr_cluster<2>, sm) != cudaSuccess) return -3;
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = cl;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    cfg.gridDim = dim3((unsigned)(nbatch * cl));
+    cfg.blockDim = dim3(256);
+    cfg.dynamicSmemBytes = sm;
+    cfg.stream = st;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    if (cudaLaunchKernelEx(&cfg, k_cpqr_cluster<2>, d_desc, mode) != cudaSuccess) return -3;
+  } else if (max_m <= CPQR_TPC_MAXM) {
     const int thr = tu.cpqr_threads == 128 ? 128 : 256;
     k_cpqr<true, CPQR_CB><<<nbatch, thr, (size_t)max_m * sizeof(double2), st>>>(d_desc, mode);
   } else if (tu.cpqr_cb == 2) {
