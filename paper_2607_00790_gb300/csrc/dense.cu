@@ -14,6 +14,8 @@
 
 #include "cplx.cuh"
 #include "dense.h"
+#include "rowswap.cuh"
+#include "tri.cuh"
 
 #define GT 32  // GEMM tile (GT x GT outputs per CTA)
 #define GK 16  // GEMM k-chunk
@@ -199,27 +201,144 @@ __global__ void k_lu_trsm_row(const LuDesc* __restrict__ d, int j0, int jb) {
 }
 
 // ------------------------------------------------------------- triangular solves ----
-// B <- op(T)^-1 B for a diagonal block [j0, j0+jb) of T (lower unit or upper non-unit),
-// RHS columns in parallel.
-__global__ void k_trsm_diag(const TrsmDesc* __restrict__ d, int j0, int jb, int fwd) {
+// B <- op(T)^-1 B for a diagonal block [j0, j0 + jb) of T (jb <= 32; lower unit or upper non-unit).
+// The block is staged as a lower triangle S (rows and columns reversed for a backward solve) with
+// the reciprocals of its diagonal, zero rows and columns beyond the matrix.
+struct TrsmStage {
+  double2 S[32][33];  // S[t][i]: column t, row i of the triangle
+  double2 inv[32];
+};
+__device__ __forceinline__ void trsm_stage(TrsmStage& D, const TrsmDesc& q, int j0, int jb, bool fwd, bool unit) {
+  const int b = min(jb, q.n - j0);
+  const double2 zero = make_double2(0.0, 0.0);
+  for (int e = threadIdx.x; e < 32 * 32; e += blockDim.x) {
+    const int a = e & 31, c = e >> 5;  // element (a, c) of the stored block
+    const bool in = a < b && c < b;
+    const double2 v = in ? q.T[(j0 + a) + (int64_t)(j0 + c) * q.ldt] : zero;
+    int i = q.trans ? c : a, t = q.trans ? a : c;
+    if (in && !fwd) {
+      i = b - 1 - i;
+      t = b - 1 - t;
+    }
+    D.S[t][i] = v;  // read where i > t only
+    if (i == t) D.inv[i] = unit || !in ? make_double2(1.0, 0.0) : cdiv(make_double2(1.0, 0.0), v);
+  }
+  __syncthreads();
+}
+
+// Few columns (up to a few thousand in the launch): one warp per column, its row `lane` in each
+// lane's register: about 2 us a block, where a thread per column takes 512 dependent steps.
+__global__ void __launch_bounds__(128) k_trsm_diag_warp(const TrsmDesc* __restrict__ d, int j0, int jb, int fwd) {
+  __shared__ TrsmStage D;
+  const TrsmDesc q = d[blockIdx.y];
+  const int lane = threadIdx.x & 31;
+  if (j0 >= q.n || (int)blockIdx.x * 4 >= q.nrhs) return;
+  const bool unit = (fwd != 0) != (q.trans != 0);  // L and L^T have a unit diagonal
+  trsm_stage(D, q, j0, jb, fwd != 0, unit);
+  const int b = min(jb, q.n - j0), row = j0 + (fwd ? lane : b - 1 - lane);
+  for (int c = blockIdx.x * 4 + (threadIdx.x >> 5); c < q.nrhs; c += gridDim.x * 4) {
+    double2* col = q.B + (int64_t)c * q.ldb;
+    double2 x = lane < b ? col[row] : make_double2(0.0, 0.0);
+    const double2 iv = D.inv[lane];
+    for (int t = 0; t < b; ++t) {
+      double2 xt;
+      xt.x = __shfl_sync(0xFFFFFFFFu, x.x, t);
+      xt.y = __shfl_sync(0xFFFFFFFFu, x.y, t);
+      if (!unit) {
+        const double2 it = D.inv[t];
+        xt = cmul(xt, it);
+      }
+      if (lane > t) x = cfms(D.S[t][lane], xt, x);
+    }
+    if (!unit) x = cmul(x, iv);
+    if (lane < b) col[row] = x;
+  }
+}
+
+// Many columns: one thread per column held in shared memory (the triangle's entries are broadcast
+// reads), so every lane of the FP64 pipe works.
+#define TRSM_COLS 64
+__global__ void __launch_bounds__(TRSM_COLS) k_trsm_diag(const TrsmDesc* __restrict__ d, int j0, int jb, int fwd) {
+  __shared__ TrsmStage D;
+  extern __shared__ double2 sx[];  // [32][TRSM_COLS + 1]: row i of the thread's column
+  const TrsmDesc q = d[blockIdx.y];
+  if (j0 >= q.n || (int)blockIdx.x * TRSM_COLS >= q.nrhs) return;
+  const bool unit = (fwd != 0) != (q.trans != 0);
+  trsm_stage(D, q, j0, jb, fwd != 0, unit);
+  const int b = min(jb, q.n - j0), tid = threadIdx.x;
+  for (int c0 = blockIdx.x * TRSM_COLS; c0 < q.nrhs; c0 += gridDim.x * TRSM_COLS) {
+    const int nc = min(TRSM_COLS, q.nrhs - c0);
+    __syncthreads();
+    for (int e = tid; e < 32 * TRSM_COLS; e += TRSM_COLS) {
+      const int i = e & 31, c = e >> 5;
+      if (i < b && c < nc) sx[(fwd ? i : b - 1 - i) * (TRSM_COLS + 1) + c] = q.B[j0 + i + (int64_t)(c0 + c) * q.ldb];
+    }
+    __syncthreads();
+    if (tid < nc) {
+      for (int i = 0; i < b; ++i) {
+        double2 s = sx[i * (TRSM_COLS + 1) + tid], s2 = make_double2(0.0, 0.0);
+        int t = 0;
+        for (; t + 1 < i; t += 2) {  // two chains
+          s = cfms(D.S[t][i], sx[t * (TRSM_COLS + 1) + tid], s);
+          s2 = cfms(D.S[t + 1][i], sx[(t + 1) * (TRSM_COLS + 1) + tid], s2);
+        }
+        if (t < i) s = cfms(D.S[t][i], sx[t * (TRSM_COLS + 1) + tid], s);
+        s.x += s2.x;
+        s.y += s2.y;
+        sx[i * (TRSM_COLS + 1) + tid] = unit ? s : cmul(s, D.inv[i]);
+      }
+    }
+    __syncthreads();
+    for (int e = tid; e < 32 * TRSM_COLS; e += TRSM_COLS) {
+      const int i = e & 31, c = e >> 5;
+      if (i < b && c < nc) q.B[j0 + i + (int64_t)(c0 + c) * q.ldb] = sx[(fwd ? i : b - 1 - i) * (TRSM_COLS + 1) + c];
+    }
+  }
+}
+
+// The update after a solved block for a few right-hand sides (nrhs <= TRSM_FEW): a thread per row,
+// 64 rows a CTA, so no lane works on columns that are not there (a 32 x 32 product tile spends
+// 31/32 of the FP64 pipe on them at one right-hand side).  Arguments as for k_trsm_update.
+#define TRSM_FEW 8
+__global__ void __launch_bounds__(64) k_trsm_update_few(const TrsmDesc* __restrict__ d, int j0, int jb, int lower) {
+  __shared__ double2 sT[32][65];
+  __shared__ double2 sb[32][TRSM_FEW];
   const TrsmDesc q = d[blockIdx.y];
   if (j0 >= q.n) return;
-  const int je = min(j0 + jb, q.n);
-  const bool unit = (fwd != 0) != (q.trans != 0);  // L and L^T have a unit diagonal
-  const int64_t si = q.trans ? q.ldt : 1, st = q.trans ? 1 : q.ldt;  // op(T)(i,t) = T[i*si + t*st]
-  for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < q.nrhs; c += gridDim.x * blockDim.x) {
-    double2* col = q.B + (int64_t)c * q.ldb;
-    if (fwd) {
-      for (int i = j0; i < je; ++i) {
-        double2 s = col[i];
-        for (int t = j0; t < i; ++t) s = cfms(q.T[i * si + t * st], col[t], s);
-        col[i] = unit ? s : cdiv(s, q.T[i * si + i * st]);
+  const int je = min(j0 + jb, q.n), kb = je - j0;
+  const int m = lower ? q.n - je : j0, r0 = lower ? je : 0;
+  if (m <= 0 || q.nrhs <= 0) return;
+  for (int e = threadIdx.x; e < 32 * TRSM_FEW; e += 64) {
+    const int t = e & 31, c = e >> 5;
+    sb[t][c] = t < kb && c < q.nrhs ? q.B[j0 + t + (int64_t)c * q.ldb] : make_double2(0.0, 0.0);
+  }
+  for (int i0 = blockIdx.x * 64; i0 < m; i0 += gridDim.x * 64) {
+    const int mm = min(64, m - i0);
+    __syncthreads();
+    if (q.trans) {  // op(T)[r0 + i, j0 + t] = T[j0 + t, r0 + i]: contiguous in t
+      for (int e = threadIdx.x; e < 32 * 64; e += 64) {
+        const int t = e & 31, i = e >> 5;
+        sT[t][i] = t < kb && i < mm ? q.T[j0 + t + (int64_t)(r0 + i0 + i) * q.ldt] : make_double2(0.0, 0.0);
       }
     } else {
-      for (int i = je - 1; i >= j0; --i) {
-        double2 s = col[i];
-        for (int t = i + 1; t < je; ++t) s = cfms(q.T[i * si + t * st], col[t], s);
-        col[i] = unit ? s : cdiv(s, q.T[i * si + i * st]);
+      const int i = threadIdx.x;
+      for (int t = 0; t < 32; ++t)
+        sT[t][i] = t < kb && i < mm ? q.T[r0 + i0 + i + (int64_t)(j0 + t) * q.ldt] : make_double2(0.0, 0.0);
+    }
+    __syncthreads();
+    if ((int)threadIdx.x < mm) {
+      const int i = threadIdx.x;
+#pragma unroll
+      for (int c = 0; c < TRSM_FEW; ++c) {
+        if (c >= q.nrhs) break;
+        double2* o = q.B + r0 + i0 + i + (int64_t)c * q.ldb;
+        double2 s = *o, s2 = make_double2(0.0, 0.0);
+#pragma unroll 4
+        for (int t = 0; t < 32; t += 2) {
+          s = cfms(sT[t][i], sb[t][c], s);
+          s2 = cfms(sT[t + 1][i], sb[t + 1][c], s2);
+        }
+        *o = make_double2(s.x + s2.x, s.y + s2.y);
       }
     }
   }
@@ -247,35 +366,18 @@ __global__ void __launch_bounds__(256) k_trsm_update(const TrsmDesc* __restrict_
   }
 }
 
-// Apply the LU row interchanges to B (forward order).
-__global__ void k_apply_piv(const TrsmDesc* __restrict__ d) {
+// LU row interchanges on B, forward (P B) or, inverse, undone (P^T B): blocks of 256 swaps as
+// gathers, one warp per column.
+__global__ void __launch_bounds__(256) k_apply_piv(const TrsmDesc* __restrict__ d, int inverse) {
+  __shared__ SwapLists S;
   const TrsmDesc q = d[blockIdx.y];
-  for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < q.nrhs; c += gridDim.x * blockDim.x) {
-    double2* col = q.B + (int64_t)c * q.ldb;
-    for (int j = 0; j < q.n; ++j) {
-      int p = q.piv[j];
-      if (p != j) {
-        double2 t = col[j];
-        col[j] = col[p];
-        col[p] = t;
-      }
-    }
-  }
-}
-
-// Undo the LU row interchanges (reverse order): B <- P^T B.
-__global__ void k_apply_piv_inv(const TrsmDesc* __restrict__ d) {
-  const TrsmDesc q = d[blockIdx.y];
-  for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < q.nrhs; c += gridDim.x * blockDim.x) {
-    double2* col = q.B + (int64_t)c * q.ldb;
-    for (int j = q.n - 1; j >= 0; --j) {
-      int p = q.piv[j];
-      if (p != j) {
-        double2 t = col[j];
-        col[j] = col[p];
-        col[p] = t;
-      }
-    }
+  if ((int)blockIdx.x * 8 >= q.nrhs) return;
+  const int nblk = (q.n + 255) / 256;
+  for (int k = 0; k < nblk; ++k) {
+    const int j0 = (inverse ? nblk - 1 - k : k) * 256, nb = min(256, q.n - j0);
+    swap_lists(S, q.piv + j0, q.n, j0, nb);
+    for (int c = blockIdx.x * 8 + (threadIdx.x >> 5); c < q.nrhs; c += gridDim.x * 8)
+      swap_column(S, nb, q.B + (int64_t)c * q.ldb, inverse != 0);
   }
 }
 
@@ -1065,29 +1167,29 @@ int wsbm_trsm_batched(const TrsmDesc* d_desc, int nbatch, int max_n, int max_nrh
         return rc;
     return 0;
   }
-  dim3 gd(tiles_x((max_nrhs + 127) / 128), nbatch);
-  if (lower) {
-    for (int j0 = 0; j0 < max_n; j0 += WSBM_NB) {
-      k_trsm_diag<<<gd, 128, 0, st>>>(d_desc, j0, WSBM_NB, 1);
-      wsbm_count_launch();
-      int m = max_n - j0 - WSBM_NB;
-      if (m > 0) {
-        int64_t t = (int64_t)((m + GT - 1) / GT) * ((max_nrhs + GT - 1) / GT);
-        k_trsm_update<<<dim3(tiles_x(t), nbatch), 256, 0, st>>>(d_desc, j0, WSBM_NB, 1);
-        wsbm_count_launch();
-      }
+  // blocks of WSBM_NB rows: the diagonal block, then the update of the rows still to solve.  One
+  // warp per column while the columns are few (measured equal at about 4000 on 152 SMs)
+  const bool warps = (int64_t)nbatch * max_nrhs <= (int64_t)wsbm_sm_count() * 24;
+  const size_t smx = (size_t)32 * (TRSM_COLS + 1) * sizeof(double2);
+  if (!warps && wsbm_smem_optin((const void*)k_trsm_diag, 64 * 1024) != cudaSuccess) return -3;
+  const int nblk = (max_n + WSBM_NB - 1) / WSBM_NB;
+  for (int k = 0; k < nblk; ++k) {
+    const int j0 = (lower ? k : nblk - 1 - k) * WSBM_NB;
+    if (warps)
+      k_trsm_diag_warp<<<dim3(tiles_x((max_nrhs + 3) / 4), nbatch), 128, 0, st>>>(d_desc, j0, WSBM_NB, lower);
+    else
+      k_trsm_diag<<<dim3(tiles_x((max_nrhs + TRSM_COLS - 1) / TRSM_COLS), nbatch), TRSM_COLS, smx, st>>>(
+          d_desc, j0, WSBM_NB, lower);
+    wsbm_count_launch();
+    const int m = lower ? max_n - j0 - WSBM_NB : j0;
+    if (m <= 0) continue;
+    if (max_nrhs <= TRSM_FEW) {
+      k_trsm_update_few<<<dim3(tiles_x((m + 63) / 64), nbatch), 64, 0, st>>>(d_desc, j0, WSBM_NB, lower);
+    } else {
+      const int64_t t = (int64_t)((m + GT - 1) / GT) * ((max_nrhs + GT - 1) / GT);
+      k_trsm_update<<<dim3(tiles_x(t), nbatch), 256, 0, st>>>(d_desc, j0, WSBM_NB, lower);
     }
-  } else {
-    int last = ((max_n - 1) / WSBM_NB) * WSBM_NB;
-    for (int j0 = last; j0 >= 0; j0 -= WSBM_NB) {
-      k_trsm_diag<<<gd, 128, 0, st>>>(d_desc, j0, WSBM_NB, 0);
-      wsbm_count_launch();
-      if (j0 > 0) {
-        int64_t t = (int64_t)((j0 + GT - 1) / GT) * ((max_nrhs + GT - 1) / GT);
-        k_trsm_update<<<dim3(tiles_x(t), nbatch), 256, 0, st>>>(d_desc, j0, WSBM_NB, 0);
-        wsbm_count_launch();
-      }
-    }
+    wsbm_count_launch();
   }
   return cudaGetLastError() == cudaSuccess ? 0 : -3;
 }
@@ -1106,8 +1208,7 @@ int wsbm_lu_solve_batched(const TrsmDesc* d_desc_lower, const TrsmDesc* d_desc_u
         return rc;
     return 0;
   }
-  dim3 gd(tiles_x((max_nrhs + 127) / 128), nbatch);
-  k_apply_piv<<<gd, 128, 0, st>>>(d_desc_lower);
+  k_apply_piv<<<dim3(tiles_x((max_nrhs + 7) / 8), nbatch), 256, 0, st>>>(d_desc_lower, 0);
   wsbm_count_launch();
   int rc = wsbm_trsm_batched(d_desc_lower, nbatch, max_n, max_nrhs, 1, st);
   if (rc) return rc;
@@ -1185,8 +1286,7 @@ int wsbm_lu_solve_t_batched(const TrsmDesc* d_desc, int nbatch, int max_n, int m
   if (rc) return rc;
   rc = wsbm_trsm_batched(d_desc, nbatch, max_n, max_nrhs, 0, st);  // L^T, backward
   if (rc) return rc;
-  dim3 gd(tiles_x((max_nrhs + 127) / 128), nbatch);
-  k_apply_piv_inv<<<gd, 128, 0, st>>>(d_desc);
+  k_apply_piv<<<dim3(tiles_x((max_nrhs + 7) / 8), nbatch), 256, 0, st>>>(d_desc, 1);
   wsbm_count_launch();
   return cudaGetLastError() == cudaSuccess ? 0 : -3;
 }
@@ -1224,108 +1324,90 @@ __global__ void k_lut_swap(const LuSolveDesc* __restrict__ d, int j0, int jb) {
 }
 
 // X = inverse of the unit lower (upper = 0) or of the upper (upper = 1, non-unit) triangle of
-// the diagonal block A[j0 : j0+jb, j0 : j0+jb] of item blockIdx.y; X: jb x jb (ld jb) at
-// X + blockIdx.y * ldx_item.  One thread per column j: x_ij from the rows before (lower) or
-// after (upper) it.
-__global__ void k_lut_trinv(const LuSolveDesc* __restrict__ d, int j0, int jb, int upper,
-                            double2* __restrict__ Xall, int64_t ldx_item) {
+// the diagonal block A[j0 : j0+jb, j0 : j0+jb] (jb <= 64) of item blockIdx.y; X: jb x jb (ld jb) at
+// X + blockIdx.y * ldx_item.  One warp per column, 16 columns a CTA.
+__global__ void __launch_bounds__(512) k_lut_trinv(const LuSolveDesc* __restrict__ d, int j0, int jb, int upper,
+                                                   double2* __restrict__ Xall, int64_t ldx_item) {
+  __shared__ double2 stage[32 * 64];
+  __shared__ double2 dinv[32];
   const LuSolveDesc q = d[blockIdx.y];
-  const int j = blockIdx.x * blockDim.x + threadIdx.x;
   if (j0 >= q.n) return;
-  const int b = min(jb, q.n - j0);
-  if (j >= b) return;
+  const int b = min(jb, q.n - j0), j = blockIdx.x * 16 + (threadIdx.x >> 5);
+  if ((int)blockIdx.x * 16 >= b) return;
   double2* x = Xall + blockIdx.y * ldx_item + (int64_t)j * b;
   const double2* T = q.A + j0 + (int64_t)j0 * q.lda;
-  const double2 one = make_double2(1.0, 0.0), zero = make_double2(0.0, 0.0);
-  if (!upper) {
-    for (int i = 0; i < j; ++i) x[i] = zero;
-    x[j] = one;
-    for (int i = j + 1; i < b; ++i) {
-      double2 s = zero;
-      for (int t = j; t < i; ++t) s = cfms(T[i + (int64_t)t * q.lda], x[t], s);
-      x[i] = s;
-    }
-  } else {
-    for (int i = j + 1; i < b; ++i) x[i] = zero;
-    const double2 djj = T[j + (int64_t)j * q.lda];
-    x[j] = (djj.x == 0.0 && djj.y == 0.0) ? zero : cdiv(one, djj);
-    for (int i = j - 1; i >= 0; --i) {
-      double2 s = zero;
-      for (int t = i + 1; t <= j; ++t) s = cfms(T[i + (int64_t)t * q.lda], x[t], s);
-      const double2 dii = T[i + (int64_t)i * q.lda];
-      x[i] = (dii.x == 0.0 && dii.y == 0.0) ? zero : cdiv(s, dii);
-    }
-  }
+  const int first = blockIdx.x / 2;  // 16 columns a CTA lie in one slot of 32
+  if (upper)
+    tri_inverse_column<2, true>(T, q.lda, b, j, x, stage, dinv, true, first);
+  else
+    tri_inverse_column<2, false>(T, q.lda, b, j, x, stage, dinv, true, first);
 }
 
 // Inverses of the diagonal blocks of LU factors (unit lower L, upper U), for block triangular
 // solves whose products run on the tensor cores.  Item blockIdx.y with block width nb = q.nb,
-// block p = blockIdx.x (rows and columns p nb .. min(n, (p + 1) nb)), blockIdx.z = 0: L_pp^-1
+// block p = blockIdx.x / NCH (rows and columns p nb .. min(n, (p + 1) nb)), blockIdx.z = 0: L_pp^-1
 // into Linv + p nb^2, 1: U_pp^-1 into Uinv + p nb^2 (column-major, leading dimension nb; the
-// part outside a ragged last block is not written).  Thread j forms column j by substitution.
-// A zero diagonal entry of U leaves a zero row in U_pp^-1.
-__global__ void k_lu_dinv(const DinvDesc* __restrict__ d) {
+// part outside a ragged last block is not written).  One warp per column, 16 columns a CTA (chunk
+// blockIdx.x % NCH).  A zero diagonal entry of U leaves a zero row in U_pp^-1.
+#define DINV_CHUNKS 16  // CTAs per block: up to 256 columns
+__global__ void __launch_bounds__(512) k_lu_dinv(const DinvDesc* __restrict__ d) {
+  extern __shared__ double2 stage[];
+  __shared__ double2 dinv[32];
   const DinvDesc q = d[blockIdx.y];
-  const int nb = q.nb, p = blockIdx.x, j0 = p * nb;
+  const int nb = q.nb, p = blockIdx.x / DINV_CHUNKS, ch = blockIdx.x % DINV_CHUNKS, j0 = p * nb;
   if (j0 >= q.n) return;
-  const int b = min(nb, q.n - j0), j = threadIdx.x;
-  if (j >= b) return;
+  const int b = min(nb, q.n - j0), j = ch * 16 + (threadIdx.x >> 5);
+  if (ch * 16 >= b) return;
   const bool upper = blockIdx.z != 0;
   double2* x = (upper ? q.Uinv : q.Linv) + (int64_t)p * nb * nb + (int64_t)j * nb;
   const double2* T = q.A + j0 + (int64_t)j0 * q.lda;
-  const double2 one = make_double2(1.0, 0.0), zero = make_double2(0.0, 0.0);
-  if (!upper) {
-    for (int i = 0; i < j; ++i) x[i] = zero;
-    x[j] = one;
-    for (int i = j + 1; i < b; ++i) {
-      double2 s = zero;
-      for (int t = j; t < i; ++t) s = cfms(T[i + (int64_t)t * q.lda], x[t], s);
-      x[i] = s;
-    }
-  } else {
-    for (int i = j + 1; i < b; ++i) x[i] = zero;
-    const double2 djj = T[j + (int64_t)j * q.lda];
-    x[j] = (djj.x == 0.0 && djj.y == 0.0) ? zero : cdiv(one, djj);
-    for (int i = j - 1; i >= 0; --i) {
-      double2 s = zero;
-      for (int t = i + 1; t <= j; ++t) s = cfms(T[i + (int64_t)t * q.lda], x[t], s);
-      const double2 dii = T[i + (int64_t)i * q.lda];
-      x[i] = (dii.x == 0.0 && dii.y == 0.0) ? zero : cdiv(s, dii);
-    }
-  }
+  if (upper)
+    tri_inverse_column<8, true>(T, q.lda, b, j, x, stage, dinv, true, ch / 2);
+  else
+    tri_inverse_column<8, false>(T, q.lda, b, j, x, stage, dinv, true, ch / 2);
 }
 
 int wsbm_lu_dinv_batched(const DinvDesc* d_desc, int nitems, int max_blocks, int max_nb, cudaStream_t st) {
   if (nitems <= 0 || max_blocks <= 0) return 0;
   if (max_nb < 1 || max_nb > 256) return -1;
+  const size_t sm = (size_t)32 * 256 * sizeof(double2);
+  if (wsbm_smem_optin((const void*)k_lu_dinv, sm) != cudaSuccess) return -3;
   for (int c = 0; c < nitems; c += LAUNCH_MAX_Y) {
     const int n = std::min(LAUNCH_MAX_Y, nitems - c);
-    k_lu_dinv<<<dim3(max_blocks, n, 2), max_nb, 0, st>>>(d_desc + c);
+    k_lu_dinv<<<dim3(max_blocks * DINV_CHUNKS, n, 2), 512, sm, st>>>(d_desc + c);
     wsbm_count_launch();
   }
   return cudaGetLastError() == cudaSuccess ? 0 : -3;
 }
 
 // perm of the row interchanges piv (piv[j]: the row swapped with row j at step j, j = 0..n-1):
-// (P b)[r] = b[perm[r]].  One thread per item (the swaps are sequential).
-__global__ void k_piv_perm(const PermDesc* __restrict__ d, int nitems) {
-  const int it = blockIdx.x * blockDim.x + threadIdx.x;
-  if (it >= nitems) return;
-  const PermDesc q = d[it];
-  for (int r = 0; r < q.n; ++r) q.perm[r] = r;
-  for (int j = 0; j < q.n; ++j) {
-    const int p = q.piv[j];
-    if (p > j && p < q.n) {
-      const int t = q.perm[j];
-      q.perm[j] = q.perm[p];
-      q.perm[p] = t;
+// (P b)[r] = b[perm[r]].  One CTA per item, 256 swaps at a time.
+__global__ void __launch_bounds__(256) k_piv_perm(const PermDesc* __restrict__ d) {
+  __shared__ SwapLists S;
+  const PermDesc q = d[blockIdx.x];
+  const int t = threadIdx.x;
+  for (int r = t; r < q.n; r += 256) q.perm[r] = r;
+  for (int j0 = 0; j0 < q.n; j0 += 256) {
+    const int nb = min(256, q.n - j0);
+    swap_lists(S, q.piv + j0, q.n, j0, nb);
+    int v[2];
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int e = t + 256 * h;
+      if (e < 2 * nb && S.dst[e] >= 0) v[h] = q.perm[S.src[e]];
+    }
+    __syncthreads();
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int e = t + 256 * h;
+      if (e < 2 * nb && S.dst[e] >= 0) q.perm[S.dst[e]] = v[h];
     }
   }
 }
 
 int wsbm_piv_perm_batched(const PermDesc* d_desc, int nitems, cudaStream_t st) {
   if (nitems <= 0) return 0;
-  k_piv_perm<<<(nitems + 63) / 64, 64, 0, st>>>(d_desc, nitems);
+  k_piv_perm<<<nitems, 256, 0, st>>>(d_desc);
   wsbm_count_launch();
   return cudaGetLastError() == cudaSuccess ? 0 : -3;
 }
@@ -1410,7 +1492,7 @@ int wsbm_lu_solve_tc_batched_nb(const LuSolveDesc* h, const LuSolveDesc* d, int 
   for (int j0 = 0; j0 < maxn; j0 += nb) {
     k_lu_panel<<<nbatch, 256, 0, st>>>(d_lu, j0, nb, nullptr);
     k_lut_swap<<<dim3(tiles_x((maxnc + 127) / 128), nbatch), 128, 0, st>>>(d, j0, nb);
-    k_lut_trinv<<<dim3(1, nbatch), nb, 0, st>>>(d, j0, nb, 0, X, ldx);
+    k_lut_trinv<<<dim3((nb + 15) / 16, nbatch), 512, 0, st>>>(d, j0, nb, 0, X, ldx);
     wsbm_count_launches(3);
     // U12 = L11^-1 [A12 | B1]  (in place: the digit planes are formed before C is written)
     for (int i = 0; i < nbatch; ++i) {
@@ -1436,7 +1518,7 @@ int wsbm_lu_solve_tc_batched_nb(const LuSolveDesc* h, const LuSolveDesc* d, int 
   }
   // ---- back substitution X = U^-1 (L^-1 P B), panels from the bottom
   for (int j0 = ((maxn - 1) / nb) * nb; j0 >= 0; j0 -= nb) {
-    k_lut_trinv<<<dim3(1, nbatch), nb, 0, st>>>(d, j0, nb, 1, X, ldx);
+    k_lut_trinv<<<dim3((nb + 15) / 16, nbatch), 512, 0, st>>>(d, j0, nb, 1, X, ldx);
     wsbm_count_launch();
     for (int i = 0; i < nbatch; ++i) {
       const LuSolveDesc& q = h[i];

@@ -11,6 +11,8 @@
 
 #include "cplx.cuh"
 #include "dense.h"
+#include "rowswap.cuh"
+#include "tri.cuh"
 
 #ifndef LUB_NB
 #define LUB_NB 128      // outer panel width
@@ -189,105 +191,42 @@ __global__ void __launch_bounds__(LUB_T, 1)
   }
 }
 
-// Row interchanges piv[j0 .. j0 + nb) (nb <= 256) on the columns [a0, a1) and [b0, b1).  The nb
-// swaps are turned into one gather per column (at most 2 nb rows move): with a[j] the row whose
-// content sits in row j0 + j just before swap j, row j0 + j receives the content of row piv[j]
-// and a row below the panel the content a[j] of the last swap that names it.  One warp per
-// column, so the top nb rows are read and written contiguously (5 us a call at n = 8200).
+// Row interchanges piv[j0 .. j0 + nb) (nb <= 256) on the columns [a0, a1) and [b0, b1), as one
+// gather per column, one warp each: the top nb rows are read and written contiguously (5 us a
+// call at n = 8200).
 __global__ void __launch_bounds__(256) k_lub_rowswap(double2* __restrict__ A, int64_t lda, int n, int j0, int nb,
                                                      const int* __restrict__ piv, int a0, int a1, int b0, int b1) {
-  __shared__ int sp[256], ptr[256], src[512], dst[512];
-  const int t = threadIdx.x, lane = t & 31;
-  if (t < nb) {
-    const int p = piv[j0 + t];  // out of range only after a panel that gave up waiting
-    sp[t] = p >= j0 + t && p < n ? p : j0 + t;
-  }
-  __syncthreads();
-  int par = -1, prev = -1;
-  bool last = true;
-  if (t < nb) {
-    for (int i = 0; i < nb; ++i) {
-      const int q = sp[i];
-      if (i < t && q == j0 + t) par = i;
-      if (i < t && q == sp[t]) prev = i;
-      if (i > t && q == sp[t]) last = false;
-    }
-    ptr[t] = par >= 0 ? par : t;
-  }
-  __syncthreads();
-  for (int s = 1; s < nb; s <<= 1) {  // root of each chain by pointer jumping
-    const int v = t < nb ? ptr[ptr[t]] : 0;
-    __syncthreads();
-    if (t < nb) ptr[t] = v;
-    __syncthreads();
-  }
-  if (t < nb) {
-    const int at = j0 + ptr[t];
-    dst[t] = j0 + t;
-    src[t] = sp[t] == j0 + t ? at : (prev >= 0 ? j0 + ptr[prev] : sp[t]);
-    dst[nb + t] = sp[t] >= j0 + nb && last ? sp[t] : -1;
-    src[nb + t] = at;
-  }
-  __syncthreads();
+  __shared__ SwapLists S;
+  swap_lists(S, piv + j0, n, j0, nb);
   const int na = a1 - a0, tot = na + (b1 - b0);
-  for (int q = blockIdx.x * 8 + (t >> 5); q < tot; q += gridDim.x * 8) {
-    double2* col = A + (int64_t)(q < na ? a0 + q : b0 + (q - na)) * lda;
-    double2 v[16];
-#pragma unroll
-    for (int s = 0; s < 16; ++s) {
-      const int e = s * 32 + lane;
-      if (e < 2 * nb && dst[e] >= 0) v[s] = col[src[e]];
-    }
-    __syncwarp();
-#pragma unroll
-    for (int s = 0; s < 16; ++s) {
-      const int e = s * 32 + lane;
-      if (e < 2 * nb && dst[e] >= 0) col[dst[e]] = v[s];
-    }
-  }
+  for (int q = blockIdx.x * 8 + (threadIdx.x >> 5); q < tot; q += gridDim.x * 8)
+    swap_column(S, nb, A + (int64_t)(q < na ? a0 + q : b0 + (q - na)) * lda, false);
 }
 
-// X = L^-1 B for the unit lower triangle L of A[r0 : r0 + nb, r0 : r0 + nb] (nb <= 256), one warp
-// per column, the column spread over the lanes' registers: step t broadcasts x_t and takes
-// column t of L (contiguous) off the rows below (80 us for a 128 x 128 inverse; one thread per
-// column, whose chain of dependent loads bound it, took 1.7 ms).  B: the ncols columns at B (leading dimension
-// ldb), in place; B = NULL: the identity, X into `out` (leading dimension nb).
-__global__ void k_lub_trsm(const double2* __restrict__ A, int64_t lda, int r0, int nb, double2* B, int64_t ldb,
-                           int ncols, double2* __restrict__ out) {
-  const int lane = threadIdx.x & 31, q = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-  if (q >= ncols) return;
-  double2 x[8];
-  double2* col = B ? B + (int64_t)q * ldb : nullptr;
-#pragma unroll
-  for (int s = 0; s < 8; ++s) {
-    const int i = s * 32 + lane;
-    x[s] = i < nb ? (B ? col[i] : make_double2(i == q ? 1.0 : 0.0, 0.0)) : make_double2(0.0, 0.0);
-  }
+// X = L^-1 B for the unit lower triangle L of A[r0 : r0 + nb, r0 : r0 + nb] (nb <= 32 NS), one warp
+// per column (tri.cuh), `cols` columns a CTA (the other warps help to stage L: the solves are bound
+// by FP64, so one column per SM until there are more columns than SMs).  B: the ncols columns at B (leading dimension ldb), in place; B = NULL: the
+// inverse itself, into `out` (leading dimension nb).
+template <int NS>
+__global__ void __launch_bounds__(128) k_lub_trsm(const double2* __restrict__ A, int64_t lda, int r0, int nb,
+                                                  double2* B, int64_t ldb, int ncols, int cols, double2* __restrict__ out) {
+  extern __shared__ double2 stage[];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, q = blockIdx.x * cols + warp;
+  const bool on = warp < cols && q < ncols;
   const double2* L = A + r0 + (int64_t)r0 * lda;
-#pragma unroll
-  for (int s = 0; s < 8; ++s) {
-    if (s * 32 >= nb) break;
-    if (!B && s * 32 + 31 < q) continue;  // leading zeros of a column of the inverse
-    const int te = min(32, nb - s * 32);
-#pragma unroll 4
-    for (int tt = 0; tt < te; ++tt) {
-      const double2* lc = L + (int64_t)(s * 32 + tt) * lda;
-      double2 xt;
-      xt.x = __shfl_sync(0xFFFFFFFFu, x[s].x, tt);
-      xt.y = __shfl_sync(0xFFFFFFFFu, x[s].y, tt);
-#pragma unroll
-      for (int s2 = s; s2 < 8; ++s2) {
-        const int i = s2 * 32 + lane;
-        if (s2 * 32 < nb && i < nb && (s2 > s || lane > tt)) x[s2] = cfms(lc[i], xt, x[s2]);
-      }
-    }
+  if (!B) {
+    tri_inverse_column<NS, false>(L, lda, nb, q, out + (int64_t)q * nb, stage, nullptr, on, (int)blockIdx.x * cols / 32);
+    return;
   }
-  double2* o = B ? col : out + (int64_t)q * nb;
+  double2 x[NS];
+  double2* col = B + (int64_t)q * ldb;
 #pragma unroll
-  for (int s = 0; s < 8; ++s) {
-    const int i = s * 32 + lane;
-    if (i < nb) o[i] = x[s];
-  }
+  for (int s = 0; s < NS; ++s)
+    x[s] = on && s * 32 + lane < nb ? col[s * 32 + lane] : make_double2(0.0, 0.0);
+  tri_solve_warp<NS, false>(L, lda, nb, x, stage, nullptr, on);
+#pragma unroll
+  for (int s = 0; s < NS; ++s)
+    if (on && s * 32 + lane < nb) col[s * 32 + lane] = x[s];
 }
 
 namespace {
@@ -321,10 +260,20 @@ int lub_swap(const LubCtx& x, int j0, int nb, int a0, int a1, int b0, int b1) {
   return 0;
 }
 
-void lub_trsm(const LubCtx& x, int r0, int nb, double2* B, int ncols, double2* out) {
-  const int wpb = ncols > wsbm_sm_count() * 4 ? 4 : 1;
-  k_lub_trsm<<<(ncols + wpb - 1) / wpb, 32 * wpb, 0, x.st>>>(x.A, x.lda, r0, nb, B, x.lda, ncols, out);
+template <int NS>
+int lub_trsm_ns(const LubCtx& x, int r0, int nb, double2* B, int ncols, double2* out) {
+  const size_t sm = (size_t)32 * 32 * NS * sizeof(double2);
+  if (wsbm_smem_optin((const void*)k_lub_trsm<NS>, sm) != cudaSuccess) return -3;
+  const int cols = std::min(4, (ncols + wsbm_sm_count() - 1) / wsbm_sm_count());
+  k_lub_trsm<NS><<<(ncols + cols - 1) / cols, 128, sm, x.st>>>(x.A, x.lda, r0, nb, B, x.lda, ncols, cols, out);
   wsbm_count_launch();
+  return 0;
+}
+int lub_trsm(const LubCtx& x, int r0, int nb, double2* B, int ncols, double2* out) {
+  if (nb <= 32) return lub_trsm_ns<1>(x, r0, nb, B, ncols, out);
+  if (nb <= 64) return lub_trsm_ns<2>(x, r0, nb, B, ncols, out);
+  if (nb <= 128) return lub_trsm_ns<4>(x, r0, nb, B, ncols, out);
+  return lub_trsm_ns<8>(x, r0, nb, B, ncols, out);
 }
 
 // factor columns [c0, c1) of rows [c0, n); row swaps across the whole outer panel
@@ -351,7 +300,7 @@ int lub_rec(const LubCtx& x, int c0, int c1, int base) {
   const int mid = c0 + ((w / 2 + base - 1) / base) * base;
   if (int rc = lub_rec(x, c0, mid, base)) return rc;
   // A[c0:mid, mid:c1] = L11^-1 A[c0:mid, mid:c1];  A[mid:n, mid:c1] -= A[mid:n, c0:mid] A[c0:mid, mid:c1]
-  lub_trsm(x, c0, mid - c0, x.A + c0 + (int64_t)mid * x.lda, c1 - mid, nullptr);
+  if (int rc = lub_trsm(x, c0, mid - c0, x.A + c0 + (int64_t)mid * x.lda, c1 - mid, nullptr)) return rc;
   const double2 mone = make_double2(-1.0, 0.0), one = make_double2(1.0, 0.0);
   if (int rc = wsbm_zgemm_tc(x.n - mid, c1 - mid, mid - c0, mone, x.A + mid + (int64_t)c0 * x.lda, x.lda,
                              x.A + c0 + (int64_t)mid * x.lda, x.lda, one, x.A + mid + (int64_t)mid * x.lda, x.lda,
@@ -421,7 +370,7 @@ int wsbm_lu_big_nb(double2* A, int64_t lda, int n, int* piv, int* d_info, void* 
       // U12 = L11^-1 A12 as a tensor-core product with the explicit inverse of the unit lower
       // L11 (the digit planes of A12 are formed before A12 is overwritten)
       const int m = n - je;
-      lub_trsm(x, j0, jb, nullptr, jb, Linv);
+      if (int rc = lub_trsm(x, j0, jb, nullptr, jb, Linv)) return rc;
       if (int rc = wsbm_zgemm_tc(jb, m, jb, one, Linv, jb, A + j0 + (int64_t)je * lda, lda, zero,
                                  A + j0 + (int64_t)je * lda, lda, ws, st))
         return rc;
