@@ -8,20 +8,22 @@
 // Thread = output node i; CTA row blockIdx.y covers the other nodes [j0, j1); per-split
 // partial sums, reduced in a fixed order by k_matvec_reduce.  Vectors in paper order.
 #define MV_THREADS 128
-#define MV_RHS 4  // right-hand sides sharing each pair's Hankel evaluations
+template <int NR>
 struct MvSlot {
-  double x, y, nx, ny, w, kap;
-  double2 u[MV_RHS], q[MV_RHS];
+  double x, y, nx, ny, w;
+  double2 u[NR], q[NR];
 };
 
-// nr <= MV_RHS columns c0 .. c0 + nr - 1 of x (column stride 2N); partial sums of column r of
-// split s at part[(s * MV_RHS + r) * 2N + row].
-template <bool TRANS>
+// nr <= NR columns c0 .. c0 + nr - 1 of x (column stride 2N; NR = 1, 2, 4 or 8 share each pair's
+// entries, absent ones are zero); partial sums of column r of split s at part[(s * NR + r) * 2N +
+// row].  Bound by the FP64 pipe: 71 operations a pair for the entries and 16 per column, so 8
+// columns at once take 199 where two passes of 4 take 270.
+template <bool TRANS, int NR>
 __global__ void __launch_bounds__(MV_THREADS)
     k_matvec(DevGeom g, Phys ph, const double2* __restrict__ xin, int nr, int64_t jspan,
              double2* __restrict__ part) {
   __shared__ HkTables T;
-  __shared__ MvSlot sj[MV_THREADS];
+  __shared__ MvSlot<NR> sj[MV_THREADS];
   hk_stage_tables(&T);
   const int64_t N = g.n;
   const int64_t i = (int64_t)blockIdx.x * MV_THREADS + threadIdx.x;
@@ -37,23 +39,22 @@ __global__ void __launch_bounds__(MV_THREADS)
     wi = g.w[i];
     ki = g.kappa[i];
   }
-  double2 a0[MV_RHS], a1[MV_RHS];
+  double2 a0[NR], a1[NR];
 #pragma unroll
-  for (int r = 0; r < MV_RHS; ++r) a0[r] = a1[r] = make_double2(0.0, 0.0);
+  for (int r = 0; r < NR; ++r) a0[r] = a1[r] = make_double2(0.0, 0.0);
   for (int64_t jc = j0; jc < j1; jc += MV_THREADS) {
     __syncthreads();
     {
       int64_t j = jc + threadIdx.x;
       if (j < j1) {
-        MvSlot& s = sj[threadIdx.x];
+        MvSlot<NR>& s = sj[threadIdx.x];
         s.x = g.x[j];
         s.y = g.y[j];
         s.nx = g.nx[j];
         s.ny = g.ny[j];
         s.w = g.w[j];
-        s.kap = g.kappa[j];
 #pragma unroll
-        for (int r = 0; r < MV_RHS; ++r) {
+        for (int r = 0; r < NR; ++r) {
           const bool on = r < nr;
           s.u[r] = on ? xin[(int64_t)r * 2 * N + j] : make_double2(0.0, 0.0);
           s.q[r] = on ? xin[(int64_t)r * 2 * N + N + j] : make_double2(0.0, 0.0);
@@ -67,7 +68,7 @@ __global__ void __launch_bounds__(MV_THREADS)
     for (int jj = 0; jj < nj; ++jj) {
       // keep the Hankel tables in shared memory: no hoisting of their loads out of the loop
       asm volatile("" ::: "memory");
-      const MvSlot& s = sj[jj];
+      const MvSlot<NR>& s = sj[jj];
       double2 e[2][2];
       if (jc + jj == i) {
         block_diag(ph, wi, ki, e);
@@ -82,21 +83,20 @@ __global__ void __launch_bounds__(MV_THREADS)
         e[1][0] = t;
       }
 #pragma unroll
-      for (int r = 0; r < MV_RHS; ++r) {
-        if (r >= nr) break;
+      for (int r = 0; r < NR; ++r) {
         const double2 u = s.u[r], q = s.q[r];
-        a0[r].x += e[0][0].x * u.x - e[0][0].y * u.y + e[0][1].x * q.x - e[0][1].y * q.y;
-        a0[r].y += e[0][0].x * u.y + e[0][0].y * u.x + e[0][1].x * q.y + e[0][1].y * q.x;
-        a1[r].x += e[1][0].x * u.x - e[1][0].y * u.y + e[1][1].x * q.x - e[1][1].y * q.y;
-        a1[r].y += e[1][0].x * u.y + e[1][0].y * u.x + e[1][1].x * q.y + e[1][1].y * q.x;
+        a0[r].x = fma(e[0][0].x, u.x, fma(-e[0][0].y, u.y, fma(e[0][1].x, q.x, fma(-e[0][1].y, q.y, a0[r].x))));
+        a0[r].y = fma(e[0][0].x, u.y, fma(e[0][0].y, u.x, fma(e[0][1].x, q.y, fma(e[0][1].y, q.x, a0[r].y))));
+        a1[r].x = fma(e[1][0].x, u.x, fma(-e[1][0].y, u.y, fma(e[1][1].x, q.x, fma(-e[1][1].y, q.y, a1[r].x))));
+        a1[r].y = fma(e[1][0].x, u.y, fma(e[1][0].y, u.x, fma(e[1][1].x, q.y, fma(e[1][1].y, q.x, a1[r].y))));
       }
     }
   }
   if (valid) {
 #pragma unroll
-    for (int r = 0; r < MV_RHS; ++r) {
+    for (int r = 0; r < NR; ++r) {
       if (r >= nr) break;
-      double2* pr = part + ((int64_t)blockIdx.y * MV_RHS + r) * 2 * N;
+      double2* pr = part + ((int64_t)blockIdx.y * NR + r) * 2 * N;
       pr[i] = a0[r];
       pr[N + i] = a1[r];
     }
@@ -104,14 +104,14 @@ __global__ void __launch_bounds__(MV_THREADS)
 }
 
 // y[:, r] = sum over the splits, in split order, for the nr columns of one launch.
-__global__ void k_matvec_reduce(int64_t N, int nsplit, int nr, const double2* __restrict__ part,
+__global__ void k_matvec_reduce(int64_t N, int nsplit, int nr, int NR, const double2* __restrict__ part,
                                 double2* __restrict__ y) {
   for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < 2 * N * nr;
        e += (int64_t)gridDim.x * blockDim.x) {
     const int64_t r = e / (2 * N), row = e % (2 * N);
     double2 s = make_double2(0.0, 0.0);
     for (int t = 0; t < nsplit; ++t) {
-      double2 v = part[((int64_t)t * MV_RHS + r) * 2 * N + row];
+      double2 v = part[((int64_t)t * NR + r) * 2 * N + row];
       s.x += v.x;
       s.y += v.y;
     }
@@ -140,11 +140,13 @@ extern "C" int wsbm_matvec(const wsbm_geom* g, const wsbm_params* p, int32_t tra
   cudaStream_t st = (cudaStream_t)stream;
   const int64_t N = g->n;
   const int64_t nti = (N + MV_THREADS - 1) / MV_THREADS;
+  const int NR = nrhs > 4 ? 8 : (nrhs > 2 ? 4 : nrhs);  // columns of one launch
+  const auto kern = trans ? (NR == 8 ? k_matvec<true, 8> : NR == 4 ? k_matvec<true, 4> : NR == 2 ? k_matvec<true, 2> : k_matvec<true, 1>)
+                          : (NR == 8 ? k_matvec<false, 8> : NR == 4 ? k_matvec<false, 4> : NR == 2 ? k_matvec<false, 2> : k_matvec<false, 1>);
   int nsm = wsbm_sm_count(), per_sm = 1;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_matvec<false>, MV_THREADS, 0) != cudaSuccess ||
-      per_sm < 1)
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, MV_THREADS, 0) != cudaSuccess || per_sm < 1)
     per_sm = 1;
-  int64_t want = (int64_t)nsm * per_sm * 8;  // about eight waves
+  int64_t want = (int64_t)nsm * per_sm * (NR == 8 ? 4 : 8);  // about eight waves (four of twice the width)
   int64_t nsplit = (want + nti - 1) / nti;
   if (nsplit < 1) nsplit = 1;
   if (nsplit > nti) nsplit = nti;
@@ -152,21 +154,16 @@ extern "C" int wsbm_matvec(const wsbm_geom* g, const wsbm_params* p, int32_t tra
   nsplit = (N + jspan - 1) / jspan;
   WsbmScratch scr(st);
   double2* part = nullptr;
-  if ((rc = scr.get((size_t)nsplit * MV_RHS * 2 * N * sizeof(double2), (void**)&part))) return rc;
+  if ((rc = scr.get((size_t)nsplit * NR * 2 * N * sizeof(double2), (void**)&part))) return rc;
   DevGeom dg = wsbm_devgeom(g);
-  for (int c = 0; c < nrhs && rc == WSBM_OK; c += MV_RHS) {
-    const int nr = nrhs - c < MV_RHS ? nrhs - c : MV_RHS;
+  for (int c = 0; c < nrhs; c += NR) {
+    const int nr = nrhs - c < NR ? nrhs - c : NR;
     const double2* xc = (const double2*)x + (int64_t)c * 2 * N;
-    if (trans)
-      k_matvec<true><<<dim3((unsigned)nti, (unsigned)nsplit), MV_THREADS, 0, st>>>(dg, ph, xc, nr, jspan, part);
-    else
-      k_matvec<false><<<dim3((unsigned)nti, (unsigned)nsplit), MV_THREADS, 0, st>>>(dg, ph, xc, nr, jspan, part);
-    wsbm_count_launch();
+    kern<<<dim3((unsigned)nti, (unsigned)nsplit), MV_THREADS, 0, st>>>(dg, ph, xc, nr, jspan, part);
     int64_t blocks = (2 * N * nr + 255) / 256;
-    k_matvec_reduce<<<grid_for(blocks), 256, 0, st>>>(N, (int)nsplit, nr, part,
-                                                     (double2*)y + (int64_t)c * 2 * N);
-    wsbm_count_launch();
-    if (cudaGetLastError() != cudaSuccess) rc = WSBM_ERR_CUDA;
+    k_matvec_reduce<<<grid_for(blocks), 256, 0, st>>>(N, (int)nsplit, nr, NR, part, (double2*)y + (int64_t)c * 2 * N);
+    wsbm_count_launches(2);
+    if (cudaGetLastError() != cudaSuccess) return WSBM_ERR_CUDA;
   }
-  return rc;
+  return WSBM_OK;
 }
