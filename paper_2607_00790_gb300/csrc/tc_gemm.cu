@@ -284,17 +284,31 @@ struct TcSrc {
   int eoff;     // first exponent
 };
 
-// Row exponents of A (m x k): one thread per row (coalesced along the column); item blockIdx.y.
-__global__ void k_tc_row_exp(const TcSrc* __restrict__ src, int* __restrict__ rexp) {
+// Row exponents of A (m x k), item blockIdx.y: 32 rows a CTA, its 32 warps over the columns (a
+// thread per row leaves a serial chain of k loads: 50 us at k = 256 against 3).
+__global__ void __launch_bounds__(1024) k_tc_row_exp(const TcSrc* __restrict__ src, int* __restrict__ rexp) {
+  __shared__ uint64_t red[32][33];
   const TcSrc q = src[blockIdx.y];
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= q.rows) return;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, i = blockIdx.x * 32 + lane;
+  if ((int)blockIdx.x * 32 >= q.rows) return;
   uint64_t mx = 0;
-  for (int l = 0; l < q.k; ++l) {
-    const double2 v = q.M[i + (int64_t)l * q.ld];
-    mx = max(mx, max(abs_bits(v.x), abs_bits(v.y)));
+  if (i < q.rows) {
+#pragma unroll 4
+    for (int l = warp; l < q.k; l += 32) {
+      const double2 v = q.M[i + (int64_t)l * q.ld];
+      mx = max(mx, max(abs_bits(v.x), abs_bits(v.y)));
+    }
   }
-  rexp[q.eoff + i] = scale_exp(mx);
+  red[warp][lane] = mx;
+  __syncthreads();
+  mx = red[lane][warp];  // row `warp` of the CTA over its 32 partial maxima
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const unsigned long long other = __shfl_xor_sync(0xFFFFFFFFu, (unsigned long long)mx, o);
+    mx = max(mx, (uint64_t)other);
+  }
+  const int r = blockIdx.x * 32 + warp;
+  if (lane == 0 && r < q.rows) rexp[q.eoff + r] = scale_exp(mx);
 }
 
 // Digit planes of A: PA[t][row][2l + c] (c = 0: Re, 1: Im), rows of Ka BF16 values (zero
@@ -809,7 +823,7 @@ int wsbm_zgemm_tc_run(const TcPlan& pl, const void* dtab_v, double2 alpha, doubl
   const TcSrc* dsa = (const TcSrc*)(dtab + (size_t)nitems * sizeof(TcItem));
   const TcSrc* dsb = dsa + nitems;
   // digit planes (the padding rows between items are never read into a stored output)
-  k_tc_row_exp<<<dim3((pl.maxm + 127) / 128, nitems), 128, 0, st>>>(dsa, exps);
+  k_tc_row_exp<<<dim3((pl.maxm + 31) / 32, nitems), 1024, 0, st>>>(dsa, exps);
   k_tc_split_a<<<dim3((pl.maxm + 31) / 32, (unsigned)((Ka / 2 + 31) / 32), nitems), 256, 0, st>>>(
       dsa, exps, PA, (int64_t)ra * Ka, Ka);
   k_tc_col_exp<<<dim3((pl.maxn + 7) / 8, nitems), 256, 0, st>>>(dsb, exps);
