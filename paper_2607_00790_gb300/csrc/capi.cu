@@ -242,6 +242,10 @@ extern "C" int wsbm_entries_raw(const wsbm_geom* g, const wsbm_params* p, const 
   if (nr == 0 || nc == 0) return WSBM_OK;
   if (!rows || !cols || !out) return WSBM_ERR_INVALID_ARG;
   cudaStream_t st = (cudaStream_t)stream;
+  if (p->formulation == WSBM_FORM_WSBM) {
+    if ((rc = wsbm_launch_entries_raw(wsbm_devgeom(g), ph, rows, nr, cols, nc, (double2*)out, st))) return rc;
+    return cudaStreamSynchronize(st) == cudaSuccess ? WSBM_OK : WSBM_ERR_CUDA;
+  }
   WsbmScratch scr(st);
   int32_t* buf = nullptr;
   PairTask* dtask = nullptr;
@@ -270,10 +274,7 @@ extern "C" int wsbm_entries_raw(const wsbm_geom* g, const wsbm_params* p, const 
     if ((rc = wsbm_launch_unknowns_to_slots(rows, nr, g->n, rnode, rpos, st))) goto done;
     if ((rc = wsbm_launch_unknowns_to_slots(cols, nc, g->n, cnode, cpos, st))) goto done;
     CK(cudaMemcpyAsync(dtask, &t, sizeof(t), cudaMemcpyHostToDevice, st));
-    if (p->formulation == WSBM_FORM_WSBM)
-      rc = wsbm_launch_pairs(dg, ph, dtask, 1, wsbm_pair_tiles(t.nr, t.nc, 0), st);
-    else
-      rc = wsbm_launch_pairs_form(p->formulation, dg, ph, dtask, 1, wsbm_pair_tiles(t.nr, t.nc, 0), st);
+    rc = wsbm_launch_pairs_form(p->formulation, dg, ph, dtask, 1, wsbm_pair_tiles(t.nr, t.nc, 0), st);
     // the task struct lives on this stack frame: wait for the copy before returning
     CK(cudaStreamSynchronize(st));
   }

@@ -178,6 +178,169 @@ __global__ void __launch_bounds__(WSBM_PAIR_THREADS)
   }
 }
 
+// ---------------------------------------------------------------- entries by index lists ----
+// Entries A[rows, cols] for arbitrary lists of unknowns, one launch without work space: a tile
+// takes RAW_F row slots and RAW_S column slots, where slot t of a list of n indices is the pair
+// (t, t + ceil(n/2)).  Lists made of the u and then the q of the same nodes (the usual request of
+// a block) have both unknowns of a node in one slot, so a node pair is evaluated once for its four
+// entries; in any other tile the four entries of a slot pair are evaluated one by one, each with
+// the part of the block that it needs (about 35 to 65 FP64 operations in place of 71).
+#define RAW_F 32
+#define RAW_S 4
+#define RAW_CLASSES 7  // fixed point beyond 20 by entry (a, b), other fixed point, series, diagonal
+
+template <int A, int B>
+__device__ __forceinline__ double2 entry_fixed(const HkTables& T, const Phys& ph, const SlotData& R, const SlotData& C,
+                                               double dx, double dy, double r2) {
+  double2 e[2][2];
+  block_fixed(T, ph, dx, dy, r2, R.nx, R.ny, C.nx, C.ny, C.w, e);
+  return e[A][B];  // the rest of the block is dead code
+}
+
+struct RawSlot {
+  SlotData d;
+  int comp;  // 0: u or first equation, 1: q or second equation; -1: no such slot
+};
+
+__device__ __forceinline__ void load_raw_slot(const DevGeom& g, const int64_t* idx, int64_t t, int64_t n, RawSlot& s) {
+  s.comp = -1;
+  if (t >= n) return;
+  const int64_t u = idx[t];
+  const int comp = u >= g.n ? 1 : 0;
+  const int32_t node = (int32_t)(u - comp * g.n);
+  s.comp = comp;
+  s.d.node = node;
+  s.d.x = g.x[node];
+  s.d.y = g.y[node];
+  s.d.nx = g.nx[node];
+  s.d.ny = g.ny[node];
+  s.d.w = g.w[node];
+  s.d.kap = g.kappa[node];
+  s.d.fx = (float)s.d.x;
+  s.d.fy = (float)s.d.y;
+}
+
+__global__ void __launch_bounds__(RAW_F* RAW_S)
+    k_entries_raw(DevGeom g, const __grid_constant__ Phys ph, const int64_t* __restrict__ rows, int64_t nr,
+                  const int64_t* __restrict__ cols, int64_t nc, double2* __restrict__ out) {
+  __shared__ HkTables T;
+  __shared__ RawSlot sr[2][RAW_F], sc[2][RAW_S];  // [half of the list][slot]
+  __shared__ int s_cnt[RAW_F * RAW_S / 32][RAW_CLASSES];
+  __shared__ int16_t s_list[RAW_F * RAW_S];
+  hk_stage_tables(&T);
+  const int tid = threadIdx.x, tx = tid & (RAW_F - 1), ty = tid / RAW_F, lane = tid & 31, warp = tid >> 5;
+  const int64_t hr = (nr + 1) / 2, hc = (nc + 1) / 2;
+  const int64_t ntr = (hr + RAW_F - 1) / RAW_F, ntiles = ntr * ((hc + RAW_S - 1) / RAW_S);
+  for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
+    const int64_t r0 = (tile % ntr) * RAW_F, c0 = (tile / ntr) * RAW_S;
+    __syncthreads();
+    if (tid < 2 * RAW_F) {
+      const int h = tid / RAW_F, t = tid % RAW_F;
+      sr[h][t].comp = -1;
+      if (r0 + t < hr) load_raw_slot(g, rows, r0 + t + h * hr, nr, sr[h][t]);
+    } else if (tid < 2 * RAW_F + 2 * RAW_S) {
+      const int h = (tid - 2 * RAW_F) / RAW_S, t = (tid - 2 * RAW_F) % RAW_S;
+      sc[h][t].comp = -1;
+      if (c0 + t < hc) load_raw_slot(g, cols, c0 + t + h * hc, nc, sc[h][t]);
+    }
+    __syncthreads();
+    // both unknowns of one node in every slot of the tile (empty slots aside)?
+    bool whole = true;
+    if (tid < RAW_F)
+      whole = sr[0][tid].comp < 0 ||
+              (sr[0][tid].comp == 0 && sr[1][tid].comp == 1 && sr[0][tid].d.node == sr[1][tid].d.node);
+    else if (tid < RAW_F + RAW_S)
+      whole = sc[0][tid - RAW_F].comp < 0 || (sc[0][tid - RAW_F].comp == 0 && sc[1][tid - RAW_F].comp == 1 &&
+                                              sc[0][tid - RAW_F].d.node == sc[1][tid - RAW_F].d.node);
+    whole = __syncthreads_and(whole);
+    for (int quad = 0; quad < (whole ? 1 : 4); ++quad) {
+      const int qr = quad & 1, qc = quad >> 1;
+      // group the pairs by evaluation path, so that a warp mixes paths only at a group boundary
+      // (the grouping only orders work: FP32 coordinates are enough)
+      int cls = RAW_CLASSES;
+      {
+        const RawSlot &R = sr[qr][tx], &C = sc[qc][ty];
+        if (R.comp >= 0 && C.comp >= 0) {
+          if (R.d.node == C.d.node) {
+            cls = 6;
+          } else {
+            const float dx = R.d.fx - C.d.fx, dy = R.d.fy - C.d.fy, r2 = fmaf(dx, dx, dy * dy);
+            cls = r2 < ph.near_r2 ? 5 : (r2 < ph.far_r2 ? 4 : (whole ? 0 : 2 * R.comp + C.comp));
+          }
+        }
+      }
+      unsigned bal[RAW_CLASSES];
+#pragma unroll
+      for (int c = 0; c < RAW_CLASSES; ++c) {
+        bal[c] = __ballot_sync(0xffffffffu, cls == c);
+        if (lane == 0) s_cnt[warp][c] = __popc(bal[c]);
+      }
+      __syncthreads();
+      int base = 0;
+#pragma unroll
+      for (int c = 0; c < RAW_CLASSES; ++c) {
+        int before = 0, total = 0;
+#pragma unroll
+        for (int w = 0; w < RAW_F * RAW_S / 32; ++w) {
+          total += s_cnt[w][c];
+          if (w < warp) before += s_cnt[w][c];
+        }
+        if (cls == c) s_list[base + before + __popc(bal[c] & ((1u << lane) - 1u))] = (int16_t)tid;
+        base += total;
+      }
+      __syncthreads();
+      if (tid < base) {
+        const int me = s_list[tid], mx = me & (RAW_F - 1), my = me / RAW_F;
+        const SlotData &R = sr[qr][mx].d, &C = sc[qc][my].d;
+        const int a = sr[qr][mx].comp, b = sc[qc][my].comp;
+        double2* o = out + (r0 + mx + qr * hr) + (c0 + my + qc * hc) * nr;
+        const double dx = __dsub_rn(R.x, C.x), dy = __dsub_rn(R.y, C.y), r2 = pair_r2(dx, dy);
+        const bool diag = R.node == C.node, fixed = !diag && pair_is_fixed(ph, r2);
+        double2 e[2][2];
+        if (fixed && !whole) {
+          double2 v;
+          if (a == 0)
+            v = b == 0 ? entry_fixed<0, 0>(T, ph, R, C, dx, dy, r2) : entry_fixed<0, 1>(T, ph, R, C, dx, dy, r2);
+          else
+            v = b == 0 ? entry_fixed<1, 0>(T, ph, R, C, dx, dy, r2) : entry_fixed<1, 1>(T, ph, R, C, dx, dy, r2);
+          *o = v;
+        } else {
+          if (diag) {
+            block_diag(ph, R.w, R.kap, e);
+          } else if (fixed) {
+            block_fixed(T, ph, dx, dy, r2, R.nx, R.ny, C.nx, C.ny, C.w, e);
+          } else {
+            PairGeom G;
+            pair_geom(R.x, R.y, R.nx, R.ny, C.x, C.y, C.nx, C.ny, ph, G);
+            block_offdiag(T, ph, G, C.w, e);
+          }
+          if (whole) {
+            double2* o2 = o + hc * nr;
+            o[0] = e[0][0];
+            o[hr] = e[1][0];
+            o2[0] = e[0][1];
+            o2[hr] = e[1][1];
+          } else {
+            *o = a == 0 ? (b == 0 ? e[0][0] : e[0][1]) : (b == 0 ? e[1][0] : e[1][1]);
+          }
+        }
+      }
+      __syncthreads();
+    }
+  }
+}
+
+int wsbm_launch_entries_raw(const DevGeom& g, const Phys& ph, const int64_t* rows, int64_t nr, const int64_t* cols,
+                            int64_t nc, double2* out, cudaStream_t st) {
+  const int64_t hr = (nr + 1) / 2, hc = (nc + 1) / 2;
+  const int64_t ntiles = (hr + RAW_F - 1) / RAW_F * ((hc + RAW_S - 1) / RAW_S);
+  if (ntiles <= 0) return WSBM_OK;
+  const int64_t cap = (int64_t)wsbm_sm_count() * WSBM_ENTRY_CTAS;
+  k_entries_raw<<<(int)(ntiles < cap ? ntiles : cap), RAW_F * RAW_S, 0, st>>>(g, ph, rows, nr, cols, nc, out);
+  wsbm_count_launch();
+  return cudaGetLastError() == cudaSuccess ? WSBM_OK : WSBM_ERR_CUDA;
+}
+
 // --------------------------------------------------------------------- proxy blocks ----
 struct ProxyPt {
   double px, py, pnx, pny;

@@ -93,6 +93,10 @@ int wsbm_launch_proxy_rows_form(int form, const DevGeom& g, const Phys& ph, cons
                                 const DevGeom* geos = nullptr, const Phys* phys = nullptr);
 int64_t wsbm_pair_tiles(int32_t nr, int32_t nc, int32_t fastc, int tf = WSBM_TILE_F);
 int64_t wsbm_proxy_tiles(int32_t nn, int32_t P, int tf = WSBM_TILE_F);
+// Entries A[rows, cols] of eq. (weakly_bm) for device index lists, out column-major nr x nc: one
+// launch, no work space.
+int wsbm_launch_entries_raw(const DevGeom& g, const Phys& ph, const int64_t* rows, int64_t nr, const int64_t* cols,
+                            int64_t nc, double2* out, cudaStream_t st);
 int wsbm_launch_hankel(const double* z, int64_t n, double* out, int mixed, cudaStream_t st);
 int wsbm_launch_unknowns_to_slots(const int64_t* idx, int64_t n, int64_t N, int32_t* node,
                                   int32_t* pos, cudaStream_t st);
