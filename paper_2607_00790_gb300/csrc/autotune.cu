@@ -305,7 +305,7 @@ extern "C" int wsbm_autotune(int32_t n_box, int32_t nbox, int32_t nrhs_box, int3
             if (cudaMemcpyAsync(M, M0, (size_t)nb * m * n * 16, cudaMemcpyDeviceToDevice, st) != cudaSuccess ||
                 cudaMemsetAsync(sw, 0, (size_t)nb * per_state, st) != cudaSuccess)
               return WSBM_ERR_CUDA;
-            return wsbm_cpqr_batched(dq, nb, 1, m, st) ? WSBM_ERR_CUDA : WSBM_OK;
+            return wsbm_cpqr_batched(dq, nb, 0, 1, m, st) ? WSBM_ERR_CUDA : WSBM_OK;
           },
           &times[7 + c]);
       if (rc) {

@@ -256,7 +256,8 @@ __global__ void __launch_bounds__(128) k_trsm_diag_warp(const TrsmDesc* __restri
 }
 
 // Many columns: one thread per column held in shared memory (the triangle's entries are broadcast
-// reads), so every lane of the FP64 pipe works.
+// reads), so every lane of the FP64 pipe works.  The same operations in the same order as above: a
+// solution does not depend on how many columns share its launch.
 #define TRSM_COLS 64
 __global__ void __launch_bounds__(TRSM_COLS) k_trsm_diag(const TrsmDesc* __restrict__ d, int j0, int jb, int fwd) {
   __shared__ TrsmStage D;
@@ -276,15 +277,8 @@ __global__ void __launch_bounds__(TRSM_COLS) k_trsm_diag(const TrsmDesc* __restr
     __syncthreads();
     if (tid < nc) {
       for (int i = 0; i < b; ++i) {
-        double2 s = sx[i * (TRSM_COLS + 1) + tid], s2 = make_double2(0.0, 0.0);
-        int t = 0;
-        for (; t + 1 < i; t += 2) {  // two chains
-          s = cfms(D.S[t][i], sx[t * (TRSM_COLS + 1) + tid], s);
-          s2 = cfms(D.S[t + 1][i], sx[(t + 1) * (TRSM_COLS + 1) + tid], s2);
-        }
-        if (t < i) s = cfms(D.S[t][i], sx[t * (TRSM_COLS + 1) + tid], s);
-        s.x += s2.x;
-        s.y += s2.y;
+        double2 s = sx[i * (TRSM_COLS + 1) + tid];
+        for (int t = 0; t < i; ++t) s = cfms(D.S[t][i], sx[t * (TRSM_COLS + 1) + tid], s);
         sx[i * (TRSM_COLS + 1) + tid] = unit ? s : cmul(s, D.inv[i]);
       }
     }
@@ -298,7 +292,8 @@ __global__ void __launch_bounds__(TRSM_COLS) k_trsm_diag(const TrsmDesc* __restr
 
 // The update after a solved block for a few right-hand sides (nrhs <= TRSM_FEW): a thread per row,
 // 64 rows a CTA, so no lane works on columns that are not there (a 32 x 32 product tile spends
-// 31/32 of the FP64 pipe on them at one right-hand side).  Arguments as for k_trsm_update.
+// 31/32 of the FP64 pipe on them at one right-hand side).  Arguments as for k_trsm_update, whose
+// order of operations it keeps.
 #define TRSM_FEW 8
 __global__ void __launch_bounds__(64) k_trsm_update_few(const TrsmDesc* __restrict__ d, int j0, int jb, int lower) {
   __shared__ double2 sT[32][65];
@@ -332,13 +327,11 @@ __global__ void __launch_bounds__(64) k_trsm_update_few(const TrsmDesc* __restri
       for (int c = 0; c < TRSM_FEW; ++c) {
         if (c >= q.nrhs) break;
         double2* o = q.B + r0 + i0 + i + (int64_t)c * q.ldb;
-        double2 s = *o, s2 = make_double2(0.0, 0.0);
-#pragma unroll 4
-        for (int t = 0; t < 32; t += 2) {
-          s = cfms(sT[t][i], sb[t][c], s);
-          s2 = cfms(sT[t + 1][i], sb[t + 1][c], s2);
-        }
-        *o = make_double2(s.x + s2.x, s.y + s2.y);
+        double2 s = make_double2(0.0, 0.0);
+#pragma unroll 8
+        for (int t = 0; t < 32; ++t) s = cfma(sT[t][i], sb[t][c], s);
+        const double2 v = *o;
+        *o = make_double2(v.x - s.x, v.y - s.y);
       }
     }
   }
@@ -638,10 +631,11 @@ __global__ void __launch_bounds__(LUS_T) k_lu_solve_fused(const LuSolveDesc* __r
 #endif
 // TPC (thread per column): each thread updates whole trailing columns against the reflector
 // staged in shared memory (no warp reductions; the strided column loads stay in L1, and on
-// GB300 a warp-wide DFMA takes 16 clocks, which hides them).  Used when the reflector fits the
-// shared memory budget (m <= CPQR_TPC_MAXM).
+// GB300 a warp-wide DFMA takes 16 clocks, which hides them).  For matrices of up to CPQR_TPC_MAXM
+// rows, the sketches: 4096 of 128 x 256 take 108 ms, 195 with a warp per column; from 250 rows on
+// the two are within 3 to 12 % in large batches and the warps win in small ones.
 #ifndef CPQR_TPC_MAXM
-#define CPQR_TPC_MAXM 2048
+#define CPQR_TPC_MAXM 192
 #endif
 #define CPQR_CLUSTER_SMEM (192 * 1024)  // longest reflector of the cluster variant (12288 rows)
 // Warp variant: CB trailing columns per warp per pass (2*CB partial sums, a power of two <= 16).
@@ -652,6 +646,7 @@ __global__ void __launch_bounds__(256, CPQR_MINB) k_cpqr(const QrDesc* __restric
   extern __shared__ double2 su[];  // TPC: the reflector u = M[j:m, j]
   const QrDesc q = d[blockIdx.x];
   const int m = q.m, n = q.n;
+  if (TPC != (m <= CPQR_TPC_MAXM)) return;
   double2* M = q.A;
   const int64_t ld = q.lda;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
@@ -886,9 +881,11 @@ __global__ void __launch_bounds__(256, CPQR_MINB) k_cpqr(const QrDesc* __restric
   }
 }
 
-// One matrix per cluster of CTAs, for batches too small to fill the GPU with one CTA per matrix
-// (the upper tree levels: few boxes, the largest matrices).  The trailing columns are dealt to
-// the warps of the whole cluster, CB at a time.  Every CTA finds the pivot from the norms in
+// One matrix of more than CPQR_TPC_MAXM rows per cluster of 1 to 8 CTAs: more than one where there
+// are too few matrices to fill the GPU (the upper tree levels: few boxes, the largest matrices).
+// The trailing columns are dealt to the warps of the whole cluster, CB at a time; a column's sums
+// do not depend on which warp or how many CTAs take it, so a matrix has the same factor in every
+// batch.  Every CTA finds the pivot from the norms in
 // global memory by itself and stages the pivot column as the reflector in its own shared memory,
 // so a step costs two cluster barriers: one between that staging and the update (which overwrites
 // the pivot's slot with column j), one after the update (the ID of the 16384-node star, 64 to 256
@@ -898,8 +895,15 @@ __device__ __forceinline__ void cluster_sync_all() {
   asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
+__device__ __forceinline__ void cpqr_sync(uint32_t csize) {
+  if (csize == 1)
+    __syncthreads();
+  else
+    cluster_sync_all();
+}
+
 template <int CB>
-__global__ void __launch_bounds__(256, 3) k_cpqr_cluster(const QrDesc* __restrict__ d, int mode) {
+__global__ void __launch_bounds__(256, CB == 2 ? 3 : 2) k_cpqr_cluster(const QrDesc* __restrict__ d, int mode) {
   constexpr int SH = CB == 1 ? 4 : CB == 2 ? 3 : CB == 4 ? 2 : 1;  // 5 - log2(2 * CB)
   extern __shared__ double2 su[];  // the reflector u = (column p)[j : m]
   uint32_t rank, csize;
@@ -907,6 +911,7 @@ __global__ void __launch_bounds__(256, 3) k_cpqr_cluster(const QrDesc* __restric
   asm("mov.u32 %0, %%cluster_nctarank;" : "=r"(csize));
   const QrDesc q = d[blockIdx.x / csize];
   const int m = q.m, n = q.n;
+  if (m <= CPQR_TPC_MAXM) return;  // the thread-per-column kernel's
   double2* M = q.A;
   const int64_t ld = q.lda;
   const int tid = threadIdx.x, lane = tid & 31, nw = blockDim.x >> 5;
@@ -929,7 +934,7 @@ __global__ void __launch_bounds__(256, 3) k_cpqr_cluster(const QrDesc* __restric
       }
     }
   }
-  cluster_sync_all();
+  cpqr_sync(csize);
   const int kt = mode == 1 ? min(q.kt, kmax) : kmax;
   for (; j < kt; ++j) {
     // pivot: largest remaining norm (lowest index on ties)
@@ -991,7 +996,7 @@ __global__ void __launch_bounds__(256, 3) k_cpqr_cluster(const QrDesc* __restric
       s_tau = uu > 0.0 ? 2.0 / uu : 0.0;
       s_beta = beta;
     }
-    cluster_sync_all();
+    cpqr_sync(csize);
     const double tau = s_tau;
     if (rank == 0 && tid == 0) {
       q.tauv[j] = tau;
@@ -1085,7 +1090,7 @@ __global__ void __launch_bounds__(256, 3) k_cpqr_cluster(const QrDesc* __restric
           }
       }
     }
-    cluster_sync_all();
+    cpqr_sync(csize);
   }
   if (rank == 0 && tid == 0) {
     q.state[0] = j;
@@ -1230,38 +1235,51 @@ int wsbm_lu_solve_fused_batched(const LuSolveDesc* d_desc, int nbatch, int max_n
   return cudaGetLastError() == cudaSuccess ? 0 : -3;
 }
 
-int wsbm_cpqr_batched(const QrDesc* d_desc, int nbatch, int mode, int max_m, cudaStream_t st) {
+int wsbm_cpqr_tpc_rows() { return CPQR_TPC_MAXM; }
+
+template <int CB>
+static int launch_cpqr_cluster(const QrDesc* d_desc, int nbatch, int mode, int cl, int max_m, cudaStream_t st) {
+  const size_t sm = (size_t)max_m * sizeof(double2);
+  if (wsbm_smem_optin((const void*)k_cpqr_cluster<CB>, sm) != cudaSuccess) return -3;
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = cl;
+  at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+  cfg.gridDim = dim3((unsigned)(nbatch * cl));
+  cfg.blockDim = dim3(256);
+  cfg.dynamicSmemBytes = sm;
+  cfg.stream = st;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  wsbm_count_launch();
+  return cudaLaunchKernelEx(&cfg, k_cpqr_cluster<CB>, d_desc, mode) == cudaSuccess ? 0 : -3;
+}
+
+// The kernel is chosen per matrix, by its rows, so that its factor does not depend on the others of
+// the launch: each launch skips the matrices of the other kind.
+int wsbm_cpqr_batched(const QrDesc* d_desc, int nbatch, int nsmall, int mode, int max_m, cudaStream_t st) {
   if (nbatch <= 0) return 0;
   const WsbmTune tu = wsbm_tune_current();
-  // clusters of 2, 4 or 8 CTAs per matrix while the GPU holds them all at once (three per SM)
-  int cl = 1;
-  while (cl < 8 && (int64_t)nbatch * cl * 2 <= (int64_t)wsbm_sm_count() * 3) cl *= 2;
-  if (cl > 1 && (size_t)max_m * sizeof(double2) <= CPQR_CLUSTER_SMEM) {
-    const size_t sm = (size_t)max_m * sizeof(double2);
-    if (wsbm_smem_optin((const void*)k_cpqr_cluster<2>, sm) != cudaSuccess) return -3;
-    cudaLaunchConfig_t cfg = {};
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = cl;
-    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
-    cfg.gridDim = dim3((unsigned)(nbatch * cl));
-    cfg.blockDim = dim3(256);
-    cfg.dynamicSmemBytes = sm;
-    cfg.stream = st;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
-    if (cudaLaunchKernelEx(&cfg, k_cpqr_cluster<2>, d_desc, mode) != cudaSuccess) return -3;
-  } else if (max_m <= CPQR_TPC_MAXM) {
+  if (nsmall > 0) {
     const int thr = tu.cpqr_threads == 128 ? 128 : 256;
-    k_cpqr<true, CPQR_CB><<<nbatch, thr, (size_t)max_m * sizeof(double2), st>>>(d_desc, mode);
-  } else if (tu.cpqr_cb == 2) {
-    k_cpqr<false, 2><<<nbatch, 256, 0, st>>>(d_desc, mode);
-  } else if (tu.cpqr_cb == 8) {
-    k_cpqr<false, 8><<<nbatch, 256, 0, st>>>(d_desc, mode);
-  } else {
-    k_cpqr<false, 4><<<nbatch, 256, 0, st>>>(d_desc, mode);
+    k_cpqr<true, CPQR_CB><<<nbatch, thr, (size_t)std::min(max_m, CPQR_TPC_MAXM) * sizeof(double2), st>>>(d_desc, mode);
+    wsbm_count_launch();
   }
-  wsbm_count_launch();
+  const int nbig = nbatch - nsmall;
+  if (nbig > 0 && (size_t)max_m * sizeof(double2) <= CPQR_CLUSTER_SMEM) {
+    // 2, 4 or 8 CTAs per matrix while the GPU holds them all at once (three per SM)
+    int cl = 1;
+    while (cl < 8 && (int64_t)nbig * cl * 2 <= (int64_t)wsbm_sm_count() * 3) cl *= 2;
+    const int cb = max_m <= 2048 ? 2 : tu.cpqr_cb;
+    if (int rc = cb == 2   ? launch_cpqr_cluster<2>(d_desc, nbatch, mode, cl, max_m, st)
+                 : cb == 8 ? launch_cpqr_cluster<8>(d_desc, nbatch, mode, cl, max_m, st)
+                           : launch_cpqr_cluster<4>(d_desc, nbatch, mode, cl, max_m, st))
+      return rc;
+  } else if (nbig > 0) {  // a reflector beyond the shared memory of a CTA
+    k_cpqr<false, 4><<<nbatch, 256, 0, st>>>(d_desc, mode);
+    wsbm_count_launch();
+  }
   return cudaGetLastError() == cudaSuccess ? 0 : -3;
 }
 

@@ -67,7 +67,7 @@
 #define WSBM_TCSOLVE_WS ((size_t)4 << 30)  // digit-plane work space of one solve product launch
 #endif
 #ifndef WSBM_BIGLU_MIN
-#define WSBM_BIGLU_MIN 2048
+#define WSBM_BIGLU_MIN 512
 #endif
 #ifndef WSBM_SKETCH_CUT
 #define WSBM_SKETCH_CUT 0.25  // measured: far-field error 3.6-5.8x tol, as with the full QR
@@ -923,6 +923,12 @@ static int upload_instances(wsbm_hss* h0, const std::vector<wsbm_hss*>& hs, Inst
 // Algorithmic flops of the fused LU + solve of an n x n matrix with nrhs right-hand sides:
 // multipliers (one complex multiply, 6 flops) and trailing updates (one complex FMA, 8 flops) of
 // the LU, the forward and backward substitutions, and the pivot scalings of the back solve.
+static int small_qrs(const std::vector<QrDesc>& q) {
+  int n = 0;
+  for (const QrDesc& d : q) n += d.m <= wsbm_cpqr_tpc_rows();
+  return n;
+}
+
 static double lu_solve_flops(double n, double nrhs) {
   const double a = n * (n - 1) / 2, b = (n - 1) * n * (2 * n - 1) / 6;
   return 6 * a + 8 * b + 16 * a * nrhs + 6 * n * nrhs;
@@ -1206,7 +1212,7 @@ static int factor_levels(const std::vector<wsbm_hss*>& hs, const std::vector<int
   HC(cudaEventRecord(h0->ev[5], st));
   int qmax_m = 0;
   for (auto& q : qd) qmax_m = std::max(qmax_m, q.m);
-  HK(wsbm_cpqr_batched(dq, 2 * NB, 0, qmax_m, st));
+  HK(wsbm_cpqr_batched(dq, 2 * NB, small_qrs(qd), 0, qmax_m, st));
   HC(cudaEventRecord(h0->ev[6], st));
   *cpqr_mats = 2 * (int64_t)NB;
   std::vector<int32_t> hstate(4 * NB);
@@ -1251,7 +1257,7 @@ static int factor_levels(const std::vector<wsbm_hss*>& hs, const std::vector<int
     HK(upload(h0, redo, &dr, tmp));
     int rmax = 0;
     for (auto& q : redo) rmax = std::max(rmax, q.m);
-    HK(wsbm_cpqr_batched(dr, (int)redo.size(), 0, rmax, st));
+    HK(wsbm_cpqr_batched(dr, (int)redo.size(), small_qrs(redo), 0, rmax, st));
     std::vector<int32_t> hs2(4 * NB);
     HC(cudaMemcpyAsync(hs2.data(), state, hs2.size() * sizeof(int32_t), cudaMemcpyDeviceToHost, st));
     HC(cudaStreamSynchronize(st));
@@ -1281,7 +1287,7 @@ static int factor_levels(const std::vector<wsbm_hss*>& hs, const std::vector<int
     HK(upload(h0, more, &dm, tmp));
     int mmax = 0;
     for (auto& q : more) mmax = std::max(mmax, q.m);
-    HK(wsbm_cpqr_batched(dm, (int)more.size(), 1, mmax, st));
+    HK(wsbm_cpqr_batched(dm, (int)more.size(), small_qrs(more), 1, mmax, st));
   }
   {
     QrDesc* dfin = nullptr;  // the final descriptors (sketched sides may have been redone on M)

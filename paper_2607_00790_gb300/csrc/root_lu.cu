@@ -82,7 +82,7 @@ __global__ void __launch_bounds__(LUB_T, 1)
   double2* lcol = sm + (size_t)w * RS;
   __shared__ double2 prow[LUB_W];
   __shared__ double2 s_inv;
-  __shared__ unsigned long long red[LUB_T / 32];
+  __shared__ unsigned long long red[LUB_T / 32], keys[LUB_T / 32];
   __shared__ int s_err;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int b = blockIdx.x, G = gridDim.x;
@@ -108,58 +108,57 @@ __global__ void __launch_bounds__(LUB_T, 1)
     best = lub_warp_max(best);
     if (lane == 0) red[warp] = best;
     __syncthreads();
+    unsigned long long* row = slots + (size_t)j * LUB_MAXCTA;
     if (warp == 0) {
-      unsigned long long k = lub_warp_max(lane < LUB_T / 32 ? red[lane] : 0ull);
+      const unsigned long long k = lub_warp_max(lane < LUB_T / 32 ? red[lane] : 0ull);
       const int loc = (int)(0xFFFFFFFFu - (unsigned)k) - r0;
       double2* mine = cand + ((size_t)par * LUB_MAXCTA + b) * LUB_W;
       if (lane < w) __stcg(mine + lane, sm[lane * RS + loc]);
       if (b == 0 && lane < w) __stcg(diag + par * LUB_W + lane, sm[lane * RS + j]);
       __syncwarp();
-      unsigned long long* row = slots + (size_t)j * LUB_MAXCTA;
       if (lane == 0) st_release(row + b, k);
-      // all keys of this column (bounded)
-      unsigned long long top = 0;
-      bool ok = true;
-      for (int x = lane; x < G; x += 32) {
-        unsigned long long v = ld_acquire(row + x);
-        if (v == 0) {
-          const unsigned long long t0 = lub_time();
-          for (unsigned it = 1; (v = ld_acquire(row + x)) == 0; ++it) {
-            if ((it & 63) == 0 && (*(volatile int*)&g_lub_error || lub_time() - t0 > LUB_WAIT_NS)) {
-              atomicExch(&g_lub_error, 1);
-              ok = false;
-              break;
-            }
+    }
+    // all keys of this column, a thread each (bounded); a warp that read several in turn would wait
+    // for L2 several times
+    unsigned long long top = 0;
+    if (tid < G) {
+      top = ld_acquire(row + tid);
+      if (top == 0) {
+        const unsigned long long t0 = lub_time();
+        for (unsigned it = 1; (top = ld_acquire(row + tid)) == 0; ++it) {
+          if ((it & 63) == 0 && (*(volatile int*)&g_lub_error || lub_time() - t0 > LUB_WAIT_NS)) {
+            atomicExch(&g_lub_error, 1);
+            s_err = 1;
+            break;
           }
         }
-        top = v > top ? v : top;
       }
-      ok = __all_sync(0xFFFFFFFFu, ok);
-      top = lub_warp_max(top);
-      if (!ok) {
-        if (lane == 0) s_err = 1;
-      } else {
-        const int p = (int)(0xFFFFFFFFu - (unsigned)top), bp = (p - c0) / R;
-        if (lane < w) {
-          const double2 v = __ldcg(cand + ((size_t)par * LUB_MAXCTA + bp) * LUB_W + lane);
-          prow[lane] = v;
-          if (p != c) {
-            if (b == bp) sm[lane * RS + (p - r0)] = __ldcg(diag + par * LUB_W + lane);
-            if (b == 0) sm[lane * RS + j] = v;
-          }
-          if (lane == j) {
-            const bool zero = v.x == 0.0 && v.y == 0.0;
-            s_inv = zero ? make_double2(0.0, 0.0) : cdiv(make_double2(1.0, 0.0), v);
-            if (b == 0) {
-              piv[c] = p;
-              if (zero && info) info[0] = c + 1;
-            }
+    }
+    top = lub_warp_max(top);
+    if (lane == 0) keys[warp] = top;
+    __syncthreads();
+    if (s_err) return;
+    if (warp == 0) {
+      top = lub_warp_max(lane < LUB_T / 32 ? keys[lane] : 0ull);
+      const int p = (int)(0xFFFFFFFFu - (unsigned)top), bp = (p - c0) / R;
+      if (lane < w) {
+        const double2 v = __ldcg(cand + ((size_t)par * LUB_MAXCTA + bp) * LUB_W + lane);
+        prow[lane] = v;
+        if (p != c) {
+          if (b == bp) sm[lane * RS + (p - r0)] = __ldcg(diag + par * LUB_W + lane);
+          if (b == 0) sm[lane * RS + j] = v;
+        }
+        if (lane == j) {
+          const bool zero = v.x == 0.0 && v.y == 0.0;
+          s_inv = zero ? make_double2(0.0, 0.0) : cdiv(make_double2(1.0, 0.0), v);
+          if (b == 0) {
+            piv[c] = p;
+            if (zero && info) info[0] = c + 1;
           }
         }
       }
     }
     __syncthreads();
-    if (s_err) return;
     // rows below c: multipliers, then the rank-1 update of the columns to the right
     const int first = b == 0 ? j + 1 : 0;
     const double2 iv = s_inv;
