@@ -375,7 +375,11 @@ int wsbm_sketch(const void* A, int64_t lda, int32_t m, int32_t n, int32_t l, voi
  *   A  device complex128 m x k (lda >= m); B: k x n (ldb >= k); C: m x n (ldc >= m); all
  *      column-major; alpha, beta: host, 2 doubles (re, im) each
  *   1 <= k <= 32768
- * Work space (7 (m + 2n) 2k BF16 values, rounded up) from the library's allocator.
+ * Large products (m, n >= 512, k >= 160) are formed from the same scaled integers modulo 14 numbers
+ * instead (28 real products in place of 136, nothing dropped) and put together by the Chinese
+ * remainder theorem; same bound.
+ * Work space (7 (m + 2n) 2k BF16 values, rounded up; 28 (m + n) k for large products where the
+ * allocator has it) from the library's allocator.
  * Synchronous.  Errors: INVALID_ARG, OOM, CUDA, TIMEOUT (a bounded wait inside the kernel ran
  * out; the result is then incomplete). */
 int wsbm_zgemm(int32_t m, int32_t n, int32_t k, const double* alpha, const void* A, int64_t lda,
@@ -422,7 +426,7 @@ int wsbm_lu_dense(void* A, int64_t lda, int32_t n, int32_t* piv, void* stream);
  *   out[1]  panel width of the batched box LU, of {32, 64} (nbox boxes of n_box unknowns with
  *           nrhs_box right-hand sides each: the leaf level of a build);
  *   out[2], out[3]  outer panel width of the root LU, of {128, 256}, for roots below and from
- *           12288 unknowns; only the class of n_root is timed, the other keeps its value;
+ *           6144 unknowns; only the class of n_root is timed, the other keeps its value;
  *   out[4]  columns per warp pass of the column-pivoted QR of ID matrices of more than 2048
  *           rows, of {2, 4, 8} (152 matrices of 2560 x 128).
  * ms: host, 10 doubles or NULL: the candidates' times in that order.  Work space (two copies of

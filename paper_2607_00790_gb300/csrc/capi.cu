@@ -2,6 +2,7 @@
 #include <math.h>
 #include <string.h>
 
+#include <algorithm>
 #include <atomic>
 #include <map>
 #include <mutex>
@@ -342,10 +343,14 @@ extern "C" int wsbm_zgemm(int32_t m, int32_t n, int32_t k, const double* alpha, 
   cudaStream_t st = (cudaStream_t)stream;
   WsbmScratch scr(st);
   void* ws = nullptr;
-  int rc = scr.get(wsbm_zgemm_tc_ws_bytes(m, n, k), &ws);
+  // the work space of one piece, else (a limited allocator) the least that the product runs with
+  const size_t least = wsbm_zgemm_tc_ws_bytes(m, n, k);
+  size_t bytes = wsbm_zgemm_crt_fits(m, n, k) ? std::max(least, wsbm_zgemm_crt_ws_bytes(m, n, k)) : least;
+  int rc = scr.get(bytes, &ws);
+  if (rc == WSBM_ERR_OOM && bytes > least) rc = scr.get(bytes = least, &ws);
   if (rc) return rc;
   rc = wsbm_zgemm_tc(m, n, k, make_double2(alpha[0], alpha[1]), (const double2*)A, lda, (const double2*)B, ldb,
-                     make_double2(beta[0], beta[1]), (double2*)C, ldc, ws, st);
+                     make_double2(beta[0], beta[1]), (double2*)C, ldc, ws, bytes, st);
   if (rc == -1) return WSBM_ERR_INVALID_ARG;
   if (rc) return WSBM_ERR_CUDA;
   rc = wsbm_zgemm_tc_status(st);

@@ -33,12 +33,21 @@ struct WsbmTune {
 WsbmTune wsbm_tune_current();
 
 // tc_gemm.cu: C (m x n) = beta C + alpha A (m x k) B (k x n), complex128 column-major, on the
-// tensor cores from exact 8-bit digit planes (FP64-level accuracy).  ws: 256-byte aligned
-// device work space of wsbm_zgemm_tc_ws_bytes(m, n, k) bytes.  1 <= k <= 32768.  Returns 0,
-// -1 (bad arguments) or -3 (launch / tensor-map error); enqueues only.
+// tensor cores (FP64-level accuracy): large products from residues (crt_gemm.cu), the others from
+// exact 8-bit digit planes.  ws: 256-byte aligned device work space of ws_bytes >=
+// wsbm_zgemm_tc_ws_bytes(m, n, k) bytes (with wsbm_zgemm_crt_ws_bytes a large product runs in one
+// piece, with less in strips).  1 <= k <= 32768.  Returns 0, -1 (bad arguments) or -3 (launch /
+// tensor-map error); enqueues only.
 int wsbm_zgemm_tc(int m, int n, int k, double2 alpha, const double2* A, int64_t lda, const double2* B,
-                  int64_t ldb, double2 beta, double2* C, int64_t ldc, void* ws, cudaStream_t st);
+                  int64_t ldb, double2 beta, double2* C, int64_t ldc, void* ws, size_t ws_bytes, cudaStream_t st);
 size_t wsbm_zgemm_tc_ws_bytes(int m, int n, int k);
+// crt_gemm.cu: the product from residues alone.  Returns -2 (nothing launched) when ws_bytes is too
+// small even for strips.
+bool wsbm_zgemm_crt_fits(int m, int n, int k);
+size_t wsbm_zgemm_crt_ws_bytes(int m, int n, int k);
+int wsbm_zgemm_crt(int m, int n, int k, double2 alpha, const double2* A, int64_t lda, const double2* B, int64_t ldb,
+                   double2 beta, double2* C, int64_t ldc, void* ws, size_t ws_bytes, cudaStream_t st, int group);
+int wsbm_zgemm_crt_status();
 // Many products in one launch: C_i = beta C_i + alpha A_i B_i (sizes per item; K padded with
 // zeros to the largest k).  ws: 256-byte aligned, wsbm_zgemm_tc_batched_ws_bytes(p, n) bytes.
 // At most 65535 items.  Returns 0, -1 or -3; enqueues only (the item table is copied to ws).

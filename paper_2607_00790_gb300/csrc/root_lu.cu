@@ -21,7 +21,7 @@
 #define LUB_NB_BIG 256  // outer panel width from LUB_BIG_N on: deeper tensor-core products
 #endif
 #ifndef LUB_BIG_N
-#define LUB_BIG_N 12288
+#define LUB_BIG_N 6144  // (measured: n = 5000 equal, 8200 117 ms against 128, 16384 416 against 537)
 #endif
 #define LUB_W 32            // widest base panel: one lane per column
 #define LUB_T 256           // threads of a base-panel CTA
@@ -240,6 +240,7 @@ struct LubCtx {
   cudaStream_t st;
   int cs, ce;  // current outer panel
   void* tcws;  // work space of the tensor-core products
+  size_t tcb;  // and its size
 };
 
 // columns a base panel can take: every CTA holds its rows of them in shared memory
@@ -303,7 +304,7 @@ int lub_rec(const LubCtx& x, int c0, int c1, int base) {
   const double2 mone = make_double2(-1.0, 0.0), one = make_double2(1.0, 0.0);
   if (int rc = wsbm_zgemm_tc(x.n - mid, c1 - mid, mid - c0, mone, x.A + mid + (int64_t)c0 * x.lda, x.lda,
                              x.A + c0 + (int64_t)mid * x.lda, x.lda, one, x.A + mid + (int64_t)mid * x.lda, x.lda,
-                             x.tcws, x.st))
+                             x.tcws, x.tcb, x.st))
     return rc;
   return lub_rec(x, mid, c1, base);
 }
@@ -355,6 +356,7 @@ int wsbm_lu_big_nb(double2* A, int64_t lda, int n, int* piv, int* d_info, void* 
   x.diag = x.cand + (size_t)2 * LUB_MAXCTA * LUB_W;
   x.st = st;
   x.tcws = ws;
+  x.tcb = o_slots;
   const int base = lub_base_width(n);
   const double2 mone = make_double2(-1.0, 0.0), one = make_double2(1.0, 0.0), zero = make_double2(0.0, 0.0);
   for (int j0 = 0; j0 < n; j0 += nb) {
@@ -371,10 +373,10 @@ int wsbm_lu_big_nb(double2* A, int64_t lda, int n, int* piv, int* d_info, void* 
       const int m = n - je;
       if (int rc = lub_trsm(x, j0, jb, nullptr, jb, Linv)) return rc;
       if (int rc = wsbm_zgemm_tc(jb, m, jb, one, Linv, jb, A + j0 + (int64_t)je * lda, lda, zero,
-                                 A + j0 + (int64_t)je * lda, lda, ws, st))
+                                 A + j0 + (int64_t)je * lda, lda, ws, o_slots, st))
         return rc;
       if (int rc = wsbm_zgemm_tc(m, m, jb, mone, A + je + (int64_t)j0 * lda, lda, A + j0 + (int64_t)je * lda, lda,
-                                 one, A + je + (int64_t)je * lda, lda, ws, st))
+                                 one, A + je + (int64_t)je * lda, lda, ws, o_slots, st))
         return rc;
     }
   }

@@ -46,6 +46,7 @@
 #include <vector>
 
 #include "dense.h"
+#include "tc_ptx.cuh"
 
 #define TC_BM 128                       // output rows per tile (= TMEM lanes)
 #define TC_BN 64                        // real output columns per tile (32 complex)
@@ -64,67 +65,10 @@
 #define TC_THREADS 320                  // producer, MMA, 8 epilogue warps
 #define TC_EPI 256                      // epilogue threads (two per TMEM lane)
 #define TC_TMEM_COLS 512
-#define TC_WAIT_NS 2000000000ull        // bound of every barrier wait (2 s)
 
 static_assert(TC_STAGE_BYTES % 1024 == 0, "stage alignment");
 static_assert(TC_KC % TC_BK == 0, "chunk of whole stages");
 static_assert(TC_BK == 16 || TC_BK == 32, "rows of 32 bytes (32-byte swizzle) or 64 (64-byte swizzle)");
-
-static __device__ int g_tc_error;  // set when a bounded wait ran out
-
-// ----------------------------------------------------------------- PTX helpers ----
-__device__ __forceinline__ uint32_t smem_u32(const void* p) {
-  return (uint32_t)__cvta_generic_to_shared(p);
-}
-__device__ __forceinline__ uint64_t globaltimer() {
-  uint64_t t;
-  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-  return t;
-}
-__device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count));
-}
-__device__ __forceinline__ void mbar_expect_tx(uint32_t bar, uint32_t bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
-}
-__device__ __forceinline__ void mbar_arrive(uint32_t bar) {
-  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
-}
-__device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
-  uint32_t ok;
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-      "selp.u32 %0, 1, 0, p;\n\t}"
-      : "=r"(ok)
-      : "r"(bar), "r"(parity)
-      : "memory");
-  return ok != 0;
-}
-// Wait for the phase of parity `parity` of barrier `bar`, at most TC_WAIT_NS.
-__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity) {
-  if (mbar_try_wait(bar, parity)) return true;
-  const uint64_t t0 = globaltimer();
-  for (uint32_t it = 1;; ++it) {
-    if (mbar_try_wait(bar, parity)) return true;
-    if ((it & 255) == 0) {
-      if (*(volatile int*)&g_tc_error) return false;
-      if (globaltimer() - t0 > TC_WAIT_NS) {
-        atomicExch(&g_tc_error, 1);
-        return false;
-      }
-    }
-  }
-}
-__device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap* map, uint32_t bar, int c0,
-                                            int c1, int c2) {
-  asm volatile(
-      "cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5}], [%2];" ::"r"(dst),
-      "l"((uint64_t)map), "r"(bar), "r"(c0), "r"(c1), "r"(c2)
-      : "memory");
-}
-__device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
-__device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 
 // Shared-memory operand descriptor: K-major tile of TC_BK * 2-byte rows swizzled over the row
 // width (atoms of 8 rows, 8 * 2 TC_BK bytes apart), descriptor version 1; swizzle code 6 for
@@ -169,28 +113,6 @@ __device__ __forceinline__ void tc_sched(int e, int& t, int& u0, int& cnt) {
     case 9: t = 5, u0 = 0, cnt = 3; break;
     default: t = 6, u0 = 0, cnt = 2; break;
   }
-}
-
-__device__ __forceinline__ void tc_commit(uint32_t bar) {
-  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar)
-               : "memory");
-}
-__device__ __forceinline__ void tmem_ld8(uint32_t taddr, float* v) {
-  uint32_t r[8];
-  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
-               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
-               : "r"(taddr));
-#pragma unroll
-  for (int i = 0; i < 8; ++i) v[i] = __uint_as_float(r[i]);
-}
-__device__ __forceinline__ void tmem_ld_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
-
-// x 2^ex: exponent-field addition when x and the result are normal, else ldexp.
-__device__ __forceinline__ double scale2(double x, int ex) {
-  const long long b = __double_as_longlong(x);
-  const int e = (int)((b >> 52) & 0x7FF);
-  if (e > 0 && e + ex >= 1 && e + ex <= 2046) return __longlong_as_double(b + ((long long)ex << 52));
-  return ldexp(x, ex);
 }
 
 // (T + F 2^-16) 2^ex (F in [0, 2^16)) as the correctly rounded double (to nearest, ties to
@@ -239,16 +161,6 @@ __device__ __forceinline__ bool fixed_to_double(long long T, int F, int ex, doub
 }
 
 // --------------------------------------------------------------- digit planes ----
-// Exponent e with |v| < 2^(e-1) for every |Re|, |Im| of the row/column maximum `mx` (as raw
-// bits of a non-negative double); 0 for an all-zero row.
-__device__ __forceinline__ int scale_exp(uint64_t mxbits) {
-  if (mxbits == 0) return 0;
-  const int E = (int)(mxbits >> 52);
-  return (E > 0 ? E : 1) - 1021;
-}
-__device__ __forceinline__ uint64_t abs_bits(double v) {
-  return (uint64_t)__double_as_longlong(v) & 0x7FFFFFFFFFFFFFFFull;
-}
 // The seven balanced base-256 digits of X = v 2^(56 - e) (|v| < 2^(e-1)), most significant first.
 __device__ __forceinline__ void digits7(double v, int e, int* d) {
   const uint64_t b = (uint64_t)__double_as_longlong(v);
@@ -670,24 +582,6 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
 }
 
 // -------------------------------------------------------------------- host side ----
-typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
-                                  const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
-                                  CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-
-static EncodeTiledFn encode_fn() {
-  static std::once_flag once;
-  static EncodeTiledFn fn = nullptr;
-  std::call_once(once, [] {
-    void* p = nullptr;
-    cudaDriverEntryPointQueryResult q;
-    if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000, cudaEnableDefault, &q) ==
-            cudaSuccess &&
-        q == cudaDriverEntryPointSuccess)
-      fn = (EncodeTiledFn)p;
-  });
-  return fn;
-}
-
 static int64_t tc_ka(int k) { return ((int64_t)2 * k + TC_BK - 1) / TC_BK * TC_BK; }
 
 // Work space of a batched call: digit planes (rows of A and B' of all items, padded each to a
@@ -870,10 +764,16 @@ int wsbm_zgemm_tc_batched(const TcProduct* p, int nitems, double2 alpha, double2
 }
 
 int wsbm_zgemm_tc(int m, int n, int k, double2 alpha, const double2* A, int64_t lda, const double2* B,
-                  int64_t ldb, double2 beta, double2* C, int64_t ldc, void* ws, cudaStream_t st) {
+                  int64_t ldb, double2 beta, double2* C, int64_t ldc, void* ws, size_t ws_bytes, cudaStream_t st) {
   if (m < 0 || n < 0 || k < 0) return -1;
   if (m == 0 || n == 0) return 0;
   if (k < 1 || k > 32768) return -1;  // the 64-bit recombination is sized for K_real <= 65536
+  if (!ws || ((uintptr_t)ws & 255)) return -1;
+  const int group = wsbm_tune_current().tc_group;
+  if (wsbm_zgemm_crt_fits(m, n, k)) {
+    const int rc = wsbm_zgemm_crt(m, n, k, alpha, A, lda, B, ldb, beta, C, ldc, ws, ws_bytes, st, group);
+    if (rc != -2) return rc;
+  }
   TcProduct p;
   p.A = A;
   p.lda = lda;
@@ -885,7 +785,7 @@ int wsbm_zgemm_tc(int m, int n, int k, double2 alpha, const double2* A, int64_t 
   p.n = n;
   p.k = k;
   p.pad = 0;
-  return wsbm_zgemm_tc_batched(&p, 1, alpha, beta, ws, st);
+  return wsbm_zgemm_tc_batched_g(&p, 1, alpha, beta, ws, st, group);
 }
 
 // Error flag of the bounded waits: returns it and clears it (synchronizes the stream).
@@ -896,9 +796,10 @@ int wsbm_zgemm_tc_status(cudaStream_t st) {
   if (v) {
     const int zero = 0;
     cudaMemcpyToSymbol(g_tc_error, &zero, sizeof(int));
+    wsbm_zgemm_crt_status();
     return -5;
   }
-  return 0;
+  return wsbm_zgemm_crt_status();
 }
 
 // ------------------------------------------------ sketches Y = Omega M (Omega = +-1) ----
