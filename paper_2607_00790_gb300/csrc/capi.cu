@@ -245,6 +245,7 @@ extern "C" int wsbm_entries_raw(const wsbm_geom* g, const wsbm_params* p, const 
   cudaStream_t st = (cudaStream_t)stream;
   if (p->formulation == WSBM_FORM_WSBM) {
     if ((rc = wsbm_launch_entries_raw(wsbm_devgeom(g), ph, rows, nr, cols, nc, (double2*)out, st))) return rc;
+    // a handle passes its own stream: the caller's lists and result must be free to use on return
     return cudaStreamSynchronize(st) == cudaSuccess ? WSBM_OK : WSBM_ERR_CUDA;
   }
   WsbmScratch scr(st);
@@ -300,6 +301,12 @@ extern "C" int wsbm_proxy_block(const wsbm_geom* g, const wsbm_params* p, int32_
   if (nidx == 0) return WSBM_OK;
   if (!idx || !out) return WSBM_ERR_INVALID_ARG;
   cudaStream_t st = (cudaStream_t)stream;
+  if (p->formulation == WSBM_FORM_WSBM || side == 1) {
+    if ((rc = wsbm_launch_proxy_raw(wsbm_devgeom(g), ph, idx, nidx, side, cx, cy, rho, P, p->precision, (double2*)out,
+                                    st)))
+      return rc;
+    return cudaStreamSynchronize(st) == cudaSuccess ? WSBM_OK : WSBM_ERR_CUDA;  // complete on return, as the forms
+  }
   WsbmScratch scr(st);
   int32_t* buf = nullptr;
   ProxyTask* dtask = nullptr;
@@ -317,17 +324,14 @@ extern "C" int wsbm_proxy_block(const wsbm_geom* g, const wsbm_params* p, int32_
     t.nn = (int32_t)nidx;
     t.P = P;
     t.side = side;
-    t.tr = side == 0 ? 1 : 0;  // row block: box equations are the rows of the output
-    t.ld = side == 0 ? nidx : 2 * (int64_t)P;
+    t.tr = 1;  // box equations are the rows of the output
+    t.ld = nidx;
     t.off = 0;
     t.tile0 = 0;
     DevGeom dg = wsbm_devgeom(g);
     if ((rc = wsbm_launch_unknowns_to_slots(idx, nidx, g->n, buf, buf + nidx, st))) goto done;
     CK(cudaMemcpyAsync(dtask, &t, sizeof(t), cudaMemcpyHostToDevice, st));
-    if (side == 0 && p->formulation != WSBM_FORM_WSBM)
-      rc = wsbm_launch_proxy_rows_form(p->formulation, dg, ph, dtask, 1, wsbm_proxy_tiles(t.nn, P), st);
-    else
-      rc = wsbm_launch_proxy(dg, ph, dtask, 1, wsbm_proxy_tiles(t.nn, P), p->precision, st);
+    rc = wsbm_launch_proxy_rows_form(p->formulation, dg, ph, dtask, 1, wsbm_proxy_tiles(t.nn, P), st);
     CK(cudaStreamSynchronize(st));
   }
 done:

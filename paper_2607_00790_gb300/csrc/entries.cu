@@ -216,6 +216,9 @@ __device__ __forceinline__ void load_raw_slot(const DevGeom& g, const int64_t* i
   s.d.ny = g.ny[node];
   s.d.w = g.w[node];
   s.d.kap = g.kappa[node];
+  s.d.fnx = (float)s.d.nx;
+  s.d.fny = (float)s.d.ny;
+  s.d.fw = (float)s.d.w;
   s.d.fx = (float)s.d.x;
   s.d.fy = (float)s.d.y;
 }
@@ -421,6 +424,51 @@ __device__ __forceinline__ void proxy_col_fp64(const HkTables& T, const Phys& ph
   }
 }
 
+// The same two blocks with both arguments in the range of hankel_fixed: amplitudes and constants folded
+// into real factors of the unit-amplitude values (as block_fixed does): about half the FP64 operations
+// outside the functions themselves.  The pair is bound by the FP64 pipe (one instruction a warp in 18
+// cycles), so the count is the time.
+__device__ __forceinline__ void proxy_row_fixed(const HkTables& T, const Phys& ph, const SlotData& X, const ProxyPt& p,
+                                                double pw, double dx, double dy, double r2, double2 o[2][2]) {
+  const double ir = rsqrt3(r2), r = sqrt_from(r2, ir), z1 = ph.k1 * r;
+  const double dnu = fma(dx, p.pnx, dy * p.pny) * ir, dnx = fma(dx, X.nx, dy * X.ny) * ir;
+  const double c = dnx * dnu, m2c = fma(-2.0, c, fma(X.nx, p.pnx, X.ny * p.pny)) * ir;
+  const double a1 = pw * (0.25 * WSBM_SQRT_2_OVER_PI) * rsqrt3(z1);
+  HxUnit h;
+#pragma unroll
+  for (int s = 0; s < 2; ++s) {
+    const double k = s == 0 ? ph.k1 : ph.k0, a = s == 0 ? a1 : a1 * ph.s10;
+    hankel_fixed(T.near_, s == 0 ? z1 : ph.k0 * r, ir * (s == 0 ? ph.inv_k1 : ph.inv_k0), h);
+    // pw Phi = v (h0 + i dnu h1);  alpha pw dPhi = -w2 [h0 c + h1 m2c / (k r) + i h1 dnx]
+    const double v = a * k, vd = v * dnu, w2 = v * (s == 0 ? k * ph.inv_k0 : 1.0);
+    const double w0 = w2 * c, w1 = w2 * (s == 0 ? ph.inv_k1 : ph.inv_k0) * m2c, wd = w2 * dnx;
+    const double phr = fma(-vd, h.i1, v * h.r0), phi = fma(vd, h.r1, v * h.i0);
+    const double adr = fma(wd, h.i1, fma(-w0, h.r0, -w1 * h.r1)), adi = fma(-wd, h.r1, fma(-w0, h.i0, -w1 * h.i1));
+    if (s == 0) {
+      o[0][0] = make_double2(phr, phi);
+      o[0][1] = make_double2(-adr, -adi);
+    } else {
+      o[1][0] = make_double2(0.0, 0.0);
+      o[1][1] = make_double2(phr + adr, phi + adi);
+    }
+  }
+}
+__device__ __forceinline__ void proxy_col_fixed(const HkTables& T, const Phys& ph, const SlotData& Y, double dx, double dy,
+                                                double r2, double2 o[2][2]) {
+  const double ir = rsqrt3(r2), r = sqrt_from(r2, ir), z1 = ph.k1 * r;
+  const double a1 = Y.w * (0.25 * WSBM_SQRT_2_OVER_PI) * rsqrt3(z1);
+  const double dny = fma(dx, Y.nx, dy * Y.ny) * ir;
+  HxUnit h;
+#pragma unroll
+  for (int s = 0; s < 2; ++s) {
+    const double a = s == 0 ? a1 : a1 * ph.s10;
+    hankel_fixed(T.near_, s == 0 ? z1 : ph.k0 * r, ir * (s == 0 ? ph.inv_k1 : ph.inv_k0), h);
+    const double u = a * (s == 0 ? ph.k1 : ph.k0) * dny, q = a * (s == 0 ? ph.eps1 : ph.eps0);
+    o[s][0] = make_double2(-u * h.i1, u * h.r1);
+    o[s][1] = make_double2(q * h.i0, -q * h.r0);
+  }
+}
+
 // Mixed precision versions: z = k r formed in FP64 and reduced mod 2 pi in FP64; amplitude and
 // entry algebra in FP32.
 // sqrt of r2 > 0 for the mixed path: FP64 reciprocal-square-root seed and one Newton step
@@ -530,6 +578,45 @@ __device__ __forceinline__ void proxy_col_mixed(const HkTables& T, const Phys& p
   }
 }
 
+// One node / proxy-point block, by mode (WSBM_FP64, WSBM_MIXED or WSBM_MIXED_FINE) and side.
+template <int MODE>
+__device__ __forceinline__ void proxy_pair(const HkTables& T, const Phys& ph, int side, const SlotData& X,
+                                           const ProxyPt& p, double pw, double2 o[2][2]) {
+  if (MODE == WSBM_FP64) {
+    const double dx = side == 0 ? X.x - p.px : p.px - X.x, dy = side == 0 ? X.y - p.py : p.py - X.y;
+    const double r2 = pair_r2(dx, dy);
+    if (pair_is_fixed(ph, r2)) {
+      if (side == 0)
+        proxy_row_fixed(T, ph, X, p, pw, dx, dy, r2, o);
+      else
+        proxy_col_fixed(T, ph, X, dx, dy, r2, o);
+      return;
+    }
+  }
+  if (side == 0) {
+    if (MODE == WSBM_MIXED)
+      proxy_row_mixed(T, ph, X, p, pw, o);
+    else
+      proxy_row_fp64<MODE == WSBM_MIXED_FINE>(T, ph, X, p, pw, o);
+  } else {
+    if (MODE == WSBM_MIXED)
+      proxy_col_mixed(T, ph, X, p, o);
+    else
+      proxy_col_fp64<MODE == WSBM_MIXED_FINE>(T, ph, X, p, o);
+  }
+}
+
+__device__ __forceinline__ void load_proxy_pt(double cx, double cy, double rho, int P, int m, ProxyPt& p) {
+  double sn, cs;
+  sincospi(2.0 * (double)m / (double)P, &sn, &cs);
+  p.pnx = cs;
+  p.pny = sn;
+  p.fpnx = (float)cs;
+  p.fpny = (float)sn;
+  p.px = cx + rho * cs;
+  p.py = cy + rho * sn;
+}
+
 // MODE: WSBM_FP64, WSBM_MIXED or WSBM_MIXED_FINE
 template <int MODE, int TF>
 __global__ void __launch_bounds__(WSBM_PAIR_THREADS)
@@ -539,6 +626,7 @@ __global__ void __launch_bounds__(WSBM_PAIR_THREADS)
   __shared__ HkTables T;
   __shared__ ProxyPt sp[TF];
   __shared__ SlotData ss[TS];
+  __shared__ double s_pw;  // one FP64 division per tile, not per pair
   hk_stage_tables(&T);
   const int tx = threadIdx.x & (TF - 1);
   const int ty = threadIdx.x / TF;
@@ -556,15 +644,9 @@ __global__ void __launch_bounds__(WSBM_PAIR_THREADS)
     if (threadIdx.x < TF) {
       int m = m0 + threadIdx.x;
       if (m < tk.P) {
-        double sn, cs;
-        sincospi(2.0 * (double)m / (double)tk.P, &sn, &cs);
-        sp[threadIdx.x].pnx = cs;
-        sp[threadIdx.x].pny = sn;
-        sp[threadIdx.x].fpnx = (float)cs;
-        sp[threadIdx.x].fpny = (float)sn;
-        sp[threadIdx.x].px = tk.cx + tk.rho * cs;
-        sp[threadIdx.x].py = tk.cy + tk.rho * sn;
+        load_proxy_pt(tk.cx, tk.cy, tk.rho, tk.P, m, sp[threadIdx.x]);
       }
+      if (threadIdx.x == 0) s_pw = 2.0 * WSBM_PI * tk.rho / (double)tk.P;
     } else if (threadIdx.x < TF + TS) {
       int k = threadIdx.x - TF;
       if (s0 + k < tk.nn) load_slot(g, tk.node, tk.pos, s0 + k, ss[k]);
@@ -574,18 +656,7 @@ __global__ void __launch_bounds__(WSBM_PAIR_THREADS)
     if (m < tk.P && s < tk.nn) {
       double2 o[2][2];
       const SlotData& X = ss[ty];
-      if (tk.side == 0) {
-        double pw = 2.0 * WSBM_PI * tk.rho / (double)tk.P;
-        if (MODE == WSBM_MIXED)
-          proxy_row_mixed(T, ph, X, sp[tx], pw, o);
-        else
-          proxy_row_fp64<MODE == WSBM_MIXED_FINE>(T, ph, X, sp[tx], pw, o);
-      } else {
-        if (MODE == WSBM_MIXED)
-          proxy_col_mixed(T, ph, X, sp[tx], o);
-        else
-          proxy_col_fp64<MODE == WSBM_MIXED_FINE>(T, ph, X, sp[tx], o);
-      }
+      proxy_pair<MODE>(T, ph, tk.side, X, sp[tx], s_pw, o);
       const int bp[2] = {X.p0, X.p1};
 #pragma unroll
       for (int sgn = 0; sgn < 2; ++sgn) {
@@ -600,6 +671,77 @@ __global__ void __launch_bounds__(WSBM_PAIR_THREADS)
       }
     }
   }
+}
+
+// Proxy block of one box by index list, one launch without work space: a tile takes RAW_F proxy points
+// and RAW_S list slots, slot t being the pair (t, t + ceil(n/2)) as in k_entries_raw: a node whose two
+// unknowns share a slot is evaluated once for both.  Output of the row side nidx x 2P, of the column
+// side 2P x nidx, column-major.  1500 unknowns (750 nodes) by 712 points: 300 us before (index pass, task
+// copy, one block for each unknown, half of it dropped), 135 us with both unknowns from one block and the
+// folded factors.
+template <int MODE>
+__global__ void __launch_bounds__(RAW_F* RAW_S)
+    k_proxy_raw(DevGeom g, const __grid_constant__ Phys ph, const int64_t* __restrict__ idx, int64_t n, int side,
+                double cx, double cy, double rho, int P, double2* __restrict__ out) {
+  __shared__ HkTables T;
+  __shared__ ProxyPt sp[RAW_F];
+  __shared__ RawSlot ss[2][RAW_S];
+  hk_stage_tables(&T);
+  const int tid = threadIdx.x, tx = tid & (RAW_F - 1), ty = tid / RAW_F;
+  const int64_t h = (n + 1) / 2;
+  const int ntp = (P + RAW_F - 1) / RAW_F;
+  const int64_t ntiles = ntp * ((h + RAW_S - 1) / RAW_S);
+  const double pw = 2.0 * WSBM_PI * rho / (double)P;
+  for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
+    const int m = (int)(tile % ntp) * RAW_F + tx;
+    const int64_t t0 = (tile / ntp) * RAW_S;
+    __syncthreads();
+    if (tid < RAW_F) {
+      if (m < P) load_proxy_pt(cx, cy, rho, P, m, sp[tid]);
+    } else if (tid < RAW_F + 2 * RAW_S) {
+      const int half = (tid - RAW_F) / RAW_S, t = (tid - RAW_F) % RAW_S;
+      ss[half][t].comp = -1;
+      if (t0 + t < h) load_raw_slot(g, idx, t0 + t + half * h, n, ss[half][t]);
+    }
+    __syncthreads();
+    const RawSlot &s0 = ss[0][ty], &s1 = ss[1][ty];
+    const bool whole = s0.comp == 0 && s1.comp == 1 && s0.d.node == s1.d.node;  // the same for a warp
+    if (m < P) {
+#pragma unroll 1
+      for (int q = 0; q < (whole ? 1 : 2); ++q) {
+        const RawSlot& s = ss[q][ty];
+        if (s.comp < 0) continue;
+        double2 o[2][2];
+        proxy_pair<MODE>(T, ph, side, s.d, sp[tx], pw, o);
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {  // k1, then k0
+          const int64_t prow = (int64_t)k * P + m, t = t0 + ty;
+          auto at = [&](int64_t e) { return side == 0 ? e + prow * n : prow + e * 2 * P; };
+          if (whole) {
+            out[at(t)] = o[k][0];
+            out[at(t + h)] = o[k][1];
+          } else {
+            out[at(t + q * h)] = s.comp == 0 ? o[k][0] : o[k][1];
+          }
+        }
+      }
+    }
+  }
+}
+
+int wsbm_launch_proxy_raw(const DevGeom& g, const Phys& ph, const int64_t* idx, int64_t n, int side, double cx,
+                          double cy, double rho, int P, int mode, double2* out, cudaStream_t st) {
+  const int64_t ntiles = (int64_t)((P + RAW_F - 1) / RAW_F) * (((n + 1) / 2 + RAW_S - 1) / RAW_S);
+  const int64_t cap = (int64_t)wsbm_sm_count() * WSBM_ENTRY_CTAS;
+  const int gr = (int)(ntiles < cap ? ntiles : cap);
+  if (mode == WSBM_MIXED)
+    k_proxy_raw<WSBM_MIXED><<<gr, RAW_F * RAW_S, 0, st>>>(g, ph, idx, n, side, cx, cy, rho, P, out);
+  else if (mode == WSBM_MIXED_FINE)
+    k_proxy_raw<WSBM_MIXED_FINE><<<gr, RAW_F * RAW_S, 0, st>>>(g, ph, idx, n, side, cx, cy, rho, P, out);
+  else
+    k_proxy_raw<WSBM_FP64><<<gr, RAW_F * RAW_S, 0, st>>>(g, ph, idx, n, side, cx, cy, rho, P, out);
+  wsbm_count_launch();
+  return cudaGetLastError() == cudaSuccess ? WSBM_OK : WSBM_ERR_CUDA;
 }
 
 // -------------------------------------------------------------- Hankel test kernel ----

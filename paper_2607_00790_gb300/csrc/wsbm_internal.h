@@ -97,6 +97,9 @@ int64_t wsbm_proxy_tiles(int32_t nn, int32_t P, int tf = WSBM_TILE_F);
 // launch, no work space.
 int wsbm_launch_entries_raw(const DevGeom& g, const Phys& ph, const int64_t* rows, int64_t nr, const int64_t* cols,
                             int64_t nc, double2* out, cudaStream_t st);
+// Proxy block of one box (wsbm_proxy_block) for a device index list: one launch, no work space.
+int wsbm_launch_proxy_raw(const DevGeom& g, const Phys& ph, const int64_t* idx, int64_t n, int side, double cx,
+                          double cy, double rho, int P, int mode, double2* out, cudaStream_t st);
 int wsbm_launch_hankel(const double* z, int64_t n, double* out, int mixed, cudaStream_t st);
 int wsbm_launch_unknowns_to_slots(const int64_t* idx, int64_t n, int64_t N, int32_t* node,
                                   int32_t* pos, cudaStream_t st);
