@@ -208,26 +208,58 @@ struct TrsmStage {
   double2 S[32][33];  // S[t][i]: column t, row i of the triangle
   double2 inv[32];
 };
+__device__ __forceinline__ double2 trsm_elem(const TrsmDesc& q, int j0, int b, int e) {
+  const int a = e & 31, c = e >> 5;  // element (a, c) of the stored block
+  return a < b && c < b ? q.T[(j0 + a) + (int64_t)(j0 + c) * q.ldt] : make_double2(0.0, 0.0);
+}
+__device__ __forceinline__ void trsm_put(TrsmStage& D, const TrsmDesc& q, int b, bool fwd, int e, double2 v) {
+  const int a = e & 31, c = e >> 5;
+  int i = q.trans ? c : a, t = q.trans ? a : c;
+  if (a < b && c < b && !fwd) {
+    i = b - 1 - i;
+    t = b - 1 - t;
+  }
+  D.S[t][i] = v;  // read where i >= t only
+}
+// The reciprocals by one warp at once: a division in the loop above would run for the one diagonal lane
+// of every pass, 32 times a block.  The columns are scaled by them, which takes a complex product out
+// of every step of the chain: x_i = r_i / S_ii with r_i = b_i - sum (S_it / S_tt) r_t.
+__device__ __forceinline__ void trsm_reciprocals(TrsmStage& D, int b, bool unit) {
+  __syncthreads();
+  const int i = threadIdx.x;
+  if (unit) return;
+  if (i < 32) D.inv[i] = i >= b ? make_double2(1.0, 0.0) : cdiv(make_double2(1.0, 0.0), D.S[i][i]);
+  __syncthreads();
+  for (int e = i; e < 32 * 32; e += blockDim.x)
+    if ((e & 31) > (e >> 5)) D.S[e >> 5][e & 31] = cmul(D.S[e >> 5][e & 31], D.inv[e >> 5]);
+  __syncthreads();
+}
 __device__ __forceinline__ void trsm_stage(TrsmStage& D, const TrsmDesc& q, int j0, int jb, bool fwd, bool unit) {
   const int b = min(jb, q.n - j0);
-  const double2 zero = make_double2(0.0, 0.0);
-  for (int e = threadIdx.x; e < 32 * 32; e += blockDim.x) {
-    const int a = e & 31, c = e >> 5;  // element (a, c) of the stored block
-    const bool in = a < b && c < b;
-    const double2 v = in ? q.T[(j0 + a) + (int64_t)(j0 + c) * q.ldt] : zero;
-    int i = q.trans ? c : a, t = q.trans ? a : c;
-    if (in && !fwd) {
-      i = b - 1 - i;
-      t = b - 1 - t;
-    }
-    D.S[t][i] = v;  // read where i > t only
-    if (i == t) D.inv[i] = unit || !in ? make_double2(1.0, 0.0) : cdiv(make_double2(1.0, 0.0), v);
+  for (int e0 = threadIdx.x; e0 < 32 * 32; e0 += 8 * blockDim.x) {  // blockDim.x = 64 or 128: 8 loads in flight
+    double2 v[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) v[k] = trsm_elem(q, j0, b, e0 + k * blockDim.x);
+#pragma unroll
+    for (int k = 0; k < 8; ++k) trsm_put(D, q, b, fwd, e0 + k * blockDim.x, v[k]);
   }
-  __syncthreads();
+  trsm_reciprocals(D, b, unit);
+}
+
+// One column of the staged block by a warp, row `lane` of the solve's order in each lane's x.
+__device__ __forceinline__ double2 trsm_warp_column(const TrsmStage& D, int b, bool unit, double2 x) {
+  const int lane = threadIdx.x & 31;
+  for (int t = 0; t < b; ++t) {
+    double2 xt;
+    xt.x = __shfl_sync(0xFFFFFFFFu, x.x, t);
+    xt.y = __shfl_sync(0xFFFFFFFFu, x.y, t);
+    if (lane > t) x = cfms(D.S[t][lane], xt, x);
+  }
+  return unit ? x : cmul(x, D.inv[lane]);
 }
 
 // Few columns (up to a few thousand in the launch): one warp per column, its row `lane` in each
-// lane's register: about 2 us a block, where a thread per column takes 512 dependent steps.
+// lane's register: 32 dependent steps a block, where a thread per column takes 512.
 __global__ void __launch_bounds__(128) k_trsm_diag_warp(const TrsmDesc* __restrict__ d, int j0, int jb, int fwd) {
   __shared__ TrsmStage D;
   const TrsmDesc q = d[blockIdx.y];
@@ -238,19 +270,7 @@ __global__ void __launch_bounds__(128) k_trsm_diag_warp(const TrsmDesc* __restri
   const int b = min(jb, q.n - j0), row = j0 + (fwd ? lane : b - 1 - lane);
   for (int c = blockIdx.x * 4 + (threadIdx.x >> 5); c < q.nrhs; c += gridDim.x * 4) {
     double2* col = q.B + (int64_t)c * q.ldb;
-    double2 x = lane < b ? col[row] : make_double2(0.0, 0.0);
-    const double2 iv = D.inv[lane];
-    for (int t = 0; t < b; ++t) {
-      double2 xt;
-      xt.x = __shfl_sync(0xFFFFFFFFu, x.x, t);
-      xt.y = __shfl_sync(0xFFFFFFFFu, x.y, t);
-      if (!unit) {
-        const double2 it = D.inv[t];
-        xt = cmul(xt, it);
-      }
-      if (lane > t) x = cfms(D.S[t][lane], xt, x);
-    }
-    if (!unit) x = cmul(x, iv);
+    const double2 x = trsm_warp_column(D, b, unit, lane < b ? col[row] : make_double2(0.0, 0.0));
     if (lane < b) col[row] = x;
   }
 }
@@ -279,8 +299,10 @@ __global__ void __launch_bounds__(TRSM_COLS) k_trsm_diag(const TrsmDesc* __restr
       for (int i = 0; i < b; ++i) {
         double2 s = sx[i * (TRSM_COLS + 1) + tid];
         for (int t = 0; t < i; ++t) s = cfms(D.S[t][i], sx[t * (TRSM_COLS + 1) + tid], s);
-        sx[i * (TRSM_COLS + 1) + tid] = unit ? s : cmul(s, D.inv[i]);
+        sx[i * (TRSM_COLS + 1) + tid] = s;
       }
+      if (!unit)
+        for (int i = 0; i < b; ++i) sx[i * (TRSM_COLS + 1) + tid] = cmul(sx[i * (TRSM_COLS + 1) + tid], D.inv[i]);
     }
     __syncthreads();
     for (int e = tid; e < 32 * TRSM_COLS; e += TRSM_COLS) {
@@ -335,6 +357,129 @@ __global__ void __launch_bounds__(64) k_trsm_update_few(const TrsmDesc* __restri
       }
     }
   }
+}
+
+// One step for a few right-hand sides of a few matrices, a column a CTA: the update by the solved block
+// [j0, j0 + jb), and the next block, solved by the CTA that has just updated its rows (tiles of 32 rows
+// count from the solved block, so these are tile 0's, and stay in their registers).
+// A step is a chain of FP64 instructions, and a sub-partition takes 64 clocks for each of them, whatever
+// else it holds: so a lane has one real component of a row instead of a row (half the instructions a
+// warp), and the two halves of the rows run on two sub-partitions, the second taking the first one's
+// solutions 8 at a time.  What does not depend on B (the triangle, its reciprocals, the tile of T) is
+// fetched before the wait for the step before, by programmatic launch: T is complete by then, as the
+// first block's solve is an ordinary launch.  Every CTA waits, also one without work: a step's end has
+// to mean that all steps before it ended.  The order of operations is that of the separate kernels.
+// n = 2200, one right-hand side: 8.3 us a step (update 2.9, solve 4.2, the rest launch and exchange),
+// 27 us as two launches with a row a lane.
+#define TRSM_ST 64
+__global__ void __launch_bounds__(TRSM_ST) k_trsm_step_few(const TrsmDesc* __restrict__ d, int j0, int jb, int lower) {
+  __shared__ TrsmStage D;
+  __shared__ double2 sT[32][33];
+  __shared__ double sb[32][2], xs[16][2];  // re, im of the solved block; of the first half of the next
+  const TrsmDesc q = d[blockIdx.y];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, c = blockIdx.z;
+  const int i = 16 * warp + (lane >> 1), part = lane & 1;  // row in the order of the solve; re or im
+  const int neg = part ? 0 : -1;
+  auto flip = [](double v, int f) {  // -v where f: on the integer pipe
+    return __hiloint2double(__double2hiint(v) ^ (f & 0x80000000), __double2loint(v));
+  };
+  const int je = min(j0 + jb, q.n), kb = max(0, je - j0);  // kb = 0: this matrix begins at a later block
+  const int jn = lower ? j0 + jb : j0 - jb;
+  const int m = kb == 0 ? 0 : lower ? q.n - je : j0;
+  const bool solve = blockIdx.x == 0 && jn >= 0 && jn < q.n;
+  const int b = min(jb, q.n - jn);
+  const bool unit = (lower != 0) != (q.trans != 0);
+  const int ntile = c < q.nrhs ? max((m + 31) / 32, solve ? 1 : 0) : 0;
+  auto load_tile = [&](int tile) {  // sT[t][row of the tile, in the order of the solve]
+    const int r = lower ? je + 32 * tile : j0 - 32 * tile - 1, mm = min(32, m - 32 * tile);
+    double2 v[1024 / TRSM_ST];
+#pragma unroll
+    for (int e = 0; e < 1024 / TRSM_ST; ++e) {
+      const int o = warp + e * (TRSM_ST / 32);
+      const int a = q.trans ? o : lane, t = q.trans ? lane : o;  // op(T)[row a, j0 + t], contiguous in lane
+      const int64_t row = lower ? r + a : r - a;
+      v[e] = t < kb && a < mm ? (q.trans ? q.T[j0 + t + row * q.ldt] : q.T[row + (int64_t)(j0 + t) * q.ldt])
+                              : make_double2(0.0, 0.0);
+    }
+#pragma unroll
+    for (int e = 0; e < 1024 / TRSM_ST; ++e) {
+      const int o = warp + e * (TRSM_ST / 32);
+      sT[q.trans ? lane : o][q.trans ? o : lane] = v[e];
+    }
+  };
+  if ((int)blockIdx.x < ntile) {
+    load_tile(blockIdx.x);
+    if (solve) trsm_stage(D, q, jn, jb, lower != 0, unit);
+  }
+  cudaGridDependencySynchronize();
+  cudaTriggerProgrammaticLaunchCompletion();
+  double2* col = q.B + (int64_t)c * q.ldb;
+  for (int tile = blockIdx.x; tile < ntile; tile += gridDim.x) {
+    __syncthreads();
+    if (tile != (int)blockIdx.x) load_tile(tile);
+    const bool last = tile == 0 && solve;
+    const int mm = last ? b : min(32, m - 32 * tile);
+    const int row = lower ? jn + 32 * tile + i : last ? jn + b - 1 - i : j0 - 32 * tile - 1 - i;
+    double x = i < mm ? __ldcg((const double*)(col + row) + part) : 0.0;
+    if (kb > 0) {
+      const int t = threadIdx.x >> 1;
+      sb[t][part] = t < kb ? __ldcg((const double*)(col + j0 + t) + part) : 0.0;
+      __syncthreads();
+      double s = 0.0;
+#pragma unroll 8
+      for (int t = 0; t < 32; ++t) {  // cfma, one component
+        const double2 v = sT[t][i];
+        s = fma(v.x, sb[t][part], fma(flip(v.y, neg), sb[t][1 - part], s));
+      }
+      x -= s;
+    }
+    if (last) {
+      auto take = [&](int t, double own, double other) {  // cfms, one component
+        const double2 v = D.S[t][i];
+        if (i > t) x = fma(-v.x, own, fma(flip(v.y, ~neg), other, x));
+      };
+      auto solve16 = [&](int t0, int t1) {  // rows t0 .. t1 - 1 of this warp's 16
+        for (int t = t0; t < t1; ++t) {
+          const int l = 2 * (t & 15);
+          const double own = __shfl_sync(0xFFFFFFFFu, x, l + part), other = __shfl_sync(0xFFFFFFFFu, x, l + 1 - part);
+          take(t, own, other);
+        }
+      };
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        if (warp == 0) {
+          solve16(8 * h, min(b, 8 * h + 8));
+          if (i >= 8 * h && i < 8 * h + 8) xs[i][part] = x;
+        }
+        asm volatile("bar.sync %0, 64;" ::"r"(1 + h) : "memory");
+        if (warp == 1) {
+#pragma unroll
+          for (int k = 0; k < 8; ++k)
+            if (8 * h + k < b) take(8 * h + k, xs[8 * h + k][part], xs[8 * h + k][1 - part]);
+        }
+      }
+      if (warp == 1) solve16(16, b);
+      if (!unit) {
+        const double y = __shfl_xor_sync(0xFFFFFFFFu, x, 1);
+        const double2 r = cmul(part ? make_double2(y, x) : make_double2(x, y), D.inv[i]);
+        x = part ? r.y : r.x;
+      }
+    }
+    if (i < mm) ((double*)(col + row))[part] = x;
+  }
+}
+
+static cudaError_t launch_trsm_step(dim3 grid, const TrsmDesc* d, int j0, int lower, cudaStream_t st) {
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute attr;
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(TRSM_ST);
+  cfg.stream = st;
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, k_trsm_step_few, d, j0, WSBM_NB, lower);
 }
 
 // Update after a solved diagonal block: lower: B[je:n] -= T[je:n, j0:je] B[j0:je];
@@ -1178,17 +1323,22 @@ int wsbm_trsm_batched(const TrsmDesc* d_desc, int nbatch, int max_n, int max_nrh
   const size_t smx = (size_t)32 * (TRSM_COLS + 1) * sizeof(double2);
   if (!warps && wsbm_smem_optin((const void*)k_trsm_diag, 64 * 1024) != cudaSuccess) return -3;
   const int nblk = (max_n + WSBM_NB - 1) / WSBM_NB;
+  const bool few = max_nrhs <= TRSM_FEW, steps = warps && few;
   for (int k = 0; k < nblk; ++k) {
     const int j0 = (lower ? k : nblk - 1 - k) * WSBM_NB;
-    if (warps)
-      k_trsm_diag_warp<<<dim3(tiles_x((max_nrhs + 3) / 4), nbatch), 128, 0, st>>>(d_desc, j0, WSBM_NB, lower);
-    else
-      k_trsm_diag<<<dim3(tiles_x((max_nrhs + TRSM_COLS - 1) / TRSM_COLS), nbatch), TRSM_COLS, smx, st>>>(
-          d_desc, j0, WSBM_NB, lower);
-    wsbm_count_launch();
+    if (k == 0 || !steps) {  // a step solves the block after it
+      if (warps)
+        k_trsm_diag_warp<<<dim3(tiles_x((max_nrhs + 3) / 4), nbatch), 128, 0, st>>>(d_desc, j0, WSBM_NB, lower);
+      else
+        k_trsm_diag<<<dim3(tiles_x((max_nrhs + TRSM_COLS - 1) / TRSM_COLS), nbatch), TRSM_COLS, smx, st>>>(
+            d_desc, j0, WSBM_NB, lower);
+      wsbm_count_launch();
+    }
     const int m = lower ? max_n - j0 - WSBM_NB : j0;
     if (m <= 0) continue;
-    if (max_nrhs <= TRSM_FEW) {
+    if (steps) {
+      if (launch_trsm_step(dim3(tiles_x((m + 31) / 32), nbatch, max_nrhs), d_desc, j0, lower, st) != cudaSuccess) return -3;
+    } else if (few) {
       k_trsm_update_few<<<dim3(tiles_x((m + 63) / 64), nbatch), 64, 0, st>>>(d_desc, j0, WSBM_NB, lower);
     } else {
       const int64_t t = (int64_t)((m + GT - 1) / GT) * ((max_nrhs + GT - 1) / GT);
