@@ -82,6 +82,56 @@ __global__ void __launch_bounds__(256) k_gemm(const GemmDesc* __restrict__ d, in
   }
 }
 
+// The same for a few columns (n <= GEMM_FEW), a column per blockIdx.z: a warp has 16 rows, a lane one
+// real component of one, so no lane works on columns that are not there and a step of the sum costs two
+// FP64 instructions a warp (64 clocks each on its sub-partition) in place of 32.  Operands come from
+// L1/L2, GF_K steps ahead of the sum.  The order of operations is k_gemm's.
+#define GEMM_FEW 8
+#define GF_K 8
+__global__ void __launch_bounds__(128) k_gemm_few(const GemmDesc* __restrict__ d) {
+  const GemmDesc g = d[blockIdx.y];
+  const int lane = threadIdx.x & 31, part = lane & 1, c = blockIdx.z, neg = part ? 0 : (int)0x80000000;
+  if (c >= g.n) return;
+  const double* B = (const double*)(g.B + (int64_t)c * g.ldb);
+  const int64_t sa = g.ta ? 1 : g.lda;
+  for (int r0 = blockIdx.x * 64 + (threadIdx.x >> 5) * 16; r0 < g.m; r0 += gridDim.x * 64) {
+    const int i = r0 + (lane >> 1);
+    const double2* A = g.A + (int64_t)min(i, g.m - 1) * (g.ta ? g.lda : 1);
+    double acc = 0.0;
+    double2 a[GF_K], na[GF_K];
+    double own[GF_K], oth[GF_K], nown[GF_K], noth[GF_K];
+    auto load = [&](int t0, double2(&x)[GF_K], double(&u)[GF_K], double(&v)[GF_K]) {
+#pragma unroll
+      for (int t = 0; t < GF_K; ++t) {
+        const bool in = t0 + t < g.k;
+        x[t] = in ? A[(t0 + t) * sa] : make_double2(0.0, 0.0);
+        u[t] = in ? B[2 * (t0 + t) + part] : 0.0;
+        v[t] = in ? B[2 * (t0 + t) + 1 - part] : 0.0;
+      }
+    };
+    load(0, a, own, oth);
+    for (int t0 = 0; t0 < g.k; t0 += GF_K) {
+      load(t0 + GF_K, na, nown, noth);
+#pragma unroll
+      for (int t = 0; t < GF_K; ++t) {  // cfma, one component
+        const double ay = __hiloint2double(__double2hiint(a[t].y) ^ neg, __double2loint(a[t].y));
+        acc = fma(a[t].x, own[t], fma(ay, oth[t], acc));
+        a[t] = na[t];
+        own[t] = nown[t];
+        oth[t] = noth[t];
+      }
+    }
+    // the complex epilogue of k_gemm: each lane of a pair forms it and keeps its component
+    const bool in = i < g.m, beta0 = g.beta.x == 0.0 && g.beta.y == 0.0;
+    double* p = (double*)(g.C + i + (int64_t)c * g.ldc) + part;
+    const double old = in && !beta0 ? *p : 0.0;
+    const double acc2 = __shfl_xor_sync(0xFFFFFFFFu, acc, 1), old2 = __shfl_xor_sync(0xFFFFFFFFu, old, 1);
+    double2 v = cmul(g.alpha, part ? make_double2(acc2, acc) : make_double2(acc, acc2));
+    if (!beta0) v = cfma(g.beta, part ? make_double2(old2, old) : make_double2(old, old2), v);
+    if (in) *p = part ? v.y : v.x;
+  }
+}
+
 // LU trailing update at panel j0 (width jb): A22 -= A21 * A12.
 __global__ void __launch_bounds__(256) k_lu_update(const LuDesc* __restrict__ d, int j0, int jb) {
   const LuDesc q = d[blockIdx.y];
@@ -1271,9 +1321,16 @@ int wsbm_gemm_batched(const GemmDesc* d_desc, int nbatch, int max_m, int max_n, 
         return rc;
     return 0;
   }
-  int64_t t = (int64_t)((max_m + GT - 1) / GT) * ((max_n + GT - 1) / GT);
-  dim3 grid(tiles_x(t), nbatch);
-  k_gemm<<<grid, 256, 0, st>>>(d_desc, nbatch);
+  if (max_n <= 0) return 0;
+  // few columns: a 32 x 32 tile would leave 3/4 of its lanes (8 columns) to 31/32 (one) without work
+  // (one column of the box solves at N = 4096: 162 us a launch as tiles, 18 us here)
+  if (max_n <= GEMM_FEW) {
+    k_gemm_few<<<dim3(tiles_x((max_m + 63) / 64), nbatch, max_n), 128, 0, st>>>(d_desc);
+  } else {
+    int64_t t = (int64_t)((max_m + GT - 1) / GT) * ((max_n + GT - 1) / GT);
+    dim3 grid(tiles_x(t), nbatch);
+    k_gemm<<<grid, 256, 0, st>>>(d_desc, nbatch);
+  }
   wsbm_count_launch();
   return cudaGetLastError() == cudaSuccess ? 0 : -3;
 }
