@@ -1097,6 +1097,12 @@ __device__ __forceinline__ void cpqr_sync(uint32_t csize) {
     cluster_sync_all();
 }
 
+// Norms in an order that integers have: negative zero and NaN never win.
+__device__ __forceinline__ long long cpqr_norm_key(double v) {
+  const long long b = __double_as_longlong(v);
+  return (b & 0x7fffffffffffffffll) > 0x7ff0000000000000ll ? -1 : b;
+}
+
 template <int CB>
 __global__ void __launch_bounds__(256, CB == 2 ? 3 : 2) k_cpqr_cluster(const QrDesc* __restrict__ d, int mode) {
   constexpr int SH = CB == 1 ? 4 : CB == 2 ? 3 : CB == 4 ? 2 : 1;  // 5 - log2(2 * CB)
@@ -1111,8 +1117,9 @@ __global__ void __launch_bounds__(256, CB == 2 ? 3 : 2) k_cpqr_cluster(const QrD
   const int64_t ld = q.lda;
   const int tid = threadIdx.x, lane = tid & 31, nw = blockDim.x >> 5;
   const int gw = (int)rank * nw + (tid >> 5), gn = (int)csize * nw;  // this warp and all warps of the cluster
-  __shared__ double sval[8], ssum[8];
-  __shared__ int sidx[8];
+  __shared__ long long sval[8];
+  __shared__ double ssum[8];
+  __shared__ int sidx[8], s_stop;
   __shared__ double s_tau;
   __shared__ double2 s_beta;
   const int kmax = min(m, n);
@@ -1132,11 +1139,12 @@ __global__ void __launch_bounds__(256, CB == 2 ? 3 : 2) k_cpqr_cluster(const QrD
   cpqr_sync(csize);
   const int kt = mode == 1 ? min(q.kt, kmax) : kmax;
   for (; j < kt; ++j) {
-    // pivot: largest remaining norm (lowest index on ties)
-    double best = -1.0;
+    // pivot: largest remaining norm (lowest index on ties), compared by bits on the integer pipe: an
+    // FP64 instruction of a warp takes its sub-partition 64 clocks, a compare too
+    long long best = -1;
     int p = j;
     for (int c = j + tid; c < n; c += blockDim.x) {
-      const double v = __ldcg(q.norm2 + c);
+      const long long v = cpqr_norm_key(__ldcg(q.norm2 + c));
       if (v > best) {
         best = v;
         p = c;
@@ -1144,7 +1152,7 @@ __global__ void __launch_bounds__(256, CB == 2 ? 3 : 2) k_cpqr_cluster(const QrD
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
-      const double ob = __shfl_xor_sync(0xffffffffu, best, o);
+      const long long ob = __shfl_xor_sync(0xffffffffu, best, o);
       const int oi = __shfl_xor_sync(0xffffffffu, p, o);
       if (ob > best || (ob == best && oi < p)) {
         best = ob;
@@ -1163,10 +1171,6 @@ __global__ void __launch_bounds__(256, CB == 2 ? 3 : 2) k_cpqr_cluster(const QrD
         best = sval[w];
         p = sidx[w];
       }
-    const double nrm = sqrt(fmax(best, 0.0));
-    if (j == 0 && rank == 0 && tid == 0) q.rdiag0[0] = nrm;
-    const double r00 = j == 0 ? nrm : __ldcg(q.rdiag0);
-    if (mode == 0 && (nrm <= q.tol * r00 || nrm == 0.0)) break;  // the same in every CTA
     // reflector from x = column p; |x| recomputed exactly
     const int mm = m - j;
     double s = 0.0;
@@ -1179,19 +1183,32 @@ __global__ void __launch_bounds__(256, CB == 2 ? 3 : 2) k_cpqr_cluster(const QrD
     for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
     if (lane == 0) ssum[tid >> 5] = s;
     __syncthreads();
-    if (tid == 0) {
-      double t = 0.0;
-      for (int w = 0; w < nw; ++w) t += ssum[w];
-      const double xn = sqrt(t);
+    // the scalars, a lane for each root and each quotient: one root and one quotient long
+    if (tid < 32) {
+      double t = lane < nw ? ssum[lane] : 0.0;
+#pragma unroll
+      for (int o = 4; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
       const double2 x0 = su[0];
-      const double a0 = sqrt(cabs2(x0));
-      const double2 beta = a0 > 0.0 ? make_double2(-x0.x / a0 * xn, -x0.y / a0 * xn) : make_double2(-xn, 0.0);
-      su[0] = make_double2(x0.x - beta.x, x0.y - beta.y);
+      const double rt = sqrt(lane == 1 ? cabs2(x0) : t);
+      const double xn = __shfl_sync(0xffffffffu, rt, 0), a0 = __shfl_sync(0xffffffffu, rt, 1);
       const double uu = 2.0 * xn * (xn + a0);  // u^H u = 2 |x| (|x| + |x0|)
-      s_tau = uu > 0.0 ? 2.0 / uu : 0.0;
-      s_beta = beta;
+      const double qt = (lane == 0 ? -x0.x : lane == 1 ? -x0.y : 2.0) / (lane < 2 ? a0 : uu);
+      const double bx = __shfl_sync(0xffffffffu, qt, 0), by = __shfl_sync(0xffffffffu, qt, 1);
+      const double tq = __shfl_sync(0xffffffffu, qt, 2);
+      if (lane == 0) {
+        const double2 beta = a0 > 0.0 ? make_double2(bx * xn, by * xn) : make_double2(-xn, 0.0);
+        su[0] = make_double2(x0.x - beta.x, x0.y - beta.y);
+        s_tau = uu > 0.0 ? tq : 0.0;
+        s_beta = beta;
+      }
+    } else if (tid == 32) {  // beside them, the stopping rule: the same in every CTA
+      const double nrm = sqrt(best > 0 ? __longlong_as_double(best) : 0.0);
+      if (j == 0 && rank == 0) q.rdiag0[0] = nrm;
+      const double r00 = j == 0 ? nrm : __ldcg(q.rdiag0);
+      s_stop = mode == 0 && (nrm <= q.tol * r00 || nrm == 0.0);
     }
     cpqr_sync(csize);
+    if (s_stop) break;
     const double tau = s_tau;
     if (rank == 0 && tid == 0) {
       q.tauv[j] = tau;
@@ -1239,11 +1256,12 @@ __global__ void __launch_bounds__(256, CB == 2 ? 3 : 2) k_cpqr_cluster(const QrD
           acc[0] += __shfl_xor_sync(0xffffffffu, acc[0], o);
         }
       }
+      acc[0] *= tau;
       double2 w[CB], top[CB];
 #pragma unroll
       for (int v = 0; v < CB; ++v) {
-        w[v].x = tau * __shfl_sync(0xffffffffu, acc[0], v << SH);
-        w[v].y = tau * __shfl_sync(0xffffffffu, acc[0], (CB + v) << SH);
+        w[v].x = __shfl_sync(0xffffffffu, acc[0], v << SH);
+        w[v].y = __shfl_sync(0xffffffffu, acc[0], (CB + v) << SH);
         top[v] = make_double2(0.0, 0.0);
       }
       for (int i = lane; i < mm; i += 32) {
@@ -1257,33 +1275,40 @@ __global__ void __launch_bounds__(256, CB == 2 ? 3 : 2) k_cpqr_cluster(const QrD
           }
       }
       // remaining norms: downdated by the new row-j entry, recomputed exactly once cancellation
-      // has eaten half their digits
+      // has eaten half their digits; column v's in lane v
+      double2 mine = make_double2(0.0, 0.0);
 #pragma unroll
       for (int v = 0; v < CB; ++v) {
-        if (v >= nc) break;
-        const int c = c0 + v, cs = c == p ? j : c;
-        const double rj = __shfl_sync(0xffffffffu, cabs2(top[v]), 0);
-        const double nf = __ldcg(q.nref + cs);
-        double nv = __ldcg(q.norm2 + cs) - rj;
-        __syncwarp();
-        if (nv <= 1e-8 * nf) {
+        const double tx = __shfl_sync(0xffffffffu, top[v].x, 0), ty = __shfl_sync(0xffffffffu, top[v].y, 0);
+        if (lane == v) mine = make_double2(tx, ty);
+      }
+      const bool on = lane < nc;
+      const int lc = c0 + lane, ls = lc == p ? j : lc;
+      const double nf = on ? __ldcg(q.nref + ls) : 0.0;
+      double nv = (on ? __ldcg(q.norm2 + ls) : 1.0) - cabs2(mine);
+      const unsigned redo = __ballot_sync(0xffffffffu, on && nv <= 1e-8 * nf);  // orders the stores above, too
+#pragma unroll
+      for (int v = 0; v < CB; ++v)
+        if (redo >> v & 1) {
           double ns = 0.0;
-          const double2* col = M + (int64_t)c * ld;
+          const double2* col = M + (int64_t)(c0 + v) * ld;
           for (int i = j + 1 + lane; i < m; i += 32) ns += cabs2(col[i]);
           for (int o = 16; o > 0; o >>= 1) ns += __shfl_xor_sync(0xffffffffu, ns, o);
-          nv = ns;
-          if (lane == 0) q.nref[c] = ns;
-        } else if (cs != c && lane == 0) {
-          q.nref[c] = nf;
-        }
-        if (lane == 0) q.norm2[c] = fmax(nv, 0.0);
-        if (cs != c)  // rows above j of R: plain interchange of columns j and p
-          for (int i = lane; i < j; i += 32) {
-            const double2 t = M[i + (int64_t)j * ld];
-            M[i + (int64_t)j * ld] = M[i + (int64_t)p * ld];
-            M[i + (int64_t)p * ld] = t;
+          if (lane == v) {
+            nv = ns;
+            q.nref[lc] = ns;
           }
+        }
+      if (on) {
+        if (ls != lc && !(redo >> lane & 1)) q.nref[lc] = nf;
+        q.norm2[lc] = fmax(nv, 0.0);
       }
+      if (c0 <= p && p < c0 + nc)  // rows above j of R: plain interchange of columns j and p
+        for (int i = lane; i < j; i += 32) {
+          const double2 t = M[i + (int64_t)j * ld];
+          M[i + (int64_t)j * ld] = M[i + (int64_t)p * ld];
+          M[i + (int64_t)p * ld] = t;
+        }
     }
     cpqr_sync(csize);
   }
