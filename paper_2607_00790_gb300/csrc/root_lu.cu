@@ -40,13 +40,11 @@ __device__ __forceinline__ unsigned long long lub_key(double2 v, int row) {
   return (hi << 32) | (unsigned long long)(0xFFFFFFFFu - (unsigned)row);
 }
 
+// by 32-bit reductions of the halves: about 80 clocks, a tree of 64-bit shuffles 400, four times a column
 __device__ __forceinline__ unsigned long long lub_warp_max(unsigned long long best) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    const unsigned long long x = __shfl_xor_sync(0xFFFFFFFFu, best, o);
-    best = x > best ? x : best;
-  }
-  return best;
+  const unsigned hi = (unsigned)(best >> 32), mh = __reduce_max_sync(0xFFFFFFFFu, hi);
+  const unsigned ml = __reduce_max_sync(0xFFFFFFFFu, hi == mh ? (unsigned)best : 0u);
+  return (unsigned long long)mh << 32 | ml;
 }
 
 __device__ __forceinline__ unsigned long long ld_acquire(const unsigned long long* p) {
@@ -67,9 +65,10 @@ __device__ __forceinline__ unsigned long long lub_time() {
 // cooperative launch, R consecutive rows each (R >= w), held in shared memory from the first to
 // the last column.  Per column every CTA publishes its best candidate (key) and that candidate's
 // panel row; every CTA then reads all the keys, takes the winner's row as the pivot row and
-// updates its own rows, so a column costs one exchange through L2 instead of two launches: about
-// 6 us a column at n = 8200 (49 ms in all; the launches per column and their gaps took 100 ms).
-// Bound by that exchange (release, 152 polled keys, one row read); the FP64 work is 1 us of it.
+// updates its own rows, so a column costs one exchange through L2 instead of two launches.  Bound by
+// that exchange (release, 152 polled keys, one row read): 4.7 us a column at n = 8200, 39 ms in all.
+// Only the next column is updated before its candidate is published, the others while it travels (with
+// the whole update first, and 64-bit reductions, 6.4 us; launches per column and their gaps 100 ms).
 //   slots  key slots [w][LUB_MAXCTA], zero on entry (a key is never zero)
 //   cand   published rows [2][LUB_MAXCTA][32]; a slot of one parity is rewritten two columns
 //          later, after every CTA has published the column between (and so has read it)
@@ -98,10 +97,8 @@ __global__ void __launch_bounds__(LUB_T, 1)
     const unsigned long long k = lub_key(sm[i], r0 + i);
     best = k > best ? k : best;
   }
-  // rows per pass of the update: threads in groups of `span` rows, the groups over the columns
-  int span = 32;
-  while (span < cnt && span < LUB_T) span *= 2;
-  const int ng = LUB_T / span, g = tid / span, ri = tid - g * span;
+  const int nchunk = (cnt + 31) / 32;
+  int prev = 0;  // first row below the last pivot's: rows from here on await its update
 
   for (int j = 0; j < w; ++j) {
     const int c = c0 + j, par = j & 1;
@@ -109,14 +106,41 @@ __global__ void __launch_bounds__(LUB_T, 1)
     if (lane == 0) red[warp] = best;
     __syncthreads();
     unsigned long long* row = slots + (size_t)j * LUB_MAXCTA;
+    // column j is up to date, the columns after it await the update by the last pivot: warp 0 applies it
+    // to the candidate's row (and to row c) alone and publishes, the other warps to the rows in shared
+    // memory, while the candidates travel
+    unsigned long long k = 0;
+    double2 vloc, vdiag, lloc, ldiag, pr;
     if (warp == 0) {
-      const unsigned long long k = lub_warp_max(lane < LUB_T / 32 ? red[lane] : 0ull);
+      k = lub_warp_max(lane < LUB_T / 32 ? red[lane] : 0ull);
       const int loc = (int)(0xFFFFFFFFu - (unsigned)k) - r0;
-      double2* mine = cand + ((size_t)par * LUB_MAXCTA + b) * LUB_W;
-      if (lane < w) __stcg(mine + lane, sm[lane * RS + loc]);
-      if (b == 0 && lane < w) __stcg(diag + par * LUB_W + lane, sm[lane * RS + j]);
+      if (lane < w) {
+        vloc = sm[lane * RS + loc];
+        if (b == 0) vdiag = sm[lane * RS + j];
+      }
+      if (j > 0) {
+        pr = prow[lane];
+        lloc = lcol[loc];
+        if (b == 0) ldiag = lcol[j];
+      }
+    }
+    __syncthreads();
+    if (warp == 0) {
+      if (j > 0 && lane > j && lane < w) {
+        vloc = cfms(lloc, pr, vloc);
+        if (b == 0) vdiag = cfms(ldiag, pr, vdiag);
+      }
+      if (lane < w) {
+        __stcg(cand + ((size_t)par * LUB_MAXCTA + b) * LUB_W + lane, vloc);
+        if (b == 0) __stcg(diag + par * LUB_W + lane, vdiag);
+      }
       __syncwarp();
       if (lane == 0) st_release(row + b, k);
+    } else if (j > 0) {
+      for (int e = warp - 1; e < nchunk * (w - 1 - j); e += LUB_T / 32 - 1) {
+        const int i = (e % nchunk) * 32 + lane, t = j + 1 + e / nchunk;
+        if (i >= prev && i < cnt) sm[t * RS + i] = cfms(lcol[i], prow[t], sm[t * RS + i]);
+      }
     }
     // all keys of this column, a thread each (bounded); a warp that read several in turn would wait
     // for L2 several times
@@ -159,29 +183,23 @@ __global__ void __launch_bounds__(LUB_T, 1)
       }
     }
     __syncthreads();
-    // rows below c: multipliers, then the rank-1 update of the columns to the right
+    // rows below c: multipliers, and the next column with its candidate; the rest follows the publication
     const int first = b == 0 ? j + 1 : 0;
     const double2 iv = s_inv;
+    best = 0;
     for (int i = tid; i < cnt; i += LUB_T)
       if (i >= first) {
         const double2 l = cmul(sm[j * RS + i], iv);
         sm[j * RS + i] = l;
         lcol[i] = l;
-      }
-    __syncthreads();
-    best = 0;
-    for (int i = ri; i < cnt; i += span) {
-      if (i < first) continue;
-      const double2 l = lcol[i];
-      for (int t = j + 1 + g; t < w; t += ng) {
-        const double2 v = cfms(l, prow[t], sm[t * RS + i]);
-        sm[t * RS + i] = v;
-        if (t == j + 1) {
-          const unsigned long long k = lub_key(v, r0 + i);
-          best = k > best ? k : best;
+        if (j + 1 < w) {
+          const double2 v = cfms(l, prow[j + 1], sm[(j + 1) * RS + i]);
+          sm[(j + 1) * RS + i] = v;
+          const unsigned long long x = lub_key(v, r0 + i);
+          best = x > best ? x : best;
         }
       }
-    }
+    prev = first;
   }
   __syncthreads();
   for (int e = tid; e < R * w; e += LUB_T) {
