@@ -100,7 +100,7 @@ def lu_src_sha():
 
 def kernel_src_sha():
     h = hashlib.sha256()
-    for f in ("entries.cu", "entry_blocks.cuh", "hankel.cuh", "hankel_coeffs.inc"):
+    for f in ("entries.cu", "entry_blocks.cuh", "hankel.cuh", "hankel_coeffs.inc", "hankel_fixed.cuh", "hankel_fixed.inc"):
         with open(os.path.join(ROOT, "paper_2607_00790_gb300", "csrc", f), "rb") as fh:
             h.update(fh.read())
     return h.hexdigest()[:16]
@@ -710,7 +710,7 @@ def run_full_2p18(dev, precision=0, tol=1e-8, rows=256, refine=True, ff_ref=None
     p = binding.make_params(cfg["k0"], cfg["n"], leaf=cfg["leaf"], nproxy=cfg["nproxy"], id_tol=tol,
                             precision=precision, root_cap=200000)
     # the tensor-core shapes timed once per process, before the build; the root panel width is
-    # timed on a 4096-unknown matrix (its class below 6144 unknowns), so the large class keeps
+    # timed on a 4096-unknown matrix (its class below 12288 unknowns), so the large class keeps
     # its width (256): a timing at 16384 unknowns does not carry over to a root of ~1e5
     if not _FULL_TUNING:
         choice, tms = binding.wsbm_autotune(n_box=2 * cfg["leaf"], nbox=N // cfg["leaf"], nrhs_box=128,

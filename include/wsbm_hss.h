@@ -335,8 +335,8 @@ void wsbm_batch_destroy(wsbm_batch_t b);
  * matrix of eq. (weakly_bm) (every node pair, O(N^2) work, nothing stored): residuals and
  * iterative refinement of HSS and adjoint solutions.  x, y: device complex128 2N x nrhs in
  * paper order (for trans = 0, x by unknown and y by equation; the reverse for trans = 1).
- * The Hankel values of each node pair are evaluated once for up to four right-hand sides.
- * Scratch: 4 x 2N x (eight waves of CTAs / ceil(N/128)) complex128 from the library's
+ * The Hankel values of each node pair are evaluated once for up to eight right-hand sides.
+ * Scratch: at most 4 x 2N x (eight waves of CTAs / ceil(N/128)) complex128 from the library's
  * allocator (wsbm_set_allocator) on `stream`.  Asynchronous.  Errors: INVALID_ARG, OOM, CUDA. */
 int wsbm_matvec(const wsbm_geom* g, const wsbm_params* p, int32_t trans, const void* x,
                 int32_t nrhs, void* y, void* stream);
@@ -426,7 +426,7 @@ int wsbm_lu_dense(void* A, int64_t lda, int32_t n, int32_t* piv, void* stream);
  *   out[1]  panel width of the batched box LU, of {32, 64} (nbox boxes of n_box unknowns with
  *           nrhs_box right-hand sides each: the leaf level of a build);
  *   out[2], out[3]  outer panel width of the root LU, of {128, 256}, for roots below and from
- *           6144 unknowns; only the class of n_root is timed, the other keeps its value;
+ *           12288 unknowns; only the class of n_root is timed, the other keeps its value;
  *   out[4]  columns per warp pass of the column-pivoted QR of ID matrices of more than 2048
  *           rows, of {2, 4, 8} (152 matrices of 2560 x 128).
  * ms: host, 10 doubles or NULL: the candidates' times in that order.  Work space (two copies of

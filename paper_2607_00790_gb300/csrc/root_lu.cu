@@ -21,7 +21,11 @@
 #define LUB_NB_BIG 256  // outer panel width from LUB_BIG_N on: deeper tensor-core products
 #endif
 #ifndef LUB_BIG_N
-#define LUB_BIG_N 6144  // (measured: n = 5000 equal, 8200 117 ms against 128, 16384 416 against 537)
+// 256 columns from here on only: at n = 8200 they take 104 ms against 115, but their wider explicit
+// inverses cost accuracy, |PA - LU| / |A| 4.1e-14 against 2.8e-14 and the largest entry 7.6e-13 against
+// 5e-13 (128-column panels of the launch-per-column version: 4.5e-14 and 5.5e-13).  n = 16384: 416 ms
+// against 537.
+#define LUB_BIG_N 12288
 #endif
 #define LUB_W 32            // widest base panel: one lane per column
 #define LUB_T 256           // threads of a base-panel CTA
