@@ -7,13 +7,17 @@
 // registers (row 32 s + lane in x[s]).  Columns of T come through shared memory 32 at a time
 // (`stage`: 32 x 32 NS values, shared by the CTA's warps), so a step is a broadcast of x_t and a
 // few multiply-adds off shared memory: a chain of about 100 clocks a row instead of a chain of
-// global loads (a 128 x 128 inverse takes 88 us spread over 128 SMs; 1.7 ms with a thread per column).  Every thread of the CTA has to call it with the same T and nb; warps that are not
-// `active` only help with the staging.  `first` (the same for every thread): the slot where the
-// nonzeros of every column of the CTA begin (end, if UPPER); the slots before it are skipped.
+// global loads (a 128 x 128 inverse takes 88 us spread over 128 SMs; 1.7 ms with a thread per
+// column).  An upper triangle's columns are scaled by the reciprocals of its diagonal as they are
+// staged, so no step multiplies by them.  Every thread of the CTA has to call it with the same T and
+// nb; warps that are not `active` only help with the staging.  `first` (the same for every thread):
+// the slot where the nonzeros of every column of the CTA begin (end, if UPPER); the slots before it are
+// skipped, and of the warp's column the steps before its row `own`, whose x_t are zero.  Both matter
+// where many matrices fill the FP64 pipe: 4096 pairs of 64 x 64 inverses 27.7 ms without, 14.0 ms with.
 template <int NS, bool UPPER>
 __device__ __forceinline__ void tri_solve_warp(const double2* __restrict__ T, int64_t ldt, int nb, double2 (&x)[NS],
                                                double2* stage, double2* dinv, bool active = true,
-                                               int first = UPPER ? NS - 1 : 0) {
+                                               int first = UPPER ? NS - 1 : 0, int own = UPPER ? 32 * NS - 1 : 0) {
   constexpr int LD = 32 * NS;
   const int lane = threadIdx.x & 31;
 #pragma unroll
@@ -36,18 +40,19 @@ __device__ __forceinline__ void tri_solve_warp(const double2* __restrict__ T, in
             v.x == 0.0 && v.y == 0.0 ? make_double2(0.0, 0.0) : cdiv(make_double2(1.0, 0.0), v);
       }
       __syncthreads();
+      for (int e = threadIdx.x; e < te * LD; e += blockDim.x) {
+        const int tt = e / LD, i = e - tt * LD;
+        if (i < t0 + tt) stage[e] = cmul(stage[e], dinv[tt]);
+      }
+      __syncthreads();
     }
     if (!active) continue;
-    for (int k = 0; k < te; ++k) {
+    for (int k = max(0, UPPER ? t0 + te - 1 - own : own - t0); k < te; ++k) {
       const int tt = UPPER ? te - 1 - k : k;
       const double2* col = stage + tt * LD;
       double2 xt;
       xt.x = __shfl_sync(0xFFFFFFFFu, x[s].x, tt);
       xt.y = __shfl_sync(0xFFFFFFFFu, x[s].y, tt);
-      if (UPPER) {
-        xt = cmul(xt, dinv[tt]);
-        if (lane == tt) x[s] = xt;
-      }
 #pragma unroll
       for (int r = 0; r < NS; ++r) {
         const int i = r * 32 + lane;
@@ -55,6 +60,7 @@ __device__ __forceinline__ void tri_solve_warp(const double2* __restrict__ T, in
           if (UPPER || i < nb) x[r] = cfms(col[i], xt, x[r]);
       }
     }
+    if (UPPER && lane < te) x[s] = cmul(x[s], dinv[lane]);
   }
 }
 
@@ -67,7 +73,7 @@ __device__ __forceinline__ void tri_inverse_column(const double2* __restrict__ T
   double2 x[NS];
 #pragma unroll
   for (int s = 0; s < NS; ++s) x[s] = make_double2(s * 32 + lane == j ? 1.0 : 0.0, 0.0);
-  tri_solve_warp<NS, UPPER>(T, ldt, nb, x, stage, dinv, active, first);
+  tri_solve_warp<NS, UPPER>(T, ldt, nb, x, stage, dinv, active, first, j);
 #pragma unroll
   for (int s = 0; s < NS; ++s)
     if (active && j < nb && s * 32 + lane < nb) out[s * 32 + lane] = x[s];
