@@ -34,12 +34,12 @@ UNIT = "entries/s"
 # for the kernel sources with the recorded hash; when the sources change the traffic figure is
 # withheld until re-measured.
 KERNEL_COUNTS = {
-    "src_sha": "39971b7a6cb47b86",
+    "src_sha": "6fec8f827c2ae62f",
     # 16384-node star, leaf level (bench.py --profile-case), tiles of 16 x 8 node pairs (the
     # autotuned shape; the proxy kernel's per-pair count includes its proxy-point set-up, which
     # depends on the tile width): 4.16 M / 4.24 M pairs
-    "k_proxy": {"tf": 16, "fp64_flops_per_pair": 244.5, "dram_bytes_per_pair": 50.1},
-    "k_pairs": {"tf": 16, "fp64_flops_per_pair": 323.9, "dram_bytes_per_pair": 50.8},
+    "k_proxy": {"tf": 16, "fp64_flops_per_pair": 81.8, "dram_bytes_per_pair": 50.2},
+    "k_pairs": {"tf": 16, "fp64_flops_per_pair": 100.5, "dram_bytes_per_pair": 50.3},
     # DRAM traffic of the column-pivoted QR per ID matrix of this workload, keyed by the hash of
     # its dense.cu section and the matrix rows it was measured on (1024 sketches of 128 rows,
     # 65536-node star)
