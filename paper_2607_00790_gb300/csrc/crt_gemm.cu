@@ -24,14 +24,14 @@
 //
 // Error: the rounding of X to 56 bits, as in tc_gemm.cu; nothing is dropped.
 //
-// Kernel: clusters of two CTAs, persistent over 128 x 96 complex tiles, 48 columns each.  The pair
-// shares every A tile: each loads half of it and multicasts it to both.  Warp 0 issues the TMA loads (a
+// Kernel: one CTA per SM, persistent over 128 x 48 complex tiles.  Warp 0 issues the TMA loads (a
 // 5-stage ring of 32-deep K blocks of four planes, 64-byte swizzled rows), warp 1 the MMAs (128 x 48 x
 // 16, the four accumulators in turn) into two TMEM buffers (P+ and P- of two moduli each); warps 4-11
 // reduce them: two threads per row, 24 columns each, 6 registers of running sums per entry (setmaxnreg
 // moves the registers over; 64 columns a CTA spill).  Bound by the instructions of that reduction (about
-// 25 issue slots per entry and modulus, 160 to make the double), 6 clocks per entry and SM; loads and
-// MMAs alone take 1.3 of the 2.5 ms at 8192 x 8192 x 256.
+// 25 issue slots per entry and modulus, 160 to make the double), 6 clocks per entry and SM: 2.44 ms at
+// 8192 x 8192 x 256.  Every CTA loads whole A tiles: pairs of CTAs that shared them were no faster (2.5
+// ms), since the loads are not the bound, and each had to outlive the other's arrivals.
 #include <stdint.h>
 #include <string.h>
 
@@ -43,7 +43,7 @@
 #define CR_NP 14             // moduli
 #define CR_PL (2 * CR_NP)    // planes per operand
 #define CR_BM 128            // rows per tile
-#define CR_BN 48             // complex columns per CTA (two CTAs side by side)
+#define CR_BN 48             // complex columns per tile
 #define CR_TC (CR_BN / 2)    // columns per epilogue thread: 6 CR_TC registers of running sums
 #define CR_BK 32             // K values per stage (64-byte rows)
 #define CR_G 4               // planes per stage: P+ and P- of two moduli
@@ -83,24 +83,10 @@ struct CrtArgs {
   double2 alpha, beta;
   int m, n, kb;             // kb: K blocks of CR_BK
   int mode;                 // 0: C = A B, 1: C -= A B, 2: general
-  int tiles_m, tiles_n;     // 128 x 96 tiles
+  int tiles_m, tiles_n;     // 128 x 48 tiles
   int group;                // row tiles per raster group
 };
 
-__device__ __forceinline__ void tma_load_3d_pair(uint32_t dst, const CUtensorMap* map, uint32_t bar, int c0, int c1,
-                                                 int c2) {
-  asm volatile(
-      "cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes.multicast::cluster [%0], [%1, {%3, "
-      "%4, %5}], [%2], %6;" ::"r"(dst),
-      "l"((uint64_t)map), "r"(bar), "r"(c0), "r"(c1), "r"(c2), "h"((uint16_t)3)
-      : "memory");
-}
-__device__ __forceinline__ void commit_pair(uint32_t bar) {
-  asm volatile(
-      "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(bar),
-      "h"((uint16_t)3)
-      : "memory");
-}
 // K-major tile of 64-byte rows, 64-byte swizzle (atoms of 8 rows, 512 bytes apart).
 __device__ __forceinline__ uint64_t cr_desc(uint32_t addr) {
   return (uint64_t)((addr >> 4) & 0x3FFF) | (uint64_t)1 << 16 | (uint64_t)(512 >> 4) << 32 | (uint64_t)1 << 46 |
@@ -115,9 +101,6 @@ __device__ __forceinline__ void cr_mma(uint32_t d_tmem, uint64_t a, uint64_t b, 
       "setp.ne.b32 p, %4, 0;\n\t"
       "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem),
       "l"(a), "l"(b), "r"(idesc), "r"(accum));
-}
-__device__ __forceinline__ void cr_cluster_sync() {
-  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
 // ------------------------------------------------------------------ residues ----
@@ -391,7 +374,7 @@ __device__ __forceinline__ void crt_finish(const CrtArgs& a, uint64_t (&fr)[CR_T
   }
 }
 
-__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(CR_THREADS, 1)
+__global__ void __launch_bounds__(CR_THREADS, 1)
     k_zgemm_crt(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB,
                 const __grid_constant__ CrtArgs a) {
   extern __shared__ unsigned char smem_raw[];
@@ -403,14 +386,13 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(CR_THREADS, 1)
                  tempty0 = tfull0 + 8 * CR_NBUF;
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(gbase + CR_STAGES * CR_STAGE + 16 * CR_STAGES + 16 * CR_NBUF);
   const int warp = threadIdx.x / 32, lane = threadIdx.x & 31;
-  const int rank = blockIdx.x & 1, ncl = gridDim.x >> 1;
   const int ntiles = a.tiles_m * a.tiles_n;
   const int nchunks = (a.kb + CR_KC / CR_BK - 1) / (CR_KC / CR_BK);
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < CR_STAGES; ++s) {
       mbar_init(full0 + 8 * s, 1);
-      mbar_init(empty0 + 8 * s, 2);  // both CTAs have read the stage
+      mbar_init(empty0 + 8 * s, 1);
     }
     for (int s = 0; s < CR_NBUF; ++s) {
       mbar_init(tfull0 + 8 * s, 1);
@@ -424,7 +406,6 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(CR_THREADS, 1)
   }
   tc_fence_before();
   __syncthreads();
-  cr_cluster_sync();  // the other CTA's barriers are initialized
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
 
@@ -442,7 +423,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(CR_THREADS, 1)
       // -------------------------------------------------------------- TMA producer
       uint32_t it = 0;
       bool ok = true;
-      for (int t = blockIdx.x >> 1; t < ntiles && ok; t += ncl) {
+      for (int t = blockIdx.x; t < ntiles && ok; t += gridDim.x) {
         int tm, tn;
         coords(t, tm, tn);
         for (int kc = 0; kc < a.kb && ok; kc += CR_KC / CR_BK) {
@@ -455,9 +436,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(CR_THREADS, 1)
               mbar_expect_tx(full, CR_STAGE);
 #pragma unroll
               for (int q = 0; q < CR_G; ++q) {
-                tma_load_3d_pair(sa + q * CR_A_BYTES + rank * (CR_A_BYTES / 2), &mapA, full, kb * CR_BK,
-                                 tm * CR_BM + rank * (CR_BM / 2), g * CR_G + q);
-                tma_load_3d(sb + q * CR_B_BYTES, &mapB, full, kb * CR_BK, (tn * 2 + rank) * CR_BN, g * CR_G + q);
+                tma_load_3d(sa + q * CR_A_BYTES, &mapA, full, kb * CR_BK, tm * CR_BM, g * CR_G + q);
+                tma_load_3d(sb + q * CR_B_BYTES, &mapB, full, kb * CR_BK, tn * CR_BN, g * CR_G + q);
               }
             }
         }
@@ -472,7 +452,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(CR_THREADS, 1)
       // -------------------------------------------------------------- MMA issuer
       uint32_t it = 0, u = 0;
       bool ok = true;
-      for (int t = blockIdx.x >> 1; t < ntiles && ok; t += ncl) {
+      for (int t = blockIdx.x; t < ntiles && ok; t += gridDim.x) {
         for (int kc = 0; kc < a.kb && ok; kc += CR_KC / CR_BK) {
           const int ke = min(a.kb, kc + CR_KC / CR_BK);
           for (int g = 0; g < CR_PL / CR_G && ok; ++g, ++u) {
@@ -490,7 +470,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(CR_THREADS, 1)
                 for (int q = 0; q < CR_G; ++q)  // four accumulators in turn: no product waits for the last
                   cr_mma(tmem + (b * CR_G + q) * 64, cr_desc(sa + q * CR_A_BYTES) + 2 * kk,
                          cr_desc(sb + q * CR_B_BYTES) + 2 * kk, kb > kc || kk > 0 ? 1u : 0u);
-              commit_pair(empty0 + 8 * s);
+              tc_commit(empty0 + 8 * s);
             }
             if (ok) tc_commit(tfull0 + 8 * b);
           }
@@ -504,7 +484,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(CR_THREADS, 1)
     const uint32_t tq = tmem + ((uint32_t)(quad * 32) << 16) + half * CR_TC;
     uint32_t u = 0;
     bool ok = true;
-    for (int t = blockIdx.x >> 1; t < ntiles && ok; t += ncl) {
+    for (int t = blockIdx.x; t < ntiles && ok; t += gridDim.x) {
       int tm, tn;
       coords(t, tm, tn);
       uint64_t fr[CR_TC], fi[CR_TC];
@@ -546,7 +526,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(CR_THREADS, 1)
       }
       if (!ok) break;
       // scales of this thread's row and of column j0 + lane (dealt out by shuffles)
-      const int i = tm * CR_BM + quad * 32 + lane, j0 = (tn * 2 + rank) * CR_BN + half * CR_TC;
+      const int i = tm * CR_BM + quad * 32 + lane, j0 = tn * CR_BN + half * CR_TC;
       const int2 er = i < a.m ? a.rexp[i] : make_int2(0, -1000);
       const int2 ecl = lane < CR_TC && j0 + lane < a.n ? a.cexp[j0 + lane] : make_int2(0, -1000);
       // crt_fix is needed only for extreme scales, or where a row and a column have few significant bits
@@ -561,7 +541,6 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(CR_THREADS, 1)
   }
   tc_fence_before();
   __syncthreads();
-  cr_cluster_sync();  // no load into, or arrival at, the other CTA is outstanding
   if (warp == 1) {
     tc_fence_after();
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512));
@@ -633,34 +612,6 @@ static int crt_map(CUtensorMap* map, void* planes, int64_t rows, int64_t Kp, int
              : -3;
 }
 
-// Clusters of the product kernel that the device holds at once (per device, thread safe).
-static int crt_clusters() {
-  static std::mutex mu;
-  static int count[64];
-  int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return std::max(1, wsbm_sm_count() / 2);
-  std::lock_guard<std::mutex> lk(mu);
-  if (!count[dev]) {
-    cudaLaunchConfig_t cfg = {};
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = 2;
-    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
-    cfg.gridDim = dim3(2 * wsbm_sm_count());
-    cfg.blockDim = dim3(CR_THREADS);
-    cfg.dynamicSmemBytes = CR_SMEM;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
-    int n = 0;
-    if (cudaOccupancyMaxActiveClusters(&n, k_zgemm_crt, &cfg) != cudaSuccess || n < 1) {
-      cudaGetLastError();
-      n = std::max(1, wsbm_sm_count() / 2);
-    }
-    count[dev] = n;
-  }
-  return count[dev];
-}
-
 static int64_t crt_kp(int k) { return ((int64_t)std::min(k, CR_KMAX) + CR_BK - 1) / CR_BK * CR_BK; }
 static size_t crt_up(size_t b) { return (b + 255) & ~(size_t)255; }
 static size_t crt_bytes(int64_t m, int64_t n, int64_t Kp) {
@@ -669,9 +620,9 @@ static size_t crt_bytes(int64_t m, int64_t n, int64_t Kp) {
 
 size_t wsbm_zgemm_crt_ws_bytes(int m, int n, int k) { return crt_bytes(m, n, crt_kp(k)); }
 
-// Measured against the digit planes: 8192 x 8192 x 256 2.63 ms against 3.60, x 512 4.62 / 6.35, x 128
+// Measured against the digit planes: 8192 x 8192 x 256 2.55 ms against 3.60, x 512 4.50 / 6.34, x 128
 // 2.04 / 2.11 (the reduction of the sums, 6 clocks per entry and SM, does not shrink with k), 1024 x
-// 1024 x 128 0.118 / 0.100; small or thin results leave clusters idle.
+// 1024 x 128 0.118 / 0.100; small or thin results leave SMs idle.
 bool wsbm_zgemm_crt_fits(int m, int n, int k) { return k >= 160 && m >= 512 && n >= 512; }
 
 // ws_bytes may be less than wsbm_zgemm_crt_ws_bytes: the longer side then goes through in strips
@@ -722,14 +673,14 @@ int wsbm_zgemm_crt(int m, int n, int k, double2 alpha, const double2* A, int64_t
                                                                                   PA);
           wsbm_count_launches(2);
         }
-        if (crt_map(&ma, PA, mm, kp, CR_BM / 2)) return -3;
+        if (crt_map(&ma, PA, mm, kp, CR_BM)) return -3;
         a.C = C + i0 + (int64_t)j0 * ldc;
         a.m = mm;
         a.n = nn;
         a.tiles_m = (mm + CR_BM - 1) / CR_BM;
-        a.tiles_n = (nn + 2 * CR_BN - 1) / (2 * CR_BN);
+        a.tiles_n = (nn + CR_BN - 1) / CR_BN;
         const int64_t tiles = (int64_t)a.tiles_m * a.tiles_n;
-        const int grid = 2 * (int)std::min<int64_t>(tiles, crt_clusters());
+        const int grid = (int)std::min<int64_t>(tiles, wsbm_sm_count());
         k_zgemm_crt<<<grid, CR_THREADS, CR_SMEM, st>>>(ma, mb, a);
         wsbm_count_launch();
       }
