@@ -1329,7 +1329,8 @@ __global__ void __launch_bounds__(256, CB == 2 ? 3 : 2) k_cpqr_cluster(const QrD
       const int lc = c0 + lane, ls = lc == p ? j : lc;
       const double nf = on ? __ldcg(q.nref + ls) : 0.0;
       double nv = (on ? __ldcg(q.norm2 + ls) : 1.0) - cabs2(mine);
-      const unsigned redo = __ballot_sync(0xffffffffu, on && nv <= 1e-8 * nf);  // orders the stores above, too
+      const unsigned redo = __ballot_sync(0xffffffffu, on && nv <= 1e-8 * nf);
+      if (redo) __syncwarp();  // a vote does not order memory: the sums below read other lanes' stores
 #pragma unroll
       for (int v = 0; v < CB; ++v)
         if (redo >> v & 1) {
