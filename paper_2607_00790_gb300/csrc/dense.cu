@@ -875,7 +875,7 @@ __global__ void __launch_bounds__(LUS_T) k_lu_solve_fused(const LuSolveDesc* __r
 #ifndef CPQR_TPC_MAXM
 #define CPQR_TPC_MAXM 192
 #endif
-#define CPQR_CLUSTER_SMEM (192 * 1024)  // longest reflector of the cluster variant (12288 rows)
+#define CPQR_CLUSTER_MAXM 12288  // rows of the cluster variant: a reflector of 192 KB in shared memory
 // Warp variant: CB trailing columns per warp per pass (2*CB partial sums, a power of two <= 16).
 template <bool TPC, int CB>
 __global__ void __launch_bounds__(256, CPQR_MINB) k_cpqr(const QrDesc* __restrict__ d, int mode) {
@@ -884,7 +884,7 @@ __global__ void __launch_bounds__(256, CPQR_MINB) k_cpqr(const QrDesc* __restric
   extern __shared__ double2 su[];  // TPC: the reflector u = M[j:m, j]
   const QrDesc q = d[blockIdx.x];
   const int m = q.m, n = q.n;
-  if (TPC != (m <= CPQR_TPC_MAXM)) return;
+  if (TPC ? m > CPQR_TPC_MAXM : m <= CPQR_CLUSTER_MAXM) return;
   double2* M = q.A;
   const int64_t ld = q.lda;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
@@ -1119,7 +1119,7 @@ __global__ void __launch_bounds__(256, CPQR_MINB) k_cpqr(const QrDesc* __restric
   }
 }
 
-// One matrix of more than CPQR_TPC_MAXM rows per cluster of 1 to 8 CTAs: more than one where there
+// One matrix of more than CPQR_TPC_MAXM and at most CPQR_CLUSTER_MAXM rows per cluster of 1 to 8 CTAs: more than one where there
 // are too few matrices to fill the GPU (the upper tree levels: few boxes, the largest matrices).
 // The trailing columns are dealt to the warps of the whole cluster, CB at a time; a column's sums
 // do not depend on which warp or how many CTAs take it, so a matrix has the same factor in every
@@ -1155,7 +1155,7 @@ __global__ void __launch_bounds__(256, CB == 2 ? 3 : 2) k_cpqr_cluster(const QrD
   asm("mov.u32 %0, %%cluster_nctarank;" : "=r"(csize));
   const QrDesc q = d[blockIdx.x / csize];
   const int m = q.m, n = q.n;
-  if (m <= CPQR_TPC_MAXM) return;  // the thread-per-column kernel's
+  if (m <= CPQR_TPC_MAXM || m > CPQR_CLUSTER_MAXM) return;  // another kernel's
   double2* M = q.A;
   const int64_t ld = q.lda;
   const int tid = threadIdx.x, lane = tid & 31, nw = blockDim.x >> 5;
@@ -1515,7 +1515,7 @@ int wsbm_cpqr_tpc_rows() { return CPQR_TPC_MAXM; }
 
 template <int CB>
 static int launch_cpqr_cluster(const QrDesc* d_desc, int nbatch, int mode, int cl, int max_m, cudaStream_t st) {
-  const size_t sm = (size_t)max_m * sizeof(double2);
+  const size_t sm = (size_t)std::min(max_m, CPQR_CLUSTER_MAXM) * sizeof(double2);
   if (wsbm_smem_optin((const void*)k_cpqr_cluster<CB>, sm) != cudaSuccess) return -3;
   cudaLaunchConfig_t cfg = {};
   cudaLaunchAttribute at[1];
@@ -1533,7 +1533,7 @@ static int launch_cpqr_cluster(const QrDesc* d_desc, int nbatch, int mode, int c
 }
 
 // The kernel is chosen per matrix, by its rows, so that its factor does not depend on the others of
-// the launch: each launch skips the matrices of the other kind.
+// the launch: each launch skips the matrices of the other kinds.
 int wsbm_cpqr_batched(const QrDesc* d_desc, int nbatch, int nsmall, int mode, int max_m, cudaStream_t st) {
   if (nbatch <= 0) return 0;
   const WsbmTune tu = wsbm_tune_current();
@@ -1543,7 +1543,7 @@ int wsbm_cpqr_batched(const QrDesc* d_desc, int nbatch, int nsmall, int mode, in
     wsbm_count_launch();
   }
   const int nbig = nbatch - nsmall;
-  if (nbig > 0 && (size_t)max_m * sizeof(double2) <= CPQR_CLUSTER_SMEM) {
+  if (nbig > 0) {
     // 2, 4 or 8 CTAs per matrix while the GPU holds them all at once (three per SM)
     int cl = 1;
     while (cl < 8 && (int64_t)nbig * cl * 2 <= (int64_t)wsbm_sm_count() * 3) cl *= 2;
@@ -1552,7 +1552,8 @@ int wsbm_cpqr_batched(const QrDesc* d_desc, int nbatch, int nsmall, int mode, in
                  : cb == 8 ? launch_cpqr_cluster<8>(d_desc, nbatch, mode, cl, max_m, st)
                            : launch_cpqr_cluster<4>(d_desc, nbatch, mode, cl, max_m, st))
       return rc;
-  } else if (nbig > 0) {  // a reflector beyond the shared memory of a CTA
+  }
+  if (max_m > CPQR_CLUSTER_MAXM) {
     k_cpqr<false, 4><<<nbatch, 256, 0, st>>>(d_desc, mode);
     wsbm_count_launch();
   }

@@ -63,3 +63,13 @@ def test_norms_after_cancellation(m):
         assert np.all(np.abs(norm2[kt:] - left) <= 40 * EPS / 1e-8 * left)
         R = np.linalg.qr(A, mode="r")
         assert np.all(np.abs(np.abs(beta[:kt]) - np.abs(np.diag(R))[:kt]) <= m * n * EPS)
+
+
+@pytest.mark.parametrize("m", [150, 193, 300])
+@pytest.mark.parametrize("other", [64, 2100, 12288, 12289])
+def test_factor_does_not_depend_on_its_batch(m, other):
+    """Beside a matrix that another kernel, or another width of the same kernel, takes."""
+    A, B = graded(m, 41), graded(other, 6)
+    alone, beside = cpqr([A], 6)[0], cpqr([A, B], 6)[0]
+    for x, y in zip(alone, beside):
+        assert np.array_equal(x, y)
