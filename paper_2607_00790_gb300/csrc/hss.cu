@@ -297,21 +297,27 @@ __global__ void k_split_uq(const double2* __restrict__ x, double2* __restrict__ 
 // Far field: one CTA per observation angle, all right-hand sides, reduction over nodes.
 //   u_inf = e^{i pi/4}/sqrt(8 pi k0) sum_j w_j [-i k0 (xh.n_j) u_j - eps0 q_j] e^{-i k0 xh.x_j}
 // For a few right-hand sides: bound by the FP64 pipe (a sine and cosine per node and angle, 8
-// operations per right-hand side); the many go through the product below.
+// operations per right-hand side); the many go through the product below.  bad (NULL: everything):
+// only the rows with bad[angle] != 0 and the columns with bad[nang + column] != 0.
 #define FF_CHUNK 8
 __global__ void __launch_bounds__(256) k_farfield(DevGeom g, double k0, double eps0,
                                                   const double2* __restrict__ u,
                                                   const double2* __restrict__ q, int nrhs,
                                                   const double* __restrict__ ang, int nang,
-                                                  double2* __restrict__ out) {
+                                                  const int* __restrict__ bad, double2* __restrict__ out) {
   __shared__ double2 red[FF_CHUNK][256 / 32];
   const int a = blockIdx.x;
+  const bool row = !bad || bad[a];
   double ca, sa;
   sincos(ang[a], &sa, &ca);
   const int64_t N = g.n;
   const double pr = 1.0 / sqrt(8.0 * 3.14159265358979323846 * k0);
   const double2 pref = make_double2(pr * 0.70710678118654752440, pr * 0.70710678118654752440);
   for (int c0 = 0; c0 < nrhs; c0 += FF_CHUNK) {
+    if (!row) {
+      const int c = c0 + (int)threadIdx.x;
+      if (!__syncthreads_or(threadIdx.x < FF_CHUNK && c < nrhs && bad[nang + c])) continue;
+    }
     double2 acc[FF_CHUNK];
 #pragma unroll
     for (int c = 0; c < FF_CHUNK; ++c) acc[c] = make_double2(0.0, 0.0);
@@ -341,7 +347,7 @@ __global__ void __launch_bounds__(256) k_farfield(DevGeom g, double k0, double e
       if (lane == 0) red[c][wp] = v;
     }
     __syncthreads();
-    if (threadIdx.x < FF_CHUNK && c0 + threadIdx.x < nrhs) {
+    if (threadIdx.x < FF_CHUNK && c0 + threadIdx.x < nrhs && (row || bad[nang + c0 + threadIdx.x])) {
       double2 v = make_double2(0.0, 0.0);
       for (int k = 0; k < 256 / 32; ++k) {
         v.x += red[threadIdx.x][k].x;
@@ -359,11 +365,13 @@ __global__ void __launch_bounds__(256) k_farfield(DevGeom g, double k0, double e
 // the right factor, since q is of the order k0 u) have the same magnitude, as the row and column
 // scaling of the product wants.  The nodes are cut into chunks of S, one product each (K = 2S), so
 // that the few tiles of a nang x nrhs result still fill the GPU; the partial results are summed in
-// chunk order.  A sine and cosine per node and angle in all, 11.8 -> 1.5 ms for 360 angles, 64
+// chunk order.  Two sines and cosines per node and angle in all, 11.8 -> 1.5 ms for 360 angles, 64
 // right-hand sides and 16384 nodes (the kernel above repeats them for every 8 columns and spends
-// 8 FP64 operations per column).
+// 8 FP64 operations per column).  The digits of the product have no infinity and no NaN: rows and columns
+// that hold one are marked in bad[angle] and bad[nang + column] and formed by the kernel above.
 __global__ void __launch_bounds__(256) k_ff_rows(DevGeom g, double k0, int64_t j0, int64_t nn, int S,
-                                                 const double* __restrict__ ang, int nang, double2* __restrict__ E) {
+                                                 const double* __restrict__ ang, int nang, double2* __restrict__ E,
+                                                 int* __restrict__ bad) {
   const double pr = 0.70710678118654752440 / sqrt(8.0 * 3.14159265358979323846 * k0);
   for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < nn * nang;
        e += (int64_t)gridDim.x * blockDim.x) {
@@ -374,6 +382,7 @@ __global__ void __launch_bounds__(256) k_ff_rows(DevGeom g, double k0, int64_t j
     sincos(k0 * (ca * g.x[j] + sa * g.y[j]), &s, &c);
     const double w = pr * g.w[j], xn = ca * g.nx[j] + sa * g.ny[j];
     const double2 f = make_double2(w * (c + s), w * (c - s));  // (1 + i) w e^{-i ...}
+    if (!isfinite(xn * f.x) || !isfinite(xn * f.y)) bad[a] = 1;
     const int64_t ch = jj / S, i = jj - ch * S, sz = min((int64_t)S, nn - ch * S);
     double2* o = E + 2 * ch * S * nang + a;
     o[i * nang] = make_double2(xn * f.y, -xn * f.x);
@@ -382,15 +391,17 @@ __global__ void __launch_bounds__(256) k_ff_rows(DevGeom g, double k0, int64_t j
 }
 __global__ void __launch_bounds__(256) k_ff_cols(double k0, double eps0, int64_t N, int64_t j0, int64_t nn, int S,
                                                  const double2* __restrict__ u, const double2* __restrict__ q,
-                                                 int nrhs, double2* __restrict__ B) {
+                                                 int nrhs, double2* __restrict__ B, int* __restrict__ bad) {
   for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < nn * nrhs;
        e += (int64_t)gridDim.x * blockDim.x) {
     const int64_t c = e / nn, jj = e - c * nn;
     const int64_t ch = jj / S, i = jj - ch * S, sz = min((int64_t)S, nn - ch * S);
     double2* o = B + 2 * ch * S * nrhs + c * 2 * sz + i;
     const double2 uv = u[j0 + jj + c * N], qv = q[j0 + jj + c * N];
-    o[0] = make_double2(k0 * uv.x, k0 * uv.y);
-    o[sz] = make_double2(eps0 * qv.x, eps0 * qv.y);
+    const double2 b0 = make_double2(k0 * uv.x, k0 * uv.y), b1 = make_double2(eps0 * qv.x, eps0 * qv.y);
+    if (!isfinite(b0.x) || !isfinite(b0.y) || !isfinite(b1.x) || !isfinite(b1.y)) bad[c] = 1;
+    o[0] = b0;
+    o[sz] = b1;
   }
 }
 __global__ void __launch_bounds__(256) k_ff_sum(const double2* __restrict__ part, int nch, int64_t n, int add,
@@ -2886,20 +2897,25 @@ static int farfield_product(wsbm_hss* h, const double2* u, const double2* q, int
   TmpMem tmp(h);
   double2 *E = nullptr, *B = nullptr, *C = nullptr;
   void* ws = nullptr;
+  int* bad = nullptr;
   if (dalloc(h, (size_t)2 * pass * nang * sizeof(double2), (void**)&E, tmp.v) ||
       dalloc(h, (size_t)2 * pass * nrhs * sizeof(double2), (void**)&B, tmp.v) ||
-      dalloc(h, (size_t)nch * nang * nrhs * sizeof(double2), (void**)&C, tmp.v) || dalloc(h, tcb, &ws, tmp.v))
+      dalloc(h, (size_t)nch * nang * nrhs * sizeof(double2), (void**)&C, tmp.v) || dalloc(h, tcb, &ws, tmp.v) ||
+      dalloc(h, ((size_t)nang + nrhs) * sizeof(int), (void**)&bad, tmp.v))
     return WSBM_ERR_OOM;
+  HC(cudaMemsetAsync(bad, 0, ((size_t)nang + nrhs) * sizeof(int), st));
   for (int64_t j0 = 0; j0 < N; j0 += pass) {
     const int64_t nn = std::min(pass, N - j0);
-    k_ff_rows<<<gridfor(nn * nang), 256, 0, st>>>(h->g, h->ph.k0, j0, nn, S, ang, nang, E);
-    k_ff_cols<<<gridfor(nn * nrhs), 256, 0, st>>>(h->ph.k0, h->ph.eps0, N, j0, nn, S, u, q, nrhs, B);
+    k_ff_rows<<<gridfor(nn * nang), 256, 0, st>>>(h->g, h->ph.k0, j0, nn, S, ang, nang, E, bad);
+    k_ff_cols<<<gridfor(nn * nrhs), 256, 0, st>>>(h->ph.k0, h->ph.eps0, N, j0, nn, S, u, q, nrhs, B, bad + nang);
     const int n = items(nn, E, B, C);
     if (wsbm_zgemm_tc_batched(p.data(), n, make_double2(1.0, 0.0), make_double2(0.0, 0.0), ws, st))
       return WSBM_ERR_CUDA;
     k_ff_sum<<<gridfor((int64_t)nang * nrhs), 256, 0, st>>>(C, n, (int64_t)nang * nrhs, j0 > 0, out);
     wsbm_count_launches(3);
   }
+  k_farfield<<<nang, 256, 0, st>>>(h->g, h->ph.k0, h->ph.eps0, u, q, nrhs, ang, nang, bad, out);
+  wsbm_count_launch();
   return cudaGetLastError() == cudaSuccess ? WSBM_OK : WSBM_ERR_CUDA;
 }
 
@@ -2915,7 +2931,7 @@ extern "C" int wsbm_farfield(wsbm_hss_t h, const void* u, const void* q, int32_t
     const int rc = farfield_product(h, cu, cq, nrhs, angles, nang, (double2*)out);
     if (rc != WSBM_ERR_OOM) return rc;
   }
-  k_farfield<<<nang, 256, 0, h->st>>>(h->g, h->ph.k0, h->ph.eps0, cu, cq, nrhs, angles, nang, (double2*)out);
+  k_farfield<<<nang, 256, 0, h->st>>>(h->g, h->ph.k0, h->ph.eps0, cu, cq, nrhs, angles, nang, nullptr, (double2*)out);
   wsbm_count_launch();
   return cudaGetLastError() == cudaSuccess ? WSBM_OK : WSBM_ERR_CUDA;
 }
