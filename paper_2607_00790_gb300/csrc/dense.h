@@ -48,6 +48,8 @@ size_t wsbm_zgemm_crt_ws_bytes(int m, int n, int k);
 int wsbm_zgemm_crt(int m, int n, int k, double2 alpha, const double2* A, int64_t lda, const double2* B, int64_t ldb,
                    double2 beta, double2* C, int64_t ldc, void* ws, size_t ws_bytes, cudaStream_t st, int group);
 int wsbm_zgemm_crt_status();
+// Lets one bounded wait run out (2 s), for tests of what the callers make of it.
+int wsbm_tc_expire_wait(cudaStream_t st);
 // Many products in one launch: C_i = beta C_i + alpha A_i B_i (sizes per item; K padded with
 // zeros to the largest k).  ws: 256-byte aligned, wsbm_zgemm_tc_batched_ws_bytes(p, n) bytes.
 // At most 65535 items.  Returns 0, -1 or -3; enqueues only (the item table is copied to ws).

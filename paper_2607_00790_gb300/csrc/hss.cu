@@ -2916,7 +2916,10 @@ static int farfield_product(wsbm_hss* h, const double2* u, const double2* q, int
   }
   k_farfield<<<nang, 256, 0, st>>>(h->g, h->ph.k0, h->ph.eps0, u, q, nrhs, ang, nang, bad, out);
   wsbm_count_launch();
-  return cudaGetLastError() == cudaSuccess ? WSBM_OK : WSBM_ERR_CUDA;
+  if (cudaGetLastError() != cudaSuccess) return WSBM_ERR_CUDA;
+  // a bounded wait of the product that ran out leaves an incomplete pattern
+  const int t = wsbm_zgemm_tc_status(st);
+  return t == 0 ? WSBM_OK : t == -5 ? WSBM_ERR_TIMEOUT : WSBM_ERR_CUDA;
 }
 
 extern "C" int wsbm_farfield(wsbm_hss_t h, const void* u, const void* q, int32_t nrhs,

@@ -802,6 +802,18 @@ int wsbm_zgemm_tc_status(cudaStream_t st) {
   return wsbm_zgemm_crt_status();
 }
 
+// A wait on a barrier at which nothing arrives: it gives up after TC_WAIT_NS and leaves the error flag
+// set, as a product that hung would.
+__global__ void k_tc_expire() {
+  __shared__ uint64_t bar;
+  mbar_init(smem_u32(&bar), 1);
+  mbar_wait(smem_u32(&bar), 0);
+}
+int wsbm_tc_expire_wait(cudaStream_t st) {
+  k_tc_expire<<<1, 1, 0, st>>>();
+  return cudaGetLastError() == cudaSuccess ? 0 : -3;
+}
+
 // ------------------------------------------------ sketches Y = Omega M (Omega = +-1) ----
 // Y_i (l_i x n_i) = Omega[:l_i, :m_i] M_i (m_i x n_i complex) with Omega_rc = -1 when bit 0 of
 // the sketch hash of (r, c, seed) is set, else +1, shared by every item.  Omega is exact in BF16

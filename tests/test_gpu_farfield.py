@@ -56,3 +56,19 @@ def test_angles_without_a_direction(solver):
     got = solver.farfield(_t(u), _t(q), _t(ang)).cpu().numpy()
     rest = [a for a in range(NANG) if a not in (4, 12)]
     assert np.isnan(got[[4, 12]]).all() and np.array_equal(got[rest], plain[rest])
+
+
+def test_a_wait_that_runs_out_is_reported(solver):
+    """By the call whose product it may have cut short, and by no later one."""
+    import ctypes
+
+    import torch
+    u, q, ang = densities()
+    plain = solver.farfield(_t(u), _t(q), _t(ang)).cpu().numpy()
+    lib = ctypes.CDLL(binding.LIB_PATH)
+    assert lib["_Z19wsbm_tc_expire_waitP11CUstream_st"](None) == 0
+    torch.cuda.synchronize()
+    with pytest.raises(binding.WsbmError) as e:
+        solver.farfield(_t(u), _t(q), _t(ang))
+    assert e.value.code == -5  # WSBM_ERR_TIMEOUT
+    assert np.array_equal(solver.farfield(_t(u), _t(q), _t(ang)).cpu().numpy(), plain)
