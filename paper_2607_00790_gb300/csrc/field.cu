@@ -23,12 +23,15 @@ struct FldSlot {
 };
 
 // ---- side of the targets.  The Gauss sum is 0 or 1 up to the quadrature error, so FP32 decides
-// it nearly everywhere: coordinate differences from (hi, lo) FP32 pairs, sums of 128 terms in FP32,
-// the sums of those in FP64.  A target whose sum lies within FLD_SIDE_EPS sum_j w_j/r_j of the
-// threshold (every rounding error above is below a tenth of that), or that meets a node closer than
-// FP32 resolves, is summed again in FP64.  0.1 ms for 3001 targets and 16384 nodes, where one FP64
+// it nearly everywhere: coordinate differences from (hi, lo) FP32 pairs taken relative to the first
+// node (a curve far from the origin loses no digits), sums of 128 terms in FP32, the sums of those in
+// FP64.  A target whose sum lies within FLD_SIDE_EPS sum_j w_j/r_j of the threshold (every rounding
+// error above is below a tenth of that), or that has a node at a distance whose square is near the ends
+// of FP32's range (or beyond, or zero: FLD_R2_MIN, FLD_R2_MAX), is summed again in FP64.  0.1 ms for 3001 targets and 16384 nodes, where one FP64
 // thread per target took 10.4 ms.
 #define FLD_SIDE_EPS 1e-4f
+#define FLD_R2_MIN 1e-30f
+#define FLD_R2_MAX 1e30f
 struct SideSlot {
   float xh, xl, yh, yl, nx, ny, w;
 };
@@ -39,7 +42,8 @@ __global__ void __launch_bounds__(FLD_THREADS)
   __shared__ SideSlot sj[FLD_THREADS];
   const int64_t t = (int64_t)blockIdx.x * FLD_THREADS + threadIdx.x;
   const double px = t < nt ? tx[t] : 0.0, py = t < nt ? ty[t] : 0.0;
-  const float pxh = (float)px, pyh = (float)py, pxl = (float)(px - (double)pxh), pyl = (float)(py - (double)pyh);
+  const double x0 = g.x[0], y0 = g.y[0], qx = px - x0, qy = py - y0;
+  const float pxh = (float)qx, pyh = (float)qy, pxl = (float)(qx - (double)pxh), pyl = (float)(qy - (double)pyh);
   const int64_t j0 = (int64_t)blockIdx.y * jspan, j1 = min(g.n, j0 + jspan);
   double acc = 0.0, mag = 0.0;
   for (int64_t jc = j0; jc < j1; jc += FLD_THREADS) {
@@ -47,7 +51,7 @@ __global__ void __launch_bounds__(FLD_THREADS)
     const int64_t j = jc + threadIdx.x;
     if (j < j1) {
       SideSlot& s = sj[threadIdx.x];
-      const double x = g.x[j], y = g.y[j];
+      const double x = g.x[j] - x0, y = g.y[j] - y0;
       s.xh = (float)x;
       s.xl = (float)(x - (double)s.xh);
       s.yh = (float)y;
@@ -63,10 +67,11 @@ __global__ void __launch_bounds__(FLD_THREADS)
       const SideSlot& s = sj[jj];
       const float dx = (pxh - s.xh) + (pxl - s.xl), dy = (pyh - s.yh) + (pyl - s.yl);
       const float r2 = fmaf(dx, dx, dy * dy);
-      const float ir = rsqrtf(r2);  // infinite at r2 = 0: the FP64 sum decides
+      const float ir = rsqrtf(r2);
       const float wr = s.w * ir;
       a = fmaf(wr * ir, fmaf(dx, s.nx, dy * s.ny), a);
-      m += fabsf(wr);
+      // an infinite m leaves the decision to the FP64 sum, whatever became of the term
+      m += r2 > FLD_R2_MIN && r2 < FLD_R2_MAX ? fabsf(wr) : __int_as_float(0x7F800000);
     }
     acc += (double)a;
     mag += (double)m;
@@ -89,7 +94,7 @@ __global__ void __launch_bounds__(FLD_THREADS)
       mag += v.y;
     }
   const double off = fabs(acc + WSBM_PI);  // 2 pi |sum - 1/2|
-  const bool sure = off > (double)FLD_SIDE_EPS * mag;  // false for infinities and NaN
+  const bool sure = off > (double)FLD_SIDE_EPS * mag;  // false for an infinite or NaN mag
   unsure[threadIdx.x] = t < nt && !sure;
   if (t < nt && sure) side[t] = (-acc / (2.0 * WSBM_PI)) > 0.5 ? 1 : 0;
   __syncthreads();
