@@ -66,8 +66,14 @@
 #ifndef WSBM_TCSOLVE_WS
 #define WSBM_TCSOLVE_WS ((size_t)4 << 30)  // digit-plane work space of one solve product launch
 #endif
+// Roots from here on take the LU whose updates run on the tensor cores, one after another; smaller ones
+// share the launches of the batched FP64 LU, so that many small curves cost little more than one (a rule on
+// the count would make a curve's factors depend on its batch).  Batched / one after another, ms: n = 700
+// 10.1 / 4.4 for one root, 58 / 284 for 64; n = 1400 34.9 / 9.4 and 428 / 600; n = 2000 71 / 14 and 1230 /
+// 915.  The FP64 LU is a little more accurate too (n = 640: |PA - LU| 5.6e-15 |A| against 6.2e-15, largest
+// entry 4.4e-14 against 1.0e-13).
 #ifndef WSBM_BIGLU_MIN
-#define WSBM_BIGLU_MIN 512
+#define WSBM_BIGLU_MIN 2048
 #endif
 #ifndef WSBM_SKETCH_CUT
 #define WSBM_SKETCH_CUT 0.25  // measured: far-field error 3.6-5.8x tol, as with the full QR
@@ -1730,7 +1736,7 @@ static int factor_roots(const std::vector<wsbm_hss*>& hs, double ms_out[2]) {
       HK(upload(h0, small, &ds, tmp));
       HK(wsbm_lu_batched(ds, (int)small.size(), maxs, nullptr, st));
     }
-    if (wsb && wsbm_lu_big_status(st) != 0) return WSBM_ERR_TIMEOUT;
+    if (wsbm_lu_big_status(st) != 0) return WSBM_ERR_TIMEOUT;  // of the box factors' products, too
   }
   HC(cudaEventRecord(h0->ev[2], st));
   HC(cudaStreamSynchronize(st));
