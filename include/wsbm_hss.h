@@ -340,9 +340,10 @@ void wsbm_batch_destroy(wsbm_batch_t b);
  * matrix of eq. (weakly_bm) (every node pair, O(N^2) work, nothing stored): residuals and
  * iterative refinement of HSS and adjoint solutions.  x, y: device complex128 2N x nrhs in
  * paper order (for trans = 0, x by unknown and y by equation; the reverse for trans = 1).
- * The Hankel values of each node pair are evaluated once for up to eight right-hand sides.
- * Scratch: at most 4 x 2N x (eight waves of CTAs / ceil(N/128)) complex128 from the library's
- * allocator (wsbm_set_allocator) on `stream`.  Asynchronous.  Errors: INVALID_ARG, OOM, CUDA. */
+ * The Hankel values of each node pair are evaluated once for up to eight right-hand sides; a column of
+ * y does not depend on the others.
+ * Scratch: 8 x 2N x (32 CTAs per SM / ceil(N/128)) complex128 from the library's allocator
+ * (wsbm_set_allocator) on `stream`, 4, 2 or 1 x for fewer columns or where the allocator has no more.  Asynchronous.  Errors: INVALID_ARG, OOM, CUDA. */
 int wsbm_matvec(const wsbm_geom* g, const wsbm_params* p, int32_t trans, const void* x,
                 int32_t nrhs, void* y, void* stream);
 

@@ -9,6 +9,9 @@
 // partial sums, reduced in a fixed order by k_matvec_reduce.  Vectors in paper order.
 #define MV_THREADS 128
 #define MV_FLUSH 16  // divides MV_THREADS
+// CTAs per SM.  N = 16384, one and eight columns: 45.5 and 96.5 ms, 47.8 and 95.5 with 16 (a last wave that
+// is nearly empty), 48.4 and 101.7 with 8
+#define MV_WANT 32
 template <int NR>
 struct MvSlot {
   double x, y, nx, ny, w;
@@ -147,13 +150,8 @@ extern "C" int wsbm_matvec(const wsbm_geom* g, const wsbm_params* p, int32_t tra
   cudaStream_t st = (cudaStream_t)stream;
   const int64_t N = g->n;
   const int64_t nti = (N + MV_THREADS - 1) / MV_THREADS;
-  const int NR = nrhs > 4 ? 8 : (nrhs > 2 ? 4 : nrhs);  // columns of one launch
-  const auto kern = trans ? (NR == 8 ? k_matvec<true, 8> : NR == 4 ? k_matvec<true, 4> : NR == 2 ? k_matvec<true, 2> : k_matvec<true, 1>)
-                          : (NR == 8 ? k_matvec<false, 8> : NR == 4 ? k_matvec<false, 4> : NR == 2 ? k_matvec<false, 2> : k_matvec<false, 1>);
-  int nsm = wsbm_sm_count(), per_sm = 1;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, MV_THREADS, 0) != cudaSuccess || per_sm < 1)
-    per_sm = 1;
-  int64_t want = (int64_t)nsm * per_sm * (NR == 8 ? 4 : 8);  // about eight waves (four of twice the width)
+  // the split, hence a column's rounding, depends on N alone and not on how many columns come along
+  const int64_t want = (int64_t)wsbm_sm_count() * MV_WANT;
   int64_t nsplit = (want + nti - 1) / nti;
   if (nsplit < 1) nsplit = 1;
   if (nsplit > nti) nsplit = nti;
@@ -161,7 +159,11 @@ extern "C" int wsbm_matvec(const wsbm_geom* g, const wsbm_params* p, int32_t tra
   nsplit = (N + jspan - 1) / jspan;
   WsbmScratch scr(st);
   double2* part = nullptr;
-  if ((rc = scr.get((size_t)nsplit * NR * 2 * N * sizeof(double2), (void**)&part))) return rc;
+  int NR = nrhs > 4 ? 8 : (nrhs > 2 ? 4 : nrhs);  // columns of one launch, fewer where the scratch is short
+  while ((rc = scr.get((size_t)nsplit * NR * 2 * N * sizeof(double2), (void**)&part)) == WSBM_ERR_OOM && NR > 1) NR /= 2;
+  if (rc) return rc;
+  const auto kern = trans ? (NR == 8 ? k_matvec<true, 8> : NR == 4 ? k_matvec<true, 4> : NR == 2 ? k_matvec<true, 2> : k_matvec<true, 1>)
+                          : (NR == 8 ? k_matvec<false, 8> : NR == 4 ? k_matvec<false, 4> : NR == 2 ? k_matvec<false, 2> : k_matvec<false, 1>);
   DevGeom dg = wsbm_devgeom(g);
   for (int c = 0; c < nrhs; c += NR) {
     const int nr = nrhs - c < NR ? nrhs - c : NR;
