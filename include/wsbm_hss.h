@@ -343,7 +343,8 @@ void wsbm_batch_destroy(wsbm_batch_t b);
  * The Hankel values of each node pair are evaluated once for up to eight right-hand sides; a column of
  * y does not depend on the others.
  * Scratch: 8 x 2N x (32 CTAs per SM / ceil(N/128)) complex128 from the library's allocator
- * (wsbm_set_allocator) on `stream`, 4, 2 or 1 x for fewer columns or where the allocator has no more.  Asynchronous.  Errors: INVALID_ARG, OOM, CUDA. */
+ * (wsbm_set_allocator) on `stream`, 4, 2 or 1 x for fewer columns or where the allocator has no
+ * more.  Asynchronous.  Errors: INVALID_ARG, OOM, CUDA. */
 int wsbm_matvec(const wsbm_geom* g, const wsbm_params* p, int32_t trans, const void* x,
                 int32_t nrhs, void* y, void* stream);
 
@@ -353,8 +354,8 @@ int wsbm_matvec(const wsbm_geom* g, const wsbm_params* p, int32_t trans, const v
  * the total field), interior points the total field eps1 S_k1[q] - D_k1[u].  tx, ty: device
  * doubles; out: device complex128 nt x nrhs; inside: device int8 nt, 1 for interior points
  * (Gauss test of the Laplace double layer).  The trapezoidal sums are accurate a few node
- * spacings away from the curve; no near-singular quadrature is applied.  Scratch from the
- * library's allocator (wsbm_set_allocator) on `stream`; asynchronous.  Errors: INVALID_ARG, OOM, CUDA. */
+ * spacings away from the curve; no near-singular quadrature is applied.  A column of out does not
+ * depend on the others.  Scratch from the library's allocator (wsbm_set_allocator) on `stream`; asynchronous.  Errors: INVALID_ARG, OOM, CUDA. */
 int wsbm_field(const wsbm_geom* g, const wsbm_params* p, const void* u, const void* q,
                int32_t nrhs, const double* tx, const double* ty, int64_t nt, void* out,
                int8_t* inside, void* stream);

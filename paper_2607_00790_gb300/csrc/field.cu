@@ -17,6 +17,8 @@
 namespace {
 
 #define FLD_THREADS 128
+// CTAs per SM.  16384 nodes, 3001 targets, 1 and 8 columns: 4.0 and 8.58 ms (16: 3.9 and 8.78; 8: 4.1 and 8.78)
+#define FLD_WANT 32
 
 struct FldSlot {
   double x, y, nx, ny, w;
@@ -247,17 +249,17 @@ extern "C" int wsbm_field(const wsbm_geom* g, const wsbm_params* p, const void* 
   cudaStream_t st = (cudaStream_t)stream;
   const int64_t N = g->n;
   const int64_t nti = (nt + FLD_THREADS - 1) / FLD_THREADS;
-  const int nr = nrhs > 4 ? 8 : (nrhs > 2 ? 4 : nrhs);  // right-hand sides per launch
-  const int per_sm = nr == 8 ? 2 : 4;                   // resident CTAs per SM
-  // about eight waves (four of the 8-column kernel, whose partial sums are twice as wide), at least
-  // 128 sources a CTA
-  const int64_t want = (int64_t)wsbm_sm_count() * per_sm * (nr == 8 ? 4 : 8);
+  // the split, hence a column's rounding, depends on N and the targets alone and not on how many columns
+  // come along: at least 128 sources a CTA
+  const int64_t want = (int64_t)wsbm_sm_count() * FLD_WANT;
   int64_t nsplit = std::max<int64_t>(1, std::min<int64_t>((want + nti - 1) / nti, (N + 127) / 128));
   const int64_t jspan = ((N + nsplit - 1) / nsplit + FLD_THREADS - 1) / FLD_THREADS * FLD_THREADS;
   nsplit = (N + jspan - 1) / jspan;
   WsbmScratch scr(st);
   double2* part = nullptr;
-  if ((rc = scr.get((size_t)nsplit * nt * nr * sizeof(double2), (void**)&part))) return rc;
+  int nr = nrhs > 4 ? 8 : (nrhs > 2 ? 4 : nrhs);  // right-hand sides per launch, fewer where the scratch is short
+  while ((rc = scr.get((size_t)nsplit * nt * nr * sizeof(double2), (void**)&part)) == WSBM_ERR_OOM && nr > 1) nr /= 2;
+  if (rc) return rc;
   DevGeom dg = wsbm_devgeom(g);
   const dim3 grid((unsigned)nti, (unsigned)nsplit);
   k_field_side<<<grid, FLD_THREADS, 0, st>>>(dg, tx, ty, nt, jspan, part);

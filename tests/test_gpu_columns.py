@@ -61,3 +61,15 @@ def test_matvec_with_little_memory():
         binding.use_torch_allocator(False)
     assert asked == [asked[3] * f for f in (8, 4, 2, 1)] and not held
     assert np.array_equal(got, full)
+
+
+@pytest.mark.parametrize("N,nt", [(300, 70), (5000, 129), (20000, 1000)])
+def test_field_columns(N, nt):
+    g, keep, p, z, rng = problem(N, 2, N, 12)
+    t, s = rng.uniform(0, 2 * np.pi, nt), rng.uniform(0.2, 3.0, nt)
+    r = s * (1 + 0.3 * np.cos(5 * t))
+    pts = _t(r * np.cos(t)), _t(r * np.sin(t))
+    full = binding.field(g, p, _t(z[0]), _t(z[1]), *pts)[0].cpu().numpy()
+    for n in COUNTS:
+        got = binding.field(g, p, _t(z[0, :, :n]), _t(z[1, :, :n]), *pts)[0].cpu().numpy()
+        assert np.array_equal(got, full[:, :n]), n
