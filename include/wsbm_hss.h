@@ -355,7 +355,8 @@ int wsbm_matvec(const wsbm_geom* g, const wsbm_params* p, int32_t trans, const v
  * doubles; out: device complex128 nt x nrhs; inside: device int8 nt, 1 for interior points
  * (Gauss test of the Laplace double layer).  The trapezoidal sums are accurate a few node
  * spacings away from the curve; no near-singular quadrature is applied.  A column of out does not
- * depend on the others.  Scratch from the library's allocator (wsbm_set_allocator) on `stream`; asynchronous.  Errors: INVALID_ARG, OOM, CUDA. */
+ * depend on the others.  Scratch from the library's allocator (wsbm_set_allocator) on `stream`;
+ * asynchronous.  Errors: INVALID_ARG, OOM, CUDA. */
 int wsbm_field(const wsbm_geom* g, const wsbm_params* p, const void* u, const void* q,
                int32_t nrhs, const double* tx, const double* ty, int64_t nt, void* out,
                int8_t* inside, void* stream);

@@ -625,8 +625,23 @@ size_t wsbm_zgemm_crt_ws_bytes(int m, int n, int k) { return crt_bytes(m, n, crt
 // 1024 x 128 0.118 / 0.100; small or thin results leave SMs idle.
 bool wsbm_zgemm_crt_fits(int m, int n, int k) { return k >= 160 && m >= 512 && n >= 512; }
 
+// Do the column-major blocks X (xr x xc) and Y (yr x yc) share an element?  Exact for equal leading
+// dimensions (two blocks of one matrix), else by the ranges of their addresses.
+static bool blocks_meet(const double2* X, int64_t ldx, int64_t xr, int64_t xc, const double2* Y, int64_t ldy, int64_t yr,
+                        int64_t yc) {
+  const uintptr_t x0 = (uintptr_t)X, x1 = (uintptr_t)(X + (xc - 1) * ldx + xr);
+  const uintptr_t y0 = (uintptr_t)Y, y1 = (uintptr_t)(Y + (yc - 1) * ldy + yr);
+  if (x1 <= y0 || y1 <= x0) return false;
+  if (ldx != ldy || (y0 - x0) % sizeof(double2)) return true;
+  const int64_t d = ((int64_t)y0 - (int64_t)x0) / (int64_t)sizeof(double2);
+  const int64_t dr = ((d % ldx) + ldx) % ldx, dc = (d - dr) / ldx;  // Y begins dr rows and dc columns after X
+  auto meet = [&](int64_t r, int64_t c) { return r < xr && r + yr > 0 && c < xc && c + yc > 0; };
+  return meet(dr, dc) || meet(dr - ldx, dc + 1);
+}
+
 // ws_bytes may be less than wsbm_zgemm_crt_ws_bytes: the longer side then goes through in strips
-// (-2 if not even a strip of 512 fits: nothing was launched).
+// (-2 if not even a strip of 512 fits, or if C is written piece by piece while A or B, which it overlaps,
+// is still to be read: nothing was launched).
 int wsbm_zgemm_crt(int m, int n, int k, double2 alpha, const double2* A, int64_t lda, const double2* B, int64_t ldb,
                    double2 beta, double2* C, int64_t ldc, void* ws, size_t ws_bytes, cudaStream_t st, int group) {
   const int64_t Kp = crt_kp(k);
@@ -636,6 +651,9 @@ int wsbm_zgemm_crt(int m, int n, int k, double2 alpha, const double2* A, int64_t
     if (x <= 512) return -2;
     x = (x / 2 + 127) / 128 * 128;
   }
+  if ((k > CR_KMAX || ms < m || ns < n) &&
+      (blocks_meet(A, lda, m, k, C, ldc, m, n) || blocks_meet(B, ldb, k, n, C, ldc, m, n)))
+    return -2;
   __nv_bfloat16 *PA = (__nv_bfloat16*)ws,
                 *PB = (__nv_bfloat16*)((char*)ws + crt_up((size_t)CR_PL * ms * Kp * 2));
   int2* exps = (int2*)((char*)PB + crt_up((size_t)CR_PL * ns * Kp * 2));
