@@ -383,7 +383,7 @@ int wsbm_sketch(const void* A, int64_t lda, int32_t m, int32_t n, int32_t l, voi
  *   A  device complex128 m x k (lda >= m); B: k x n (ldb >= k); C: m x n (ldc >= m); all
  *      column-major; alpha, beta: host, 2 doubles (re, im) each
  *   1 <= k <= 32768
- * Large products (m, n >= 512, k >= 160) are formed from the same scaled integers modulo 14 numbers
+ * Large products (m, n >= 512, k >= 160, and tiles enough for the whole GPU) are formed from the same scaled integers modulo 14 numbers
  * instead (28 real products in place of 136, nothing dropped) and put together by the Chinese
  * remainder theorem; same bound.
  * Work space (7 (m + 2n) 2k BF16 values, rounded up; 28 (m + n) k for large products where the

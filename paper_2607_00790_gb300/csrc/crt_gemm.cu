@@ -620,10 +620,18 @@ static size_t crt_bytes(int64_t m, int64_t n, int64_t Kp) {
 
 size_t wsbm_zgemm_crt_ws_bytes(int m, int n, int k) { return crt_bytes(m, n, crt_kp(k)); }
 
-// Measured against the digit planes: 8192 x 8192 x 256 2.55 ms against 3.60, x 512 4.50 / 6.34, x 128
-// 2.04 / 2.11 (the reduction of the sums, 6 clocks per entry and SM, does not shrink with k), 1024 x
-// 1024 x 128 0.118 / 0.100; small or thin results leave SMs idle.
-bool wsbm_zgemm_crt_fits(int m, int n, int k) { return k >= 160 && m >= 512 && n >= 512; }
+// Against the digit planes: large products 8192 x 8192 x 256 2.55 ms against 3.60, x 512 4.50 / 6.34; below k
+// = 160 the reduction of the sums, 6 clocks per entry and SM, does not shrink with k (8192 x 8192 x 128 2.04 /
+// 2.11).  Smaller results by the waves that their tiles take (128 x 48 here, 128 x 32 there), one of which takes
+// up to 1.2 of the other's time with the splits.  Measured for k = 160 to 1000, us at k = 256: 768 x 768 (one
+// wave each) 67 / 59, 1024 x 1024 (2, 2) 101 / 87, 1200 x 1200 (2, 3) 105 / 117, 1300 x 1300 (3, 3) 141 / 122,
+// 1600 x 1600 (3, 5) 147 / 191, 4000 x 512 (3, 4) 157 / 172, 6000 x 512 (4, 5) 204 / 217.
+bool wsbm_zgemm_crt_fits(int m, int n, int k) {
+  if (k < 160 || m < 512 || n < 512) return false;
+  const int64_t rows = (m + 127) / 128, sms = wsbm_sm_count();
+  const int64_t here = (rows * ((n + 47) / 48) + sms - 1) / sms, there = (rows * ((n + 31) / 32) + sms - 1) / sms;
+  return 6 * here <= 5 * there;
+}
 
 // Do the column-major blocks X (xr x xc) and Y (yr x yc) share an element?  Exact for equal leading
 // dimensions (two blocks of one matrix), else by the ranges of their addresses.
