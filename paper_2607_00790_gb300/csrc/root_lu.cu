@@ -21,10 +21,9 @@
 #define LUB_NB_BIG 256  // outer panel width from LUB_BIG_N on: deeper tensor-core products
 #endif
 #ifndef LUB_BIG_N
-// 256 columns from here on only: at n = 8200 they take 104 ms against 115, but their wider explicit
-// inverses cost accuracy, |PA - LU| / |A| 4.1e-14 against 2.8e-14 and the largest entry 7.6e-13 against
-// 5e-13 (128-column panels of the launch-per-column version: 4.5e-14 and 5.5e-13).  n = 16384: 416 ms
-// against 537.
+// 256 columns from here on only: at n = 8200 they take 95 ms against 107, but their wider explicit
+// inverses cost accuracy (random matrix, rms of PA - LU over |A|: 4.4e-14 against 2.7e-14; 2.75e-14 with
+// the launch-per-column version).  n = 12288: 200 ms against 245, n = 16384: 368 against 489.
 #define LUB_BIG_N 12288
 #endif
 #define LUB_W 32            // widest base panel: one lane per column
@@ -70,9 +69,13 @@ __device__ __forceinline__ unsigned long long lub_time() {
 // the last column.  Per column every CTA publishes its best candidate (key) and that candidate's
 // panel row; every CTA then reads all the keys, takes the winner's row as the pivot row and
 // updates its own rows, so a column costs one exchange through L2 instead of two launches.  Bound by
-// that exchange (release, 152 polled keys, one row read): 4.7 us a column at n = 8200, 39 ms in all.
+// that exchange (release, 152 polled keys, one row read): 3.8 us a column at n = 8200, 31 ms in all.
 // Only the next column is updated before its candidate is published, the others while it travels (with
 // the whole update first, and 64-bit reductions, 6.4 us; launches per column and their gaps 100 ms).
+// The others take the pivots two at a time, j even and j + 1, their products summed before the one
+// subtraction: an entry is rounded at its own size once a pair (a multiply-add per product would round it
+// four times).  1/2 on the diagonal, rms of PA - LU there in ulp(1/2): n = 2048 0.91, 8200 1.68 (a pivot at a
+// time 1.43, 2.08; 8-column panels with products between them 0.89, 1.63).
 //   slots  key slots [w][LUB_MAXCTA], zero on entry (a key is never zero)
 //   cand   published rows [2][LUB_MAXCTA][32]; a slot of one parity is rewritten two columns
 //          later, after every CTA has published the column between (and so has read it)
@@ -82,8 +85,7 @@ __global__ void __launch_bounds__(LUB_T, 1)
                 double2* cand, double2* diag, int* __restrict__ piv, int* __restrict__ info) {
   extern __shared__ double2 sm[];
   const int RS = R | 1;  // odd stride: a row read across the columns meets no bank twice
-  double2* lcol = sm + (size_t)w * RS;
-  __shared__ double2 prow[LUB_W];
+  __shared__ double2 prow[4][LUB_W];  // rows of the last four pivots, by column modulo 4
   __shared__ double2 s_inv;
   __shared__ unsigned long long red[LUB_T / 32], keys[LUB_T / 32];
   __shared__ int s_err;
@@ -101,49 +103,56 @@ __global__ void __launch_bounds__(LUB_T, 1)
     const unsigned long long k = lub_key(sm[i], r0 + i);
     best = k > best ? k : best;
   }
-  const int nchunk = (cnt + 31) / 32;
   int prev = 0;  // first row below the last pivot's: rows from here on await its update
+  // a lane per real component where a step waits for the result: half the FP64 instructions a warp
+  const int part = lane & 1;
+  auto flip = [part](double v) {  // -v for the real part: on the integer pipe
+    return __hiloint2double(__double2hiint(v) ^ (part ? 0 : (int)0x80000000), __double2loint(v));
+  };
+  auto comp = [part](const double2& v, int other) { return (part ^ other) ? v.y : v.x; };
+  auto dot = [&](double x, const double2& l, const double2& u) {  // x plus the product's component
+    return fma(l.x, comp(u, 0), fma(flip(l.y), comp(u, 1), x));
+  };
 
   for (int j = 0; j < w; ++j) {
-    const int c = c0 + j, par = j & 1;
+    const int c = c0 + j;
     best = lub_warp_max(best);
     if (lane == 0) red[warp] = best;
     __syncthreads();
     unsigned long long* row = slots + (size_t)j * LUB_MAXCTA;
-    // column j is up to date, the columns after it await the update by the last pivot: warp 0 applies it
-    // to the candidate's row (and to row c) alone and publishes, the other warps to the rows in shared
-    // memory, while the candidates travel
+    // Column j is up to date.  At an even j the columns after it await the pivots j - 2 and j - 1: those
+    // before `half` take them now, the others at j + 1, when all await pivot j as well.
+    const int je = j & ~1, half = je + 1 + max(2, (w - je) / 2);
+    const bool pair = je > 0, odd = j & 1;
+    const double2 *ra = prow[(je - 2) & 3], *rb = prow[(je - 1) & 3], *rc = prow[je & 3];
+    // The candidate's row (warps 0 and 1) is published complete, but for the columns from `half` on at an odd
+    // j; row c (warps 2 and 3 of its CTA) as the rows in shared memory will be after this update.
     unsigned long long k = 0;
-    double2 vloc, vdiag, lloc, ldiag, pr;
-    if (warp == 0) {
+    if (warp < (b == 0 ? 4 : 2)) {
       k = lub_warp_max(lane < LUB_T / 32 ? red[lane] : 0ull);
-      const int loc = (int)(0xFFFFFFFFu - (unsigned)k) - r0;
-      if (lane < w) {
-        vloc = sm[lane * RS + loc];
-        if (b == 0) vdiag = sm[lane * RS + j];
-      }
-      if (j > 0) {
-        pr = prow[lane];
-        lloc = lcol[loc];
-        if (b == 0) ldiag = lcol[j];
+      const bool mine = warp < 2;
+      const int loc = mine ? (int)(0xFFFFFFFFu - (unsigned)k) - r0 : j, t = 16 * (warp & 1) + (lane >> 1);
+      if (t < w) {
+        double x = comp(sm[t * RS + loc], 0);
+        if (t > j) {
+          if (mine && odd) {
+            if (t < half) x -= dot(0.0, sm[je * RS + loc], rc[t]);
+          } else if (pair && (mine || (t >= half) == odd)) {
+            x -= dot(dot(0.0, sm[(je - 1) * RS + loc], rb[t]), sm[(je - 2) * RS + loc], ra[t]);
+          }
+        }
+        double2* o = mine ? cand + ((size_t)(j & 1) * LUB_MAXCTA + b) * LUB_W : diag + (j & 1) * LUB_W;
+        __stcg((double*)(o + t) + part, x);
       }
     }
     __syncthreads();
-    if (warp == 0) {
-      if (j > 0 && lane > j && lane < w) {
-        vloc = cfms(lloc, pr, vloc);
-        if (b == 0) vdiag = cfms(ldiag, pr, vdiag);
-      }
-      if (lane < w) {
-        __stcg(cand + ((size_t)par * LUB_MAXCTA + b) * LUB_W + lane, vloc);
-        if (b == 0) __stcg(diag + par * LUB_W + lane, vdiag);
-      }
-      __syncwarp();
-      if (lane == 0) st_release(row + b, k);
-    } else if (j > 0) {
-      for (int e = warp - 1; e < nchunk * (w - 1 - j); e += LUB_T / 32 - 1) {
-        const int i = (e % nchunk) * 32 + lane, t = j + 1 + e / nchunk;
-        if (i >= prev && i < cnt) sm[t * RS + i] = cfms(lcol[i], prow[t], sm[t * RS + i]);
+    if (tid == 0) st_release(row + b, k);
+    if (pair) {  // while the candidates travel
+      const int t0 = odd ? half : j + 1, t1 = odd ? w : min(half, w), rows = cnt - prev;
+      for (int e = tid; e < rows * (t1 - t0); e += LUB_T) {  // (row, column) packed: no lane without a row
+        const int q = e / rows, i = prev + e - q * rows, t = t0 + q;
+        const double2 v = cfma(sm[(je - 2) * RS + i], ra[t], cmul(sm[(je - 1) * RS + i], rb[t])), x = sm[t * RS + i];
+        sm[t * RS + i] = make_double2(x.x - v.x, x.y - v.y);
       }
     }
     // all keys of this column, a thread each (bounded); a warp that read several in turn would wait
@@ -170,12 +179,10 @@ __global__ void __launch_bounds__(LUB_T, 1)
       top = lub_warp_max(lane < LUB_T / 32 ? keys[lane] : 0ull);
       const int p = (int)(0xFFFFFFFFu - (unsigned)top), bp = (p - c0) / R;
       if (lane < w) {
-        const double2 v = __ldcg(cand + ((size_t)par * LUB_MAXCTA + bp) * LUB_W + lane);
-        prow[lane] = v;
-        if (p != c) {
-          if (b == bp) sm[lane * RS + (p - r0)] = __ldcg(diag + par * LUB_W + lane);
-          if (b == 0) sm[lane * RS + j] = v;
-        }
+        const double2 v = __ldcg(cand + ((size_t)(j & 1) * LUB_MAXCTA + bp) * LUB_W + lane);
+        prow[j & 3][lane] = v;
+        if (p != c && b == bp) sm[lane * RS + (p - r0)] = __ldcg(diag + (j & 1) * LUB_W + lane);
+        if (b == 0) sm[lane * RS + j] = v;
         if (lane == j) {
           const bool zero = v.x == 0.0 && v.y == 0.0;
           s_inv = zero ? make_double2(0.0, 0.0) : cdiv(make_double2(1.0, 0.0), v);
@@ -191,18 +198,35 @@ __global__ void __launch_bounds__(LUB_T, 1)
     const int first = b == 0 ? j + 1 : 0;
     const double2 iv = s_inv;
     best = 0;
-    for (int i = tid; i < cnt; i += LUB_T)
-      if (i >= first) {
-        const double2 l = cmul(sm[j * RS + i], iv);
-        sm[j * RS + i] = l;
-        lcol[i] = l;
-        if (j + 1 < w) {
-          const double2 v = cfms(l, prow[j + 1], sm[(j + 1) * RS + i]);
-          sm[(j + 1) * RS + i] = v;
-          const unsigned long long x = lub_key(v, r0 + i);
+    for (int i0 = first; i0 < cnt; i0 += LUB_T / 2) {  // the same for every lane
+      const int i = i0 + (tid >> 1), ii = min(i, cnt - 1);
+      const double2 a = sm[j * RS + ii];
+      const double l = fma(comp(a, 0), iv.x, flip(comp(a, 1) * iv.y)), lo = __shfl_xor_sync(0xFFFFFFFFu, l, 1);
+      __syncwarp();
+      if (i < cnt) ((double*)&sm[j * RS + i])[part] = l;
+      if (j + 1 < w) {
+        const double2 u1 = prow[j & 3][j + 1];
+        double s = fma(part ? lo : l, comp(u1, 0), flip((part ? l : lo) * comp(u1, 1)));
+        if (odd) s = dot(s, sm[je * RS + ii], rc[j + 1]);
+        const double v = comp(sm[(j + 1) * RS + ii], 0) - s;
+        const int h = __double2hiint(v) & 0x7fffffff, ho = __shfl_xor_sync(0xFFFFFFFFu, h, 1);
+        if (i < cnt) {
+          ((double*)&sm[(j + 1) * RS + i])[part] = v;
+          const unsigned long long x = (unsigned long long)max(h, ho) << 32 | (0xFFFFFFFFu - (unsigned)(r0 + i));
           best = x > best ? x : best;
         }
       }
+    }
+    // an odd j's pivot row from `half` on (at most 15 columns), by the last warp, a lane per component
+    const int t = half + (lane >> 1);
+    if (warp == LUB_T / 32 - 1 && odd && t < w) {
+      double2* r = prow[j & 3];
+      double x = comp(r[t], 0);
+      if (pair) x -= dot(dot(0.0, r[je - 1], rb[t]), r[je - 2], ra[t]);
+      x -= dot(0.0, r[je], rc[t]);
+      ((double*)&r[t])[part] = x;
+      if (b == 0) ((double*)&sm[t * RS + j])[part] = x;
+    }
     prev = first;
   }
   __syncthreads();
@@ -269,7 +293,7 @@ struct LubCtx {
 int lub_base_width(int n) {
   const int64_t per = std::max<int64_t>(LUB_MINROWS, (n + wsbm_sm_count() - 1) / wsbm_sm_count()) + 1;
   for (int w = LUB_W; w > 1; w /= 2)
-    if (per * (w + 1) * (int64_t)sizeof(double2) <= LUB_SMEM) return w;
+    if (per * w * (int64_t)sizeof(double2) <= LUB_SMEM) return w;
   return 1;
 }
 
@@ -305,7 +329,7 @@ int lub_rec(const LubCtx& x, int c0, int c1, int base) {
     int rows = x.n - c0, nsm = std::min(wsbm_sm_count(), LUB_MAXCTA);
     int R = std::max(LUB_MINROWS, (rows + nsm - 1) / nsm);
     int G = (rows + R - 1) / R, width = w, c = c0;
-    size_t smem = ((size_t)w * (R | 1) + R) * sizeof(double2);
+    size_t smem = (size_t)w * (R | 1) * sizeof(double2);
     if (wsbm_smem_optin((const void*)k_lub_panel, LUB_SMEM) != cudaSuccess) return -3;
     double2* A = x.A;
     int64_t lda = x.lda;
