@@ -269,10 +269,10 @@ int wsbm_refine(wsbm_hss_t h, int32_t trans, const void* rhs, int32_t nrhs, void
  * u_inf(a) = e^{i pi/4}/sqrt(8 pi k0) sum_j w_j [-i k0 (xh.n_j) u_j - eps0 q_j] e^{-i k0 xh.x_j}.
  * u, q: device complex128 N x nrhs; angles: device doubles; out: device complex128
  * nang x nrhs.
- * From 8 right-hand sides, 8 angles and 256 nodes on the sum is a product on the tensor cores (error
- * bound of wsbm_zgemm, infinities and NaN as in the sum), unless its work space cannot be had or the
- * stream is being captured: then a column's last bits are not those of fewer right-hand sides, and
- * the call is synchronous.  Otherwise asynchronous.  Errors: INVALID_ARG, CUDA, TIMEOUT (a bounded
+ * For many right-hand sides (8 and more; the more, the smaller N and nang) the sum is a product on
+ * the tensor cores (error bound of wsbm_zgemm, infinities and NaN as in the sum), unless its work space
+ * cannot be had or the stream is being captured: then a column's last bits are not those of fewer
+ * right-hand sides, and the call is synchronous.  Otherwise asynchronous.  Errors: INVALID_ARG, CUDA, TIMEOUT (a bounded
  * wait inside the product ran out; out is then incomplete). */
 int wsbm_farfield(wsbm_hss_t h, const void* u, const void* q, int32_t nrhs, const double* angles,
                   int32_t nang, void* out);

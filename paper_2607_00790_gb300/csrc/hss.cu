@@ -2872,6 +2872,16 @@ extern "C" int wsbm_rhs_planewave(wsbm_hss_t h, const double* angles, int32_t na
   return cudaGetLastError() == cudaSuccess ? WSBM_OK : WSBM_ERR_CUDA;
 }
 
+// Whether the product is the cheaper form.  Microseconds, measured for N = 256 .. 16384, 1 .. 128 right-hand
+// sides and 8 .. 360 angles: the kernel takes 30 and 8.3 per pass of an SM over 256 nodes, 8 columns and one
+// angle; the product 150 (a dozen launches and the wait for its flag) and 0.2 per 1000 pairs of node and angle.
+// N = 256, 8 columns, 90 angles: kernel 46, product 149; N = 8192: 255, 312; N = 16384, 8 angles: 471, 242;
+// N = 2048, 16 columns, 360 angles: 440, 312.
+static bool farfield_as_product(int64_t N, int nrhs, int nang) {
+  const double passes = (double)((N + 255) / 256 * ((nrhs + 7) / 8)) * std::max(1.0, (double)nang / wsbm_sm_count());
+  return nrhs >= 8 && nang >= 8 && N >= 256 && 150.0 + 2e-4 * (double)N * nang < 30.0 + 8.3 * passes;
+}
+
 // WSBM_ERR_OOM: nothing was launched.
 static int farfield_product(wsbm_hss* h, const double2* u, const double2* q, int nrhs, const double* ang, int nang,
                             double2* out) {
@@ -2934,9 +2944,9 @@ extern "C" int wsbm_farfield(wsbm_hss_t h, const void* u, const void* q, int32_t
   if (nrhs == 0 || nang == 0) return WSBM_OK;
   if (!u || !q || !angles || !out) return WSBM_ERR_INVALID_ARG;
   const double2 *cu = (const double2*)u, *cq = (const double2*)q;
-  // from 8 right-hand sides on as a product, unless its work space cannot be had or the stream is
-  // being captured (the product's item table is copied from host memory of this call)
-  if (nrhs >= 8 && nang >= 8 && h->N >= 256) {
+  // unless the product's work space cannot be had or the stream is being captured (the item table is
+  // copied from host memory of this call)
+  if (farfield_as_product(h->N, nrhs, nang)) {
     const int rc = farfield_product(h, cu, cq, nrhs, angles, nang, (double2*)out);
     if (rc != WSBM_ERR_OOM) return rc;
   }

@@ -7,7 +7,7 @@ import oracle
 from paper_2607_00790_gb300 import binding, inputs
 
 pytestmark = pytest.mark.gpu
-N, NRHS, NANG = 300, 20, 13
+N, NRHS, NANG = 300, 200, 13
 
 
 def _t(a):
@@ -72,3 +72,46 @@ def test_a_wait_that_runs_out_is_reported(solver):
         solver.farfield(_t(u), _t(q), _t(ang))
     assert e.value.code == -5  # WSBM_ERR_TIMEOUT
     assert np.array_equal(solver.farfield(_t(u), _t(q), _t(ang)).cpu().numpy(), plain)
+
+
+def test_rule():
+    """The product where it is the cheaper form (measured on 152 SMs), the kernel (one launch) elsewhere."""
+    import ctypes
+
+    import torch
+    if torch.cuda.get_device_properties(0).multi_processor_count != 152:
+        pytest.skip("measured on 152 SMs")
+    count = ctypes.CDLL(binding.LIB_PATH)["_Z17wsbm_launch_countv"]
+    count.restype = ctypes.c_int64
+    for n in (256, 1024, 4096, 16384):
+        c = inputs.star(n)
+        g, keep = binding.make_geom(c)
+        s = binding.Solver(g, binding.make_params(float(inputs.k0_for_density(c)), 1.5))
+        for nrhs, nang, product in ((1, 360, False), (8, 360, False), (8, 8, n > 2048), (16, 36, n > 2048), (16, 360, n > 2048),
+                                    (64, 8, n > 256), (64, 360, True), (200, 8, True), (9, 7, False)):
+            u = torch.ones(nrhs, n, dtype=torch.complex128, device="cuda").T
+            a = torch.linspace(0, 6, nang, dtype=torch.float64, device="cuda")
+            before = count()
+            s.farfield(u, u, a)
+            assert (count() - before > 1) == product, (n, nrhs, nang)
+        s.close()
+
+
+@pytest.mark.parametrize("n,nrhs,nang", [(256, 129, 8), (257, 200, 131), (300, 193, 9), (511, 65, 129), (1000, 64, 360)])
+def test_product_at_its_edges(n, nrhs, nang):
+    c = inputs.star(n)
+    ph = oracle.Physics(inputs.k0_for_density(c), n=1.5)
+    g, keep = binding.make_geom(c)
+    rng = np.random.default_rng(nrhs)
+    u, q = (rng.standard_normal((n, nrhs)) + 1j * rng.standard_normal((n, nrhs)) for _ in range(2))
+    ang = rng.uniform(0, 2 * np.pi, nang)
+    s = binding.Solver(g, binding.make_params(ph.k0, 1.5))
+    got = s.farfield(_t(u), _t(q), _t(ang)).cpu().numpy()
+    s.close()
+    ref = oracle.farfield(c, ph, u, q, ang).reshape(got.shape)
+    k0, w = ph.k0, c["w"][:, None]
+    terms = (w * (k0 * np.abs(u) + np.abs(q))).sum(0) / np.sqrt(8 * np.pi * k0)
+    # an ulp or two of the phase k0 r in each term on both sides, and the rounding of the product:
+    # 2^-53 of a row's largest factor times a column's (about 16 times the mean product here)
+    tol = np.finfo(np.float64).eps * (16 * k0 * np.hypot(c["x"], c["y"]).max() + 256)
+    assert np.all(np.abs(got - ref) <= tol * terms)
