@@ -12,6 +12,8 @@
 // level in one launch).
 #include <math.h>
 
+#include <algorithm>
+
 #include "entry_blocks.cuh"
 
 #define PAIR_CLASSES 4  // far, middle, near, diagonal (k_pairs)
@@ -180,11 +182,13 @@ __global__ void __launch_bounds__(WSBM_PAIR_THREADS)
 
 // ---------------------------------------------------------------- entries by index lists ----
 // Entries A[rows, cols] for arbitrary lists of unknowns, one launch without work space: a tile
-// takes RAW_F row slots and RAW_S column slots, where slot t of a list of n indices is the pair
+// takes TR row slots and TC column slots (128 pairs), where slot t of a list of n indices is the pair
 // (t, t + ceil(n/2)).  Lists made of the u and then the q of the same nodes (the usual request of
 // a block) have both unknowns of a node in one slot, so a node pair is evaluated once for its four
 // entries; in any other tile the four entries of a slot pair are evaluated one by one, each with
-// the part of the block that it needs (about 35 to 65 FP64 operations in place of 71).
+// the part of the block that it needs (about 35 to 65 FP64 operations in place of 71): by a CTA each while
+// the tiles are too few to fill the GPU.  Tiles of 32 x 4 slots, of 4 x 32 where there are few rows (8 rows by
+// 30000 columns: 91 us, 308 with 32 x 4).
 #define RAW_F 32
 #define RAW_S 4
 #define RAW_CLASSES 7  // fixed point beyond 20 by entry (a, b), other fixed point, series, diagonal
@@ -223,40 +227,41 @@ __device__ __forceinline__ void load_raw_slot(const DevGeom& g, const int64_t* i
   s.d.fy = (float)s.d.y;
 }
 
-__global__ void __launch_bounds__(RAW_F* RAW_S)
+template <int TR, int TC>
+__global__ void __launch_bounds__(TR* TC)
     k_entries_raw(DevGeom g, const __grid_constant__ Phys ph, const int64_t* __restrict__ rows, int64_t nr,
                   const int64_t* __restrict__ cols, int64_t nc, double2* __restrict__ out) {
   __shared__ HkTables T;
-  __shared__ RawSlot sr[2][RAW_F], sc[2][RAW_S];  // [half of the list][slot]
-  __shared__ int s_cnt[RAW_F * RAW_S / 32][RAW_CLASSES];
-  __shared__ int16_t s_list[RAW_F * RAW_S];
+  __shared__ RawSlot sr[2][TR], sc[2][TC];  // [half of the list][slot]
+  __shared__ int s_cnt[TR * TC / 32][RAW_CLASSES];
+  __shared__ int16_t s_list[TR * TC];
   hk_stage_tables(&T);
-  const int tid = threadIdx.x, tx = tid & (RAW_F - 1), ty = tid / RAW_F, lane = tid & 31, warp = tid >> 5;
+  const int tid = threadIdx.x, tx = tid & (TR - 1), ty = tid / TR, lane = tid & 31, warp = tid >> 5;
   const int64_t hr = (nr + 1) / 2, hc = (nc + 1) / 2;
-  const int64_t ntr = (hr + RAW_F - 1) / RAW_F, ntiles = ntr * ((hc + RAW_S - 1) / RAW_S);
+  const int64_t ntr = (hr + TR - 1) / TR, ntiles = ntr * ((hc + TC - 1) / TC);
   for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
-    const int64_t r0 = (tile % ntr) * RAW_F, c0 = (tile / ntr) * RAW_S;
+    const int64_t r0 = (tile % ntr) * TR, c0 = (tile / ntr) * TC;
     __syncthreads();
-    if (tid < 2 * RAW_F) {
-      const int h = tid / RAW_F, t = tid % RAW_F;
+    if (tid < 2 * TR) {
+      const int h = tid / TR, t = tid % TR;
       sr[h][t].comp = -1;
       if (r0 + t < hr) load_raw_slot(g, rows, r0 + t + h * hr, nr, sr[h][t]);
-    } else if (tid < 2 * RAW_F + 2 * RAW_S) {
-      const int h = (tid - 2 * RAW_F) / RAW_S, t = (tid - 2 * RAW_F) % RAW_S;
+    } else if (tid < 2 * TR + 2 * TC) {
+      const int h = (tid - 2 * TR) / TC, t = (tid - 2 * TR) % TC;
       sc[h][t].comp = -1;
       if (c0 + t < hc) load_raw_slot(g, cols, c0 + t + h * hc, nc, sc[h][t]);
     }
     __syncthreads();
     // both unknowns of one node in every slot of the tile (empty slots aside)?
     bool whole = true;
-    if (tid < RAW_F)
+    if (tid < TR)
       whole = sr[0][tid].comp < 0 ||
               (sr[0][tid].comp == 0 && sr[1][tid].comp == 1 && sr[0][tid].d.node == sr[1][tid].d.node);
-    else if (tid < RAW_F + RAW_S)
-      whole = sc[0][tid - RAW_F].comp < 0 || (sc[0][tid - RAW_F].comp == 0 && sc[1][tid - RAW_F].comp == 1 &&
-                                              sc[0][tid - RAW_F].d.node == sc[1][tid - RAW_F].d.node);
+    else if (tid < TR + TC)
+      whole = sc[0][tid - TR].comp < 0 || (sc[0][tid - TR].comp == 0 && sc[1][tid - TR].comp == 1 &&
+                                              sc[0][tid - TR].d.node == sc[1][tid - TR].d.node);
     whole = __syncthreads_and(whole);
-    for (int quad = 0; quad < (whole ? 1 : 4); ++quad) {
+    for (int quad = blockIdx.y; quad < (whole ? 1 : 4); quad += gridDim.y) {
       const int qr = quad & 1, qc = quad >> 1;
       // group the pairs by evaluation path, so that a warp mixes paths only at a group boundary
       // (the grouping only orders work: FP32 coordinates are enough)
@@ -284,7 +289,7 @@ __global__ void __launch_bounds__(RAW_F* RAW_S)
       for (int c = 0; c < RAW_CLASSES; ++c) {
         int before = 0, total = 0;
 #pragma unroll
-        for (int w = 0; w < RAW_F * RAW_S / 32; ++w) {
+        for (int w = 0; w < TR * TC / 32; ++w) {
           total += s_cnt[w][c];
           if (w < warp) before += s_cnt[w][c];
         }
@@ -293,7 +298,7 @@ __global__ void __launch_bounds__(RAW_F* RAW_S)
       }
       __syncthreads();
       if (tid < base) {
-        const int me = s_list[tid], mx = me & (RAW_F - 1), my = me / RAW_F;
+        const int me = s_list[tid], mx = me & (TR - 1), my = me / TR;
         const SlotData &R = sr[qr][mx].d, &C = sc[qc][my].d;
         const int a = sr[qr][mx].comp, b = sc[qc][my].comp;
         double2* o = out + (r0 + mx + qr * hr) + (c0 + my + qc * hc) * nr;
@@ -336,10 +341,16 @@ __global__ void __launch_bounds__(RAW_F* RAW_S)
 int wsbm_launch_entries_raw(const DevGeom& g, const Phys& ph, const int64_t* rows, int64_t nr, const int64_t* cols,
                             int64_t nc, double2* out, cudaStream_t st) {
   const int64_t hr = (nr + 1) / 2, hc = (nc + 1) / 2;
-  const int64_t ntiles = (hr + RAW_F - 1) / RAW_F * ((hc + RAW_S - 1) / RAW_S);
+  const bool wide = hr < RAW_F && hc > hr;
+  const int64_t tr = wide ? RAW_S : RAW_F, tc = wide ? RAW_F : RAW_S;
+  const int64_t ntiles = ((hr + tr - 1) / tr) * ((hc + tc - 1) / tc);
   if (ntiles <= 0) return WSBM_OK;
   const int64_t cap = (int64_t)wsbm_sm_count() * WSBM_ENTRY_CTAS;
-  k_entries_raw<<<(int)(ntiles < cap ? ntiles : cap), RAW_F * RAW_S, 0, st>>>(g, ph, rows, nr, cols, nc, out);
+  const dim3 grid((unsigned)std::min(ntiles, cap), 4 * ntiles <= cap ? 4 : 1);
+  if (wide)
+    k_entries_raw<RAW_S, RAW_F><<<grid, RAW_F * RAW_S, 0, st>>>(g, ph, rows, nr, cols, nc, out);
+  else
+    k_entries_raw<RAW_F, RAW_S><<<grid, RAW_F * RAW_S, 0, st>>>(g, ph, rows, nr, cols, nc, out);
   wsbm_count_launch();
   return cudaGetLastError() == cudaSuccess ? WSBM_OK : WSBM_ERR_CUDA;
 }
