@@ -135,7 +135,7 @@ extern "C" int wsbm_autotune(int32_t n_box, int32_t nbox, int32_t nrhs_box, int3
       cudaEventElapsedTime(&v, tm.a, tm.b);
       best = v < best ? v : best;
     }
-    if (wsbm_lu_big_status(st) != 0) return WSBM_ERR_TIMEOUT;
+    if (wsbm_lu_big_status(st, n_root) != 0) return WSBM_ERR_TIMEOUT;
     *out_ms = best;
     return WSBM_OK;
   };

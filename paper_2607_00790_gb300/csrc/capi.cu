@@ -349,7 +349,8 @@ extern "C" int wsbm_zgemm(int32_t m, int32_t n, int32_t k, const double* alpha, 
   void* ws = nullptr;
   // the work space of one piece, else (a limited allocator) the least that the product runs with
   const size_t least = wsbm_zgemm_tc_ws_bytes(m, n, k);
-  size_t bytes = wsbm_zgemm_crt_fits(m, n, k) ? std::max(least, wsbm_zgemm_crt_ws_bytes(m, n, k)) : least;
+  const bool residues = wsbm_zgemm_crt_fits(m, n, k);
+  size_t bytes = residues ? std::max(least, wsbm_zgemm_crt_ws_bytes(m, n, k)) : least;
   int rc = scr.get(bytes, &ws);
   if (rc == WSBM_ERR_OOM && bytes > least) rc = scr.get(bytes = least, &ws);
   if (rc) return rc;
@@ -357,7 +358,7 @@ extern "C" int wsbm_zgemm(int32_t m, int32_t n, int32_t k, const double* alpha, 
                      make_double2(beta[0], beta[1]), (double2*)C, ldc, ws, bytes, st);
   if (rc == -1) return WSBM_ERR_INVALID_ARG;
   if (rc) return WSBM_ERR_CUDA;
-  rc = wsbm_zgemm_tc_status(st);
+  rc = wsbm_zgemm_tc_status(st, residues);
   return rc == 0 ? WSBM_OK : (rc == -5 ? WSBM_ERR_TIMEOUT : WSBM_ERR_CUDA);
 }
 
@@ -372,7 +373,7 @@ extern "C" int wsbm_lu_dense(void* A, int64_t lda, int32_t n, int32_t* piv, void
   rc = wsbm_lu_big((double2*)A, lda, n, piv, nullptr, ws, st);
   if (rc == -1) return WSBM_ERR_INVALID_ARG;
   if (rc) return WSBM_ERR_CUDA;
-  rc = wsbm_lu_big_status(st);
+  rc = wsbm_lu_big_status(st, n);
   return rc == 0 ? WSBM_OK : (rc == -5 ? WSBM_ERR_TIMEOUT : WSBM_ERR_CUDA);
 }
 

@@ -88,8 +88,8 @@ int wsbm_zgemm_tc_run(const TcPlan& pl, const void* dtab, double2 alpha, double2
 size_t wsbm_sketch_tc_ws_bytes(const TcProduct* p, int nitems);
 int wsbm_sketch_tc(const TcProduct* p, int nitems, uint32_t seed, void* ws, cudaStream_t st);
 // Synchronizes the stream and returns -5 (and clears the flag) if a bounded wait of the GEMM
-// kernel ran out since the last call, else 0 (-3 on a CUDA error).
-int wsbm_zgemm_tc_status(cudaStream_t st);
+// kernel ran out since the last call, else 0 (-3 on a CUDA error).  residues: of products from residues, too.
+int wsbm_zgemm_tc_status(cudaStream_t st, bool residues = false);
 
 // C = alpha * op(A) * B + beta * C  (column-major, op(A) m x k, B k x n, C m x n);
 // op(A) = A (ta = 0, A stored m x k) or A^T (ta = 1, A stored k x m).
@@ -200,8 +200,9 @@ int wsbm_lu_big(double2* A, int64_t lda, int n, int* piv, int* d_info, void* ws,
 int wsbm_lu_big_nb(double2* A, int64_t lda, int n, int* piv, int* d_info, void* ws, cudaStream_t st, int nb);
 int wsbm_lu_big_large_n();  // n from which the root LU takes the large-class panel width
 size_t wsbm_lu_big_ws_bytes(int n);
-// wsbm_zgemm_tc_status for a large LU: the waits of its panels and of its products.
-int wsbm_lu_big_status(cudaStream_t st);
+// wsbm_zgemm_tc_status for a large LU of n unknowns (the largest, if several): the waits of its panels and
+// of its products.
+int wsbm_lu_big_status(cudaStream_t st, int n);
 int wsbm_trsm_batched(const TrsmDesc* d_desc, int nbatch, int max_n, int max_nrhs, int lower,
                       cudaStream_t st);
 int wsbm_lu_solve_batched(const TrsmDesc* d_desc_lower, const TrsmDesc* d_desc_upper, int nbatch,

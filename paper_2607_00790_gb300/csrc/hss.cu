@@ -1736,7 +1736,7 @@ static int factor_roots(const std::vector<wsbm_hss*>& hs, double ms_out[2]) {
       HK(upload(h0, small, &ds, tmp));
       HK(wsbm_lu_batched(ds, (int)small.size(), maxs, nullptr, st));
     }
-    if (wsbm_lu_big_status(st) != 0) return WSBM_ERR_TIMEOUT;  // of the box factors' products, too
+    if (wsbm_lu_big_status(st, maxn) != 0) return WSBM_ERR_TIMEOUT;  // of the box factors' products, too
   }
   HC(cudaEventRecord(h0->ev[2], st));
   HC(cudaStreamSynchronize(st));

@@ -431,8 +431,8 @@ int wsbm_lu_big_nb(double2* A, int64_t lda, int n, int* piv, int* d_info, void* 
 
 // Error flags of the bounded waits of the panel and of its products: reads and clears both
 // (synchronizes the stream).
-int wsbm_lu_big_status(cudaStream_t st) {
-  const int rc = wsbm_zgemm_tc_status(st);
+int wsbm_lu_big_status(cudaStream_t st, int n) {
+  const int rc = wsbm_zgemm_tc_status(st, n > 512);  // smaller results never come from residues
   if (rc == -3) return rc;
   int v = 0;
   if (cudaMemcpyFromSymbol(&v, g_lub_error, sizeof(int)) != cudaSuccess) return -3;

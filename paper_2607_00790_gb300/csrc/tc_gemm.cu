@@ -788,18 +788,19 @@ int wsbm_zgemm_tc(int m, int n, int k, double2 alpha, const double2* A, int64_t 
   return wsbm_zgemm_tc_batched_g(&p, 1, alpha, beta, ws, st, group);
 }
 
-// Error flag of the bounded waits: returns it and clears it (synchronizes the stream).
-int wsbm_zgemm_tc_status(cudaStream_t st) {
+// Error flag of the bounded waits: returns it and clears it (synchronizes the stream).  residues: of
+// products from residues, too; a read takes 10 us, so only where there can have been one.
+int wsbm_zgemm_tc_status(cudaStream_t st, bool residues) {
   if (cudaStreamSynchronize(st) != cudaSuccess) return -3;
   int v = 0;
   if (cudaMemcpyFromSymbol(&v, g_tc_error, sizeof(int)) != cudaSuccess) return -3;
   if (v) {
     const int zero = 0;
     cudaMemcpyToSymbol(g_tc_error, &zero, sizeof(int));
-    wsbm_zgemm_crt_status();
+    if (residues) wsbm_zgemm_crt_status();
     return -5;
   }
-  return wsbm_zgemm_crt_status();
+  return residues ? wsbm_zgemm_crt_status() : 0;
 }
 
 // A wait on a barrier at which nothing arrives: it gives up after TC_WAIT_NS and leaves the error flag
