@@ -870,8 +870,8 @@ __global__ void __launch_bounds__(LUS_T) k_lu_solve_fused(const LuSolveDesc* __r
 // TPC (thread per column): each thread updates whole trailing columns against the reflector
 // staged in shared memory (no warp reductions; the strided column loads stay in L1, and on
 // GB300 a warp-wide DFMA takes 16 clocks, which hides them).  For matrices of up to CPQR_TPC_MAXM
-// rows, the sketches: 4096 of 128 x 256 take 108 ms, 195 with a warp per column; from 250 rows on
-// the two are within 3 to 12 % in large batches and the warps win in small ones.
+// rows, the sketches: 4096 of 128 x 256 take 88 ms; from there on the two are within 4 % in large
+// batches and the warps win in small ones.
 #ifndef CPQR_TPC_MAXM
 #define CPQR_TPC_MAXM 192
 #endif
@@ -1146,8 +1146,8 @@ __device__ __forceinline__ long long cpqr_norm_key(double v) {
   return (b & 0x7fffffffffffffffll) > 0x7ff0000000000000ll ? -1 : b;
 }
 
-template <int CB>
-__global__ void __launch_bounds__(256, CB == 2 ? 3 : 2) k_cpqr_cluster(const QrDesc* __restrict__ d, int mode) {
+template <int CB, int MINB>
+__global__ void __launch_bounds__(256, MINB) k_cpqr_cluster(const QrDesc* __restrict__ d, int mode) {
   constexpr int SH = CB == 1 ? 4 : CB == 2 ? 3 : CB == 4 ? 2 : 1;  // 5 - log2(2 * CB)
   extern __shared__ double2 su[];  // the reflector u = (column p)[j : m]
   uint32_t rank, csize;
@@ -1513,10 +1513,10 @@ int wsbm_lu_solve_fused_batched(const LuSolveDesc* d_desc, int nbatch, int max_n
 
 int wsbm_cpqr_tpc_rows() { return CPQR_TPC_MAXM; }
 
-template <int CB>
+template <int CB, int MINB>
 static int launch_cpqr_cluster(const QrDesc* d_desc, int nbatch, int mode, int cl, int max_m, cudaStream_t st) {
   const size_t sm = (size_t)std::min(max_m, CPQR_CLUSTER_MAXM) * sizeof(double2);
-  if (wsbm_smem_optin((const void*)k_cpqr_cluster<CB>, sm) != cudaSuccess) return -3;
+  if (wsbm_smem_optin((const void*)k_cpqr_cluster<CB, MINB>, sm) != cudaSuccess) return -3;
   cudaLaunchConfig_t cfg = {};
   cudaLaunchAttribute at[1];
   at[0].id = cudaLaunchAttributeClusterDimension;
@@ -1529,7 +1529,7 @@ static int launch_cpqr_cluster(const QrDesc* d_desc, int nbatch, int mode, int c
   cfg.attrs = at;
   cfg.numAttrs = 1;
   wsbm_count_launch();
-  return cudaLaunchKernelEx(&cfg, k_cpqr_cluster<CB>, d_desc, mode) == cudaSuccess ? 0 : -3;
+  return cudaLaunchKernelEx(&cfg, k_cpqr_cluster<CB, MINB>, d_desc, mode) == cudaSuccess ? 0 : -3;
 }
 
 // The kernel is chosen per matrix, by its rows, so that its factor does not depend on the others of
@@ -1547,10 +1547,14 @@ int wsbm_cpqr_batched(const QrDesc* d_desc, int nbatch, int nsmall, int mode, in
     // 2, 4 or 8 CTAs per matrix while the GPU holds them all at once (three per SM)
     int cl = 1;
     while (cl < 8 && (int64_t)nbig * cl * 2 <= (int64_t)wsbm_sm_count() * 3) cl *= 2;
+    // columns a warp takes at a time (its sums are the same): 4 share the reductions of short columns, 2 give
+    // a matrix alone more warps (4096 of 256 x 256: 204 ms with 4, 231 with 2, 196 in the thread-per-column
+    // kernel; 1200 of 400 x 300: 136, 144, 137; one of 500 x 400: 8.2, 5.8, 49)
     const int cb = max_m <= 2048 ? 2 : tu.cpqr_cb;
-    if (int rc = cb == 2   ? launch_cpqr_cluster<2>(d_desc, nbatch, mode, cl, max_m, st)
-                 : cb == 8 ? launch_cpqr_cluster<8>(d_desc, nbatch, mode, cl, max_m, st)
-                           : launch_cpqr_cluster<4>(d_desc, nbatch, mode, cl, max_m, st))
+    if (int rc = cl == 1 && max_m <= 800 ? launch_cpqr_cluster<4, 3>(d_desc, nbatch, mode, cl, max_m, st)
+                 : cb == 2               ? launch_cpqr_cluster<2, 3>(d_desc, nbatch, mode, cl, max_m, st)
+                 : cb == 8               ? launch_cpqr_cluster<8, 2>(d_desc, nbatch, mode, cl, max_m, st)
+                                         : launch_cpqr_cluster<4, 2>(d_desc, nbatch, mode, cl, max_m, st))
       return rc;
   }
   if (max_m > CPQR_CLUSTER_MAXM) {

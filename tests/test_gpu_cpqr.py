@@ -73,3 +73,13 @@ def test_factor_does_not_depend_on_its_batch(m, other):
     alone, beside = cpqr([A], 6)[0], cpqr([A, B], 6)[0]
     for x, y in zip(alone, beside):
         assert np.array_equal(x, y)
+
+
+@pytest.mark.parametrize("m", [193, 500, 800, 801])
+def test_factor_in_a_large_batch(m):
+    """Alone it has a cluster and narrow passes, among 300 a CTA and wide ones."""
+    A = graded(m, 41)
+    alone, many = cpqr([A], 17)[0], cpqr([A] * 300, 17)
+    for got in (many[0], many[299]):
+        for x, y in zip(alone, got):
+            assert np.array_equal(x, y)
