@@ -70,7 +70,9 @@ __device__ __forceinline__ bool pair_is_fixed(const Phys& ph, double r2) {
   return h > ph.fix_lo && h < ph.fix_hi;
 }
 
-// 1/sqrt(x) to about an ulp for normal x: hardware seed (23 bits) and one third-order step.
+// 1/sqrt(x) to an ulp for normal x: the hardware's seed y (rsqrt.approx.ftz.f64, about 22 bits) and one
+// step of third order.  With e = 1 - x y^2, 1/sqrt(x) = y (1 - e)^(-1/2) = y (1 + e/2 + 3 e^2/8 + O(e^3)),
+// the binomial series; the next term, 5 e^3/16, is below 2^-60.
 __device__ __forceinline__ double rsqrt3(double x) {
   double y;
   asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
@@ -84,7 +86,8 @@ __device__ __forceinline__ double rsqrt3_any(double x) {
   return h >= 0x00100000 && h < 0x7FF00000 ? rsqrt3(x) : rsqrt(x);
 }
 
-// sqrt(x), correctly rounded, from y = 1/sqrt(x): x y plus half its residual times y.
+// sqrt(x) from y = 1/sqrt(x) by one Newton step: r = x y, then r + (x - r^2) y / 2, the residual from a
+// fused multiply-add.  Correctly rounded wherever compared with sqrt().
 __device__ __forceinline__ double sqrt_from(double x, double y) {
   const double r = x * y;
   return fma(fma(-r, r, x), __hiloint2double(__double2hiint(y) - 0x100000, __double2loint(y)), r);

@@ -49,7 +49,6 @@ struct HkF {
 // (divergent interval indices within a warp would serialise constant-bank reads).
 struct HkTables {
   HxNear near_;
-  double asy[4][HK_DEG_T + 1];
   double ser[4][HK_NSER];
   double sn[HK_DEG_SC + 1];
   double cs[HK_DEG_SC + 1];
@@ -68,7 +67,6 @@ __device__ __forceinline__ void hk_stage_tables(HkTables* t) {
   hk_copy(&t->near_.c[0][0][0], &hx_near_c[0][0][0], HX_NIV * 4 * (HX_DEG_N + 1));
   hk_copy(t->near_.lo, hx_near_lo, HX_NIV);
   hk_copy(t->near_.sh, hx_near_sh, HX_NIV);
-  hk_copy(&t->asy[0][0], &hk_asy[0][0], 4 * (HK_DEG_T + 1));
   hk_copy(&t->ser[0][0], &hk_ser[0][0], 4 * HK_NSER);
   hk_copy(t->sn, hk_sin, HK_DEG_SC + 1);
   hk_copy(t->cs, hk_cos, HK_DEG_SC + 1);
@@ -150,7 +148,6 @@ __device__ __forceinline__ int hk_interval_hi(int hi) {
   for (int k = 0; k < HK_NIV - 1; ++k) iv += (hi >= lim[k]) ? 1 : 0;
   return iv;
 }
-__device__ __forceinline__ int hk_interval(double z) { return hk_interval_hi(__double2hiint(z)); }
 
 // e^{i(z - pi/4)} = E + iF.  z - pi/4 = w + k pi/2 with |w| <= pi/4: k = rint(2z/pi - 1/2),
 // w = z - (k + 1/2) pi/2 by two fused multiply-adds with a two-part pi/2, then

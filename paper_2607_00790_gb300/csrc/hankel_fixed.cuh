@@ -6,7 +6,7 @@
 // formed as 64-bit fractions and only the four results become doubles, by integer operations as
 // well.  Each result is within about 2^-58 of the modulus before that rounding, where the FP64
 // evaluation loses a few 2^-53.  The matrix-free product of 16384 nodes took 103.8 ms with the FP64
-// evaluator (185 FP64 operations a pair, the pipe 90 % busy) and takes 47.8 ms with this one (71 and
+// evaluator (185 FP64 operations a pair, the pipe 90 % busy) and takes 45.5 ms with this one (71 and
 // 16 for the product).
 //
 //   phase   z = m 2^e (53-bit m): m times the 96-bit 2/pi, shifted, gives 2 z / pi modulo 4 to

@@ -250,8 +250,8 @@ __global__ void __launch_bounds__(256) k_lub_rowswap(double2* __restrict__ A, in
 
 // X = L^-1 B for the unit lower triangle L of A[r0 : r0 + nb, r0 : r0 + nb] (nb <= 32 NS), one warp
 // per column (tri.cuh), `cols` columns a CTA (the other warps help to stage L: the solves are bound
-// by FP64, so one column per SM until there are more columns than SMs).  B: the ncols columns at B (leading dimension ldb), in place; B = NULL: the
-// inverse itself, into `out` (leading dimension nb).
+// by FP64, so one column per SM until there are more columns than SMs).  B: the ncols columns at B (leading
+// dimension ldb), in place; B = NULL: the inverse itself, into `out` (leading dimension nb).
 template <int NS>
 __global__ void __launch_bounds__(128) k_lub_trsm(const double2* __restrict__ A, int64_t lda, int r0, int nb,
                                                   double2* B, int64_t ldb, int ncols, int cols, double2* __restrict__ out) {
