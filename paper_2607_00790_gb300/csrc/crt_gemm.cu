@@ -56,6 +56,10 @@
 #define CR_SMEM (CR_STAGES * CR_STAGE + 256 + 1024)
 #define CR_THREADS 384
 #define CR_EPI 256
+// registers a thread of the four warps that issue and of the epilogue, out of those of the launch (168 each):
+// an increase beyond the launch's total would wait for ever, so crt_registers() checks it
+#define CR_REGS_ISSUE 40
+#define CR_REGS_EPI 232
 #define CR_NBUF 2            // TMEM buffers of CR_G x 64 columns (the accumulators use CR_BN of each 64)
 #define CR_FEWBITS 40        // a row or column of values of at most so many significant bits
 #define CR_LOW_NONE 1000000  // lowest set bit of an all-zero row or column
@@ -418,7 +422,7 @@ __global__ void __launch_bounds__(CR_THREADS, 1)
   };
 
   if (warp < 4) {
-    asm volatile("setmaxnreg.dec.sync.aligned.u32 40;");
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(CR_REGS_ISSUE));
     if (warp == 0 && lane == 0) {
       // -------------------------------------------------------------- TMA producer
       uint32_t it = 0;
@@ -479,7 +483,7 @@ __global__ void __launch_bounds__(CR_THREADS, 1)
     }
   } else {
     // ---------------------------------------------------------------- epilogue (warps 4-11)
-    asm volatile("setmaxnreg.inc.sync.aligned.u32 232;");
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(CR_REGS_EPI));
     const int quad = warp & 3, half = (warp - 4) >> 2;  // TMEM lanes, and which half of the columns
     const uint32_t tq = tmem + ((uint32_t)(quad * 32) << 16) + half * CR_TC;
     uint32_t u = 0;
@@ -612,6 +616,19 @@ static int crt_map(CUtensorMap* map, void* planes, int64_t rows, int64_t Kp, int
              : -3;
 }
 
+// The kernel was compiled with the registers that its warps share out.
+static bool crt_registers() {
+  static const bool ok = [] {
+    cudaFuncAttributes a;
+    if (cudaFuncGetAttributes(&a, k_zgemm_crt) != cudaSuccess) {
+      cudaGetLastError();
+      return false;
+    }
+    return a.numRegs * CR_THREADS >= (CR_THREADS - CR_EPI) * CR_REGS_ISSUE + CR_EPI * CR_REGS_EPI;
+  }();
+  return ok;
+}
+
 static int64_t crt_kp(int k) { return ((int64_t)std::min(k, CR_KMAX) + CR_BK - 1) / CR_BK * CR_BK; }
 static size_t crt_up(size_t b) { return (b + 255) & ~(size_t)255; }
 static size_t crt_bytes(int64_t m, int64_t n, int64_t Kp) {
@@ -648,10 +665,11 @@ static bool blocks_meet(const double2* X, int64_t ldx, int64_t xr, int64_t xc, c
 }
 
 // ws_bytes may be less than wsbm_zgemm_crt_ws_bytes: the longer side then goes through in strips
-// (-2 if not even a strip of 512 fits, or if C is written piece by piece while A or B, which it overlaps,
+// (-2 if not even a strip of 512 fits, if the registers do not suffice, or if C is written piece by piece while A or B, which it overlaps,
 // is still to be read: nothing was launched).
 int wsbm_zgemm_crt(int m, int n, int k, double2 alpha, const double2* A, int64_t lda, const double2* B, int64_t ldb,
                    double2 beta, double2* C, int64_t ldc, void* ws, size_t ws_bytes, cudaStream_t st, int group) {
+  if (!crt_registers()) return -2;
   const int64_t Kp = crt_kp(k);
   int ms = m, ns = n;
   while (crt_bytes(ms, ns, Kp) > ws_bytes) {
