@@ -200,6 +200,11 @@ int wsbm_lu_big(double2* A, int64_t lda, int n, int* piv, int* d_info, void* ws,
 int wsbm_lu_big_nb(double2* A, int64_t lda, int n, int* piv, int* d_info, void* ws, cudaStream_t st, int nb);
 int wsbm_lu_big_large_n();  // n from which the root LU takes the large-class panel width
 size_t wsbm_lu_big_ws_bytes(int n);
+// The same for several matrices in step (host descriptors by falling n, at most wsbm_lu_big_multi_max(h,
+// count) of them): the factors that each has alone.
+int wsbm_lu_big_multi(const LuDesc* h, int count, void* ws, cudaStream_t st);
+int wsbm_lu_big_multi_max(const LuDesc* h, int count);  // how many of them, from the first, can go together
+size_t wsbm_lu_big_multi_ws_bytes(const LuDesc* h, int count);
 // wsbm_zgemm_tc_status for a large LU of n unknowns (the largest, if several): the waits of its panels and
 // of its products.
 int wsbm_lu_big_status(cudaStream_t st, int n);

@@ -45,8 +45,6 @@
 #ifndef WSBM_LU_TC_MIN
 #define WSBM_LU_TC_MIN 128
 #endif
-// Dense roots of at least this order are factored by the LU whose trailing updates run on
-// the tensor cores (wsbm_lu_big); smaller ones by the batched FP64 blocked LU.
 // Solves with at least WSBM_TCSOLVE_RHS right-hand sides run their products on the tensor
 // cores, and their LU solves of box factors of at least WSBM_LU_TC_MIN unknowns as block solves
 // there (WSBM_TCSOLVE_NB rows per block); the LU solves of dense roots of at least
@@ -66,14 +64,12 @@
 #ifndef WSBM_TCSOLVE_WS
 #define WSBM_TCSOLVE_WS ((size_t)4 << 30)  // digit-plane work space of one solve product launch
 #endif
-// Roots from here on take the LU whose updates run on the tensor cores, one after another; smaller ones
-// share the launches of the batched FP64 LU, so that many small curves cost little more than one (a rule on
-// the count would make a curve's factors depend on its batch).  Batched / one after another, ms: n = 700
-// 10.1 / 4.4 for one root, 58 / 284 for 64; n = 1400 34.9 / 9.4 and 428 / 600; n = 2000 71 / 14 and 1230 /
-// 915.  The FP64 LU is a little more accurate too (n = 640: |PA - LU| 5.6e-15 |A| against 6.2e-15, largest
-// entry 4.4e-14 against 1.0e-13).
+// Roots from here on take the LU whose updates run on the tensor cores, those of a batch in step (root_lu.cu);
+// smaller ones the batched FP64 LU.  FP64 / in step, ms: n = 512 6.1 / 3.1 for one root, 24 / 15 for 64; n = 700
+// 10 / 4.4 and 58 / 23; n = 1400 35 / 9.1 and 428 / 66 (591 one after another); n = 3000 169 / 22 and 4018 / 311.
+// The pivots are the largest to within 2^-20; |PA - LU| of a random matrix of 640 is 5.3e-15 |A| against 5.6e-15.
 #ifndef WSBM_BIGLU_MIN
-#define WSBM_BIGLU_MIN 2048
+#define WSBM_BIGLU_MIN 512
 #endif
 #ifndef WSBM_SKETCH_CUT
 #define WSBM_SKETCH_CUT 0.25  // measured: far-field error 3.6-5.8x tol, as with the full QR
@@ -1713,24 +1709,34 @@ static int factor_roots(const std::vector<wsbm_hss*>& hs, double ms_out[2]) {
     h0->stats.pairs_evaluated += pb.pairs;
     h0->stats.pairs_pairs += pb.pairs;
   }
-  // large roots: one at a time through the LU whose trailing updates run on the tensor cores;
+  // large roots: in step through the LU whose trailing updates run on the tensor cores;
   // the others in one batched blocked LU
   {
-    std::vector<LuDesc> small;
+    std::vector<LuDesc> small, big;
     int maxs = 0;
-    size_t wsb = 0;
-    for (auto& l : lus)
-      if (l.n >= WSBM_BIGLU_MIN) wsb = std::max(wsb, wsbm_lu_big_ws_bytes(l.n));
-    void* ws = nullptr;
-    if (wsb) HK(dalloc(h0, wsb, &ws, tmp));
     for (auto& l : lus) {
       if (l.n >= WSBM_BIGLU_MIN) {
-        if (wsbm_lu_big(l.A, l.lda, l.n, l.piv, nullptr, ws, st)) return WSBM_ERR_CUDA;
+        big.push_back(l);
       } else {
         small.push_back(l);
         maxs = std::max(maxs, l.n);
       }
     }
+    std::stable_sort(big.begin(), big.end(), [](const LuDesc& a, const LuDesc& b) { return a.n > b.n; });
+    const int nbig = (int)big.size();
+    int cap = nbig;  // fewer in step where the allocator has no more work space
+    auto group = [&](int i) { return std::min(cap, wsbm_lu_big_multi_max(&big[i], nbig - i)); };
+    void* ws = nullptr;
+    while (nbig > 0) {
+      size_t need = 0;
+      for (int i = 0; i < nbig; i += group(i)) need = std::max(need, wsbm_lu_big_multi_ws_bytes(&big[i], group(i)));
+      const int rc = dalloc(h0, need, &ws, tmp);
+      if (rc == WSBM_OK) break;
+      if (rc != WSBM_ERR_OOM || cap == 1) return rc;
+      cap = (cap + 1) / 2;
+    }
+    for (int i = 0; i < nbig; i += group(i))
+      if (wsbm_lu_big_multi(&big[i], group(i), ws, st)) return WSBM_ERR_CUDA;
     if (!small.empty()) {
       LuDesc* ds = nullptr;
       HK(upload(h0, small, &ds, tmp));

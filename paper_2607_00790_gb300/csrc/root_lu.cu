@@ -1,4 +1,6 @@
-// LU with partial pivoting of one large complex matrix (the dense root of a build).
+// LU with partial pivoting of large complex matrices (the dense roots of a build): one, or the roots of
+// several curves in step, panel by panel in the same launches.  Every kernel works on a matrix without regard
+// to the others, so the factors of a root do not depend on its company.
 //
 // Right-looking, outer panels of LUB_NB columns (LUB_NB_BIG for large n, where the deeper
 // tensor-core products pay for the longer panels).  An outer panel is factored recursively by
@@ -8,6 +10,8 @@
 // for wsbm_lu_batched.  Pivot: the row of largest max(|re|, |im|) compared on the upper 32 bits
 // of its bit pattern (within 2^-20 of the largest), first row on ties.
 #include <algorithm>
+#include <climits>
+#include <vector>
 
 #include "cplx.cuh"
 #include "dense.h"
@@ -30,10 +34,25 @@
 #define LUB_T 256           // threads of a base-panel CTA
 #define LUB_MINROWS 32      // fewest rows per CTA (the base panel's pivot rows all start in CTA 0)
 #define LUB_MAXCTA 256      // CTAs a base panel can use (key slots per column)
+#define LUB_MAXB 16         // matrices in step (their descriptors are kernel arguments)
 #define LUB_SMEM (200 * 1024)
 #define LUB_WAIT_NS 2000000000ull  // bound of every wait (2 s)
 
 static __device__ int g_lub_error;  // set when a bounded wait ran out
+
+struct LubItem {
+  double2* A;
+  int64_t lda;
+  int n;
+  int *piv, *info;
+  unsigned long long* slots;  // [outer panel's columns][LUB_MAXCTA]
+  double2 *cand, *diag, *inv;
+};
+struct LubBatch {
+  LubItem it[LUB_MAXB];     // by falling n
+  int first[LUB_MAXB + 1];  // base panel: first CTA of each
+  int R;                    // base panel: rows per CTA
+};
 
 __device__ __forceinline__ unsigned long long lub_key(double2 v, int row) {
   const unsigned long long m = 0x7fffffffffffffffull;
@@ -64,9 +83,9 @@ __device__ __forceinline__ unsigned long long lub_time() {
   return t;
 }
 
-// Base panel: columns [c0, c0 + w) (w <= 32) of rows [c0, n), rows spread over the CTAs of one
+// Base panel: columns [c0, min(c1, n)) (at most 32) of rows [c0, n), rows spread over the CTAs of one
 // cooperative launch, R consecutive rows each (R >= w), held in shared memory from the first to
-// the last column.  Per column every CTA publishes its best candidate (key) and that candidate's
+// the last column.  Several matrices share the launch, each with CTAs of its own that wait for one another only.  Per column every CTA publishes its best candidate (key) and that candidate's
 // panel row; every CTA then reads all the keys, takes the winner's row as the pivot row and
 // updates its own rows, so a column costs one exchange through L2 instead of two launches.  Bound by
 // that exchange (release, 152 polled keys, one row read): 3.8 us a column at n = 8200, 31 ms in all.
@@ -81,16 +100,23 @@ __device__ __forceinline__ unsigned long long lub_time() {
 //          later, after every CTA has published the column between (and so has read it)
 //   diag   row c as its owner holds it before the swap, [2][32]
 __global__ void __launch_bounds__(LUB_T, 1)
-    k_lub_panel(double2* __restrict__ A, int64_t lda, int n, int c0, int w, int R, unsigned long long* slots,
-                double2* cand, double2* diag, int* __restrict__ piv, int* __restrict__ info) {
+    k_lub_panel(const __grid_constant__ LubBatch q, int c0, int c1, int slot0) {
   extern __shared__ double2 sm[];
+  int it = 0;
+  while ((int)blockIdx.x >= q.first[it + 1]) ++it;
+  double2* __restrict__ A = q.it[it].A;
+  const int64_t lda = q.it[it].lda;
+  const int n = q.it[it].n, w = min(c1, n) - c0, R = q.R;
+  unsigned long long* slots = q.it[it].slots + (size_t)slot0 * LUB_MAXCTA;
+  double2 *cand = q.it[it].cand, *diag = q.it[it].diag;
+  int *__restrict__ piv = q.it[it].piv, *__restrict__ info = q.it[it].info;
   const int RS = R | 1;  // odd stride: a row read across the columns meets no bank twice
   __shared__ double2 prow[4][LUB_W];  // rows of the last four pivots, by column modulo 4
   __shared__ double2 s_inv;
   __shared__ unsigned long long red[LUB_T / 32], keys[LUB_T / 32];
   __shared__ int s_err;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int b = blockIdx.x, G = gridDim.x;
+  const int b = (int)blockIdx.x - q.first[it], G = q.first[it + 1] - q.first[it];
   const int r0 = c0 + b * R, cnt = min(R, n - r0);
   for (int e = tid; e < R * w; e += LUB_T) {
     const int t = e / R, i = e - t * R;
@@ -236,57 +262,181 @@ __global__ void __launch_bounds__(LUB_T, 1)
   }
 }
 
-// Row interchanges piv[j0 .. j0 + nb) (nb <= 256) on the columns [a0, a1) and [b0, b1), as one
-// gather per column, one warp each: the top nb rows are read and written contiguously (5 us a
-// call at n = 8200).
-__global__ void __launch_bounds__(256) k_lub_rowswap(double2* __restrict__ A, int64_t lda, int n, int j0, int nb,
-                                                     const int* __restrict__ piv, int a0, int a1, int b0, int b1) {
+// Row interchanges piv[j0 .. min(j0 + nb, n)) (nb <= 256) on the columns [a0, a1) and [b0, min(b1, n)), as
+// one gather per column, one warp each: the top nb rows are read and written contiguously (5 us a
+// call at n = 8200).  Matrix blockIdx.y.
+__global__ void __launch_bounds__(256)
+    k_lub_rowswap(const __grid_constant__ LubBatch q, int j0, int nb, int a0, int a1, int b0, int b1) {
   __shared__ SwapLists S;
-  swap_lists(S, piv + j0, n, j0, nb);
-  const int na = a1 - a0, tot = na + (b1 - b0);
-  for (int q = blockIdx.x * 8 + (threadIdx.x >> 5); q < tot; q += gridDim.x * 8)
-    swap_column(S, nb, A + (int64_t)(q < na ? a0 + q : b0 + (q - na)) * lda, false);
+  const LubItem& x = q.it[blockIdx.y];
+  const int jb = min(nb, x.n - j0), na = a1 - a0, tot = na + max(0, min(b1, x.n) - b0);
+  if ((int)blockIdx.x * 8 >= tot) return;
+  swap_lists(S, x.piv + j0, x.n, j0, jb);
+  for (int c = blockIdx.x * 8 + (threadIdx.x >> 5); c < tot; c += gridDim.x * 8)
+    swap_column(S, jb, x.A + (int64_t)(c < na ? a0 + c : b0 + (c - na)) * x.lda, false);
 }
 
 // X = L^-1 B for the unit lower triangle L of A[r0 : r0 + nb, r0 : r0 + nb] (nb <= 32 NS), one warp
 // per column (tri.cuh), `cols` columns a CTA (the other warps help to stage L: the solves are bound
-// by FP64, so one column per SM until there are more columns than SMs).  B: the ncols columns at B (leading
-// dimension ldb), in place; B = NULL: the inverse itself, into `out` (leading dimension nb).
+// by FP64, so one column per SM until there are more columns than SMs).  B: the columns [b0, min(b1, n)) of A's
+// rows r0 .. r0 + nb - 1, in place; b0 < 0: the inverse itself, into `inv` (leading dimension nb).  Matrix
+// blockIdx.y.
 template <int NS>
-__global__ void __launch_bounds__(128) k_lub_trsm(const double2* __restrict__ A, int64_t lda, int r0, int nb,
-                                                  double2* B, int64_t ldb, int ncols, int cols, double2* __restrict__ out) {
+__global__ void __launch_bounds__(128)
+    k_lub_trsm(const __grid_constant__ LubBatch p, int r0, int nb, int b0, int b1, int cols) {
   extern __shared__ double2 stage[];
+  const LubItem& m = p.it[blockIdx.y];
+  const int ncols = b0 < 0 ? nb : min(b1, m.n) - b0;
+  if ((int)blockIdx.x * cols >= ncols) return;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, q = blockIdx.x * cols + warp;
   const bool on = warp < cols && q < ncols;
-  const double2* L = A + r0 + (int64_t)r0 * lda;
-  if (!B) {
-    tri_inverse_column<NS, false>(L, lda, nb, q, out + (int64_t)q * nb, stage, nullptr, on, (int)blockIdx.x * cols / 32);
+  const double2* L = m.A + r0 + (int64_t)r0 * m.lda;
+  if (b0 < 0) {
+    tri_inverse_column<NS, false>(L, m.lda, nb, q, m.inv + (int64_t)q * nb, stage, nullptr, on, (int)blockIdx.x * cols / 32);
     return;
   }
   double2 x[NS];
-  double2* col = B + (int64_t)q * ldb;
+  double2* col = m.A + r0 + (int64_t)(b0 + q) * m.lda;
 #pragma unroll
   for (int s = 0; s < NS; ++s)
     x[s] = on && s * 32 + lane < nb ? col[s * 32 + lane] : make_double2(0.0, 0.0);
-  tri_solve_warp<NS, false>(L, lda, nb, x, stage, nullptr, on);
+  tri_solve_warp<NS, false>(L, m.lda, nb, x, stage, nullptr, on);
 #pragma unroll
   for (int s = 0; s < NS; ++s)
     if (on && s * 32 + lane < nb) col[s * 32 + lane] = x[s];
 }
 
 namespace {
-struct LubCtx {
-  double2* A;
-  int64_t lda;
-  int n;
-  int* piv;
-  int* info;
-  unsigned long long* slots;  // [LUB_NB_BIG][LUB_MAXCTA], by column of the outer panel
-  double2 *cand, *diag;
+// Matrices in step.  Panels are those of the largest; a smaller one leaves with the panel that reaches its
+// last column, whose part beyond it is empty.
+struct Lub {
+  LubBatch q;
+  int count, nb, base;
   cudaStream_t st;
-  int cs, ce;  // current outer panel
-  void* tcws;  // work space of the tensor-core products
-  size_t tcb;  // and its size
+  int cs;                       // first column of the outer panel
+  void* ws;                     // work space of the tensor-core products
+  size_t wsb;                   // and its size
+  std::vector<TcProduct> prod;  // the products of one step
+
+  int n(int i) const { return q.it[i].n; }
+  int beyond(int c) const {  // matrices of more than c columns
+    int k = 0;
+    while (k < count && n(k) > c) ++k;
+    return k;
+  }
+
+  int panel(int c0, int c1) {
+    const int k = beyond(c0), nsm = std::min(wsbm_sm_count(), LUB_MAXCTA);
+    int64_t rows = 0;
+    for (int i = 0; i < k; ++i) rows += n(i) - c0;
+    int R = (int)std::max<int64_t>(LUB_MINROWS, (rows + nsm - 1) / nsm);
+    for (;; ++R) {
+      q.first[0] = 0;
+      for (int i = 0; i < k; ++i) q.first[i + 1] = q.first[i] + (n(i) - c0 + R - 1) / R;
+      if (q.first[k] <= nsm) break;
+    }
+    q.R = R;
+    const size_t smem = (size_t)(c1 - c0) * (R | 1) * sizeof(double2);
+    if (smem > LUB_SMEM || wsbm_smem_optin((const void*)k_lub_panel, LUB_SMEM) != cudaSuccess) return -3;
+    int slot0 = c0 - cs;
+    void* args[] = {&q, &c0, &c1, &slot0};
+    if (cudaLaunchCooperativeKernel((const void*)k_lub_panel, dim3(q.first[k]), dim3(LUB_T), args, smem, st) != cudaSuccess)
+      return -3;
+    wsbm_count_launch();
+    return 0;
+  }
+
+  void swap(int j0, int w, int a0, int a1, int b0, int b1) {
+    const int k = beyond(j0), tot = (a1 - a0) + std::max(0, std::min(b1, n(0)) - b0);
+    if (tot <= 0) return;
+    const int cap = std::max(1, wsbm_sm_count() * 4 / k);
+    k_lub_rowswap<<<dim3(std::min((tot + 7) / 8, cap), k), 256, 0, st>>>(q, j0, w, a0, a1, b0, b1);
+    wsbm_count_launch();
+  }
+
+  template <int NS>
+  int trsm_ns(int r0, int w, int b0, int b1, int k) {
+    const size_t sm = (size_t)32 * 32 * NS * sizeof(double2);
+    if (wsbm_smem_optin((const void*)k_lub_trsm<NS>, sm) != cudaSuccess) return -3;
+    const int ncols = b0 < 0 ? w : std::min(b1, n(0)) - b0;
+    const int cols = std::min(4, (ncols * k + wsbm_sm_count() - 1) / wsbm_sm_count());
+    k_lub_trsm<NS><<<dim3((ncols + cols - 1) / cols, k), 128, sm, st>>>(q, r0, w, b0, b1, cols);
+    wsbm_count_launch();
+    return 0;
+  }
+  int trsm(int r0, int w, int b0, int b1, int k) {  // on the first k matrices
+    if (w <= 32) return trsm_ns<1>(r0, w, b0, b1, k);
+    if (w <= 64) return trsm_ns<2>(r0, w, b0, b1, k);
+    if (w <= 128) return trsm_ns<4>(r0, w, b0, b1, k);
+    return trsm_ns<8>(r0, w, b0, b1, k);
+  }
+
+  void add(const double2* A, int64_t lda, const double2* B, int64_t ldb, double2* C, int64_t ldc, int m, int nn, int k) {
+    if (m > 0 && nn > 0) prod.push_back({A, lda, B, ldb, C, ldc, m, nn, k, 0});
+  }
+  int run(double alpha, double beta) {
+    int rc = 0;
+    const double2 a = make_double2(alpha, 0.0), b = make_double2(beta, 0.0);
+    if (prod.size() == 1) {
+      const TcProduct& t = prod[0];
+      rc = wsbm_zgemm_tc(t.m, t.n, t.k, a, t.A, t.lda, t.B, t.ldb, b, t.C, t.ldc, ws, wsb, st);
+    } else if (!prod.empty()) {
+      rc = wsbm_zgemm_tc_batched(prod.data(), (int)prod.size(), a, b, ws, st);
+    }
+    prod.clear();
+    return rc;
+  }
+
+  // factor columns [c0, c1) of rows [c0, n); row swaps across the whole outer panel
+  int rec(int c0, int c1) {
+    if (beyond(c0) == 0) return 0;
+    if (c1 - c0 <= base) {
+      if (int rc = panel(c0, c1)) return rc;
+      swap(c0, c1 - c0, cs, c0, c1, cs + nb);
+      return 0;
+    }
+    const int mid = c0 + (c1 - c0) / 2, k = beyond(mid);
+    if (int rc = rec(c0, mid)) return rc;
+    if (k == 0) return 0;
+    // A[c0:mid, mid:c1] = L11^-1 A[c0:mid, mid:c1];  A[mid:n, mid:c1] -= A[mid:n, c0:mid] A[c0:mid, mid:c1]
+    if (int rc = trsm(c0, mid - c0, mid, c1, k)) return rc;
+    for (int i = 0; i < k; ++i) {
+      const LubItem& x = q.it[i];
+      add(x.A + mid + (int64_t)c0 * x.lda, x.lda, x.A + c0 + (int64_t)mid * x.lda, x.lda,
+          x.A + mid + (int64_t)mid * x.lda, x.lda, x.n - mid, std::min(c1, x.n) - mid, mid - c0);
+    }
+    if (int rc = run(-1.0, 1.0)) return rc;
+    return rec(mid, c1);
+  }
+
+  int factor() {
+    for (int j0 = 0; j0 < n(0); j0 += nb) {
+      const int je = j0 + nb, k = beyond(je);
+      cs = j0;
+      if (cudaMemsetAsync(q.it[0].slots, 0, (size_t)beyond(j0) * nb * LUB_MAXCTA * sizeof(unsigned long long), st) !=
+          cudaSuccess)
+        return -3;
+      if (int rc = rec(j0, je)) return rc;
+      swap(j0, nb, 0, j0, je, INT_MAX);
+      if (k == 0) continue;
+      // U12 = L11^-1 A12 as a tensor-core product with the explicit inverse of the unit lower
+      // L11 (the digit planes of A12 are formed before A12 is overwritten)
+      if (int rc = trsm(j0, nb, -1, 0, k)) return rc;
+      for (int i = 0; i < k; ++i) {
+        const LubItem& x = q.it[i];
+        double2* U = x.A + j0 + (int64_t)je * x.lda;
+        add(x.inv, nb, U, x.lda, U, x.lda, nb, x.n - je, nb);
+      }
+      if (int rc = run(1.0, 0.0)) return rc;
+      for (int i = 0; i < k; ++i) {
+        const LubItem& x = q.it[i];
+        add(x.A + je + (int64_t)j0 * x.lda, x.lda, x.A + j0 + (int64_t)je * x.lda, x.lda,
+            x.A + je + (int64_t)je * x.lda, x.lda, x.n - je, x.n - je, nb);
+      }
+      if (int rc = run(-1.0, 1.0)) return rc;
+    }
+    return cudaGetLastError() == cudaSuccess ? 0 : -3;
+  }
 };
 
 // columns a base panel can take: every CTA holds its rows of them in shared memory
@@ -297,73 +447,38 @@ int lub_base_width(int n) {
   return 1;
 }
 
-int lub_swap(const LubCtx& x, int j0, int nb, int a0, int a1, int b0, int b1) {
-  const int tot = (a1 - a0) + (b1 - b0);
-  if (tot <= 0) return 0;
-  k_lub_rowswap<<<std::min((tot + 7) / 8, wsbm_sm_count() * 4), 256, 0, x.st>>>(x.A, x.lda, x.n, j0, nb, x.piv, a0,
-                                                                               a1, b0, b1);
-  wsbm_count_launch();
-  return 0;
-}
-
-template <int NS>
-int lub_trsm_ns(const LubCtx& x, int r0, int nb, double2* B, int ncols, double2* out) {
-  const size_t sm = (size_t)32 * 32 * NS * sizeof(double2);
-  if (wsbm_smem_optin((const void*)k_lub_trsm<NS>, sm) != cudaSuccess) return -3;
-  const int cols = std::min(4, (ncols + wsbm_sm_count() - 1) / wsbm_sm_count());
-  k_lub_trsm<NS><<<(ncols + cols - 1) / cols, 128, sm, x.st>>>(x.A, x.lda, r0, nb, B, x.lda, ncols, cols, out);
-  wsbm_count_launch();
-  return 0;
-}
-int lub_trsm(const LubCtx& x, int r0, int nb, double2* B, int ncols, double2* out) {
-  if (nb <= 32) return lub_trsm_ns<1>(x, r0, nb, B, ncols, out);
-  if (nb <= 64) return lub_trsm_ns<2>(x, r0, nb, B, ncols, out);
-  if (nb <= 128) return lub_trsm_ns<4>(x, r0, nb, B, ncols, out);
-  return lub_trsm_ns<8>(x, r0, nb, B, ncols, out);
-}
-
-// factor columns [c0, c1) of rows [c0, n); row swaps across the whole outer panel
-int lub_rec(const LubCtx& x, int c0, int c1, int base) {
-  const int w = c1 - c0;
-  if (w <= base) {
-    int rows = x.n - c0, nsm = std::min(wsbm_sm_count(), LUB_MAXCTA);
-    int R = std::max(LUB_MINROWS, (rows + nsm - 1) / nsm);
-    int G = (rows + R - 1) / R, width = w, c = c0;
-    size_t smem = (size_t)w * (R | 1) * sizeof(double2);
-    if (wsbm_smem_optin((const void*)k_lub_panel, LUB_SMEM) != cudaSuccess) return -3;
-    double2* A = x.A;
-    int64_t lda = x.lda;
-    int n = x.n;
-    unsigned long long* slots = x.slots + (size_t)(c0 - x.cs) * LUB_MAXCTA;
-    double2 *cand = x.cand, *diag = x.diag;
-    int *piv = x.piv, *info = x.info;
-    void* args[] = {&A, &lda, &n, &c, &width, &R, &slots, &cand, &diag, &piv, &info};
-    if (cudaLaunchCooperativeKernel((const void*)k_lub_panel, dim3(G), dim3(LUB_T), args, smem, x.st) != cudaSuccess)
-      return -3;
-    wsbm_count_launch();
-    return lub_swap(x, c0, w, x.cs, c0, c1, x.ce);
+// work space: the products' planes, then key slots, published rows and L11^-1 of each matrix
+constexpr size_t lub_slot_bytes = (size_t)LUB_NB_BIG * LUB_MAXCTA * sizeof(unsigned long long);
+constexpr size_t lub_cand_bytes = (size_t)2 * (LUB_MAXCTA + 1) * LUB_W * sizeof(double2);
+constexpr size_t lub_inv_bytes = (size_t)LUB_NB_BIG * LUB_NB_BIG * sizeof(double2);
+size_t lub_product_bytes(const LuDesc* h, int count) {
+  size_t b = wsbm_zgemm_tc_ws_bytes(h[0].n, h[0].n, LUB_NB_BIG);  // either panel width fits
+  if (count > 1) {
+    std::vector<TcProduct> p(count);
+    for (int i = 0; i < count; ++i) p[i] = {nullptr, 0, nullptr, 0, nullptr, 0, h[i].n, h[i].n, LUB_NB, 0};
+    b = std::max(b, wsbm_zgemm_tc_batched_ws_bytes(p.data(), count));
   }
-  const int mid = c0 + ((w / 2 + base - 1) / base) * base;
-  if (int rc = lub_rec(x, c0, mid, base)) return rc;
-  // A[c0:mid, mid:c1] = L11^-1 A[c0:mid, mid:c1];  A[mid:n, mid:c1] -= A[mid:n, c0:mid] A[c0:mid, mid:c1]
-  if (int rc = lub_trsm(x, c0, mid - c0, x.A + c0 + (int64_t)mid * x.lda, c1 - mid, nullptr)) return rc;
-  const double2 mone = make_double2(-1.0, 0.0), one = make_double2(1.0, 0.0);
-  if (int rc = wsbm_zgemm_tc(x.n - mid, c1 - mid, mid - c0, mone, x.A + mid + (int64_t)c0 * x.lda, x.lda,
-                             x.A + c0 + (int64_t)mid * x.lda, x.lda, one, x.A + mid + (int64_t)mid * x.lda, x.lda,
-                             x.tcws, x.tcb, x.st))
-    return rc;
-  return lub_rec(x, mid, c1, base);
+  return (b + 255) & ~(size_t)255;
 }
 
-// work space behind the products' planes: key slots, published rows, L11^-1
-size_t lub_layout(int n, size_t* o_slots, size_t* o_cand, size_t* o_inv) {
-  size_t b = (wsbm_zgemm_tc_ws_bytes(n, n, LUB_NB_BIG) + 255) & ~(size_t)255;  // either panel width fits
-  *o_slots = b;
-  b += (size_t)LUB_NB_BIG * LUB_MAXCTA * sizeof(unsigned long long);
-  *o_cand = b;
-  b += (size_t)2 * (LUB_MAXCTA + 1) * LUB_W * sizeof(double2);
-  *o_inv = b;
-  return b + (size_t)LUB_NB_BIG * LUB_NB_BIG * sizeof(double2) + 256;
+int lub_run(const LuDesc* h, int count, int* d_info, void* ws, cudaStream_t st, int nb) {
+  Lub x;
+  x.count = count;
+  x.nb = nb;
+  x.base = std::min(lub_base_width(h[0].n), nb);
+  x.st = st;
+  x.ws = ws;
+  x.wsb = lub_product_bytes(h, count);
+  char* slots = (char*)ws + x.wsb;
+  char* cand = slots + count * lub_slot_bytes;
+  char* inv = cand + count * lub_cand_bytes;
+  for (int i = 0; i < count; ++i) {
+    double2* c = (double2*)(cand + i * lub_cand_bytes);
+    x.q.it[i] = {h[i].A, h[i].lda, h[i].n, h[i].piv, d_info,
+                 (unsigned long long*)slots + (size_t)i * nb * LUB_MAXCTA,  // without a gap: one memset
+                 c, c + (size_t)2 * LUB_MAXCTA * LUB_W, (double2*)(inv + i * lub_inv_bytes)};
+  }
+  return x.factor();
 }
 }  // namespace
 
@@ -375,9 +490,37 @@ static int lub_nb(int n) {
   return n >= LUB_BIG_N ? t.root_nb_large : t.root_nb_mid;
 }
 
+size_t wsbm_lu_big_multi_ws_bytes(const LuDesc* h, int count) {
+  if (count <= 0 || h[0].n <= 0) return 256;
+  return lub_product_bytes(h, count) + count * (lub_slot_bytes + lub_cand_bytes + lub_inv_bytes) + 256;
+}
+
 size_t wsbm_lu_big_ws_bytes(int n) {
-  size_t a, b, c;
-  return lub_layout(n, &a, &b, &c);
+  const LuDesc d = {nullptr, n, nullptr, n, 0};
+  return wsbm_lu_big_multi_ws_bytes(&d, 1);
+}
+
+int wsbm_lu_big_multi_max(const LuDesc* h, int count) {
+  if (lub_nb(h[0].n) != LUB_NB) return 1;  // wide panels are worth their launches alone
+  const int nsm = std::min(wsbm_sm_count(), LUB_MAXCTA);
+  int64_t rows = 0;
+  int k = 0;
+  // rows a CTA has to hold of 32 columns when every matrix rounds up to whole CTAs
+  for (; k < std::min(count, LUB_MAXB); ++k) {
+    rows += h[k].n;
+    if (lub_nb(h[k].n) != LUB_NB) break;
+    if (k > 0 && (nsm <= k + 1 || ((rows + nsm - k - 2) / (nsm - k - 1) + 1) * LUB_W * (int64_t)sizeof(double2) > LUB_SMEM))
+      break;
+  }
+  return std::max(k, 1);
+}
+
+int wsbm_lu_big_multi(const LuDesc* h, int count, void* ws, cudaStream_t st) {
+  if (count <= 0) return 0;
+  if (!h || !ws || ((uintptr_t)ws & 255) || count > wsbm_lu_big_multi_max(h, count)) return -1;
+  for (int i = 0; i < count; ++i)
+    if (!h[i].A || !h[i].piv || h[i].n <= 0 || h[i].lda < h[i].n || (i && h[i].n > h[i - 1].n)) return -1;
+  return lub_run(h, count, nullptr, ws, st, lub_nb(h[0].n));
 }
 
 int wsbm_lu_big(double2* A, int64_t lda, int n, int* piv, int* d_info, void* ws, cudaStream_t st) {
@@ -388,45 +531,8 @@ int wsbm_lu_big_nb(double2* A, int64_t lda, int n, int* piv, int* d_info, void* 
   if (n <= 0) return 0;
   if (!A || !piv || !ws || lda < n || ((uintptr_t)ws & 255)) return -1;
   if (nb != LUB_NB && nb != LUB_NB_BIG) return -1;
-  size_t o_slots, o_cand, o_inv;
-  lub_layout(n, &o_slots, &o_cand, &o_inv);
-  double2* Linv = (double2*)((char*)ws + o_inv);
-  LubCtx x;
-  x.A = A;
-  x.lda = lda;
-  x.n = n;
-  x.piv = piv;
-  x.info = d_info;
-  x.slots = (unsigned long long*)((char*)ws + o_slots);
-  x.cand = (double2*)((char*)ws + o_cand);
-  x.diag = x.cand + (size_t)2 * LUB_MAXCTA * LUB_W;
-  x.st = st;
-  x.tcws = ws;
-  x.tcb = o_slots;
-  const int base = lub_base_width(n);
-  const double2 mone = make_double2(-1.0, 0.0), one = make_double2(1.0, 0.0), zero = make_double2(0.0, 0.0);
-  for (int j0 = 0; j0 < n; j0 += nb) {
-    const int jb = std::min(nb, n - j0), je = j0 + jb;
-    x.cs = j0;
-    x.ce = je;
-    if (cudaMemsetAsync(x.slots, 0, (size_t)jb * LUB_MAXCTA * sizeof(unsigned long long), st) != cudaSuccess)
-      return -3;
-    if (int rc = lub_rec(x, j0, je, base)) return rc;
-    lub_swap(x, j0, jb, 0, j0, je, n);
-    if (je < n) {
-      // U12 = L11^-1 A12 as a tensor-core product with the explicit inverse of the unit lower
-      // L11 (the digit planes of A12 are formed before A12 is overwritten)
-      const int m = n - je;
-      if (int rc = lub_trsm(x, j0, jb, nullptr, jb, Linv)) return rc;
-      if (int rc = wsbm_zgemm_tc(jb, m, jb, one, Linv, jb, A + j0 + (int64_t)je * lda, lda, zero,
-                                 A + j0 + (int64_t)je * lda, lda, ws, o_slots, st))
-        return rc;
-      if (int rc = wsbm_zgemm_tc(m, m, jb, mone, A + je + (int64_t)j0 * lda, lda, A + j0 + (int64_t)je * lda, lda,
-                                 one, A + je + (int64_t)je * lda, lda, ws, o_slots, st))
-        return rc;
-    }
-  }
-  return cudaGetLastError() == cudaSuccess ? 0 : -3;
+  const LuDesc d = {A, lda, piv, n, 0};
+  return lub_run(&d, 1, d_info, ws, st, nb);
 }
 
 // Error flags of the bounded waits of the panel and of its products: reads and clears both
