@@ -34,16 +34,16 @@ UNIT = "entries/s"
 # for the kernel sources with the recorded hash; when the sources change the traffic figure is
 # withheld until re-measured.
 KERNEL_COUNTS = {
-    "src_sha": "6fec8f827c2ae62f",
+    "src_sha": "4086c37b777a63d5",
     # 16384-node star, leaf level (bench.py --profile-case), tiles of 16 x 8 node pairs (the
     # autotuned shape; the proxy kernel's per-pair count includes its proxy-point set-up, which
     # depends on the tile width): 4.16 M / 4.24 M pairs
-    "k_proxy": {"tf": 16, "fp64_flops_per_pair": 81.8, "dram_bytes_per_pair": 50.2},
+    "k_proxy": {"tf": 16, "fp64_flops_per_pair": 81.8, "dram_bytes_per_pair": 50.3},
     "k_pairs": {"tf": 16, "fp64_flops_per_pair": 100.5, "dram_bytes_per_pair": 50.3},
     # DRAM traffic of the column-pivoted QR per ID matrix of this workload, keyed by the hash of
     # its dense.cu section and the matrix rows it was measured on (1024 sketches of 128 rows,
     # 65536-node star)
-    "k_cpqr": {"src_sha": "efa00c1011a862ff", "rows": 128, "dram_bytes_per_matrix": 6.30e7},
+    "k_cpqr": {"src_sha": "b05a64a619ed1265", "rows": 128, "dram_bytes_per_matrix": 6.46e7},
     # DRAM traffic of the two fused LU + solve launches of a leaf level (box LU with D^-1 L of
     # 256 unknowns, and Dhat), per factored matrix: 25.71 GB over the 1024 matrices of the
     # 512 leaf boxes of the same star at N = 65536 (boxes of the same size and ranks)
