@@ -81,43 +81,39 @@ __global__ void __launch_bounds__(FLD_THREADS)
   if (t < nt) part[(int64_t)blockIdx.y * nt + t] = make_double2(acc, mag);
 }
 
-// side[t] = 1 inside, 0 outside
+// side[t] = 1 inside, 0 outside: a warp per target, so that targets summed again in FP64 spread over the GPU
+// (500 targets on the nodes of a curve of 500: a CTA per 128 targets took as long as the field itself).
 __global__ void __launch_bounds__(FLD_THREADS)
     k_field_side_finish(DevGeom g, const double* __restrict__ tx, const double* __restrict__ ty, int64_t nt,
                         int nsplit, const double2* __restrict__ part, int8_t* __restrict__ side) {
-  __shared__ double red[FLD_THREADS];
-  __shared__ int unsure[FLD_THREADS];
-  const int64_t t0 = (int64_t)blockIdx.x * FLD_THREADS, t = t0 + threadIdx.x;
+  const int lane = threadIdx.x & 31;
+  const int64_t t = (int64_t)blockIdx.x * (FLD_THREADS / 32) + (threadIdx.x >> 5);
+  if (t >= nt) return;
+  auto sum = [](double v) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xFFFFFFFFu, v, o);
+    return v;
+  };
   double acc = 0.0, mag = 0.0;
-  if (t < nt)
-    for (int p = 0; p < nsplit; ++p) {
-      const double2 v = part[(int64_t)p * nt + t];
-      acc += v.x;
-      mag += v.y;
-    }
+  for (int p = lane; p < nsplit; p += 32) {
+    const double2 v = part[(int64_t)p * nt + t];
+    acc += v.x;
+    mag += v.y;
+  }
+  acc = sum(acc);
+  mag = sum(mag);
   const double off = fabs(acc + WSBM_PI);  // 2 pi |sum - 1/2|
-  const bool sure = off > (double)FLD_SIDE_EPS * mag;  // false for an infinite or NaN mag
-  unsure[threadIdx.x] = t < nt && !sure;
-  if (t < nt && sure) side[t] = (-acc / (2.0 * WSBM_PI)) > 0.5 ? 1 : 0;
-  __syncthreads();
-  for (int q = 0; q < FLD_THREADS; ++q) {
-    if (!unsure[q]) continue;
-    const double px = tx[t0 + q], py = ty[t0 + q];
-    double s = 0.0;
-    for (int64_t j = threadIdx.x; j < g.n; j += FLD_THREADS) {
+  if (!(off > (double)FLD_SIDE_EPS * mag)) {  // also an infinite or NaN mag
+    const double px = tx[t], py = ty[t];
+    acc = 0.0;
+    for (int64_t j = lane; j < g.n; j += 32) {
       const double dx = px - g.x[j], dy = py - g.y[j];
       const double r2 = dx * dx + dy * dy;
-      if (r2 > 0.0) s += g.w[j] * (dx * g.nx[j] + dy * g.ny[j]) / r2;
+      if (r2 > 0.0) acc += g.w[j] * (dx * g.nx[j] + dy * g.ny[j]) / r2;
     }
-    red[threadIdx.x] = s;
-    __syncthreads();
-    for (int h = FLD_THREADS / 2; h > 0; h >>= 1) {
-      if (threadIdx.x < h) red[threadIdx.x] += red[threadIdx.x + h];
-      __syncthreads();
-    }
-    if (threadIdx.x == 0) side[t0 + q] = (-red[0] / (2.0 * WSBM_PI)) > 0.5 ? 1 : 0;
-    __syncthreads();
+    acc = sum(acc);
   }
+  if (lane == 0) side[t] = (-acc / (2.0 * WSBM_PI)) > 0.5 ? 1 : 0;
 }
 
 // Partial sums over the sources [j0, j1) of CTA row blockIdx.y, for the nc <= NR right-hand sides
@@ -263,7 +259,7 @@ extern "C" int wsbm_field(const wsbm_geom* g, const wsbm_params* p, const void* 
   DevGeom dg = wsbm_devgeom(g);
   const dim3 grid((unsigned)nti, (unsigned)nsplit);
   k_field_side<<<grid, FLD_THREADS, 0, st>>>(dg, tx, ty, nt, jspan, part);
-  k_field_side_finish<<<(unsigned)nti, FLD_THREADS, 0, st>>>(dg, tx, ty, nt, (int)nsplit, part, inside);
+  k_field_side_finish<<<(unsigned)((nt + FLD_THREADS / 32 - 1) / (FLD_THREADS / 32)), FLD_THREADS, 0, st>>>(dg, tx, ty, nt, (int)nsplit, part, inside);
   wsbm_count_launches(2);
   const double2 *cu = (const double2*)u, *cq = (const double2*)q;
   for (int c0 = 0; c0 < nrhs; c0 += nr) {
