@@ -70,6 +70,7 @@ __global__ void __launch_bounds__(MV_THREADS)
       }
     }
     __syncthreads();
+    const unsigned mask = __ballot_sync(0xFFFFFFFFu, valid);
     if (!valid) continue;
     const int nj = (int)min((int64_t)MV_THREADS, j1 - jc);
 #pragma unroll 1
@@ -78,12 +79,22 @@ __global__ void __launch_bounds__(MV_THREADS)
       asm volatile("" ::: "memory");
       const MvSlot<NR>& s = sj[jj];
       double2 e[2][2];
-      if (jc + jj == i) {
+      // block (i, j): row node i, column node j; TRANS: block (j, i), applied transposed.  A warp with pairs
+      // out of the fixed-point range takes the general path for all of its pairs: half the way through both
+      // would cost more (64 nodes, 15 a wavelength: 983 us, now 870; 2000 nodes: 1766, 1637)
+      const bool diag = jc + jj == i;
+      const double sx = TRANS ? s.x : xi, sy = TRANS ? s.y : yi, tx = TRANS ? xi : s.x, ty = TRANS ? yi : s.y;
+      const double snx = TRANS ? s.nx : nxi, sny = TRANS ? s.ny : nyi, tnx = TRANS ? nxi : s.nx, tny = TRANS ? nyi : s.ny;
+      const double w = TRANS ? wi : s.w, dx = __dsub_rn(sx, tx), dy = __dsub_rn(sy, ty), r2 = pair_r2(dx, dy);
+      const bool fixed = __all_sync(mask, diag || pair_is_fixed(ph, r2));
+      if (diag) {
         block_diag(ph, wi, ki, e);
-      } else if (!TRANS) {  // block (i, j): row node i, column node j
-        pair_block(T, ph, xi, yi, nxi, nyi, s.x, s.y, s.nx, s.ny, s.w, e);
-      } else {  // block (j, i), applied transposed
-        pair_block(T, ph, s.x, s.y, s.nx, s.ny, xi, yi, nxi, nyi, wi, e);
+      } else if (fixed) {
+        block_fixed(T, ph, dx, dy, r2, snx, sny, tnx, tny, w, e);
+      } else {
+        PairGeom G;
+        pair_geom(sx, sy, snx, sny, tx, ty, tnx, tny, ph, G);
+        block_offdiag(T, ph, G, w, e);
       }
       if (TRANS) {
         double2 t = e[0][1];
