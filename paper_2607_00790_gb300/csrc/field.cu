@@ -120,7 +120,7 @@ __global__ void __launch_bounds__(FLD_THREADS)
 // starting at column c0.  part: nsplit x nt x NR complex128.  Bound by the FP64 pipe: 31 operations
 // a pair (Hankel values in fixed point, one reciprocal square root each for 1/r and the amplitude,
 // the side's signs and constants folded into two factors) and 8 per right-hand side.  16384 nodes, 3001
-// targets, 8 columns: 8.4 ms (25 ms in two launches of 4 columns with FP64 Hankel values).
+// targets, 8 columns: 8.5 ms (25 ms in two launches of 4 columns with FP64 Hankel values).
 template <int NR>
 __global__ void __launch_bounds__(FLD_THREADS)
     k_field(DevGeom g, Phys ph, const double2* __restrict__ u, const double2* __restrict__ q, int nc, int c0,

@@ -933,15 +933,16 @@ static int upload_instances(wsbm_hss* h0, const std::vector<wsbm_hss*>& hs, Inst
 // Compress and factor one tree level of each item (a curve and its level): every phase is one
 // launch over all boxes of all items (entries, proxy blocks, IDs, LU, D^-1 L, Dhat).  All
 // handles share one stream.  Candidates (cr, cc) of every box must be set.
-// Algorithmic flops of the fused LU + solve of an n x n matrix with nrhs right-hand sides:
-// multipliers (one complex multiply, 6 flops) and trailing updates (one complex FMA, 8 flops) of
-// the LU, the forward and backward substitutions, and the pivot scalings of the back solve.
+// How many of them the thread-per-column QR takes.
 static int small_qrs(const std::vector<QrDesc>& q) {
   int n = 0;
   for (const QrDesc& d : q) n += d.m <= wsbm_cpqr_tpc_rows();
   return n;
 }
 
+// Algorithmic flops of the fused LU + solve of an n x n matrix with nrhs right-hand sides:
+// multipliers (one complex multiply, 6 flops) and trailing updates (one complex FMA, 8 flops) of
+// the LU, the forward and backward substitutions, and the pivot scalings of the back solve.
 static double lu_solve_flops(double n, double nrhs) {
   const double a = n * (n - 1) / 2, b = (n - 1) * n * (2 * n - 1) / 6;
   return 6 * a + 8 * b + 16 * a * nrhs + 6 * n * nrhs;
