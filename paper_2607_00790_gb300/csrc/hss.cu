@@ -930,10 +930,7 @@ static int upload_instances(wsbm_hss* h0, const std::vector<wsbm_hss*>& hs, Inst
   return upload(h0, p, &ia->phys, tmp);
 }
 
-// Compress and factor one tree level of each item (a curve and its level): every phase is one
-// launch over all boxes of all items (entries, proxy blocks, IDs, LU, D^-1 L, Dhat).  All
-// handles share one stream.  Candidates (cr, cc) of every box must be set.
-// How many of them the thread-per-column QR takes.
+// How many of the matrices the thread-per-column QR takes.
 static int small_qrs(const std::vector<QrDesc>& q) {
   int n = 0;
   for (const QrDesc& d : q) n += d.m <= wsbm_cpqr_tpc_rows();
@@ -948,6 +945,9 @@ static double lu_solve_flops(double n, double nrhs) {
   return 6 * a + 8 * b + 16 * a * nrhs + 6 * n * nrhs;
 }
 
+// Compress and factor one tree level of each item (a curve and its level): every phase is one
+// launch over all boxes of all items (entries, proxy blocks, IDs, LU, D^-1 L, Dhat).  All
+// handles share one stream.  Candidates (cr, cc) of every box must be set.
 static int factor_levels(const std::vector<wsbm_hss*>& hs, const std::vector<int>& levels,
                          double ms_out[5], int64_t* cpqr_mats, double* cpqr_flops,
                          int64_t sketch_out[2], double* sketch_ms, double lu_out[4]) {
